@@ -312,6 +312,31 @@ def test_revived_vertices_do_not_keep_old_in_edges(B):
     B.summarize_destroy(ctx)
 
 
+@pytest.mark.parametrize("length", [31, 513, 16385])
+def test_rows_pointing_at_many_revived_vertices_are_purged_once(B, length):
+    # rows of every scan tier hold several entries into each of many vertices
+    # that die and come back: in one batch, and dead for a batch in between
+    rng = np.random.default_rng(length)
+    n = 400
+    back = rng.permutation(np.arange(8, n))[:150]
+    src = np.concatenate([np.zeros(length, np.int64), rng.integers(1, 8, 900), rng.integers(8, n, 300)]).astype(np.int32)
+    dst = rng.integers(0, n, len(src)).astype(np.int32)
+    lab = rng.integers(0, 3, len(src)).astype(np.int32)
+    vl = rng.integers(0, 2, n).astype(np.int32)
+    state = dict(n=n, alive=np.ones(n, np.uint8), vlabel=vl, src=src, dst=dst, elabel=lab)
+    ctx = B.summarize_init_coo(n, _dev(src), _dev(dst), _dev(lab), _dev(vl), options=B.default_options(k_incremental=2))
+    B.apply_updates(ctx, _dev(np.zeros((0, 4), np.int32)))
+    kill = [[3, v, 0, 0] for v in back]
+    add = [[2, v, 0, int(vl[v])] for v in back]
+    edges = [[0, int(u), int(w), 1] for u, w in zip(rng.integers(0, 8, 60), rng.choice(back, 60))]
+    for ops in (kill, add + edges, kill[:70] + add[:70] + edges[:30], kill + add):
+        ops = np.array(ops, np.int32)
+        state = oracle.apply_ops(state, ops)
+        B.apply_updates(ctx, _dev(ops))
+        check_partition(B, ctx, state, 2)
+    B.summarize_destroy(ctx)
+
+
 def test_vertex_joining_a_singleton_block_one_level_down(B):
     """Vertices alone in their block one level down are not re-hashed; when another
     vertex later joins that block, the singleton must be compared again (here u is
