@@ -76,6 +76,23 @@ def test_powerlaw_scaled_spans_every_bucket(B):
     assert stats["n_hub"] > 0 and stats["n_mid"] > 0 and stats["n_small"] > 0
 
 
+@pytest.mark.parametrize("m", [1, 2047, 2048, 2049, 152 * 7 * 2048 + 1])
+def test_unsorted_list_tiles(B, m):
+    # sizes around a tile of the unsorted build and past one pass of its grid;
+    # a third of the edges leave vertex 0, and the highest vertex has some
+    rng = np.random.default_rng(m)
+    n = max(2, m // 9)
+    src = rng.integers(0, n, m).astype(np.int32)
+    src[rng.random(m) < 0.33] = 0
+    src[0] = n - 1
+    src[m // 2:m // 2 + 70] = n // 2                      # a run inside the disorder
+    dst = rng.integers(0, n, m).astype(np.int32)
+    lab = rng.integers(0, 2, m).astype(np.int32)
+    vl = rng.integers(0, 2, n).astype(np.int32)
+    g = dict(n=n, src=src, dst=dst, elabel=lab, vlabel=vl)
+    check(B, g, (2,))
+
+
 @pytest.mark.parametrize("order", ["sorted", "shuffled", "descending", "one_swap"])
 def test_edge_list_order_does_not_matter(B, order):
     # a list sorted by source takes the run-based placement, any other the
