@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "prof.cuh"
+#include "rounds.cuh"
 
 namespace bisim {
 
@@ -394,31 +395,42 @@ bisim_status dense_rounds_begin(bisim_ctx* ctx, cudaStream_t s, const uint8_t* k
 // consecutive rounds prove the fixpoint, since every round refines the
 // previous partition.
 bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int64_t prev,
-                              int32_t* out_rounds, int32_t* out_executed, int64_t* out_blocks, bool allow_graph) {
+                              int32_t* out_rounds, int32_t* out_executed, int64_t* out_blocks, bool allow_graph,
+                              bool allow_loop, bool from_p0) {
     cudaError_t e;
     const bool fixpoint = k == BISIM_FIXPOINT;
     const int32_t limit = fixpoint ? cap : k;
     int32_t rounds = limit, executed = 0;
     bool done = limit <= 0;
-    if (!done && allow_graph && dense_graph_usable(ctx)) {
-        // the round loop on the device: one graph launch
+    // on the device as far as it goes: one round of the kernels of every class and
+    // the cooperative loop, then (while rows above 256 edges stay listed) the
+    // captured graph; a hash collision ends either one's last round here
+    const bool device_loop = round_loop_usable(ctx);
+    bool collided = false;
+    for (int part = 0; part < 2 && !done && !collided && device_loop; ++part) {
+        if (part == 0 ? !allow_loop : !allow_graph) continue;
         GraphRounds g{};
-        bisim_status st = dense_graph_rounds(ctx, s, limit, fixpoint, prev, &g);
+        bisim_status st = part == 0 ? dense_round_then_loop(ctx, s, limit, fixpoint, prev, from_p0, &g)
+                                    : dense_graph_rounds(ctx, s, limit - executed, fixpoint, prev, &g);
         if (st != BISIM_OK) return st;
-        executed = g.executed;
-        if (g.stop == 1) {
-            rounds = g.rounds;
+        const int32_t before = executed;
+        executed += g.executed;
+        if (g.stop == kStopDone) {
+            rounds = fixpoint ? before + g.rounds : limit;
             prev = g.blocks;
             done = true;
+        } else if (g.stop == kStopWideRows) {
+            prev = g.blocks;
         } else {
             // the last round met a hash collision (or an error): finish it here
             int64_t blocks = 0;
             if ((st = dense_finish_round(ctx, s, &blocks)) != BISIM_OK) return st;
-            if (blocks == prev) {
+            if (blocks == g.prev) {
                 rounds = fixpoint ? executed - 1 : k;
                 done = true;
             }
             prev = blocks;
+            collided = true;
         }
     }
     for (int32_t i = executed; !done && i < limit; ++i) {
@@ -444,16 +456,41 @@ bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
     return BISIM_OK;
 }
 
+// The cooperative loop takes the first round too when it covers every row and
+// the graph has at most this many vertices: above it the first round's list is
+// long enough to fill the kernels of the single classes, which keep twice the
+// warps resident.
+constexpr int64_t kLoopStartMax = int64_t{1} << 20;
+
+bisim_status dense_rounds_all(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
+                              int32_t* out_executed, int64_t* out_blocks, bool allow_graph) {
+    bisim_status st;
+    int64_t prev = 0, dropped = 0;
+    const int32_t limit = k == BISIM_FIXPOINT ? cap : k;
+    if ((st = dense_prepare(ctx, s)) != BISIM_OK) return st;
+    const bool from_p0 = limit > 0 && round_loop_usable(ctx) && round_loop_covers(ctx) &&
+                         ctx->dbegin[kDClasses] <= kLoopStartMax;
+    if (from_p0) {
+        if (ctx->opt.mem_budget_bytes > 0 && ctx->device_bytes > ctx->opt.mem_budget_bytes)
+            return set_error(ctx, BISIM_ENOMEM, "context exceeds the memory budget");
+        dense_mark_dead(ctx, s);
+        ctx->cur = 0;
+        prev = ctx->last_blocks;
+    } else if ((st = dense_rounds_begin(ctx, s, nullptr, &prev, &dropped)) != BISIM_OK) {
+        return st;
+    }
+    return dense_rounds_run(ctx, k, cap, s, prev, out_rounds, out_executed, out_blocks, allow_graph, true, from_p0);
+}
+
 // Resets to P_0 and refines (see dense_rounds_run); batched contexts go to
 // segment_rounds.
 bisim_status run_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
                         int32_t* out_executed, int64_t* out_blocks, bool allow_graph) {
     if (segment_usable(ctx)) return segment_rounds(ctx, k, cap, s, out_rounds, out_executed, out_blocks);
-    int64_t prev = 0, dropped = 0;
-    bisim_status st = dense_rounds_begin(ctx, s, nullptr, &prev, &dropped);
-    if (st != BISIM_OK) return st;
+    int64_t prev = 0;
     int32_t rounds = 0, executed = 0;
-    if ((st = dense_rounds_run(ctx, k, cap, s, prev, &rounds, &executed, &prev, allow_graph)) != BISIM_OK) return st;
+    bisim_status st;
+    if ((st = dense_rounds_all(ctx, k, cap, s, &rounds, &executed, &prev, allow_graph)) != BISIM_OK) return st;
     ctx->cur_k = rounds;
     ctx->stats.rounds = rounds;
     ctx->stats.rounds_executed = executed;

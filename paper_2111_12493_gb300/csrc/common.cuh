@@ -516,8 +516,9 @@ bisim_status apply_ops_to_store(bisim_ctx* ctx, const bisim_op* d_ops, int64_t n
 
 // ----------------------------------------------------------------------------- rounds (api.cu)
 
-// allow_graph: the loop may run as the captured graph (callers that rebuild the
-// layout for every call, like the full recompute of an update batch, pass false).
+// allow_graph: rounds that the cooperative loop does not take may run as the
+// captured graph (callers that rebuild the layout for every call, like the full
+// recompute of an update batch, pass false).
 bisim_status run_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
                         int32_t* out_executed, int64_t* out_blocks, bool allow_graph = true);
 // The two halves of the dense path of run_rounds: reset to P_0 and list the
@@ -526,8 +527,14 @@ bisim_status run_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, 
 // out_dropped the live vertices left out (counted as blocks by the rounds).
 bisim_status dense_rounds_begin(bisim_ctx* ctx, cudaStream_t s, const uint8_t* keep_graph, int64_t* out_prev,
                                 int64_t* out_dropped);
+// allow_loop: the cooperative loop may run (it wants every SM to itself);
+// from_p0: dense_rounds_begin was left out because that loop starts from P_0.
 bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int64_t prev,
-                              int32_t* out_rounds, int32_t* out_executed, int64_t* out_blocks, bool allow_graph);
+                              int32_t* out_rounds, int32_t* out_executed, int64_t* out_blocks, bool allow_graph,
+                              bool allow_loop = false, bool from_p0 = false);
+// Both halves over every live vertex, by the route the graph's rows allow.
+bisim_status dense_rounds_all(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
+                              int32_t* out_executed, int64_t* out_blocks, bool allow_graph);
 bisim_status refresh_after_edit(bisim_ctx* ctx, cudaStream_t s);
 
 // ----------------------------------------------------------------------------- dense rounds (dense.cu)
@@ -577,10 +584,15 @@ struct GraphRounds {
     int32_t executed;     // rounds run on the device
     int32_t rounds;       // r when stop == 1
     int64_t blocks;       // block count after the last round
-    int32_t stop;         // 1 done, 2 the last round needs its collision levels, 3 device error
+    int64_t prev;         // block count before it
+    int32_t stop;         // kStop* (rounds.cuh): 1 done, 2 the last round needs its collision levels, 3 device error
 };
-// Whether the rounds may run as the captured device-side loop.
-bool dense_graph_usable(const bisim_ctx* ctx);
+// One round through the kernels of every class, then the cooperative loop
+// (rounds.cu) for as long as no row above 256 edges is listed; with from_p0 the
+// cooperative loop alone, from P_0. One synchronisation. out->stop is
+// kStopWideRows when the loop left the rest of the rounds.
+bisim_status dense_round_then_loop(bisim_ctx* ctx, cudaStream_t s, int32_t limit, bool fixpoint, int64_t prev_blocks,
+                                   bool from_p0, GraphRounds* out);
 // Runs up to `limit` rounds from P[0] as one graph launch (the loop checks the
 // block count on the device); the result is in P[0] unless stop == 2.
 bisim_status dense_graph_rounds(bisim_ctx* ctx, cudaStream_t s, int32_t limit, bool fixpoint, int64_t prev_blocks,

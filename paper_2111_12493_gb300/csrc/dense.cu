@@ -34,6 +34,7 @@
 
 #include "common.cuh"
 #include "prof.cuh"
+#include "rounds.cuh"
 
 namespace bisim {
 
@@ -1290,39 +1291,16 @@ __global__ void __launch_bounds__(kThreads) k_dense_compare_cta(const int2* __re
 
 // ----------------------------------------------------------------------------- device-side round loop
 
-// State of the round loop run by the captured graph (device memory).
-struct LoopState {
-    unsigned long long prev_blocks;   // block count of the partition the next round refines
-    unsigned long long blocks;        // block count after the last round
-    int32_t executed;                 // rounds run
-    int32_t limit;                    // rounds allowed
-    int32_t fixpoint;                 // 1: stop as soon as a round keeps the block count
-    int32_t rounds;                   // the result r (k, or the fixpoint round)
-    int32_t stop;                     // 0 go on, 1 done, 2 a hash collision to resolve on the host, 3 error
-    int32_t pad;
-};
-
 // After a round: decide whether the loop goes on (the while condition of the graph).
 __global__ void k_round_check(const DevState* __restrict__ st, LoopState* L, cudaGraphConditionalHandle cond) {
-    const unsigned long long blocks = st->blocks;
-    const int32_t executed = L->executed + 1;
-    int32_t stop = 0;
-    if (st->error != 0u) {
-        stop = 3;
-    } else if (st->unresolved != 0u) {
-        stop = 2;                     // the host finishes this round's collision levels
-    } else if (blocks == L->prev_blocks) {
-        stop = 1;                     // P_{i+1} refines P_i with as many blocks: the fixpoint
-        L->rounds = L->fixpoint ? executed - 1 : L->limit;
-    } else if (executed >= L->limit) {
-        stop = 1;
-        L->rounds = L->limit;
-    }
-    if (stop < 2) L->prev_blocks = blocks;
-    L->blocks = blocks;
-    L->executed = executed;
-    L->stop = stop;
-    cudaGraphSetConditional(cond, stop == 0 ? 1u : 0u);
+    loop_advance(*L, st->blocks, st->unresolved, st->error);
+    cudaGraphSetConditional(cond, L->stop == kStopNo ? 1u : 0u);
+}
+
+// The same after a round launched outside the graph, which starts from `init`.
+__global__ void k_round_settle(const DevState* __restrict__ st, LoopState* L, LoopState init) {
+    loop_advance(init, st->blocks, st->unresolved, st->error);
+    *L = init;
 }
 
 // Start of a captured round: the table is blanked when the epoch of this
@@ -2084,17 +2062,14 @@ TableRef fixed_table(const bisim_ctx* ctx) {
 // renumbering over the active list), the loop check, and the end of the round
 // (P_{i+1} of the listed vertices copied into the input buffer, the list
 // compacted). The body reads P[0] and writes P[1].
-bisim_status build_round_graph(bisim_ctx* ctx) {
+bisim_status build_round_graph(bisim_ctx* ctx, cudaStream_t s) {
     set_attributes();
     cudaError_t e;
     if (ctx->capture_stream == nullptr &&
         (e = cudaStreamCreateWithFlags(reinterpret_cast<cudaStream_t*>(&ctx->capture_stream), cudaStreamNonBlocking)))
         return cuda_error(ctx, e, "create capture stream");
-    if (ctx->dloop == nullptr) {
-        if ((e = ctx_alloc(ctx, &ctx->dloop, sizeof(LoopState), nullptr))) return cuda_error(ctx, e, "alloc loop state");
-        static_assert(sizeof(LoopState) <= 256, "pinned blocks hold 256 bytes");
-        if ((ctx->hloop = pinned_take()) == nullptr) return set_error(ctx, BISIM_ENOMEM, "pinned loop state mirror");
-    }
+    bisim_status st;
+    if ((st = round_loop_state(ctx, s)) != BISIM_OK) return st;
     cudaStream_t cs = static_cast<cudaStream_t>(ctx->capture_stream);
     cudaGraph_t g = nullptr;
     if ((e = cudaGraphCreate(&g, 0))) return cuda_error(ctx, e, "create round graph");
@@ -2160,15 +2135,40 @@ bisim_status build_round_graph(bisim_ctx* ctx) {
 
 }  // namespace
 
-bool dense_graph_usable(const bisim_ctx* ctx) {
-    return ctx->dense_ready && ctx->n > 0 && !prof_enabled() &&
-           !(ctx->opt.flags & (BISIM_FLAG_EAGER | BISIM_FLAG_L2_PIN));
+bisim_status dense_round_then_loop(bisim_ctx* ctx, cudaStream_t s, int32_t limit, bool fixpoint, int64_t prev_blocks,
+                                   bool from_p0, GraphRounds* out) {
+    LoopState init{};
+    init.prev_blocks = static_cast<unsigned long long>(prev_blocks);
+    init.limit = limit;
+    init.fixpoint = fixpoint ? 1 : 0;
+    init.rounds = limit;
+    bisim_status st;
+    set_attributes();                          // a collision's levels on the host need them too
+    if (!from_p0) {
+        if ((st = round_loop_state(ctx, s)) != BISIM_OK) return st;
+        launch_round(ctx, s, level_table(ctx, s));
+        LoopState* L = static_cast<LoopState*>(ctx->dloop);
+        BISIM_SITE(site_ck, "round_check");
+        {
+            Launch Lk(site_ck, s, 0, 0, 0.0);
+            k_round_settle<<<1, 1, 0, s>>>(ctx->dstate, L, init);
+        }
+        launch_round_end(ctx, s, dense_view(ctx), &L->stop);
+    }
+    LoopState r;
+    if ((st = round_loop(ctx, s, from_p0, init, class_counts(ctx), &r)) != BISIM_OK) return st;
+    out->executed = r.executed;
+    out->rounds = r.rounds;
+    out->blocks = static_cast<int64_t>(r.blocks);
+    out->prev = static_cast<int64_t>(r.prev_blocks);
+    out->stop = r.stop;
+    return BISIM_OK;
 }
 
 bisim_status dense_graph_rounds(bisim_ctx* ctx, cudaStream_t s, int32_t limit, bool fixpoint, int64_t prev_blocks,
                                 GraphRounds* out) {
     bisim_status st;
-    if (ctx->round_graph == nullptr && (st = build_round_graph(ctx)) != BISIM_OK) return st;
+    if (ctx->round_graph == nullptr && (st = build_round_graph(ctx, s)) != BISIM_OK) return st;
     LoopState* h = static_cast<LoopState*>(ctx->hloop);
     std::memset(h, 0, sizeof(*h));
     h->prev_blocks = static_cast<unsigned long long>(prev_blocks);
@@ -2187,6 +2187,7 @@ bisim_status dense_graph_rounds(bisim_ctx* ctx, cudaStream_t s, int32_t limit, b
     out->executed = h->executed;
     out->rounds = h->rounds;
     out->blocks = static_cast<int64_t>(h->blocks);
+    out->prev = static_cast<int64_t>(h->prev_blocks);
     out->stop = h->stop;
     return BISIM_OK;
 }

@@ -1,0 +1,65 @@
+// The device-side round loop: its state, shared by the cooperative kernel
+// (rounds.cu) and the captured graph (dense.cu).
+#pragma once
+
+#include "common.cuh"
+
+namespace bisim {
+
+// Why a loop of rounds ended on the device.
+enum : int32_t {
+    kStopNo = 0,
+    kStopDone = 1,
+    kStopCollision = 2,     // the last round's hash collisions are left to the host
+    kStopError = 3,         // error bits in the status word
+    kStopWideRows = 4,      // cooperative kernel: rows above 256 edges are listed; nothing was done
+    kStopLost = 5,          // cooperative kernel: no result came back
+};
+
+// State of a run of rounds (device memory, and its pinned mirror).
+struct LoopState {
+    unsigned long long prev_blocks;   // block count of the partition the next round refines
+    unsigned long long blocks;        // block count after the last round
+    int32_t executed;                 // rounds run
+    int32_t limit;                    // rounds allowed
+    int32_t fixpoint;                 // 1: stop as soon as a round keeps the block count
+    int32_t rounds;                   // the result r (k, or the fixpoint round)
+    int32_t stop;                     // kStop*
+    int32_t epoch;                    // cooperative kernel: the table epoch of its last round
+};
+
+// The state after a round that ended with `blocks` blocks and the given
+// unresolved positions and error bits.
+__host__ __device__ inline void loop_advance(LoopState& L, unsigned long long blocks, unsigned unresolved,
+                                             unsigned error) {
+    L.executed += 1;
+    if (error != 0u) {
+        L.stop = kStopError;
+    } else if (unresolved != 0u) {
+        L.stop = kStopCollision;
+    } else if (blocks == L.prev_blocks) {     // P_{i+1} refines P_i with as many blocks: the fixpoint
+        L.stop = kStopDone;
+        L.rounds = L.fixpoint ? L.executed - 1 : L.limit;
+    } else if (L.executed >= L.limit) {
+        L.stop = kStopDone;
+        L.rounds = L.limit;
+    }
+    if (L.stop < kStopCollision) L.prev_blocks = blocks;
+    L.blocks = blocks;
+}
+
+// Whether runs of rounds may go through the cooperative kernel at all.
+bool round_loop_usable(const bisim_ctx* ctx);
+// Whether it covers the whole graph (no live vertex above 256 edges).
+bool round_loop_covers(const bisim_ctx* ctx);
+// Allocates the loop state and its mirror.
+bisim_status round_loop_state(bisim_ctx* ctx, cudaStream_t s);
+// Runs the loop: from P_0 with every live vertex listed (start; `init` is the
+// state to begin with), or from the current list and the loop state in device
+// memory. The result is in P[0] unless out->stop is kStopCollision or
+// kStopError: then the last round stands as the host-driven levels expect it.
+// `ccount`: the list's per-class survivor counters. Synchronises s.
+bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopState& init, unsigned long long* ccount,
+                        LoopState* out);
+
+}  // namespace bisim

@@ -700,11 +700,9 @@ bisim_status segment_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t
     const bool any_big = n_small < ctx->n_graphs;
     if (any_big && (n_small == 0 || limit <= 0)) {
         // every graph above the split: the union's round kernels alone
-        int64_t prev = 0, dropped = 0, blocks = 0;
+        int64_t blocks = 0;
         int32_t rounds = 0, executed = 0;
-        if ((st = dense_rounds_begin(ctx, s, nullptr, &prev, &dropped)) != BISIM_OK ||
-            (st = dense_rounds_run(ctx, k, cap, s, prev, &rounds, &executed, &blocks, true)) != BISIM_OK)
-            return st;
+        if ((st = dense_rounds_all(ctx, k, cap, s, &rounds, &executed, &blocks, true)) != BISIM_OK) return st;
         ctx->cur_k = rounds;
         ctx->stats.rounds = rounds;
         ctx->stats.rounds_executed = executed;

@@ -1,0 +1,114 @@
+"""The cooperative round loop at the edges of what it takes: row lengths around
+its groups, list lengths around a CTA and the grid, the epoch cycle of the table,
+hash collisions that hand a round back to the host, and rows it leaves to the
+kernels of the wide classes. Partitions and rounds equal the oracle's."""
+
+import numpy as np
+import pytest
+
+import oracle
+from test_gpu_parity import B, check  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def rows_graph(n, degree, seed, copies=3, n_labels=2):
+    """n vertices of out-degree `degree` - 1, `degree` or `degree` + 1; groups of `copies` vertices share a row (in
+    another order, one entry doubled), so that many pairs need the exact comparison."""
+    rng = np.random.default_rng(seed)
+    src, dst, lab = [], [], []
+    for v0 in range(0, n, copies):
+        d = max(0, degree + int(rng.integers(-1, 2)))
+        t, l = rng.integers(0, n, d), rng.integers(0, n_labels, d)
+        for v in range(v0, min(n, v0 + copies)):
+            o = rng.permutation(d)
+            if d > 1 and v % 2:
+                o[0] = o[1]                                # a repeated entry in place of one: another set
+            src.append(np.full(d, v)); dst.append(t[o]); lab.append(l[o])
+    cat = lambda a: np.concatenate(a).astype(np.int32) if a else np.zeros(0, np.int32)  # noqa: E731
+    return dict(n=n, src=cat(src), dst=cat(dst), elabel=cat(lab), vlabel=rng.integers(0, 2, n).astype(np.int32))
+
+
+def path_graph(lengths, marked=()):
+    n = int(sum(lengths))
+    ends = np.cumsum(lengths) - 1
+    v = np.setdiff1d(np.arange(n), ends)
+    vl = np.zeros(n, np.int32)
+    vl[list(marked)] = 1
+    return dict(n=n, src=v.astype(np.int32), dst=(v + 1).astype(np.int32), elabel=np.zeros(len(v), np.int32), vlabel=vl)
+
+
+@pytest.mark.parametrize("n", [1, 33, 1024, 1025, 6000])
+@pytest.mark.parametrize("degree", [1, 8, 16, 32])
+def test_row_lengths_of_every_group(B, n, degree):
+    check(B, rows_graph(n, degree, seed=n + degree), [1, 2, oracle.FIXPOINT])
+
+
+@pytest.mark.parametrize("degree", [64, 200, 255])
+def test_rows_of_the_warp_classes(B, degree):
+    check(B, rows_graph(2100, degree, seed=degree), [2, oracle.FIXPOINT])
+
+
+@pytest.mark.parametrize("k", [1, 2, 14, 15, 16, 31])
+def test_rounds_around_the_epoch_cycle(B, k):
+    check(B, path_graph([40] * 30 + [7, 1, 90], marked=(3, 600)), [k])
+
+
+@pytest.mark.parametrize("bits", [3, 9, 16])
+@pytest.mark.parametrize("n,degree", [(300, 3), (3000, 9), (3000, 40)])
+def test_collisions_hand_the_round_back(B, bits, n, degree):
+    check(B, rows_graph(n, degree, seed=bits), [1, 3, oracle.FIXPOINT], options=B.default_options(hash_bits=bits))
+
+
+def test_collisions_in_a_late_round(B):
+    # few blocks at first, so the narrow hash collides only rounds later
+    g = path_graph([60] * 200, marked=(5, 4000, 7001))
+    check(B, g, [oracle.FIXPOINT], options=B.default_options(hash_bits=13))
+
+
+def test_a_popular_signature_over_many_ctas(B):
+    # 200k vertices with one signature in round 1 (a hot table slot), dead vertices among them
+    n = 200_000
+    rng = np.random.default_rng(4)
+    alive = np.ones(n, np.uint8)
+    alive[rng.integers(100, n, 500)] = 0
+    src = np.flatnonzero(alive[:-1] & (np.arange(n - 1) % 7 != 0)).astype(np.int32)
+    g = dict(n=n, src=src, dst=rng.integers(0, 100, len(src)).astype(np.int32), elabel=np.zeros(len(src), np.int32),
+             vlabel=np.zeros(n, np.int32))
+    check(B, g, [1, oracle.FIXPOINT], alive=alive)
+
+
+@pytest.mark.parametrize("wide", [257, 9000])
+def test_wide_rows_that_stay_listed_leave_the_loop(B, wide):
+    # twins with equal rows are never alone: a wide pair keeps every round in the kernels of its class
+    rng = np.random.default_rng(wide)
+    base = path_graph([30] * 500)
+    n = base["n"]
+    t = rng.integers(0, n, wide)
+    src = np.concatenate([base["src"], np.full(wide, 2), np.full(wide, 32)]).astype(np.int32)
+    dst = np.concatenate([base["dst"], t, t[::-1]]).astype(np.int32)
+    g = dict(base, src=src, dst=dst, elabel=np.zeros(len(src), np.int32))
+    check(B, g, [1, 5, oracle.FIXPOINT])
+
+
+def test_wide_rows_that_become_alone_enter_the_loop(B):
+    rng = np.random.default_rng(8)
+    base = path_graph([30] * 500)
+    n = base["n"]
+    src = np.concatenate([base["src"], np.full(700, 2), np.full(10_000, 32)]).astype(np.int32)
+    dst = np.concatenate([base["dst"], rng.integers(0, n, 10_700)]).astype(np.int32)
+    g = dict(base, src=src, dst=dst, elabel=np.zeros(len(src), np.int32))
+    check(B, g, [1, 2, 17, oracle.FIXPOINT])
+
+
+def test_resident_context_alternates_routes(B):
+    # the same context by the loop, host-driven, and again: nothing of one run leaks into the next
+    g = path_graph([25] * 300, marked=(11,))
+    dev = [__import__("torch").from_numpy(g[k]).cuda() for k in ("src", "dst", "elabel", "vlabel")]
+    ctx = B.summarize_init_coo(g["n"], *dev)
+    for k in (3, oracle.FIXPOINT, 0, 40, 1, oracle.FIXPOINT):
+        rounds, blocks = B.bisim_iterate(ctx, k, 10_000)
+        want, wr, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], k, 10_000)
+        assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want) and rounds == wr
+        assert blocks == len(np.unique(want))
+    B.summarize_destroy(ctx)
