@@ -152,12 +152,13 @@ __device__ __forceinline__ uint32_t table_insert_at(const TableRef& t, uint64_t 
             }
             if ((cur & kSlotKeyMask) == tag) {                  // same fingerprint: keep the smaller vertex
                 // popular signatures are inserted by many vertices; the plain
-                // read above skips the atomic when a smaller one is recorded
-                while (static_cast<uint32_t>(v) < static_cast<uint32_t>(cur)) {
-                    const unsigned long long prev = atomicCAS(&t.slots[pos].w, cur, want);
-                    if (prev == cur) break;
-                    cur = prev;
-                }
+                // read above skips the atomic when a smaller one is recorded.
+                // A slot keeps its tag for the rest of the epoch, so the
+                // smaller word is the smaller vertex, and a minimum without a
+                // result does it: nothing waits and nothing is tried again (a
+                // compare-and-swap loop lost to the slot's other vertices took
+                // most of a round with blocks of 500 members, 39 us of 77)
+                if (static_cast<uint32_t>(v) < static_cast<uint32_t>(cur)) atomicMin(&t.slots[pos].w, want);
                 return static_cast<uint32_t>(pos);
             }
             break;                                               // another signature: probe on
@@ -343,6 +344,7 @@ struct bisim_ctx {
     void* copy_events[4] = {nullptr, nullptr, nullptr, nullptr};   // buffers ready; sources, targets, labels copied
     void* dloop = nullptr;                           // loop state on the device
     void* hloop = nullptr;                           // its pinned host mirror
+    int32_t loop_copy = 0;                           // cooperative loop: which copy of its counters the next launch uses
     int64_t round_graph_launches = 0;                // kernels in one captured round
 
     // batched contexts: the persistent per-graph kernel (segment.cu)

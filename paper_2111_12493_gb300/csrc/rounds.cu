@@ -4,19 +4,29 @@
 // What it replaces is a loop of about a dozen kernels a round. Each of those is
 // near empty once the list is short (a late round of a power-law graph) or the
 // graph is small, and a round then costs its launches: 77 us on 300k vertices in
-// paths, 60 us on 10k vertices. Here a round is two phases with a grid barrier
-// after each, one CTA of 1024 threads per SM (fewer on small graphs, and no
-// barrier but the CTA's own when one CTA holds them all):
-//   A  of the previous round's list, the entries that are not alone in their
-//      block go on the new list; each computes its signature and enters the table
-//   B  every entry of the new list is confirmed against its slot's smallest
-//      vertex by an exact comparison, inside the thread for rows of at most
-//      eight edges, in the warp for longer ones
+// paths, 60 us on 10k vertices. Here a round is two or three phases with a grid
+// barrier after each, one CTA per SM (on small graphs one cluster, or one CTA):
+//   A  the entries of the list that are not alone in their block compute their
+//      signatures
+//   B  every entry is confirmed by an exact comparison, inside the thread for
+//      rows of at most eight edges, in the warp for longer ones: in a round that
+//      splits most blocks against the smallest vertex of its slot of the
+//      signature table (which phase A filled), else against the smallest vertex
+//      of its present block; those that differ from it enter the table
+//   C  (only then, and only them) and are confirmed against their slots
+//
+// The list is cut among the CTAs at the start and each keeps its part to the end
+// (dealt in units of up to 32 entries, rotated from row to row so that no period
+// of the graph lands on one CTA), so that no list position is handed out by an
+// atomic and no entry waits for one: thousands of warps on one address are what
+// bounded the phases with a shared list. A barrier carries the CTAs' counts, so
+// every CTA knows the totals and takes the same decision: another round, done, or
+// back to the host at a hash collision (with the state the host-driven levels
+// expect).
+//
 // The two partition buffers alternate as input and output; a vertex that leaves
 // the list writes its final block into the other one, so both agree on every
-// vertex that is not listed. After B all CTAs read the same counts and take the
-// same decision: another round, done, or back to the host at a hash collision
-// (with the state the host-driven levels expect).
+// vertex that is not listed.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -30,28 +40,44 @@ namespace bisim {
 
 namespace {
 
-constexpr int kLoopThreads = 1024;
+constexpr int kLoopThreads = 1024;        // at most; 512 for short lists
 constexpr int kLoopWarps = kLoopThreads / 32;
 constexpr int kLoopGroups = 4;            // degree <= 8, <= 16, <= 32, <= 256: classes 0-4, 5, 6, 7-9
 constexpr int kHotSlots = 64;
+constexpr int kSeenSlots = 1024;
 constexpr int kLoopWarpSet = 512;         // slots of a warp's set: twice the longest row
 constexpr unsigned kSpinLimit = 1u << 22; // polls of a barrier before the kernel gives up (seconds)
+constexpr int kUnits = 4;                 // work units a warp takes between two flushes of the CTA
+constexpr int kStage = kUnits * 32;
+constexpr uint8_t kCold = 255;
+
+// Values of an entry's `own` flag. 1 with joined = 0: alone in its block.
+constexpr uint8_t kMember = 0;            // not its block's smallest vertex
+constexpr uint8_t kOwner = 1;             // the smallest vertex; joined says whether others are in the block
+constexpr uint8_t kOwnerLeft = 3;         // ... and some left since: joined may be out of date
+constexpr uint8_t kOwnerAsks = 5;         // ... and this round those that stay set it anew
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Counters of one round; three of them rotate, so that one can be cleared
-// while the others are read.
-struct RoundSet {
-    unsigned long long blocks;            // listed vertices that are their block's id
-    unsigned cnt[kLoopGroups];            // entries of the round's list per group
+// What one barrier carries: the CTAs' listed (high half) and owned entries
+// added up, and the union of their kAny* flags.
+struct __align__(16) BarrierSum {
+    unsigned long long counts;
+    unsigned long long flags;
+};
+
+// What a launch leaves behind is cleared by the next one, which uses the other copy.
+struct LoopCopy {
+    BarrierSum sum[3];                          // of barrier k: sum[k % 3]
+    unsigned arrived;                           // barrier arrivals since the launch
+    unsigned gcount[kLoopGroups];               // list entries per group, when the list goes back to the host
+    unsigned gcursor[kLoopGroups];
     unsigned unresolved;
     unsigned error;
 };
 
 struct LoopCtl {
-    RoundSet set[3];
-    unsigned arrived;                     // barrier arrivals since the launch
-    unsigned left;                        // CTAs that returned
+    LoopCopy copy[2];
     unsigned abort;                       // a barrier gave up
 };
 
@@ -76,6 +102,7 @@ struct LoopView {
     uint64_t nslots;
     uint32_t epoch;                       // the table's last epoch (kEpochCycle: blank it first)
     int32_t* unresolved;
+    int32_t* split;                       // entries that left their block's smallest vertex this round
     DevState* st;
     LoopCtl* ctl;
     LoopState* L;
@@ -83,22 +110,39 @@ struct LoopView {
     int64_t gb[kLoopGroups + 1];          // first position of each group
     int64_t n_live;
     int32_t n;
+    int32_t copy;                         // which LoopCopy this launch uses
+    int32_t cluster;                      // the grid is one cluster
     int32_t start;                        // 1: from P_0 with every live position listed; 0: from act[0] / aoff and *L
     LoopState init;                       // start: the loop state to begin with
 };
 
+struct Shared {
+    unsigned long long hot_key[kHotSlots];
+    unsigned hot_min[kHotSlots];
+    uint32_t hot_slot[kHotSlots];
+    int32_t stage_pos[kLoopWarps][kStage];    // the warp's short rows that stay listed
+    uint8_t stage_hot[kLoopWarps][kStage];    // their hot slot, or kCold (already in the table)
+    unsigned wcnt[kLoopWarps];
+    unsigned wbase[kLoopWarps];
+    unsigned zero[kLoopWarps];
+    int32_t seen[kSeenSlots];                 // positions whose joined flag this CTA has set this round
+    unsigned next_cnt[kLoopGroups];           // entries of the next list so far
+    unsigned split;                           // entries of the split list so far
+    unsigned owned;                           // entries that are their block's id
+    unsigned error;                           // kErr* bits
+    unsigned flags;                           // barrier result: kAny* of all CTAs
+    unsigned total[2];                        // barrier result: listed, owned
+    int ok;
+};
+
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 
-__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Pair value of a packed word over the labelling P, which other CTAs write
-// between barriers: read through L2.
+// Pair value of a packed word. Arrays that one phase writes and a later one
+// reads (partitions, signatures, flags, slots, lists) are read with plain loads:
+// every barrier's acquire makes the SM's L1 forget them, and within a phase L1
+// serves what all vertices of a large block read.
 __device__ __forceinline__ uint64_t word_value(unsigned long long w, const int32_t* P) {
-    return pair_value(static_cast<int32_t>(w >> 32), __ldcg(P + static_cast<uint32_t>(w)));
+    return pair_value(static_cast<int32_t>(w >> 32), P[static_cast<uint32_t>(w)]);
 }
 
 // Sum and number of the distinct values among the lanes that have one (every lane gets both).
@@ -113,52 +157,142 @@ __device__ __forceinline__ void distinct_of_warp(uint64_t val, bool has, uint64_
     *cnt = static_cast<unsigned>(__popc(__ballot_sync(0xffffffffu, first)));
 }
 
-struct Shared {
-    unsigned long long hot_key[2][kHotSlots];
-    unsigned hot_min[2][kHotSlots];
-    uint32_t hot_slot[kHotSlots];
-    unsigned wcnt[kLoopWarps];
-    unsigned wbase[kLoopWarps];
-    unsigned long long wsum[kLoopWarps];
-    unsigned zero[kLoopWarps];
-    int ok;
-};
+// ----------------------------------------------------------------------------- barrier
 
-// Grid barrier number `k` (from 1) of this launch; false when it gave up.
-__device__ bool grid_barrier(LoopCtl* c, unsigned k, Shared& sh) {
-    __syncthreads();
-    if (gridDim.x == 1) return true;
+constexpr unsigned kAnySplit = 1u, kAnyUnresolved = 2u, kAnyError = 4u;
+
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void add_release(unsigned* p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Grid barrier number `k` (from 1) of this launch; false when it gave up. One
+// counter and one poller per CTA: 2.9k cycles for 152 CTAs with stores in
+// flight, against 7k to 9k when every CTA reads a word of every other, 4.2k with
+// one CTA collecting and 3.1k of the runtime's grid sync. A grid that is one
+// cluster uses the cluster's barrier.
+__device__ bool arrive_and_wait(const LoopView& V, unsigned k, Shared& sh) {
+    LoopCopy* c = &V.ctl->copy[V.copy];
+    if (V.cluster) {
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+        return true;
+    }
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
+    }
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&c->arrived, 1u);
+        sh.ok = 1;
+        add_release(&c->arrived, 1u);
         const unsigned target = gridDim.x * k;
         unsigned spin = 0;
-        bool ok = true;
         while (load_acquire(&c->arrived) < target) {
-            if (++spin > kSpinLimit || load_acquire(&c->abort) != 0u) {
-                atomicExch(&c->abort, 1u);
-                ok = false;
+            if (++spin > kSpinLimit || ((spin & 255u) == 0u && load_acquire(&V.ctl->abort) != 0u)) {
+                atomicExch(&V.ctl->abort, 1u);
+                sh.ok = 0;
                 break;
             }
         }
-        __threadfence();
-        sh.ok = ok ? 1 : 0;
     }
     __syncthreads();
     return sh.ok != 0;
 }
 
-// The current list: group g's entries are base[g][0 .. cnt[g]), or (identity)
-// the positions from first[g] on.
+__device__ bool grid_barrier(const LoopView& V, unsigned k, Shared& sh) {
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) V.ctl->copy[V.copy].sum[(k + 1) % 3] = BarrierSum{0ull, 0ull};
+    return arrive_and_wait(V, k, sh);
+}
+
+// The same with the sum of all CTAs' counts and the union of their flags, in
+// sh.total and sh.flags. Three sums rotate: that of barrier k + 1 is cleared
+// before anyone leaves barrier k, and was last read before anyone reached k - 1.
+__device__ bool grid_barrier(const LoopView& V, unsigned k, unsigned flags, unsigned listed, unsigned owned,
+                             Shared& sh) {
+    LoopCopy* c = &V.ctl->copy[V.copy];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (blockIdx.x == 0) c->sum[(k + 1) % 3] = BarrierSum{0ull, 0ull};
+        atomicAdd(&c->sum[k % 3].counts, (static_cast<unsigned long long>(listed) << 32) | owned);
+        if (flags) atomicOr(&c->sum[k % 3].flags, static_cast<unsigned long long>(flags));
+    }
+    const bool fine = arrive_and_wait(V, k, sh);
+    if (threadIdx.x == 0) {
+        const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2*>(&c->sum[k % 3]));
+        sh.total[0] = static_cast<unsigned>(t.x >> 32);
+        sh.total[1] = static_cast<unsigned>(t.x);
+        sh.flags = static_cast<unsigned>(t.y);
+    }
+    __syncthreads();
+    return fine;
+}
+
+// ----------------------------------------------------------------------------- list
+
+// The CTA's part of the list. Group g was dealt at the start in units of
+// 1 << shift[g] entries, a row of one unit per CTA at a time; entry j of this
+// CTA's part sits where its j-th dealt entry sat, in `buf` (null: the list is
+// every position in order) from base[g] on.
 struct List {
-    const int32_t* base[kLoopGroups];
-    int64_t cnt[kLoopGroups];
-    bool identity;
+    const int32_t* buf;
+    int64_t base[kLoopGroups];
+    unsigned cnt[kLoopGroups];            // entries of this CTA
+    unsigned shift[kLoopGroups];
 };
 
-__device__ __forceinline__ int32_t list_at(const LoopView& V, const List& l, int g, int64_t i) {
-    return l.identity ? static_cast<int32_t>(V.gb[g] + i) : __ldcg(l.base[g] + i);
+__device__ __forceinline__ int64_t dealt(const List& l, int g, unsigned j) {
+    const unsigned row = j >> l.shift[g];
+    const unsigned turn = (blockIdx.x + row * 61u) % gridDim.x;
+    return ((static_cast<int64_t>(row) * gridDim.x + turn) << l.shift[g]) + (j & ((1u << l.shift[g]) - 1u));
 }
+
+// How many of `count` entries are dealt to this CTA.
+__device__ __forceinline__ unsigned dealt_count(int64_t count, unsigned shift) {
+    const int64_t units = (count + (1 << shift) - 1) >> shift;
+    if (units == 0) return 0u;
+    const int64_t rows = (units + gridDim.x - 1) / gridDim.x;
+    const unsigned turn = (blockIdx.x + static_cast<unsigned>(rows - 1) * 61u) % gridDim.x;
+    const int64_t u = (rows - 1) * gridDim.x + turn;               // this CTA's unit of the last row
+    const int64_t last = u >= units ? 0 : min(static_cast<int64_t>(1) << shift, count - (u << shift));
+    return static_cast<unsigned>(((rows - 1) << shift) + last);
+}
+
+__device__ __forceinline__ int32_t list_at(const List& l, int g, unsigned j) {
+    const int64_t at = l.base[g] + dealt(l, g, j);
+    return l.buf ? l.buf[at] : static_cast<int32_t>(at);
+}
+
+// Entry i of the CTA's groups in turn: its place among all entries.
+__device__ __forceinline__ int64_t place_of(const List& l, unsigned i, int* group, unsigned* j) {
+    int g = 0;
+#pragma unroll
+    for (int q = 0; q < kLoopGroups - 1; ++q) {
+        if (g == q && i >= l.cnt[q]) {
+            i -= l.cnt[q];
+            g = q + 1;
+        }
+    }
+    *group = g;
+    *j = i;
+    return dealt(l, g, i);
+}
+
+__device__ __forceinline__ unsigned list_size(const List& l) { return l.cnt[0] + l.cnt[1] + l.cnt[2] + l.cnt[3]; }
+
+__device__ __forceinline__ int32_t entry_of(const List& l, unsigned i) {
+    int g;
+    unsigned j;
+    const int64_t place = place_of(l, i, &g, &j);
+    const int64_t at = l.base[g] + place;
+    return l.buf ? l.buf[at] : static_cast<int32_t>(at);
+}
+
+// ----------------------------------------------------------------------------- table
 
 // Table insert of the lanes with `on`. Lanes of one hash (and region) enter as
 // one, by their smallest vertex: every vertex of a popular signature would
@@ -188,6 +322,16 @@ __device__ __forceinline__ int combine(bool on, uint64_t h, int64_t base, int32_
     return rep;
 }
 
+// Table insert of the warp's lanes with `on`; returns the lane's slot.
+__device__ __forceinline__ uint32_t insert_warp(const TableRef& tt, bool on, uint64_t h, int64_t base, uint64_t mask,
+                                                int32_t v, unsigned* err) {
+    unsigned members;
+    const int rep = combine(on, h, base, v, &members);
+    uint32_t sl = ~0u;
+    if (on && rep == static_cast<int>(lane_id())) sl = table_insert_in(tt, h, v, static_cast<uint64_t>(base), mask, err);
+    return __shfl_sync(0xffffffffu, sl, rep);
+}
+
 __device__ __forceinline__ void table_span(const LoopView& V, int32_t v, int64_t* base, uint64_t* mask) {
     *base = 0;
     *mask = V.t.mask;
@@ -206,236 +350,291 @@ __device__ __forceinline__ void put_sig(const LoopView& V, int64_t pos, uint64_t
     V.sig[pos] = r;
 }
 
-// Does position `pos` go on the next list? Not when its vertex was its block's
-// id last round and no other joined it.
-__device__ __forceinline__ bool not_alone(const LoopView& V, int32_t pos) {
-    return !(__ldcg(V.own + pos) && !__ldcg(V.joined + pos));
-}
+// ----------------------------------------------------------------------------- phase A
 
-// Phase A, group 0: a thread per vertex.
-__device__ void phase_a_threads(const LoopView& V, const TableRef& tt, const List& l, bool first, const int32_t* Pin,
-                                int32_t* Pout, int32_t* next, RoundSet* rs, Shared& sh, int* parity) {
-    const int64_t count = l.cnt[0];
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kLoopThreads;
-    const int warp = static_cast<int>(threadIdx.x >> 5);
-    for (int64_t b = static_cast<int64_t>(blockIdx.x) * kLoopThreads; b < count; b += stride, *parity ^= 1) {
-        const int par = *parity;
-        const int64_t i = b + threadIdx.x;
-        bool stay = false;
-        int32_t pos = 0, v = 0;
-        uint64_t h = 0, mask = 0;
-        int64_t base = 0;
-        if (i < count) {
-            pos = list_at(V, l, 0, i);
-            stay = first || not_alone(V, pos);
-            v = __ldg(V.vert + pos);
-            const int32_t own = __ldcg(Pin + v);
-            if (!stay) {
-                Pout[v] = own;
-            } else {
-                const int64_t e0 = __ldg(V.prp + pos);
-                const int d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
-                uint64_t x[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] = j < d ? __ldcs(V.pe + e0 + j) : 0ull;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] = j < d ? word_value(x[j], Pin) : 0ull;
-                uint64_t sum = 0;
-                unsigned u = 0;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    bool fresh = j < d;
-#pragma unroll
-                    for (int q = 0; q < j; ++q) fresh = fresh && x[q] != x[j];
-                    if (fresh) {
-                        sum += x[j];
-                        ++u;
-                    }
-                }
-                const uint64_t hash = sig_hash(own, u, sum);
-                put_sig(V, pos, hash, u, own);
-                V.joined[pos] = 0;
-                h = hash & tt.hmask;
-                table_span(V, v, &base, &mask);
-            }
-        }
-        unsigned members;
-        const int rep = combine(stay, h, base, v, &members);
-        const bool doer = stay && rep == static_cast<int>(lane_id());
-        int hot = -1;
-        if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
-            // popular in the warp: combine over the CTA too
-            const int at = static_cast<int>((h ^ (h >> 29)) & (kHotSlots - 1));
-            const unsigned long long prev = atomicCAS(&sh.hot_key[par][at], 0ull, static_cast<unsigned long long>(h));
-            if (prev == 0ull || prev == h) {
-                atomicMin(&sh.hot_min[par][at], static_cast<unsigned>(v));
-                hot = at;
-            }
-        }
-        uint32_t sl = ~0u;
-        if (doer && hot < 0) sl = table_insert_in(tt, h, v, static_cast<uint64_t>(base), mask, &rs->error);
-        const unsigned stays = __ballot_sync(0xffffffffu, stay);
-        if (lane_id() == 0) sh.wcnt[warp] = static_cast<unsigned>(__popc(stays));
-        __syncthreads();
-        if (threadIdx.x < kHotSlots) {
-            const unsigned long long key = sh.hot_key[par][threadIdx.x];
-            if (key)
-                sh.hot_slot[threadIdx.x] = table_insert(tt, key, static_cast<int32_t>(sh.hot_min[par][threadIdx.x]),
-                                                        &rs->error);
-            sh.hot_key[par ^ 1][threadIdx.x] = 0ull;
-            sh.hot_min[par ^ 1][threadIdx.x] = ~0u;
-        } else if (warp == 2 && !first) {
-            const unsigned c = sh.wcnt[lane_id()];
-            unsigned inc = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane_id() >= static_cast<unsigned>(o)) inc += y;
-            }
-            unsigned at = 0;
-            if (lane_id() == 31 && inc) at = atomicAdd(&rs->cnt[0], inc);
-            at = __shfl_sync(0xffffffffu, at, 31);
-            sh.wbase[lane_id()] = at + inc - c;
-        }
-        __syncthreads();
-        if (hot >= 0) sl = sh.hot_slot[hot];
-        sl = __shfl_sync(0xffffffffu, sl, rep);
-        if (stay) {
-            V.slot[pos] = sl;
-            if (!first) next[V.gb[0] + sh.wbase[warp] + __popc(stays & ((1u << lane_id()) - 1u))] = pos;
-        }
+// What a round is: its first of the launch (every entry stays, the list is
+// kept as it is), and whether every entry enters the table.
+struct Round {
+    bool first, insert;
+    const int32_t* Pin;
+    int32_t* Pout;
+    int32_t* next;                        // buffer of the next list
+    TableRef t;
+};
+
+// Does the entry stay on the list? Not when its vertex is alone in its block.
+// An owner whose block lost members asks those that stay, once.
+__device__ __forceinline__ bool stays_listed(const LoopView& V, const Round& R, int32_t pos) {
+    if (R.first) return true;
+    const uint8_t o = V.own[pos];
+    if (o == kMember) return true;
+    if (o == kOwnerLeft) {
+        V.own[pos] = kOwnerAsks;
+        V.joined[pos] = 0;
+        return true;
     }
+    if (!V.joined[pos]) return false;
+    if (o == kOwnerAsks) V.own[pos] = kOwner;
+    return true;
 }
 
-// Phase A, groups 1 to 3: a warp takes up to 32 entries, one at a time with
-// all lanes (several at a time for rows of at most 32 edges, to keep their
-// loads in flight together); lane q keeps the result of entry q, and the lanes
-// finish all of them together. Few entries are spread over all warps.
-__device__ void phase_a_warps(const LoopView& V, const TableRef& tt, const List& l, int g, bool first,
-                              const int32_t* Pin, int32_t* Pout, int32_t* next, RoundSet* rs, Shared& sh,
-                              unsigned long long* sets) {
-    const int64_t count = l.cnt[g];
-    const int warp = static_cast<int>(threadIdx.x >> 5);
-    const unsigned lane = lane_id();
-    const int64_t warps = static_cast<int64_t>(gridDim.x) * kLoopWarps;
-    const int64_t per = min(static_cast<int64_t>(32), (count + warps - 1) / warps);
-    const int64_t gw = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x;      // neighbours on different SMs
-    for (int64_t b = gw * per; b < count; b += warps * per) {
-        bool stay = false;
-        int32_t pos = 0, v = 0, own = 0;
-        int64_t e0 = 0;
-        int d = 0;
-        if (lane < per && b + lane < count) {
-            pos = list_at(V, l, g, b + lane);
-            stay = first || not_alone(V, pos);
-            v = __ldg(V.vert + pos);
-            own = __ldcg(Pin + v);
-            if (!stay) {
-                Pout[v] = own;
-            } else {
-                e0 = __ldg(V.prp + pos);
-                d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
-            }
-        }
-        const unsigned stays = __ballot_sync(0xffffffffu, stay);
+// A unit of up to 32 short rows (group 0): a thread per vertex. The entries that
+// stay listed are staged in shared memory; the CTA's flush appends them to its
+// next list.
+__device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, const List& l, unsigned j0, Shared& sh,
+                                             int warp, int* staged) {
+    const unsigned j = j0 + lane_id();
+    const bool in = j < l.cnt[0];
+    bool stay = false;
+    int32_t pos = 0, v = 0, own = 0;
+    int64_t e0 = 0;
+    int d = 0;
+    if (in) {
+        pos = list_at(l, 0, j);
+        v = __ldg(V.vert + pos);
+        e0 = __ldg(V.prp + pos);
+        d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
+        stay = stays_listed(V, R, pos);
+        own = R.Pin[v];
+    }
+    // the list is grouped by degree, so the warp's longest row is mostly short:
+    // what lies beyond it is skipped by the warp as a whole
+    const int widest = static_cast<int>(__reduce_max_sync(0xffffffffu, stay ? static_cast<unsigned>(d) : 0u));
+    uint64_t h = 0, mask = 0;
+    int64_t base = 0;
+    if (in && !stay) R.Pout[v] = own;
+    if (stay) {
+        uint64_t x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = q < d ? __ldcs(V.pe + e0 + q) : 0ull;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < widest) x[q] = q < d ? word_value(x[q], R.Pin) : 0ull;
         uint64_t sum = 0;
-        unsigned cnt = 0;
-        if (g < 3) {
-            constexpr int kAtOnce = 4;
-            for (unsigned todo = stays; todo;) {
-                int q[kAtOnce];
-                uint64_t w[kAtOnce];
-                bool has[kAtOnce];
+        unsigned u = 0;
 #pragma unroll
-                for (int k = 0; k < kAtOnce; ++k) {
-                    q[k] = todo ? __ffs(todo) - 1 : -1;
-                    if (todo) todo &= todo - 1u;
-                    const int src = q[k] < 0 ? 0 : q[k];
-                    const int64_t e = __shfl_sync(0xffffffffu, e0, src);
-                    const int dd = __shfl_sync(0xffffffffu, d, src);
-                    has[k] = q[k] >= 0 && static_cast<int>(lane) < dd;
-                    w[k] = has[k] ? __ldcs(V.pe + e + lane) : 0ull;
-                }
+        for (int q = 0; q < 8; ++q) {
+            if (q >= widest) break;
+            bool fresh = q < d;
 #pragma unroll
-                for (int k = 0; k < kAtOnce; ++k)
-                    if (has[k]) w[k] = word_value(w[k], Pin);
-#pragma unroll
-                for (int k = 0; k < kAtOnce; ++k) {
-                    if (q[k] < 0) break;                           // the same for the whole warp
-                    uint64_t s;
-                    unsigned c;
-                    distinct_of_warp(w[k], has[k], &s, &c);
-                    if (static_cast<int>(lane) == q[k]) {
-                        sum = s;
-                        cnt = c;
-                    }
-                }
-            }
-        } else {
-            unsigned long long* tab = sets + warp * kLoopWarpSet;
-            for (unsigned todo = stays; todo; todo &= todo - 1u) {
-                const int q = __ffs(todo) - 1;
-                const int64_t e = __shfl_sync(0xffffffffu, e0, q);
-                const int dd = __shfl_sync(0xffffffffu, d, q);
-                uint64_t mv[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int j = k * 32 + static_cast<int>(lane);
-                    mv[k] = j < dd ? __ldcs(V.pe + e + j) : 0ull;
-                }
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (k * 32 + static_cast<int>(lane) < dd) mv[k] = word_value(mv[k], Pin);
-                uint32_t size = 64;
-                while (size < 2u * static_cast<uint32_t>(dd)) size <<= 1;
-                for (uint32_t j = lane; j < size; j += 32) tab[j] = 0ull;
-                if (lane == 0) sh.zero[warp] = 0u;
-                __syncwarp();
-                uint64_t s = 0;
-                unsigned c = 0;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    if (k * 32 >= dd) break;                       // the same for the whole warp
-                    const int j = k * 32 + static_cast<int>(lane);
-                    const bool fresh = j < dd && smem_set_insert(tab, size - 1, &sh.zero[warp], mv[k]);
-                    c += static_cast<unsigned>(__popc(__ballot_sync(0xffffffffu, fresh)));
-                    if (fresh) s += mv[k];
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (static_cast<int>(lane) == q) {
-                    sum = s;
-                    cnt = c;
-                }
-                __syncwarp();                                      // the set is cleared for the next row
+            for (int p = 0; p < q; ++p) fresh = fresh && x[p] != x[q];
+            if (fresh) {
+                sum += x[q];
+                ++u;
             }
         }
-        uint64_t h = 0, mask = 0;
-        int64_t base = 0;
+        const uint64_t hash = sig_hash(own, u, sum);
+        put_sig(V, pos, hash, u, own);
+        h = hash & R.t.hmask;
+    }
+    unsigned hot = kCold;
+    if (R.insert) {                                                // the same for the whole grid
         if (stay) {
-            const uint64_t hash = sig_hash(own, cnt, sum);
-            put_sig(V, pos, hash, cnt, own);
             V.joined[pos] = 0;
-            h = hash & tt.hmask;
             table_span(V, v, &base, &mask);
         }
         unsigned members;
         const int rep = combine(stay, h, base, v, &members);
-        uint32_t sl = ~0u;
-        if (stay && rep == static_cast<int>(lane))
-            sl = table_insert_in(tt, h, v, static_cast<uint64_t>(base), mask, &rs->error);
-        sl = __shfl_sync(0xffffffffu, sl, rep);
-        unsigned at = 0;
-        if (!first && stays) {
-            if (lane == 0) at = atomicAdd(&rs->cnt[g], static_cast<unsigned>(__popc(stays)));
-            at = __shfl_sync(0xffffffffu, at, 0);
+        const bool doer = stay && rep == static_cast<int>(lane_id());
+        if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
+            // popular in the warp: combine over the CTA too, at the flush
+            const unsigned at = static_cast<unsigned>(h ^ (h >> 29)) & (kHotSlots - 1);
+            const unsigned long long prev = atomicCAS(&sh.hot_key[at], 0ull, static_cast<unsigned long long>(h));
+            if (prev == 0ull || prev == h) {
+                atomicMin(&sh.hot_min[at], static_cast<unsigned>(v));
+                hot = at;
+            }
         }
+        uint32_t sl = ~0u;
+        if (doer && hot == kCold) sl = table_insert_in(R.t, h, v, static_cast<uint64_t>(base), mask, &sh.error);
+        sl = __shfl_sync(0xffffffffu, sl, rep);
+        hot = __shfl_sync(0xffffffffu, hot, rep);
+        if (stay && hot == kCold) V.slot[pos] = sl;
+    }
+    const unsigned stays = __ballot_sync(0xffffffffu, stay);
+    if (stay) {
+        const int at = *staged + __popc(stays & ((1u << lane_id()) - 1u));
+        sh.stage_pos[warp][at] = pos;
+        sh.stage_hot[warp][at] = static_cast<uint8_t>(hot);
+    }
+    *staged += __popc(stays);
+}
+
+// A unit of up to `per` rows of group g (9 to 256 edges): a warp per row, several
+// rows of at most 32 edges at a time to keep their loads in flight together.
+// Lane q keeps the result of row q, and the lanes finish all of them together.
+__device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, const List& l, int g, unsigned j0,
+                                           unsigned per, Shared& sh, int warp, unsigned long long* sets) {
+    const unsigned lane = lane_id();
+    const unsigned cnt_g = g == 3 ? l.cnt[3] : g == 2 ? l.cnt[2] : l.cnt[1];
+    bool stay = false;
+    int32_t pos = 0, v = 0, own = 0;
+    int64_t e0 = 0;
+    int d = 0;
+    if (lane < per && j0 + lane < cnt_g) {
+        pos = g == 3 ? list_at(l, 3, j0 + lane) : g == 2 ? list_at(l, 2, j0 + lane) : list_at(l, 1, j0 + lane);
+        v = __ldg(V.vert + pos);
+        e0 = __ldg(V.prp + pos);
+        d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
+        stay = stays_listed(V, R, pos);
+        own = R.Pin[v];
+        if (!stay) R.Pout[v] = own;
+    }
+    const unsigned stays = __ballot_sync(0xffffffffu, stay);
+    uint64_t sum = 0;
+    unsigned cnt = 0;
+    if (g < 3) {
+        constexpr int kAtOnce = 4;
+        for (unsigned todo = stays; todo;) {
+            int q[kAtOnce];
+            uint64_t w[kAtOnce];
+            bool has[kAtOnce];
+#pragma unroll
+            for (int k = 0; k < kAtOnce; ++k) {
+                q[k] = todo ? __ffs(todo) - 1 : -1;
+                if (todo) todo &= todo - 1u;
+                const int src = q[k] < 0 ? 0 : q[k];
+                const int64_t e = __shfl_sync(0xffffffffu, e0, src);
+                const int dd = __shfl_sync(0xffffffffu, d, src);
+                has[k] = q[k] >= 0 && static_cast<int>(lane) < dd;
+                w[k] = has[k] ? __ldcs(V.pe + e + lane) : 0ull;
+            }
+#pragma unroll
+            for (int k = 0; k < kAtOnce; ++k)
+                if (has[k]) w[k] = word_value(w[k], R.Pin);
+#pragma unroll
+            for (int k = 0; k < kAtOnce; ++k) {
+                if (q[k] < 0) break;                               // the same for the whole warp
+                uint64_t s;
+                unsigned c;
+                distinct_of_warp(w[k], has[k], &s, &c);
+                if (static_cast<int>(lane) == q[k]) {
+                    sum = s;
+                    cnt = c;
+                }
+            }
+        }
+    } else {
+        unsigned long long* tab = sets + warp * kLoopWarpSet;
+        for (unsigned todo = stays; todo; todo &= todo - 1u) {
+            const int q = __ffs(todo) - 1;
+            const int64_t e = __shfl_sync(0xffffffffu, e0, q);
+            const int dd = __shfl_sync(0xffffffffu, d, q);
+            uint64_t mv[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int j = k * 32 + static_cast<int>(lane);
+                mv[k] = j < dd ? __ldcs(V.pe + e + j) : 0ull;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k * 32 + static_cast<int>(lane) < dd) mv[k] = word_value(mv[k], R.Pin);
+            uint32_t size = 64;
+            while (size < 2u * static_cast<uint32_t>(dd)) size <<= 1;
+            for (uint32_t j = lane; j < size; j += 32) tab[j] = 0ull;
+            if (lane == 0) sh.zero[warp] = 0u;
+            __syncwarp();
+            uint64_t s = 0;
+            unsigned c = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k * 32 >= dd) break;                           // the same for the whole warp
+                const int j = k * 32 + static_cast<int>(lane);
+                const bool fresh = j < dd && smem_set_insert(tab, size - 1, &sh.zero[warp], mv[k]);
+                c += static_cast<unsigned>(__popc(__ballot_sync(0xffffffffu, fresh)));
+                if (fresh) s += mv[k];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (static_cast<int>(lane) == q) {
+                sum = s;
+                cnt = c;
+            }
+            __syncwarp();                                          // the set is cleared for the next row
+        }
+    }
+    uint64_t h = 0, mask = 0;
+    int64_t base = 0;
+    if (stay) {
+        const uint64_t hash = sig_hash(own, cnt, sum);
+        put_sig(V, pos, hash, cnt, own);
+        h = hash & R.t.hmask;
+    }
+    if (R.insert) {
         if (stay) {
-            V.slot[pos] = sl;
-            if (!first) next[V.gb[g] + at + __popc(stays & ((1u << lane) - 1u))] = pos;
+            V.joined[pos] = 0;
+            table_span(V, v, &base, &mask);
+        }
+        const uint32_t sl = insert_warp(R.t, stay, h, base, mask, v, &sh.error);
+        if (stay) V.slot[pos] = sl;
+    }
+    if (!R.first && stays) {
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&sh.next_cnt[g], static_cast<unsigned>(__popc(stays)));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(stays & ((1u << lane) - 1u));
+        if (stay) {
+            const int64_t to = g == 3 ? V.gb[3] + dealt(l, 3, at) : g == 2 ? V.gb[2] + dealt(l, 2, at) : V.gb[1] + dealt(l, 1, at);
+            R.next[to] = pos;
         }
     }
 }
+
+// Phase A over the CTA's part of the list. It is cut into units, one warp's
+// work: 32 short rows, or up to 32 longer ones (fewer when there are not enough
+// to go round). After every kUnits units the CTA enters its hot signatures, one
+// insert each, and appends its staged rows to its next list.
+__device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared& sh, unsigned long long* sets) {
+    const int warp = static_cast<int>(threadIdx.x >> 5);
+    const unsigned lane = lane_id();
+    const unsigned warps = blockDim.x / 32;
+    const unsigned per3 = max(1u, min(32u, l.cnt[3] / warps)), per2 = max(1u, min(32u, l.cnt[2] / warps)),
+                   per1 = max(1u, min(32u, l.cnt[1] / warps));
+    const unsigned end3 = (l.cnt[3] + per3 - 1) / per3, end2 = end3 + (l.cnt[2] + per2 - 1) / per2,
+                   end1 = end2 + (l.cnt[1] + per1 - 1) / per1, units = end1 + (l.cnt[0] + 31) / 32;
+    for (unsigned u0 = 0; u0 < units; u0 += warps * kUnits) {
+        int staged = 0;
+        for (int k = 0; k < kUnits; ++k) {
+            const unsigned u = u0 + k * warps + warp;
+            if (u >= units) break;                                 // the same for the whole warp
+            if (u >= end1) unit_threads(V, R, l, (u - end1) * 32, sh, warp, &staged);
+            else if (u < end3) unit_warps(V, R, l, 3, u * per3, per3, sh, warp, sets);
+            else if (u < end2) unit_warps(V, R, l, 2, (u - end3) * per2, per2, sh, warp, sets);
+            else unit_warps(V, R, l, 1, (u - end2) * per1, per1, sh, warp, sets);
+        }
+        if (lane == 0) sh.wcnt[warp] = static_cast<unsigned>(staged);
+        __syncthreads();
+        if (threadIdx.x < kHotSlots) {
+            const unsigned long long key = sh.hot_key[threadIdx.x];
+            if (key) {
+                sh.hot_slot[threadIdx.x] = table_insert(R.t, key, static_cast<int32_t>(sh.hot_min[threadIdx.x]), &sh.error);
+                sh.hot_key[threadIdx.x] = 0ull;
+                sh.hot_min[threadIdx.x] = ~0u;
+            }
+        } else if (warp == 2) {
+            const unsigned c = lane < warps ? sh.wcnt[lane] : 0u;
+            unsigned inc = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= static_cast<unsigned>(o)) inc += y;
+            }
+            const unsigned before = sh.next_cnt[0];
+            if (lane < warps) sh.wbase[lane] = before + inc - c;
+            __syncwarp();
+            if (lane == 31) sh.next_cnt[0] = before + inc;
+        }
+        __syncthreads();
+        for (int i = static_cast<int>(lane); i < staged; i += 32) {
+            const int32_t pos = sh.stage_pos[warp][i];
+            const unsigned hot = sh.stage_hot[warp][i];
+            if (hot != kCold) V.slot[pos] = sh.hot_slot[hot];
+            if (!R.first) R.next[V.gb[0] + dealt(l, 0, sh.wbase[warp] + i)] = pos;
+        }
+        if (u0 + warps * kUnits < units) __syncthreads();          // hot_slot and wcnt are written again
+    }
+}
+
+// ----------------------------------------------------------------------------- phases B and C
 
 // Is every pair value of row [ea, ea + da) among those of row [eb, eb + db)?
 // All lanes of the warp take part; at most 256 entries each.
@@ -459,261 +658,379 @@ __device__ bool row_inside(const LoopView& V, const int32_t* P, int64_t ea, int 
     return !miss;
 }
 
-// Phase B: every listed entry against its slot's representative.
-__device__ void phase_b(const LoopView& V, const List& l, const int32_t* Pin, int32_t* Pout, RoundSet* rs,
-                        Shared& sh) {
-    const int64_t c01 = l.cnt[0] + l.cnt[1], c012 = c01 + l.cnt[2], total = c012 + l.cnt[3];
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kLoopThreads;
+// One entry and the representative it is to be confirmed against.
+struct Pair {
+    int32_t pos, v, r, rpos;              // rpos < 0: nothing to confirm
+};
+
+__device__ __forceinline__ int4 record(const LoopView& V, int32_t pos) {
+    return *reinterpret_cast<const int4*>(V.sig + pos);            // hash low, hash high, |S|, own block
+}
+
+// The representative's joined flag, set once per CTA as far as a small filter
+// in shared memory remembers: the stores of a large block's vertices would queue
+// at one sector, and so would reads past L1 to see whether it is set (1M chains:
+// 35k cycles a round for this phase, against 100k and 60k). Threads that race in
+// the filter only store again.
+__device__ __forceinline__ void mark_joined(const LoopView& V, int32_t rpos, Shared& sh) {
+    volatile int32_t* seen = &sh.seen[rpos & (kSeenSlots - 1)];
+    if (*seen == rpos) return;
+    *seen = rpos;
+    V.joined[rpos] = 1;
+}
+
+// Confirms the lanes' pairs exactly: with `test`, the records a and c have
+// equal own blocks and sizes. Returns whether the entry joins the
+// representative's block; the others (and those with `push`) go on the unresolved list.
+__device__ __forceinline__ bool confirm(const LoopView& V, const Pair& p, bool test, bool push, const int4& a,
+                                        const int4& c, const Round& R) {
     const unsigned lane = lane_id();
-    unsigned long long owned = 0;
-    for (int64_t b = static_cast<int64_t>(blockIdx.x) * kLoopThreads + (threadIdx.x & ~31u); b < total; b += stride) {
-        const int64_t i = b + lane;
-        int32_t pos = -1, v = -1, r = -1, rpos = -1;
-        bool join = false, push = false, wide = false;
-        int64_t ev = 0, er = 0;
-        int dv = 0, dr = 0;
-        if (i < total) {
-            pos = i < l.cnt[0]  ? list_at(V, l, 0, i)
-                  : i < c01     ? list_at(V, l, 1, i - l.cnt[0])
-                  : i < c012    ? list_at(V, l, 2, i - c01)
-                                : list_at(V, l, 3, i - c012);
-            v = __ldg(V.vert + pos);
-            const uint32_t sv = __ldcg(V.slot + pos);
-            r = sv == ~0u ? -1 : static_cast<int32_t>(static_cast<uint32_t>(__ldcg(&V.t.slots[sv].w)));
-            if (r < 0 || r >= V.n) {                               // failed insert
-                atomicOr(&rs->error, kErrTableFull);
-                Pout[v] = -1;
-            } else if (r == v) {
-                Pout[v] = v;
-                V.own[pos] = 1;
-                ++owned;
-            } else {
-                rpos = __ldg(V.vpos + r);
-                V.own[pos] = 0;
-                const int4 a = __ldcg(reinterpret_cast<const int4*>(V.sig + pos));
-                const int4 c = __ldcg(reinterpret_cast<const int4*>(V.sig + rpos));
-                if (a.z != c.z || a.w != c.w) {                    // |S| or own block differ
-                    push = true;
-                } else if (a.z <= 1) {                             // the full hash decides (a bijection of the pair)
-                    join = a.x == c.x && a.y == c.y;
-                    push = !join;
-                } else {
-                    ev = __ldg(V.prp + pos);
-                    dv = static_cast<int>(__ldg(V.prp + pos + 1) - ev);
-                    er = __ldg(V.prp + rpos);
-                    dr = static_cast<int>(__ldg(V.prp + rpos + 1) - er);
-                    if (dv <= 8 && dr <= 8) {
-                        // S_v inside S_r with equal sizes means equal sets
-                        uint64_t x[8];
+    bool join = false, wide = false;
+    int64_t ev = 0, er = 0;
+    int dv = 0, dr = 0;
+    if (test && a.z <= 1) {                                        // the full hash decides (a bijection of the pair)
+        join = a.x == c.x && a.y == c.y;
+        push = !join;
+    } else if (test) {
+        ev = __ldg(V.prp + p.pos);
+        dv = static_cast<int>(__ldg(V.prp + p.pos + 1) - ev);
+        er = __ldg(V.prp + p.rpos);
+        dr = static_cast<int>(__ldg(V.prp + p.rpos + 1) - er);
+        if (dv <= 8 && dr <= 8) {
+            // S_v inside S_r with equal sizes means equal sets
+            uint64_t x[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) x[j] = j < dr ? __ldg(V.pe + er + j) : 0ull;
+            for (int j = 0; j < 8; ++j) x[j] = j < dr ? __ldg(V.pe + er + j) : 0ull;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) x[j] = j < dr ? word_value(x[j], Pin) : 0ull;
-                        bool all = true;
-                        for (int j = 0; j < dv; ++j) {
-                            const uint64_t y = word_value(__ldg(V.pe + ev + j), Pin);
-                            bool found = false;
+            for (int j = 0; j < 8; ++j) x[j] = j < dr ? word_value(x[j], R.Pin) : 0ull;
+            bool all = true;
+#pragma unroll 1
+            for (int j0 = 0; j0 < dv && all; j0 += 4) {            // four of v's values at a time in flight
+                uint64_t y[4];
 #pragma unroll
-                            for (int q = 0; q < 8; ++q) found = found || (q < dr && x[q] == y);
-                            all = all && found;
-                        }
-                        join = all;
-                        push = !all;
-                    } else {
-                        wide = true;
-                    }
+                for (int j = 0; j < 4; ++j) y[j] = j0 + j < dv ? __ldg(V.pe + ev + j0 + j) : 0ull;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j0 + j < dv) y[j] = word_value(y[j], R.Pin);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    bool found = j0 + j >= dv;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) found = found || (q < dr && x[q] == y[j]);
+                    all = all && found;
                 }
             }
-        }
-        for (unsigned todo = __ballot_sync(0xffffffffu, wide); todo; todo &= todo - 1u) {
-            const int q = __ffs(todo) - 1;
-            const bool same = row_inside(V, Pin, __shfl_sync(0xffffffffu, ev, q), __shfl_sync(0xffffffffu, dv, q),
-                                         __shfl_sync(0xffffffffu, er, q), __shfl_sync(0xffffffffu, dr, q));
-            if (static_cast<int>(lane) == q) {
-                join = same;
-                push = !same;
-            }
-        }
-        if (join) {
-            Pout[v] = r;
-            if (!__ldcg(V.joined + rpos)) V.joined[rpos] = 1;
-        }
-        const unsigned p = __ballot_sync(0xffffffffu, push);
-        if (p) {
-            unsigned at = 0;
-            if (lane == 0) at = atomicAdd(&rs->unresolved, static_cast<unsigned>(__popc(p)));
-            at = __shfl_sync(0xffffffffu, at, 0);
-            if (push) V.unresolved[at + __popc(p & ((1u << lane) - 1u))] = pos;
+            join = all;
+            push = !all;
+        } else {
+            wide = true;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) owned += __shfl_xor_sync(0xffffffffu, owned, o);
-    if (lane == 0) sh.wsum[threadIdx.x >> 5] = owned;
+    for (unsigned todo = __ballot_sync(0xffffffffu, wide); todo; todo &= todo - 1u) {
+        const int q = __ffs(todo) - 1;
+        const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
+        const int qdv = __shfl_sync(0xffffffffu, dv, q), qdr = __shfl_sync(0xffffffffu, dr, q);
+        const bool same = row_inside(V, R.Pin, qev, qdv, qer, qdr);
+        if (static_cast<int>(lane) == q) {
+            join = same;
+            push = !same;
+        }
+    }
+    if (join) R.Pout[p.v] = p.r;
+    const unsigned m = __ballot_sync(0xffffffffu, push);
+    if (m) {
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&V.ctl->copy[V.copy].unresolved, static_cast<unsigned>(__popc(m)));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (push) V.unresolved[at + __popc(m & ((1u << lane) - 1u))] = p.pos;
+    }
+    return join;
+}
+
+// Adds the threads' counts to the CTA's.
+__device__ __forceinline__ void add_owned(unsigned owned, Shared& sh) {
+    owned = __reduce_add_sync(0xffffffffu, owned);
+    if (lane_id() == 0 && owned) atomicAdd(&sh.owned, owned);
+}
+
+// Confirms the CTA's entries pos_of(i), i < total, against their table slots'
+// smallest vertices. (Two entries a thread at once: no faster.)
+template <class F>
+__device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, unsigned total, const F& pos_of,
+                                             Shared& sh) {
+    const unsigned lane = lane_id();
+    unsigned owned = 0;
+    for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
+        Pair p{-1, -1, -1, -1};
+        bool test = false, push = false;
+        int4 a{}, c{};
+        if (b + lane < total) {
+            p.pos = pos_of(b + lane);
+            const uint32_t sv = V.slot[p.pos];
+            p.v = __ldg(V.vert + p.pos);
+            p.r = sv == ~0u ? -1 : table_rep(V.t.slots, sv);
+            if (p.r < 0 || p.r >= V.n) {                           // failed insert
+                atomicOr(&sh.error, kErrTableFull);
+                R.Pout[p.v] = -1;
+            } else if (p.r == p.v) {
+                R.Pout[p.v] = p.v;
+                V.own[p.pos] = kOwner;
+                ++owned;
+            } else {
+                p.rpos = __ldg(V.vpos + p.r);
+                a = record(V, p.pos);
+                c = record(V, p.rpos);
+                V.own[p.pos] = kMember;
+                test = a.z == c.z && a.w == c.w;
+                push = !test;
+            }
+        }
+        if (confirm(V, p, test, push, a, c, R)) mark_joined(V, p.rpos, sh);
+    }
+    add_owned(owned, sh);
+}
+
+// Phase B of a round whose blocks mostly hold: every entry against the smallest
+// vertex b of its present block. b stays in the part of its block that keeps the
+// block's id, whatever happens to the others, so a vertex with b's signature
+// needs neither the table nor a flag; those that leave b enter the table, and b
+// asks next round whether it is alone now (see stays_listed).
+__device__ __forceinline__ void keep_or_split(const LoopView& V, const Round& R, const List& l, Shared& sh) {
+    const unsigned total = list_size(l);
+    const unsigned lane = lane_id();
+    unsigned owned = 0;
+    for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
+        const unsigned i = b + lane;
+        Pair p{-1, -1, -1, -1};
+        bool test = false, leave = false, asks = false;
+        int4 a{}, c{};
+        if (i < total) {
+            p.pos = entry_of(l, i);
+            p.v = __ldg(V.vert + p.pos);
+            a = record(V, p.pos);
+            p.r = a.w;
+            if (p.r == p.v) {
+                R.Pout[p.v] = p.v;
+                ++owned;
+            } else {
+                p.rpos = __ldg(V.vpos + p.r);
+                c = record(V, p.rpos);
+                asks = V.own[p.rpos] == kOwnerAsks;
+                test = a.x == c.x && a.y == c.y && a.z == c.z;
+                leave = !test;
+            }
+        }
+        const bool join = confirm(V, p, test, false, a, c, R);
+        if (join && asks) mark_joined(V, p.rpos, sh);
+        const unsigned leaves = __ballot_sync(0xffffffffu, leave);
+        if (leaves) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&sh.split, static_cast<unsigned>(__popc(leaves)));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(leaves & ((1u << lane) - 1u));
+            if (leave) {
+                int g;
+                unsigned j;
+                const int64_t to = place_of(l, at, &g, &j);
+                V.split[V.gb[g] + to] = p.pos;                     // one place per entry, as on the list
+                if (__ldcg(V.own + p.rpos) != kOwnerLeft) V.own[p.rpos] = kOwnerLeft;
+            }
+        }
+    }
+    add_owned(owned, sh);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long s = 0;
-        for (int w = 0; w < kLoopWarps; ++w) s += sh.wsum[w];
-        if (s) atomicAdd(&rs->blocks, s);
+    // those that leave enter the table, equal signatures of a warp as one
+    const unsigned split = sh.split;
+    for (unsigned b = threadIdx.x - lane; b < split; b += blockDim.x) {
+        const bool on = b + lane < split;
+        int32_t pos = 0, v = 0;
+        uint64_t h = 0, mask = 0;
+        int64_t base = 0;
+        if (on) {
+            int g;
+            unsigned j;
+            const int64_t from = place_of(l, b + lane, &g, &j);
+            pos = V.split[V.gb[g] + from];
+            v = __ldg(V.vert + pos);
+            h = V.sig[pos].hash & R.t.hmask;
+            table_span(V, v, &base, &mask);
+        }
+        const uint32_t sl = insert_warp(R.t, on, h, base, mask, v, &sh.error);
+        if (on) V.slot[pos] = sl;
     }
 }
 
-// Every listed position through f(pos).
-template <class F>
-__device__ __forceinline__ void for_listed(const LoopView& V, const List& l, const F& f) {
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * kLoopThreads;
-    const int64_t t = static_cast<int64_t>(blockIdx.x) * kLoopThreads + threadIdx.x;
-    int64_t before = 0;
-    for (int g = 0; g < kLoopGroups; before += l.cnt[g], ++g)
-        for (int64_t i = t; i < l.cnt[g]; i += stride) f(list_at(V, l, g, i), before + i);
+// ----------------------------------------------------------------------------- the loop
+
+// The list and the state of a round that ended in a hash collision (or an
+// error) as the host-driven levels expect them: P_i in P[0], P_{i+1} as far as
+// it is known in P[1], the list in act[0] / aoff, the counts in the status word.
+__device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int out, unsigned long long blocks,
+                          unsigned listed, unsigned* bar, Shared& sh) {
+    LoopCopy* c = &V.ctl->copy[V.copy];
+    if (threadIdx.x < kLoopGroups && l.cnt[threadIdx.x]) atomicAdd(&c->gcount[threadIdx.x], l.cnt[threadIdx.x]);
+    if (threadIdx.x == 0 && sh.error) atomicOr(&c->error, sh.error);
+    for (unsigned i = threadIdx.x; i < list_size(l); i += blockDim.x) {
+        const int32_t pos = entry_of(l, i);
+        const int32_t v = __ldg(V.vert + pos);
+        if (V.start && R.first) {
+            V.P[0][v] = V.P0[v];
+        } else if (out == 0) {
+            const int32_t x = V.P[0][v];
+            V.P[0][v] = V.P[1][v];
+            V.P[1][v] = x;
+        }
+        if (V.own[pos] > kOwner) {                                 // whether it is alone is not known: listed on
+            V.own[pos] = kOwner;
+            V.joined[pos] = 1;
+        }
+    }
+    if (!grid_barrier(V, ++*bar, sh)) return false;
+    int64_t first[kLoopGroups + 1] = {0, 0, 0, 0, 0};
+    for (int g = 0; g < kLoopGroups; ++g) first[g + 1] = first[g] + __ldcg(&c->gcount[g]);
+    const bool in_place = R.first && !V.start;
+    if (!in_place) {
+        // flat into the buffer the list is not in, then (if that is act[1]) over to act[0]
+        int32_t* flat = l.buf == V.act[1] ? V.act[0] : V.act[1];
+        if (threadIdx.x < kLoopGroups) sh.wcnt[threadIdx.x] = atomicAdd(&c->gcursor[threadIdx.x], l.cnt[threadIdx.x]);
+        __syncthreads();
+        for (int g = 0; g < kLoopGroups; ++g)
+            for (unsigned j = threadIdx.x; j < l.cnt[g]; j += blockDim.x) flat[first[g] + sh.wcnt[g] + j] = list_at(l, g, j);
+        if (!grid_barrier(V, ++*bar, sh)) return false;
+        if (flat != V.act[0])
+            for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < listed;
+                 i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+                V.act[0][i] = flat[i];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (!in_place) {
+            // the groups as classes: 0 (0 to 4), 5, 6, 7 (7 to 9)
+            V.aoff[0] = 0;
+            for (int q = 1; q <= kDClasses; ++q) V.aoff[q] = q <= 5 ? first[1] : q == 6 ? first[2] : q == 7 ? first[3] : first[4];
+            for (int q = 0; q < kDClasses; ++q) V.ccount[q] = 0ull;
+        }
+        DevState z{};
+        z.blocks = blocks;
+        z.unresolved = __ldcg(&c->unresolved);
+        z.error = __ldcg(&c->error);
+        z.listed = listed;
+        *V.st = z;
+    }
+    return true;
 }
 
 __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V) {
-    extern __shared__ unsigned long long sets[];           // kLoopWarps * kLoopWarpSet when warp-class rows exist
+    extern __shared__ unsigned long long sets[];           // a set per warp, when warp-class rows exist
     __shared__ Shared sh;
-    LoopCtl* ctl = V.ctl;
     LoopState S = V.init;
     if (!V.start) S = *V.L;
+    if (blockIdx.x == 0) {                                 // the next launch's copy starts out zero
+        unsigned* z = reinterpret_cast<unsigned*>(&V.ctl->copy[V.copy ^ 1]);
+        for (unsigned i = threadIdx.x; i < sizeof(LoopCopy) / sizeof(unsigned); i += blockDim.x) z[i] = 0u;
+    }
     List l;
-    l.identity = V.start != 0;
-    if (V.start) {
-        for (int g = 0; g < kLoopGroups; ++g) {
-            l.base[g] = nullptr;
-            l.cnt[g] = V.gb[g + 1] - V.gb[g];
-        }
-    } else {
+    l.buf = V.start ? nullptr : V.act[0];
+    const unsigned warps = gridDim.x * (blockDim.x / 32);
+#pragma unroll
+    for (int g = 0; g < kLoopGroups; ++g) {
         constexpr int c0[kLoopGroups + 1] = {0, 5, 6, 7, 10};
-        for (int g = 0; g < kLoopGroups; ++g) {
-            l.base[g] = V.act[0] + V.aoff[c0[g]];
-            l.cnt[g] = V.aoff[c0[g + 1]] - V.aoff[c0[g]];
-        }
-        if (S.stop == 0 && V.aoff[16] != V.aoff[10]) S.stop = kStopWideRows;   // rows above 256 edges are listed
+        l.base[g] = V.start ? V.gb[g] : V.aoff[c0[g]];
+        const int64_t count = V.start ? V.gb[g + 1] - V.gb[g] : V.aoff[c0[g + 1]] - V.aoff[c0[g]];
+        unsigned shift = 5;
+        while (g > 0 && shift > 0 && (count >> shift) < warps) --shift;
+        l.shift[g] = shift;
+        l.cnt[g] = dealt_count(count, shift);
     }
+    if (!V.start && S.stop == kStopNo && V.aoff[kDClasses] != V.aoff[kDMid0]) S.stop = kStopWideRows;
     if (threadIdx.x < kHotSlots) {
-        for (int p = 0; p < 2; ++p) {
-            sh.hot_key[p][threadIdx.x] = 0ull;
-            sh.hot_min[p][threadIdx.x] = ~0u;
-        }
+        sh.hot_key[threadIdx.x] = 0ull;
+        sh.hot_min[threadIdx.x] = ~0u;
     }
-    __syncthreads();
+    if (threadIdx.x == 0) sh.error = 0u;
     uint32_t ep = V.epoch;
     unsigned bar = 0;
-    int parity = 0, nbuf = V.start ? 0 : 1;                // the list buffer the next list goes to
-    bool fine = true;
-    const int32_t* Pin = V.start ? V.P0 : V.P[0];
+    int nbuf = V.start ? 0 : 1;                            // the list buffer the next list goes to
     int out = 1;
-    for (int round = 0; S.stop == 0; ++round) {
-        const bool first = round == 0;
-        RoundSet* rs = &ctl->set[round % 3];
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            RoundSet z{};
-            ctl->set[(round + 1) % 3] = z;
-        }
+    bool fine = true;
+    int64_t grown = 0, listed_before = 0;
+    Round R;
+    R.Pin = V.start ? V.P0 : V.P[0];
+    R.t = V.t;
+    for (R.first = true; S.stop == kStopNo; R.first = false) {
         if (ep == kEpochCycle) {                           // every epoch is used up: blank the table
             uint4* w = reinterpret_cast<uint4*>(V.t.slots);
-            const uint64_t st = static_cast<uint64_t>(gridDim.x) * kLoopThreads;
-            for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * kLoopThreads + threadIdx.x; i < V.nslots / 2; i += st)
+            const uint64_t st = static_cast<uint64_t>(gridDim.x) * blockDim.x;
+            for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < V.nslots / 2; i += st)
                 w[i] = make_uint4(0u, 0u, 0u, 0u);
             ep = 0;
-            if (!(fine = grid_barrier(ctl, ++bar, sh))) break;
+            if (!(fine = grid_barrier(V, ++bar, sh))) break;
         }
         ++ep;
-        TableRef tt = V.t;
-        tt.epoch = static_cast<uint64_t>(ep) << 32;
-        int32_t* Pout = V.P[out];
-        int32_t* next = V.act[nbuf];
-        for (int g = 1; g < kLoopGroups; ++g)
-            if (l.cnt[g] > 0) phase_a_warps(V, tt, l, g, first, Pin, Pout, next, rs, sh, sets);
-        phase_a_threads(V, tt, l, first, Pin, Pout, next, rs, sh, &parity);
-        if (!(fine = grid_barrier(ctl, ++bar, sh))) break;
-        if (!first) {
-            l.identity = false;
+        R.t.epoch = static_cast<uint64_t>(ep) << 32;
+        R.Pout = V.P[out];
+        R.next = V.act[nbuf];
+        // most listed vertices keep their block's smallest vertex when the last
+        // round made few new blocks: then the table is for those that do not (a
+        // chain graph's second round splits most of its million vertices after a
+        // first that made one new block for every five)
+        R.insert = R.first || grown * 32 >= listed_before;
+        for (int i = threadIdx.x; i < kSeenSlots; i += blockDim.x) sh.seen[i] = -1;
+        if (threadIdx.x < kLoopGroups) sh.next_cnt[threadIdx.x] = 0u;
+        if (threadIdx.x == 0) sh.split = sh.owned = 0u;
+        __syncthreads();
+        phase_a(V, R, l, sh, sets);
+        if (!(fine = grid_barrier(V, ++bar, sh))) break;
+        if (!R.first) {
+            l.buf = R.next;
+#pragma unroll
             for (int g = 0; g < kLoopGroups; ++g) {
-                l.base[g] = next + V.gb[g];
-                l.cnt[g] = __ldcg(&rs->cnt[g]);
+                l.base[g] = V.gb[g];
+                l.cnt[g] = sh.next_cnt[g];
             }
             nbuf ^= 1;
         }
-        phase_b(V, l, Pin, Pout, rs, sh);
-        if (!(fine = grid_barrier(ctl, ++bar, sh))) break;
-        const int64_t listed = l.cnt[0] + l.cnt[1] + l.cnt[2] + l.cnt[3];
-        const unsigned long long blocks = static_cast<unsigned long long>(V.n_live - listed) + __ldcg(&rs->blocks);
-        loop_advance(S, blocks, __ldcg(&rs->unresolved), __ldcg(&rs->error));
+        bool confirmed = R.insert;
+        if (R.insert) verify_slots(V, R, list_size(l), [&](unsigned i) { return entry_of(l, i); }, sh);
+        else keep_or_split(V, R, l, sh);
+        __syncthreads();
+        // unresolved entries are rare: every CTA looks at the counter
+        for (;;) {
+            const unsigned flags = (sh.split ? kAnySplit : 0u) | (sh.error ? kAnyError : 0u) |
+                                   (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
+            if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
+            if (confirmed || !(sh.flags & kAnySplit)) break;
+            verify_slots(V, R, sh.split, [&](unsigned i) {
+                int g;
+                unsigned j;
+                const int64_t from = place_of(l, i, &g, &j);
+                return V.split[V.gb[g] + from];
+            }, sh);
+            confirmed = true;
+            __syncthreads();
+        }
+        if (!fine) break;
+        const unsigned listed = sh.total[0];
+        const unsigned long long blocks = static_cast<unsigned long long>(V.n_live - listed) + sh.total[1];
+        grown = static_cast<int64_t>(blocks - S.prev_blocks);
+        listed_before = listed;
+        loop_advance(S, blocks, sh.flags & kAnyUnresolved, sh.flags & kAnyError);
         if (S.stop == kStopDone) {
             if (out != 0)                                  // the result belongs in P[0]
-                for_listed(V, l, [&](int32_t pos, int64_t) {
-                    const int32_t v = __ldg(V.vert + pos);
-                    V.P[0][v] = __ldcg(V.P[1] + v);
-                });
-        } else if (S.stop != 0) {
-            // back to the host within this round: P_i in P[0], P_{i+1} as far as it is
-            // known in P[1], the list in act[0] / aoff, the counts in the status word
-            int32_t* flat = V.act[1];
-            const bool in_place = first && !V.start;
-            if (!in_place) {
-                // a list in act[1]'s own regions first moves to act[0]'s
-                if (!l.identity && l.base[0] == V.act[1] + V.gb[0]) {
-                    for (int g = 0; g < kLoopGroups; ++g) {
-                        const int64_t st = static_cast<int64_t>(gridDim.x) * kLoopThreads;
-                        for (int64_t i = static_cast<int64_t>(blockIdx.x) * kLoopThreads + threadIdx.x; i < l.cnt[g]; i += st)
-                            V.act[0][V.gb[g] + i] = __ldcg(l.base[g] + i);
-                        l.base[g] = V.act[0] + V.gb[g];
-                    }
-                    if (!(fine = grid_barrier(ctl, ++bar, sh))) break;
+                for (unsigned i = threadIdx.x; i < list_size(l); i += blockDim.x) {
+                    const int32_t v = __ldg(V.vert + entry_of(l, i));
+                    V.P[0][v] = V.P[1][v];
                 }
-                for_listed(V, l, [&](int32_t pos, int64_t i) { flat[i] = pos; });
-            }
-            if (V.start && first) {
-                for_listed(V, l, [&](int32_t pos, int64_t) {
-                    const int32_t v = __ldg(V.vert + pos);
-                    V.P[0][v] = __ldg(V.P0 + v);
-                });
-            } else if (out == 0) {
-                for_listed(V, l, [&](int32_t pos, int64_t) {
-                    const int32_t v = __ldg(V.vert + pos);
-                    const int32_t a = __ldcg(V.P[0] + v), c = __ldcg(V.P[1] + v);
-                    V.P[0][v] = c;
-                    V.P[1][v] = a;
-                });
-            }
-            if (!(fine = grid_barrier(ctl, ++bar, sh))) break;
-            if (!in_place)
-                for (int64_t i = static_cast<int64_t>(blockIdx.x) * kLoopThreads + threadIdx.x; i < listed;
-                     i += static_cast<int64_t>(gridDim.x) * kLoopThreads)
-                    V.act[0][i] = __ldcg(flat + i);
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                if (!in_place) {
-                    // the groups as classes: 0 (0 to 4), 5, 6, 7 (7 to 9)
-                    const int64_t o[4] = {l.cnt[0], l.cnt[0] + l.cnt[1], l.cnt[0] + l.cnt[1] + l.cnt[2], listed};
-                    V.aoff[0] = 0;
-                    for (int c = 1; c <= kDClasses; ++c) V.aoff[c] = c <= 5 ? o[0] : c == 6 ? o[1] : c == 7 ? o[2] : o[3];
-                    for (int c = 0; c < kDClasses; ++c) V.ccount[c] = 0ull;
-                }
-                DevState z{};
-                z.blocks = blocks;
-                z.unresolved = __ldcg(&rs->unresolved);
-                z.error = __ldcg(&rs->error);
-                z.listed = static_cast<unsigned>(listed);
-                *V.st = z;
-            }
+        } else if (S.stop != kStopNo) {
+            if (!(fine = hand_back(V, l, R, out, blocks, listed, &bar, sh))) break;
         }
-        Pin = Pout;
+        R.Pin = R.Pout;
         out ^= 1;
+        __syncthreads();                                   // the counts are cleared for the next round
     }
-    // the last CTA to leave writes the result and clears the counters for the next launch
-    __syncthreads();
-    if (threadIdx.x == 0 && fine) {
-        __threadfence();
-        const unsigned left = atomicAdd(&ctl->left, 1u);
-        if (left == gridDim.x - 1) {
-            RoundSet z{};
-            for (int k = 0; k < 3; ++k) ctl->set[k] = z;
-            ctl->arrived = 0u;
-            ctl->left = 0u;
-            S.epoch = static_cast<int32_t>(ep);
-            *V.L = S;
-            *V.host = S;
-            __threadfence_system();
-        }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && fine) {
+        S.epoch = static_cast<int32_t>(ep);
+        *V.L = S;
+        *V.host = S;
+        __threadfence_system();
     }
 }
 
@@ -745,6 +1062,47 @@ cudaError_t launch_in_lane(int device, const void* kernel, unsigned grid, unsign
     if ((e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, smem, s))) return e;
     lane.last[device] = s;
     return cudaEventRecord(lane.done[device], s);
+}
+
+cudaLaunchConfig_t cluster_config(unsigned grid, unsigned threads, size_t smem) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    return cfg;
+}
+
+cudaLaunchAttribute cluster_attribute(unsigned size) {
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = size;
+    a.val.clusterDim.y = 1;
+    a.val.clusterDim.z = 1;
+    return a;
+}
+
+// The largest cluster of full SMs the device takes (16 where a GPC has them, else 8).
+int largest_cluster(int device, size_t smem) {
+    static std::mutex mu;
+    static int known[64][2] = {};
+    if (device < 0 || device >= 64) return 1;
+    std::lock_guard<std::mutex> lk(mu);
+    cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         static_cast<int>(sizeof(unsigned long long) * kLoopWarps * kLoopWarpSet));
+    int& k = known[device][smem ? 1 : 0];
+    if (k == 0) {
+        cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (k = 16; k > 1; k >>= 1) {
+            cudaLaunchConfig_t cfg = cluster_config(static_cast<unsigned>(k), kLoopThreads, smem);
+            cudaLaunchAttribute attr = cluster_attribute(static_cast<unsigned>(k));
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, k_round_loop, &cfg) == cudaSuccess && fit > 0) break;
+            cudaGetLastError();
+        }
+    }
+    return k;
 }
 
 }  // namespace
@@ -803,6 +1161,7 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     V.t.hmask = hb >= 64 ? ~0ull : ((1ull << hb) - 1ull);
     V.epoch = regions || ctx->epoch32 == 0 ? kEpochCycle : (ctx->epoch32 - 1) % kEpochCycle + 1;
     V.unresolved = ctx->ulist[0];
+    V.split = ctx->ulist[1];
     V.st = ctx->dstate;
     V.L = static_cast<LoopState*>(ctx->dloop);
     V.ctl = reinterpret_cast<LoopCtl*>(static_cast<char*>(ctx->dloop) + ls);
@@ -812,6 +1171,8 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     for (int g = 0; g <= kLoopGroups; ++g) V.gb[g] = gb[g];
     V.n_live = db[kDClasses];
     V.n = ctx->n;
+    V.copy = ctx->loop_copy;
+    ctx->loop_copy ^= 1;
     V.start = start ? 1 : 0;
     V.init = init;
     std::memset(h, 0, sizeof(*h));
@@ -820,18 +1181,32 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
     cudaError_t e;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(sizeof(unsigned long long) * kLoopWarps * kLoopWarpSet));
-    });
-    // a thread per vertex of the short rows, a warp for every four longer ones;
-    // fewer CTAs make a cheaper barrier
-    const int64_t need = std::max(cdiv(gb[1], kLoopThreads), cdiv(gb[4] - gb[1], 4 * kLoopWarps));
-    const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(sms, need)));
+    // a warp per unit of phase A as far as the SMs go, in CTAs of 512 threads while
+    // that is enough of them (16 warps an SM issue their work sooner: 15k against
+    // 30k cycles a round on 10k vertices), of 1024 above; a grid of up to one
+    // cluster is one
+    const int64_t units = cdiv(gb[1], 32) + gb[4] - gb[1];
+    const unsigned threads = units <= static_cast<int64_t>(sms) * 16 ? 512 : kLoopThreads;
+    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(sms, cdiv(units, threads / 32)));
+    const bool cluster = want > 1 && want <= largest_cluster(ctx->device, smem);
+    const unsigned grid = static_cast<unsigned>(want);
+    V.cluster = cluster ? 1 : 0;
     void* args[] = {&V};
-    if ((e = launch_in_lane(ctx->device, reinterpret_cast<const void*>(k_round_loop), grid, kLoopThreads, args, smem, s)))
+    const void* kernel = reinterpret_cast<const void*>(k_round_loop);
+    if (grid == 1 || cluster) {
+        cudaLaunchConfig_t cfg = cluster_config(grid, threads, smem);
+        cudaLaunchAttribute attr = cluster_attribute(grid);
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        cfg.stream = s;
+        e = cudaLaunchKernelExC(&cfg, kernel, args);
+    } else {
+        e = launch_in_lane(ctx->device, kernel, grid, threads, args, smem, s);
+    }
+    if (e) {
+        ctx->loop_copy ^= 1;                               // the launch that would have cleared the other copy is missing
         return cuda_error(ctx, e, "launch round loop");
+    }
     prof_add_launches(1);
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "round loop");
     *out = *h;
