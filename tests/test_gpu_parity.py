@@ -76,7 +76,7 @@ def test_powerlaw_scaled_spans_every_bucket(B):
     assert stats["n_hub"] > 0 and stats["n_mid"] > 0 and stats["n_small"] > 0
 
 
-@pytest.mark.parametrize("m", [1, 2047, 2048, 2049, 152 * 7 * 2048 + 1])
+@pytest.mark.parametrize("m", [1, 2047, 2048, 2049, 152 * 8 * 2048 + 1])
 def test_unsorted_list_tiles(B, m):
     # sizes around a tile of the unsorted build and past one pass of its grid;
     # a third of the edges leave vertex 0, and the highest vertex has some
