@@ -456,18 +456,24 @@ bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
     return BISIM_OK;
 }
 
-// The cooperative loop takes the first round too when it covers every row: it is
-// the faster one at every size measured (us to the fixpoint, before and after, on
-// uniform graphs of five edges a vertex and on chains with two extra edges: 10k
-// vertices 194 / 78 and 231 / 85, 1M 621 / 298 and 786 / 317, 4M 2142 / 979 and
-// 2460 / 983).
+// The cooperative loop takes the first round too when it covers every row and
+// the graph has at most this many vertices. Above it the first round's list is
+// long enough for the kernels of the single classes, which keep twice the warps
+// resident. us to the fixpoint with the loop from P_0 against the kernels of one
+// round first: power-law rows of at most 256 edges, 1M vertices 329 / 384, 2M
+// 524 / 544, 4M 995 / 953, 8M 1962 / 1713; uniform graphs of five edges a vertex
+// 295 / 369, 517 / 566, 974 / 1003, 2073 / 1969; chains with two extra edges
+// 324 / 416, 536 / 671, 977 / 1165, 2019 / 2326.
+constexpr int64_t kLoopStartMax = int64_t{1} << 22;
+
 bisim_status dense_rounds_all(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
                               int32_t* out_executed, int64_t* out_blocks, bool allow_graph) {
     bisim_status st;
     int64_t prev = 0, dropped = 0;
     const int32_t limit = k == BISIM_FIXPOINT ? cap : k;
     if ((st = dense_prepare(ctx, s)) != BISIM_OK) return st;
-    const bool from_p0 = limit > 0 && round_loop_usable(ctx) && round_loop_covers(ctx);
+    const bool from_p0 = limit > 0 && round_loop_usable(ctx) && round_loop_covers(ctx) &&
+                         ctx->dbegin[kDClasses] <= kLoopStartMax;
     if (from_p0) {
         if (ctx->opt.mem_budget_bytes > 0 && ctx->device_bytes > ctx->opt.mem_budget_bytes)
             return set_error(ctx, BISIM_ENOMEM, "context exceeds the memory budget");

@@ -1180,37 +1180,87 @@ __global__ void k_active_init(int32_t* __restrict__ act, int64_t n_live, int64_t
 }
 
 constexpr int kCompareGrid = 304;                      // persistent grids: two CTAs per SM
-constexpr int kCompareWarpGrid = 1216;                 // eight per SM: a warp per pair, all warps in flight
+constexpr int kCompareWarpGrid = 1216;                 // eight per SM: 32 pairs a warp, all warps in flight
 
-// Pairs whose rows have at most 32 edges: one warp per pair. Lane j holds the
-// j-th pair value of each row; S_v is inside S_r iff every value of v's row
-// matches one of r's. The pair count is read on the device.
+// Pairs whose rows have at most 32 edges, 32 pairs to a warp. A pair with at
+// most eight edges on both sides is compared by its lane: r's values in
+// registers, v's four at a time, S_v inside S_r iff each is among them (the
+// sizes are equal). The others take the whole warp one after the other: lane j
+// holds the j-th pair value of each row. (One warp per pair throughout was bound
+// by the latency of four dependent loads a pair: 0.33 of the 0.73 ms of a 1M chain
+// graph's rounds.) The pair count is read on the device.
 __global__ void __launch_bounds__(kThreads) k_dense_compare_warp(const int2* __restrict__ pairs, const DenseView D,
                                                                  int32_t* __restrict__ Pout,
                                                                  int32_t* __restrict__ next, DevState* st) {
     const unsigned count = *reinterpret_cast<volatile unsigned*>(&st->pairs);
     const unsigned lane = lane_id();
-    const unsigned warps = gridDim.x * (kThreads / 32);
-    for (unsigned i = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); i < count; i += warps) {
-        const int2 pr = pairs[i];
-        const int64_t ev = D.prp[pr.x], dv = D.prp[pr.x + 1] - ev;
-        const int64_t er = D.prp[pr.y], dr = D.prp[pr.y + 1] - er;
-        const bool ha = lane < dv, hb = lane < dr;
-        const uint64_t a = ha ? packed_pair_value(D.pe[ev + lane], D.P) : 0ull;
-        const uint64_t b = hb ? packed_pair_value(D.pe[er + lane], D.P) : 0ull;
-        if (lane == 0) atomicAdd(&st->aux, static_cast<unsigned long long>(dv + dr));
-        bool found = false;
-        for (int k = 0; k < static_cast<int>(dr); ++k) {
-            const uint64_t bk = __shfl_sync(0xffffffffu, b, k);   // every lane takes part in every shuffle
-            found = found || bk == a;
+    const unsigned threads = gridDim.x * kThreads;
+    for (unsigned b = blockIdx.x * kThreads + (threadIdx.x & ~31u); b < count; b += threads) {
+        const bool in = b + lane < count;
+        int2 pr = make_int2(0, 0);
+        int64_t ev = 0, er = 0;
+        int dv = 0, dr = 0;
+        bool same = false;
+        if (in) {
+            pr = pairs[b + lane];
+            ev = D.prp[pr.x];
+            dv = static_cast<int>(D.prp[pr.x + 1] - ev);
+            er = D.prp[pr.y];
+            dr = static_cast<int>(D.prp[pr.y + 1] - er);
         }
-        const bool miss = __any_sync(0xffffffffu, ha && !found);
-        if (lane == 0) {
-            if (!miss) {
-                Pout[D.vert[pr.x]] = D.vert[pr.y];
-                D.joined[pr.y] = 1;
+        const bool small = in && dv <= 8 && dr <= 8;
+        if (small) {
+            uint64_t x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = j < dr ? D.pe[er + j] : 0ull;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (j < dr) x[j] = packed_pair_value(x[j], D.P);
+            same = true;
+#pragma unroll 1
+            for (int j0 = 0; j0 < dv && same; j0 += 4) {
+                uint64_t y[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) y[j] = j0 + j < dv ? D.pe[ev + j0 + j] : 0ull;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (j0 + j < dv) y[j] = packed_pair_value(y[j], D.P);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    bool found = j0 + j >= dv;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) found = found || (q < dr && x[q] == y[j]);
+                    same = same && found;
+                }
             }
-            else next[atomicAdd(&st->unresolved, 1u)] = pr.x;
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, in && !small); todo; todo &= todo - 1u) {
+            const int q = __ffs(todo) - 1;
+            const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
+            const int qdv = __shfl_sync(0xffffffffu, dv, q), qdr = __shfl_sync(0xffffffffu, dr, q);
+            const bool ha = static_cast<int>(lane) < qdv, hb = static_cast<int>(lane) < qdr;
+            const uint64_t va = ha ? packed_pair_value(D.pe[qev + lane], D.P) : 0ull;
+            const uint64_t vb = hb ? packed_pair_value(D.pe[qer + lane], D.P) : 0ull;
+            bool found = false;
+            for (int k = 0; k < qdr; ++k) {
+                const uint64_t bk = __shfl_sync(0xffffffffu, vb, k);   // every lane takes part in every shuffle
+                found = found || bk == va;
+            }
+            const bool miss = __any_sync(0xffffffffu, ha && !found);
+            if (static_cast<int>(lane) == q) same = !miss;
+        }
+        const unsigned words = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(dv + dr));
+        if (lane == 0) atomicAdd(&st->aux, static_cast<unsigned long long>(words));
+        if (in && same) {
+            Pout[D.vert[pr.x]] = D.vert[pr.y];
+            D.joined[pr.y] = 1;
+        }
+        const unsigned miss = __ballot_sync(0xffffffffu, in && !same);
+        if (miss) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&st->unresolved, static_cast<unsigned>(__popc(miss)));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (in && !same) next[at + __popc(miss & lanemask_lt())] = pr.x;
         }
     }
 }
