@@ -47,6 +47,21 @@ void pinned_give(void* p) {
     g_pinned_free.push_back(p);
 }
 
+// Whether the kernels of the current device may read `p` in place: managed
+// memory, or device memory of the current device. Memory of another GPU is
+// not (no peer mapping is assumed): it is staged through a copy like host memory.
+bool device_accessible(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (a.type == cudaMemoryTypeManaged) return true;
+    if (a.type != cudaMemoryTypeDevice) return false;
+    int cur = -1;
+    return cudaGetDevice(&cur) == cudaSuccess && a.device == cur;
+}
+
 namespace {
 
 void setup_pool(int device) {
@@ -61,21 +76,6 @@ void setup_pool(int device) {
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
         }
     });
-}
-
-// Whether the kernels of the current device may read `p` in place: managed
-// memory, or device memory of the current device. Memory of another GPU is
-// not (no peer mapping is assumed): it is staged through a copy like host memory.
-bool device_accessible(const void* p) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (a.type == cudaMemoryTypeManaged) return true;
-    if (a.type != cudaMemoryTypeDevice) return false;
-    int cur = -1;
-    return cudaGetDevice(&cur) == cudaSuccess && a.device == cur;
 }
 
 // Device-resident view of a caller array: the array itself if the GPU can

@@ -443,6 +443,8 @@ namespace bisim {
 bisim_status set_error(bisim_ctx* ctx, bisim_status st, const std::string& msg);
 bisim_status cuda_error(bisim_ctx* ctx, cudaError_t e, const char* what);
 cudaError_t ctx_alloc(bisim_ctx* ctx, void** p, size_t bytes, cudaStream_t s);
+// Whether the kernels of the current device may use `p` in place (api.cu).
+bool device_accessible(const void* p);
 // 256-byte pinned host blocks from process-lifetime slabs (nullptr if none can be had).
 void* pinned_take();
 void pinned_give(void* p);

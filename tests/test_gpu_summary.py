@@ -137,3 +137,46 @@ def test_host_outputs_and_capacity(B):
     assert count.value == len(want)
     assert list(zip(*(o.numpy().tolist() for o in outs))) == want[:cap]
     B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("direction", ["DIR_FORWARD", "DIR_BOTH", "DIR_BACKWARD"])
+@pytest.mark.parametrize("k", [0, 1])
+def test_segments_of_every_length(B, direction, k):
+    # rows at the edges of the ways a block's edges are sorted (a packed warp, a
+    # warp's and a CTA's shared memory, the radix sort), repeated edges among
+    # them; at k = 0 whole label classes form segments
+    rng = np.random.default_rng(17)
+    lengths = [0, 1, 2, 7, 8, 15, 16, 17, 31, 32, 33, 63, 64, 65, 127, 129, 255, 256, 257, 511, 513, 2047, 2048, 2049, 9000]
+    lengths += [int(x) for x in rng.integers(0, 40, 300)] + [5000, 2500]
+    n = len(lengths)
+    src = np.repeat(np.arange(n), lengths).astype(np.int32)
+    dst = rng.integers(0, n, len(src)).astype(np.int32)
+    top = 2**30 - 1 if direction == "DIR_BOTH" else 2**31 - 1
+    lab = rng.choice(np.array([-top - 1, -3, 0, 1, 2, 700, top], np.int64), len(src)).astype(np.int32)
+    vl = (np.arange(n) % 9).astype(np.int32)
+    o = rng.permutation(len(src))
+    src, dst, lab = src[o], dst[o], lab[o]
+    ctx = B.summarize_init_coo(n, _dev(src), _dev(dst), _dev(lab), _dev(vl),
+                               options=B.default_options(direction=getattr(B, direction)))
+    B.bisim_iterate(ctx, k, 0)
+    P = B.get_partition(ctx).cpu().numpy()
+    assert _gpu_summary(B, ctx) == oracle.summary_edges(src, dst, lab, P)
+    B.summarize_destroy(ctx)
+
+
+def test_big_segments_whose_triples_exceed_a_word(B):
+    # 2^22 + 3 vertices (23 bits) and labels over the whole range (32 bits) with
+    # more than 512 long rows (10 bits): target, label and segment are sorted apart
+    import torch
+    n, rows, length = (1 << 22) + 3, 600, 2100
+    rng = np.random.default_rng(23)
+    src = np.repeat(rng.choice(n, rows, replace=False), length).astype(np.int32)
+    dst = rng.integers(0, n, len(src)).astype(np.int32)
+    lab = rng.choice(np.array([-2**31, -5, 0, 2**31 - 1], np.int64), len(src)).astype(np.int32)
+    dst[1::2], lab[1::2] = dst[::2], lab[::2]              # every second edge repeats the one before it
+    vl = np.arange(n, dtype=np.int32)                      # every vertex a block of its own
+    ctx = B.summarize_init_coo(n, _dev(src), _dev(dst), _dev(lab), _dev(vl))
+    got = np.stack([x.cpu().numpy() for x in B.get_summary_edges(ctx)])
+    want = np.unique(np.stack([src, lab, dst], 1).astype(np.int64), axis=0).T
+    assert np.array_equal(got, want)
+    B.summarize_destroy(ctx)
