@@ -545,8 +545,9 @@ bisim_status refresh_after_edit(bisim_ctx* ctx, cudaStream_t s);
 
 // Builds (or rebuilds after an edit) the dense round layout of the current CSR.
 bisim_status dense_prepare(bisim_ctx* ctx, cudaStream_t s);
-// The layout's positions, classes and row offsets from the out-degrees (deg[n]).
-bisim_status dense_layout_positions(bisim_ctx* ctx, const int32_t* deg, cudaStream_t s);
+// The layout's positions, classes and row offsets from the out-degrees (deg[n]);
+// with `skip` (a device word) set, nothing is laid out. Synchronises s.
+bisim_status dense_layout_positions(bisim_ctx* ctx, const int32_t* deg, cudaStream_t s, const unsigned* skip = nullptr);
 // Batched contexts: drops from the active list the positions of the graphs
 // with keep_graph[g] == 0 (marked alone, so no round kernel touches them) and
 // turns *prev from |P_0| into the count the rounds see: P_0's blocks of the

@@ -319,19 +319,22 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
     if (m > 0)
         Launch(site_val, s, 0, m, arrival ? 4.0 * m : 8.0 * m),
         k_validate_coo<<<grid, 256, 0, s>>>(src, arrival ? nullptr : dst, m, n, ctx->alive, deg, start, ctx->dstate);
+    // the layout of a sorted list follows at once (the degrees of a list that
+    // failed the check are never used, whatever they are): one read-back tells
+    // both what the check found and where the classes lie
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
-    if ((e = cudaStreamSynchronize(s))) { cudaFreeAsync(base, s); return cuda_error(ctx, e, "validate edges"); }
-    if (ctx->hstate->error & kErrBadInput) {
-        cudaFreeAsync(base, s);
-        return set_error(ctx, BISIM_EINVAL, "edge endpoint out of range [0, n) or on a dead vertex");
-    }
+    bisim_status st = dense_layout_positions(ctx, reinterpret_cast<const int32_t*>(deg), s, &ctx->dstate->unsorted);
+    if (st == BISIM_OK && (ctx->hstate->error & kErrBadInput))
+        st = set_error(ctx, BISIM_EINVAL, "edge endpoint out of range [0, n) or on a dead vertex");
     const bool sorted = ctx->hstate->unsorted == 0;
-    if (!sorted && m > 0) {
+    if (st == BISIM_OK && !sorted && m > 0) {
         cudaMemsetAsync(deg, 0, sizeof(uint32_t) * nv, s);
-        Launch(site_cnt, s, 0, m, 4.0 * m),
-        k_count_coo<<<tile_grid, kTileThreads, 0, s>>>(src, m, deg);
+        {
+            Launch L(site_cnt, s, 0, m, 4.0 * m);
+            k_count_coo<<<tile_grid, kTileThreads, 0, s>>>(src, m, deg);
+        }
+        st = dense_layout_positions(ctx, reinterpret_cast<const int32_t*>(deg), s);
     }
-    bisim_status st = dense_layout_positions(ctx, reinterpret_cast<const int32_t*>(deg), s);
     if (st != BISIM_OK) {
         cudaFreeAsync(base, s);
         return st;

@@ -76,6 +76,26 @@ def test_powerlaw_scaled_spans_every_bucket(B):
     assert stats["n_hub"] > 0 and stats["n_mid"] > 0 and stats["n_small"] > 0
 
 
+@pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 3001])
+@pytest.mark.parametrize("thresholds", [{}, dict(small_max_degree=4, mid_max_degree=300), dict(small_max_degree=0, mid_max_degree=0)])
+def test_layout_tiles_and_classes(B, n, thresholds):
+    # every degree class (hubs of several chunks among them) and dead vertices,
+    # at sizes around a tile of the layout's partition
+    rng = np.random.default_rng(n)
+    deg = rng.choice([0, 1, 2, 3, 5, 9, 17, 33, 70, 130, 300], n, p=[.2, .2, .15, .15, .1, .08, .05, .03, .02, .01, .01])
+    for i, d in zip(rng.integers(0, n, 4), (600, 2000, 5000, 9001)):
+        deg[i] = d
+    alive = (rng.random(n) > 0.1).astype(np.uint8)
+    alive[rng.integers(0, n)] = 1
+    deg[alive == 0] = 0
+    live = np.flatnonzero(alive)
+    src = np.repeat(np.arange(n), deg).astype(np.int32)
+    dst = live[rng.integers(0, len(live), len(src))].astype(np.int32)
+    g = dict(n=n, src=src, dst=dst, elabel=rng.integers(0, 3, len(src)).astype(np.int32),
+             vlabel=rng.integers(0, 2, n).astype(np.int32))
+    check(B, g, [1, oracle.FIXPOINT], options=B.default_options(**thresholds), alive=alive)
+
+
 @pytest.mark.parametrize("m", [1, 2047, 2048, 2049, 152 * 8 * 2048 + 1])
 def test_unsorted_list_tiles(B, m):
     # sizes around a tile of the unsorted build and past one pass of its grid;
