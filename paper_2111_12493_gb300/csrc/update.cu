@@ -53,7 +53,7 @@ __global__ void k_ops_check(const bisim_op* __restrict__ ops, int64_t nops, int3
         if (edge) ok = ok && o.dst >= 0 && o.dst < n;
         if (!ok) atomicOr(&st->error, kErrBadOp);
         // vertex operations sort by vertex; edge operations go last, in batch order
-        vkey[i] = (ok && !edge) ? static_cast<uint32_t>(o.src) : 0xffffffffu;
+        vkey[i] = static_cast<uint32_t>((ok && !edge) ? o.src : n);
         vval[i] = static_cast<uint64_t>(i);
         if (ok && !edge) atomicAdd(&st->aux, 1ull);
         if (ok && o.kind == BISIM_OP_VERTEX_ADD) atomicAdd(&st->pairs, 1u);
@@ -121,13 +121,12 @@ __global__ void k_vertex_final(VertexOps V, uint8_t* __restrict__ alive, int32_t
 }
 
 // Every EDGE_ADD needs both endpoints live at its position; also emits the
-// edge-key hash of every edge operation for grouping. The vertex operations
+// edge-key hash (the low bits of `hmask`) of every edge operation for grouping. The vertex operations
 // come first in the sorted order; their number is read on the device
 // (st->aux), so this runs before the host has seen the batch's checks: an
 // operation that fails them is skipped here and rejects the batch anyway.
 __global__ void k_edge_ops(VertexOps V, const uint64_t* __restrict__ vpos, int64_t nops, int32_t n,
-                           uint32_t* __restrict__ klo, uint32_t* __restrict__ khi, uint64_t* __restrict__ kval,
-                           DevState* st) {
+                           uint32_t hmask, uint32_t* __restrict__ khash, uint64_t* __restrict__ kval, DevState* st) {
     V.nv = static_cast<int64_t>(*reinterpret_cast<const volatile unsigned long long*>(&st->aux));
     const int64_t ne = nops - V.nv;
     for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < ne;
@@ -138,22 +137,8 @@ __global__ void k_edge_ops(VertexOps V, const uint64_t* __restrict__ vpos, int64
                            o.dst >= 0 && o.dst < n;
         if (valid && o.kind == BISIM_OP_EDGE_ADD && (!alive_before(V, o.src, p) || !alive_before(V, o.dst, p)))
             atomicOr(&st->error, kErrDeadEndpoint);
-        const uint64_t h = edge_key_hash(o.src, o.dst, o.label);
-        klo[j] = static_cast<uint32_t>(h);
-        khi[j] = static_cast<uint32_t>(h >> 32);
+        khash[j] = static_cast<uint32_t>(edge_key_hash(o.src, o.dst, o.label)) & hmask;
         kval[j] = p;
-    }
-}
-
-// Key-hash halves of edge operations given in some order of positions.
-__global__ void k_key_halves(const bisim_op* __restrict__ ops, const uint64_t* __restrict__ pos, int64_t ne,
-                             uint32_t* __restrict__ lo, uint32_t* __restrict__ hi) {
-    for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < ne;
-         j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const bisim_op o = ops[pos[j]];
-        const uint64_t h = edge_key_hash(o.src, o.dst, o.label);
-        if (lo) lo[j] = static_cast<uint32_t>(h);
-        if (hi) hi[j] = static_cast<uint32_t>(h >> 32);
     }
 }
 
@@ -205,15 +190,15 @@ __device__ __forceinline__ int64_t key_find(const KeyTable& T, int32_t u, int32_
 }
 
 // Every distinct key of the batch's edge operations enters the table once.
-__global__ void k_keys_insert(const bisim_op* __restrict__ ops, const uint32_t* __restrict__ khi,
-                              const uint32_t* __restrict__ klo, const uint64_t* __restrict__ kpos, int64_t ne,
+__global__ void k_keys_insert(const bisim_op* __restrict__ ops, const uint32_t* __restrict__ khash,
+                              const uint64_t* __restrict__ kpos, int64_t ne,
                               KeyTable T, int64_t* __restrict__ keyslot, unsigned* err) {
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < ne;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const bisim_op o = ops[kpos[i]];
         // first appearance of this full key within its run of equal hashes
         bool first = true;
-        for (int64_t b = i - 1; b >= 0 && khi[b] == khi[i] && klo[b] == klo[i]; --b) {
+        for (int64_t b = i - 1; b >= 0 && khash[b] == khash[i]; --b) {
             const bisim_op ob = ops[kpos[b]];
             if (ob.src == o.src && ob.dst == o.dst && ob.label == o.label) { first = false; break; }
         }
@@ -236,8 +221,8 @@ __global__ void k_keys_count(const int32_t* __restrict__ esrc, const int32_t* __
 
 // One thread per distinct key: fold its operations in batch order, starting
 // after the last deletion of an endpoint, and record the net change.
-__global__ void k_fold_keys(VertexOps V, const uint32_t* __restrict__ khi, const uint32_t* __restrict__ klo,
-                            const uint64_t* __restrict__ kpos, int64_t ne, const int64_t* __restrict__ keyslot,
+__global__ void k_fold_keys(VertexOps V, const uint32_t* __restrict__ khash, const uint64_t* __restrict__ kpos,
+                            int64_t ne, const int64_t* __restrict__ keyslot,
                             KeyTable T, const uint8_t* __restrict__ killed, AddRec* __restrict__ add,
                             unsigned long long* __restrict__ counters, uint8_t* __restrict__ rowchg) {
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < ne;
@@ -248,7 +233,7 @@ __global__ void k_fold_keys(VertexOps V, const uint32_t* __restrict__ khi, const
         const int32_t u = oa.src, w = oa.dst, l = oa.label;
         const bool dropped = killed[u] || killed[w];           // initial copies go with the deletion
         int64_t end = i;
-        while (end < ne && khi[end] == khi[i] && klo[end] == klo[i]) ++end;
+        while (end < ne && khash[end] == khash[i]) ++end;
         // a key that is only deleted removes one copy per deletion, as far as copies
         // exist: an old count at least its number of operations gives exactly that
         // (the row-store path does not count such keys; the removal stops when the
@@ -786,8 +771,7 @@ struct Batch {
     char* base = nullptr;
     VertexOps V{};
     int64_t nv = 0, ne = 0, vadds = 0;
-    const uint32_t* skhi = nullptr;
-    const uint32_t* sklo = nullptr;
+    const uint32_t* skh = nullptr;   // edge operations sorted by key hash: the hash, the position in the batch
     const uint64_t* skp = nullptr;
     KeyTable T{};
     int64_t* keyslot = nullptr;
@@ -813,8 +797,7 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     size_t bytes = 0;
     auto need = [&](size_t b) { bytes += (b + 255) & ~size_t(255); };
     need(4 * nb); need(4 * nb); need(8 * nb); need(8 * nb);          // vertex-op keys / values (x2)
-    need(4 * nb); need(4 * nb); need(4 * nb); need(4 * nb);          // edge key halves (x2 each)
-    need(8 * nb); need(8 * nb); need(8 * nb); need(8 * nb);          // edge positions (x4)
+    need(4 * nb); need(4 * nb); need(8 * nb); need(8 * nb);          // edge key hashes / positions (x2)
     need(sizeof(AddRec) * nb); need(8 * nb);                          // additions, key slots
     for (int q = 0; q < 8; ++q) need(4 * static_cast<size_t>(tsize)); // key table
     need(8 * 4);
@@ -827,14 +810,10 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     uint32_t* vk1 = reinterpret_cast<uint32_t*>(carve(4 * nb));
     uint64_t* vv0 = reinterpret_cast<uint64_t*>(carve(8 * nb));
     uint64_t* vv1 = reinterpret_cast<uint64_t*>(carve(8 * nb));
-    uint32_t* klo0 = reinterpret_cast<uint32_t*>(carve(4 * nb));
-    uint32_t* klo1 = reinterpret_cast<uint32_t*>(carve(4 * nb));
-    uint32_t* khi0 = reinterpret_cast<uint32_t*>(carve(4 * nb));
-    uint32_t* khi1 = reinterpret_cast<uint32_t*>(carve(4 * nb));
+    uint32_t* kh0 = reinterpret_cast<uint32_t*>(carve(4 * nb));
+    uint32_t* kh1 = reinterpret_cast<uint32_t*>(carve(4 * nb));
     uint64_t* kp0 = reinterpret_cast<uint64_t*>(carve(8 * nb));
     uint64_t* kp1 = reinterpret_cast<uint64_t*>(carve(8 * nb));
-    uint64_t* kp2 = reinterpret_cast<uint64_t*>(carve(8 * nb));
-    uint64_t* kp3 = reinterpret_cast<uint64_t*>(carve(8 * nb));
     B.add = reinterpret_cast<AddRec*>(carve(sizeof(AddRec) * nb));
     B.keyslot = reinterpret_cast<int64_t*>(carve(8 * nb));
     int32_t* tab_arrays[8];
@@ -850,6 +829,14 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
         return set_error(ctx, code, msg);
     };
 
+    // One sort by 24 or 32 bits of the key hash groups the edge operations: runs of
+    // equal hashes are searched for equal keys anyway, and the few keys that share
+    // a hash only lengthen a run (below 2^18 operations one in 64 shares 24 bits
+    // at most). Sorting by all 64 bits took eight radix passes, half of a
+    // 100k-operation batch's sorting.
+    const int hbits = nops <= (1 << 18) ? 24 : 32;
+    const uint32_t hmask = hbits == 32 ? ~0u : (1u << hbits) - 1u;
+
     BISIM_SITE(site_ops, "update_ops");
     // 1. check kinds and ranges; group vertex operations by vertex
     cudaMemsetAsync(ctx->dstate, 0, sizeof(DevState), s);
@@ -857,7 +844,9 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
         Launch L(site_ops, s, 0, 0, 16.0 * nops);
         k_ops_check<<<grid_for(nops, 256), 256, 0, s>>>(d_ops, nops, n, ctx->dstate, vk0, vv0);
     }
-    const int which = radix_sort_pairs(vk0, vv0, vk1, vv1, nops, 32, B.tmp, s, "update_radix");
+    int vbits = 1;                                          // keys 0 .. n
+    while (vbits < 32 && (int64_t{1} << vbits) <= n) ++vbits;
+    const int which = radix_sort_pairs(vk0, vv0, vk1, vv1, nops, vbits, B.tmp, s, "update_radix");
     const uint32_t* vkey = which ? vk1 : vk0;
     const uint64_t* vpos = which ? vv1 : vv0;
     // 2. EDGE_ADD liveness and edge-key hashes (before the host looks: one read-back
@@ -865,7 +854,7 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     if (nops > 0) {
         Launch L(site_ops, s, 0, 0, 24.0 * nops);
         B.V = VertexOps{vkey, vpos, 0, d_ops, ctx->alive};
-        k_edge_ops<<<grid_for(nops, 256), 256, 0, s>>>(B.V, vpos, nops, n, klo0, khi0, kp0, ctx->dstate);
+        k_edge_ops<<<grid_for(nops, 256), 256, 0, s>>>(B.V, vpos, nops, n, hmask, kh0, kp0, ctx->dstate);
     }
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s))) {
@@ -882,21 +871,13 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     const int64_t nv = B.nv, ne = B.ne;
 
     // ---- from here on the batch is valid and the graph changes ----
-    // stable LSD sort of the edge operations by key hash: low half, then high
-    // half; operations of one key stay in batch order
-    B.skhi = khi0;
-    B.sklo = klo0;
+    // stable sort of the edge operations by key hash: operations of one key stay
+    // in batch order
+    B.skh = kh0;
     B.skp = kp0;
-    if (ne > 0) {
-        const int wa = radix_sort_pairs(klo0, kp0, klo1, kp1, ne, 32, B.tmp, s, "update_radix");
-        const uint64_t* posA = wa ? kp1 : kp0;
-        k_key_halves<<<grid_for(ne, 256), 256, 0, s>>>(d_ops, posA, ne, nullptr, khi0);
-        cudaMemcpyAsync(kp2, posA, 8 * ne, cudaMemcpyDeviceToDevice, s);
-        const int wb = radix_sort_pairs(khi0, kp2, khi1, kp3, ne, 32, B.tmp, s, "update_radix");
-        B.skhi = wb ? khi1 : khi0;
-        B.skp = wb ? kp3 : kp2;
-        k_key_halves<<<grid_for(ne, 256), 256, 0, s>>>(d_ops, B.skp, ne, klo0, nullptr);
-        B.sklo = klo0;
+    if (ne > 0 && radix_sort_pairs(kh0, kp0, kh1, kp1, ne, hbits, B.tmp, s, "update_radix")) {
+        B.skh = kh1;
+        B.skp = kp1;
     }
     cudaMemsetAsync(killed, 0, n + 1, s);
     cudaMemsetAsync(B.counters, 0, 8 * 4, s);
@@ -908,7 +889,7 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     }
     if (ne > 0) {
         Launch L(site_ops, s, 0, 0, 32.0 * ne);
-        k_keys_insert<<<grid_for(ne, 256), 256, 0, s>>>(d_ops, B.skhi, B.sklo, B.skp, ne, B.T, B.keyslot,
+        k_keys_insert<<<grid_for(ne, 256), 256, 0, s>>>(d_ops, B.skh, B.skp, ne, B.T, B.keyslot,
                                                        &ctx->dstate->error);
     }
     return BISIM_OK;
@@ -920,7 +901,7 @@ void fold_keys(const Batch& B, const uint8_t* killed, uint8_t* rowchg, cudaStrea
     if (B.ne <= 0) return;
     BISIM_SITE(site_ops, "update_ops");
     Launch L(site_ops, s, 0, 0, 32.0 * B.ne);
-    k_fold_keys<<<grid_for(B.ne, 128), 128, 0, s>>>(B.V, B.skhi, B.sklo, B.skp, B.ne, B.keyslot, B.T, killed, B.add,
+    k_fold_keys<<<grid_for(B.ne, 128), 128, 0, s>>>(B.V, B.skh, B.skp, B.ne, B.keyslot, B.T, killed, B.add,
                                                    B.counters, rowchg);
 }
 

@@ -530,3 +530,26 @@ def test_long_streams_in_other_directions_and_with_a_label_filter(B, direction, 
                                    alive=state["alive"], direction=mode, label_filter=keep)
         assert np.array_equal(got, want), step
     B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("n_ops", [1, 31, 1000, 1024, 1025, 2049, 4096, 4097, 30_000])
+def test_batches_around_the_sorts_sizes(B, n_ops):
+    # operations on few keys and many, repeated within the batch, at the sizes
+    # where the sorts that group them change (one CTA's network, short and long tiles)
+    rng = np.random.default_rng(n_ops)
+    g = graphgen.powerlaw_graph(n=3000, m=40_000, dmax=3000, n_elabels=4, n_vlabels=3, seed=5)
+    state = dict(n=g["n"], alive=np.ones(g["n"], np.uint8), vlabel=g["vlabel"].copy(), src=g["src"], dst=g["dst"],
+                 elabel=g["elabel"])
+    ctx = B.summarize_init_coo(g["n"], _dev(g["src"]), _dev(g["dst"]), _dev(g["elabel"]), _dev(g["vlabel"]))
+    B.apply_updates(ctx, _dev(np.zeros((0, 4), np.int32)))
+    for _ in range(2):
+        e = rng.integers(0, len(state["src"]), n_ops)
+        add = np.stack([np.zeros(n_ops), rng.integers(0, 40, n_ops), rng.integers(0, g["n"], n_ops), rng.integers(0, 2, n_ops)], 1)
+        gone = np.stack([np.ones(n_ops), state["src"][e], state["dst"][e], state["elabel"][e]], 1)
+        label = np.stack([np.full(n_ops, 2), rng.integers(0, g["n"], n_ops), np.zeros(n_ops), rng.integers(0, 3, n_ops)], 1)
+        ops = np.where((rng.random(n_ops) < 0.6)[:, None], add, np.where((rng.random(n_ops) < 0.8)[:, None], gone, label))
+        ops = np.ascontiguousarray(ops.astype(np.int32))
+        state = oracle.apply_ops(state, ops)
+        B.apply_updates(ctx, _dev(ops))
+        check_partition(B, ctx, state, 2)
+    B.summarize_destroy(ctx)
