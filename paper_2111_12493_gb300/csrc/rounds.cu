@@ -1087,10 +1087,10 @@ int largest_cluster(int device, size_t smem) {
     static int known[64][2] = {};
     if (device < 0 || device >= 64) return 1;
     std::lock_guard<std::mutex> lk(mu);
-    cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(sizeof(unsigned long long) * kLoopWarps * kLoopWarpSet));
     int& k = known[device][smem ? 1 : 0];
     if (k == 0) {
+        cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(sizeof(unsigned long long) * kLoopWarps * kLoopWarpSet));
         cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         for (k = 16; k > 1; k >>= 1) {
             cudaLaunchConfig_t cfg = cluster_config(static_cast<unsigned>(k), kLoopThreads, smem);
@@ -1188,7 +1188,8 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     const int64_t units = cdiv(gb[1], 32) + gb[4] - gb[1];
     const unsigned threads = units <= static_cast<int64_t>(sms) * 16 ? 512 : kLoopThreads;
     const int64_t want = std::max<int64_t>(1, std::min<int64_t>(sms, cdiv(units, threads / 32)));
-    const bool cluster = want > 1 && want <= largest_cluster(ctx->device, smem);
+    const int cl = largest_cluster(ctx->device, smem);     // also sets the kernel's attributes, so always asked
+    const bool cluster = want > 1 && want <= cl;
     const unsigned grid = static_cast<unsigned>(want);
     V.cluster = cluster ? 1 : 0;
     void* args[] = {&V};

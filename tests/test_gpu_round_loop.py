@@ -112,3 +112,13 @@ def test_resident_context_alternates_routes(B):
         assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want) and rounds == wr
         assert blocks == len(np.unique(want))
     B.summarize_destroy(ctx)
+
+
+def test_one_cta_with_a_warp_row_as_the_first_call():
+    # in a process of its own: the kernel's attributes are set whatever graph comes first
+    import subprocess
+    import sys
+    code = ("import torch; from paper_2111_12493_gb300 import bisim as B; i = lambda a: torch.tensor(a, dtype=torch.int32).cuda();"
+            "c = B.summarize_init_coo(3, i([0] * 40 + [1]), i([k % 3 for k in range(40)] + [2]), i(list(range(40)) + [0]), i([0, 0, 0]));"
+            "assert B.bisim_iterate(c, 1)[1] == 3; assert B.get_partition(c).tolist() == [0, 1, 2]")
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300)
