@@ -166,39 +166,53 @@ struct LayoutShared {
     unsigned long long edges[32][kLayoutClasses];
 };
 
-// This thread's class, its rank among the warp's vertices of the class and the
-// edges of those before it; the warp's totals per class go to sh.
+// This thread's class; the warp's totals per class go to sh. RANK: also the
+// thread's rank among the warp's vertices of the class and the edges of those
+// before it. The sums are 32-bit unless the warp has a row that could overflow them.
+template <bool RANK>
 __device__ __forceinline__ int layout_tile(const int32_t* __restrict__ deg, const uint8_t* __restrict__ alive, int32_t n,
                                            int small_max, int mid_max, LayoutShared& sh, unsigned* rank,
                                            unsigned long long* before) {
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     const int64_t v = static_cast<int64_t>(blockIdx.x) * kLayoutTile + threadIdx.x;
-    const int64_t d = v < n ? deg[v] : 0;
+    const int32_t d = v < n ? deg[v] : 0;
     const int c = v < n ? dense_class(d, alive == nullptr || alive[v], small_max, mid_max) : kLayoutClasses;
     if (lane < kLayoutClasses) {
         sh.cnt[warp][lane] = 0u;
         sh.edges[warp][lane] = 0ull;
     }
     __syncwarp();
-    *rank = 0u;
-    *before = 0ull;
+    const bool huge = __any_sync(0xffffffffu, static_cast<uint32_t>(d) >= 1u << 27);
     for (unsigned todo = __ballot_sync(0xffffffffu, c < kLayoutClasses); todo;) {
         const int lead = __ffs(todo) - 1;
         const int lc = __shfl_sync(0xffffffffu, c, lead);
         const unsigned same = __ballot_sync(0xffffffffu, c == lc);
-        unsigned long long inc = c == lc ? static_cast<unsigned long long>(d) : 0ull;
+        unsigned long long sum;
+        if (huge) {
+            unsigned long long inc = c == lc ? static_cast<unsigned long long>(static_cast<int64_t>(d)) : 0ull;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= static_cast<unsigned>(o)) inc += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= static_cast<unsigned>(o)) inc += y;
+            }
+            if (RANK && c == lc) *before = inc - static_cast<unsigned long long>(static_cast<int64_t>(d));
+            sum = __shfl_sync(0xffffffffu, inc, 31);
+        } else if (RANK) {
+            unsigned inc = c == lc ? static_cast<unsigned>(d) : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= static_cast<unsigned>(o)) inc += y;
+            }
+            if (c == lc) *before = inc - static_cast<unsigned>(d);
+            sum = __shfl_sync(0xffffffffu, inc, 31);
+        } else {
+            sum = __reduce_add_sync(0xffffffffu, c == lc ? static_cast<unsigned>(d) : 0u);
         }
-        if (c == lc) {
-            *rank = static_cast<unsigned>(__popc(same & lanemask_lt()));
-            *before = inc - static_cast<unsigned long long>(d);
-        }
-        if (lane == 31) {
+        if (RANK && c == lc) *rank = static_cast<unsigned>(__popc(same & lanemask_lt()));
+        if (static_cast<int>(lane) == lead) {
             sh.cnt[warp][lc] = static_cast<unsigned>(__popc(same));
-            sh.edges[warp][lc] = inc;
+            sh.edges[warp][lc] = sum;
         }
         todo &= ~same;
     }
@@ -213,9 +227,7 @@ __global__ void __launch_bounds__(kLayoutTile) k_layout_count(const int32_t* __r
                                                               const unsigned* skip) {
     __shared__ LayoutShared sh;
     if (skip != nullptr && *skip) return;
-    unsigned rank;
-    unsigned long long before;
-    layout_tile(deg, alive, n, small_max, mid_max, sh, &rank, &before);
+    layout_tile<false>(deg, alive, n, small_max, mid_max, sh, nullptr, nullptr);
     const unsigned warp = threadIdx.x >> 5;
     if (warp < kLayoutClasses) {                                     // a warp per class
         const unsigned cnt = __reduce_add_sync(0xffffffffu, sh.cnt[lane_id()][warp]);
@@ -243,9 +255,9 @@ __global__ void __launch_bounds__(kLayoutTile) k_layout_place(const int32_t* __r
         at[threadIdx.x] = sums[threadIdx.x * tiles + blockIdx.x];
         eat[threadIdx.x] = sums[(kLayoutClasses + threadIdx.x) * tiles + blockIdx.x] - n;   // the counts come first: n of them
     }
-    unsigned rank;
-    unsigned long long before;
-    const int c = layout_tile(deg, alive, n, small_max, mid_max, sh, &rank, &before);
+    unsigned rank = 0u;
+    unsigned long long before = 0ull;
+    const int c = layout_tile<true>(deg, alive, n, small_max, mid_max, sh, &rank, &before);
     const unsigned warp = threadIdx.x >> 5, lane = lane_id();
     if (warp < kLayoutClasses) {                                     // a warp per class: exclusive over the 32 warps
         const unsigned x = sh.cnt[lane][warp];
@@ -387,14 +399,29 @@ __global__ void __launch_bounds__(256) k_dense_pack_rows(const int32_t* __restri
     src[lane] = act ? rp[vert[p]] : 0;
     __syncwarp();
     const int64_t o1 = off[32];
-    for (int64_t o = off[0] + lane; o < o1; o += 32) {
-        int lo = 0, hi = 31;                             // the last row starting at or before o
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= o) lo = mid; else hi = mid - 1;
+    constexpr int kAtOnce = 4;                           // words a lane looks up before it loads any of them
+    for (int64_t o = off[0] + lane; o < o1; o += 32 * kAtOnce) {
+        int64_t e[kAtOnce];
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            const int64_t w = o + 32 * k;
+            int lo = 0, hi = 31;                         // the last row starting at or before w
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (off[mid] <= w) lo = mid; else hi = mid - 1;
+            }
+            e[k] = src[lo] + (w - off[lo]);
         }
-        const int64_t e = src[lo] + (o - off[lo]);
-        pe[o] = pack_edge(elab[e], col[e]);
+        int32_t l[kAtOnce], t[kAtOnce];
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            if (o + 32 * k >= o1) break;
+            l[k] = __ldcs(elab + e[k]);
+            t[k] = __ldcs(col + e[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k)
+            if (o + 32 * k < o1) pe[o + 32 * k] = pack_edge(l[k], t[k]);
     }
 }
 
