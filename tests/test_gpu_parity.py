@@ -76,6 +76,29 @@ def test_powerlaw_scaled_spans_every_bucket(B):
     assert stats["n_hub"] > 0 and stats["n_mid"] > 0 and stats["n_small"] > 0
 
 
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+@pytest.mark.parametrize("m", [1, 3, 4, 5, 1021, 4096])
+def test_edge_arrays_at_any_alignment(B, off, m):
+    # the check of an edge list reads four edges at a time where the arrays allow it
+    rng = np.random.default_rng(m)
+    n = 50
+    src = np.sort(rng.integers(0, n, m)).astype(np.int32)
+    dst, lab = rng.integers(0, n, m).astype(np.int32), rng.integers(0, 2, m).astype(np.int32)
+    vl = rng.integers(0, 2, n).astype(np.int32)
+    want, _, _ = oracle.refine(n, src, dst, lab, vl, 2)
+    s, d = (_dev(np.concatenate([np.full(k, 7, np.int32), a]))[k:] for k, a in ((off, src), ((off + 2) % 4, dst)))
+    with B.summarize_init_coo(n, s, d, _dev(lab), _dev(vl)) as ctx:
+        B.bisim_iterate(ctx, 2)
+        assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+    for a, bad in ((src, n), (dst, -1)):
+        keep = a[m // 2]
+        a[m // 2] = bad
+        with pytest.raises(B.BisimError):
+            s, d = (_dev(np.concatenate([np.full(off, 7, np.int32), x]))[off:] for x in (src, dst))
+            B.summarize_init_coo(n, s, d, _dev(lab), _dev(vl))
+        a[m // 2] = keep
+
+
 @pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 3001])
 @pytest.mark.parametrize("thresholds", [{}, dict(small_max_degree=4, mid_max_degree=300), dict(small_max_degree=0, mid_max_degree=0)])
 def test_layout_tiles_and_classes(B, n, thresholds):
