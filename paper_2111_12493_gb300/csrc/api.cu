@@ -351,6 +351,20 @@ cudaError_t ctx_alloc(bisim_ctx* ctx, void** p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
+cudaError_t ctx_alloc_together(bisim_ctx* ctx, std::initializer_list<CtxPiece> pieces, cudaStream_t s) {
+    size_t total = 0;
+    for (const CtxPiece& x : pieces) total += (x.bytes + 255) & ~size_t(255);
+    void* base = nullptr;
+    const cudaError_t e = ctx_alloc(ctx, &base, total, s);
+    if (e) return e;
+    char* at = static_cast<char*>(base);
+    for (const CtxPiece& x : pieces) {
+        *x.p = at;
+        at += (x.bytes + 255) & ~size_t(255);
+    }
+    return cudaSuccess;
+}
+
 // Rebuilds what depends on the CSR after an update batch changed it: degree
 // buckets, signature-list capacity and the label partition.
 bisim_status refresh_after_edit(bisim_ctx* ctx, cudaStream_t s) {

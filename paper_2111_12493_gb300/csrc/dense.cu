@@ -1846,23 +1846,16 @@ bisim_status alloc_round_state(bisim_ctx* ctx, cudaStream_t s) {
     if (ctx->dvert != nullptr) return BISIM_OK;
     const size_t nv = static_cast<size_t>(std::max(ctx->n, 1));
     cudaError_t e;
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dvert), sizeof(int32_t) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dvpos), sizeof(int32_t) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dprp), sizeof(int64_t) * (nv + 1), s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dslot), sizeof(uint32_t) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dsig), sizeof(SigRec) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dpairs), sizeof(int2) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dsmall), sizeof(int2) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dwork), sizeof(unsigned long long) * kWorkWords, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->djoined), nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->downs), nv, s)))
-        return cuda_error(ctx, e, "alloc dense round state");
     ctx->n_tiles = cdiv(static_cast<int64_t>(nv), kActTile);
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dact), sizeof(int32_t) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dact2), sizeof(int32_t) * nv, s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->daoff), sizeof(int64_t) * (kDClasses + 1), s)) ||
-        (e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dtile), sizeof(int64_t) * (ctx->n_tiles + 2 + kDClasses), s)))
-        return cuda_error(ctx, e, "alloc active list");
+    if ((e = ctx_alloc_together(
+             ctx,
+             {ctx_piece(&ctx->dvert, nv), ctx_piece(&ctx->dvpos, nv), ctx_piece(&ctx->dprp, nv + 1), ctx_piece(&ctx->dslot, nv),
+              ctx_piece(&ctx->dsig, nv), ctx_piece(&ctx->dpairs, nv), ctx_piece(&ctx->dsmall, nv),
+              ctx_piece(&ctx->dwork, kWorkWords), ctx_piece(&ctx->djoined, nv), ctx_piece(&ctx->downs, nv),
+              ctx_piece(&ctx->dact, nv), ctx_piece(&ctx->dact2, nv), ctx_piece(&ctx->daoff, kDClasses + 1),
+              ctx_piece(&ctx->dtile, static_cast<size_t>(ctx->n_tiles) + 2 + kDClasses)},
+             s)))
+        return cuda_error(ctx, e, "alloc dense round state");
     return BISIM_OK;
 }
 

@@ -774,21 +774,18 @@ bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s) {
     const int64_t m = ctx->m;
     cudaError_t e;
     const size_t nv = static_cast<size_t>(std::max(n, 1));
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->P0), sizeof(int32_t) * nv, s))) return cuda_error(ctx, e, "alloc P0");
-    for (int i = 0; i < 2; ++i)
-        if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->P[i]), sizeof(int32_t) * nv, s))) return cuda_error(ctx, e, "alloc P");
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->cnt), sizeof(int32_t) * nv, s))) return cuda_error(ctx, e, "alloc cnt");
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->slot), sizeof(uint32_t) * nv, s))) return cuda_error(ctx, e, "alloc slot");
-    for (int i = 0; i < 2; ++i)
-        if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->ulist[i]), sizeof(int32_t) * nv, s))) return cuda_error(ctx, e, "alloc unresolved list");
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->dlist), sizeof(int32_t) * nv, s))) return cuda_error(ctx, e, "alloc deferred list");
     // the pair lists (skey) of the list-mode path are allocated when that path first runs
     (void)m;
     // load factor at most 0.6: 8 bytes per slot keeps the table near L2 size
     uint64_t ns = 1024;
     while (static_cast<double>(ns) * 0.6 < static_cast<double>(n)) ns <<= 1;
     ctx->nslots = ns;
-    if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->table), sizeof(Slot) * ns, s))) return cuda_error(ctx, e, "alloc signature table");
+    if ((e = ctx_alloc_together(ctx,
+                                {ctx_piece(&ctx->P0, nv), ctx_piece(&ctx->P[0], nv), ctx_piece(&ctx->P[1], nv),
+                                 ctx_piece(&ctx->cnt, nv), ctx_piece(&ctx->slot, nv), ctx_piece(&ctx->ulist[0], nv),
+                                 ctx_piece(&ctx->ulist[1], nv), ctx_piece(&ctx->dlist, nv), ctx_piece(&ctx->table, ns)},
+                                s)))
+        return cuda_error(ctx, e, "alloc refinement state");
     cudaMemsetAsync(ctx->table, 0, sizeof(Slot) * ns, s);
     if (ctx->hub_tab) cudaMemsetAsync(ctx->hub_tab, 0, sizeof(unsigned long long) * ctx->hub_tab_words, s);
     if ((e = cudaGetLastError())) return cuda_error(ctx, e, "init refine state");
