@@ -289,20 +289,6 @@ struct bisim_ctx {
     uint64_t nslots = 0;
     uint32_t epoch32 = 0;
 
-    // degree buckets
-    int32_t* class_list = nullptr;                 // vertices grouped by class
-    int64_t class_begin[bisim::kNumClasses + 1] = {};
-    int64_t class_edges[bisim::kNumClasses] = {};   // out-edges of the vertices of each class
-    int32_t* hub_list = nullptr;                   // = class_list + class_begin[kClassHub]
-    int64_t n_hub = 0;
-    int64_t* hub_toff = nullptr;                   // table offset per hub (in words)
-    uint32_t* hub_tmask = nullptr;                 // table size - 1 per hub
-    unsigned long long* hub_tab = nullptr;
-    int64_t hub_tab_words = 0;
-    bisim::HubChunk* chunks = nullptr;
-    int64_t n_chunks = 0;
-    bisim::HubAcc* hub_acc = nullptr;
-
     // dense round layout: live vertices grouped by degree class (then the dead
     // ones), their out-rows copied in that order as packed (label << 32 | target)
     bool dense_ready = false;
@@ -507,7 +493,6 @@ bisim_status csr_from_store(bisim_ctx* ctx, cudaStream_t s);
 bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s);
 // Advances the signature table's epoch (clearing the table when it wraps).
 TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s);
-bisim_status refine_round(bisim_ctx* ctx, cudaStream_t s, int64_t* out_blocks);
 // One signature round over the vertices of `B` (all of them, or the `vcount`
 // listed in `vlist` for verification): Pout[v] = smallest listed vertex with
 // v's exact signature over the labelling Pin; hout[v] (nullable) receives the
@@ -515,7 +500,6 @@ bisim_status refine_round(bisim_ctx* ctx, cudaStream_t s, int64_t* out_blocks);
 bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
                              const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s,
                              int64_t* out_blocks);
-Buckets ctx_buckets(const bisim_ctx* ctx);
 bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s);
 void pin_partition_in_l2(bisim_ctx* ctx, const int32_t* P, cudaStream_t s);
 void unpin_partition(bisim_ctx* ctx, cudaStream_t s);

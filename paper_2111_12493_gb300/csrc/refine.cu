@@ -787,7 +787,6 @@ bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s) {
                                 s)))
         return cuda_error(ctx, e, "alloc refinement state");
     cudaMemsetAsync(ctx->table, 0, sizeof(Slot) * ns, s);
-    if (ctx->hub_tab) cudaMemsetAsync(ctx->hub_tab, 0, sizeof(unsigned long long) * ctx->hub_tab_words, s);
     if ((e = cudaGetLastError())) return cuda_error(ctx, e, "init refine state");
     return BISIM_OK;
 }
@@ -807,23 +806,6 @@ bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s) {
     ctx->last_blocks = blocks;
     ctx->stats.num_blocks = blocks;
     return BISIM_OK;
-}
-
-Buckets ctx_buckets(const bisim_ctx* ctx) {
-    Buckets B;
-    B.class_list = ctx->class_list;
-    for (int c = 0; c <= kNumClasses; ++c) B.begin[c] = ctx->class_begin[c];
-    for (int c = 0; c < kNumClasses; ++c) B.edges[c] = ctx->class_edges[c];
-    B.hub_list = ctx->hub_list;
-    B.n_hub = ctx->n_hub;
-    B.chunks = ctx->chunks;
-    B.n_chunks = ctx->n_chunks;
-    B.toff = ctx->hub_toff;
-    B.tmask = ctx->hub_tmask;
-    B.tab = ctx->hub_tab;
-    B.tab_words = ctx->hub_tab_words;
-    B.acc = ctx->hub_acc;
-    return B;
 }
 
 bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
@@ -891,16 +873,6 @@ bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pi
     M.small_max = ctx->store_ready ? ctx->inc_small_max : ctx->opt.small_max_degree;
     M.mid_max = ctx->opt.mid_max_degree;
     return resolve(ctx, M, Pout, vlist, vcount, s, out_blocks);
-}
-
-bisim_status refine_round(bisim_ctx* ctx, cudaStream_t s, int64_t* out_blocks) {
-    const int32_t* P = ctx->P[ctx->cur];
-    pin_partition_in_l2(ctx, P, s);
-    bisim_status st = signature_round(ctx, ctx_buckets(ctx), P, ctx->P[ctx->cur ^ 1], nullptr, 0, nullptr, s,
-                                      out_blocks);
-    if (st != BISIM_OK) return st;
-    ctx->cur ^= 1;
-    return BISIM_OK;
 }
 
 void launch_local_ids(const bisim_ctx* ctx, int32_t* out, cudaStream_t s) {

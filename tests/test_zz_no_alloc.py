@@ -113,6 +113,56 @@ def test_noalloc_after_a_larger_call_left_the_array_dirty(B):
     _check_against_oracle(B, big)
 
 
+@pytest.mark.parametrize("wide", [False, True])
+def test_noalloc_rows_of_every_width(B, wide):
+    # rows around the widths at which a lane, a warp and a CTA take over, each twice
+    # with its entries repeated and in another order, and once with one entry changed;
+    # `wide`: a mean row beyond a lane's, which spreads the vertices over more warps
+    rng = np.random.default_rng(150)
+    widths = [0, 1, 2, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 128, 255, 256, 257, 500, 1024, 4000, 8190, 8192]
+    leaves = 200 if wide else 25_000
+    src, dst, lab = [], [], []
+    n = leaves
+    for w in widths:
+        t, l = rng.integers(0, leaves, w), rng.integers(0, 50, w)
+        if w >= 64:                                   # some of the entries are the same
+            t[: w // 3] = t[w // 2]
+            l[: w // 3] = l[w // 2]
+        for copy in range(3):
+            p = rng.permutation(w)
+            t2, l2 = t[p].copy(), l[p].copy()
+            if copy == 2 and w:
+                l2[rng.integers(0, w)] += 50
+            src.append(np.full(w, n)); dst.append(t2); lab.append(l2)
+            n += 1
+    g = dict(n=n, src=np.concatenate(src).astype(np.int32), dst=np.concatenate(dst).astype(np.int32),
+             elabel=np.concatenate(lab).astype(np.int32),
+             vlabel=np.concatenate([rng.integers(0, 40, leaves), np.zeros(n - leaves)]).astype(np.int32))
+    _check_against_oracle(B, g)
+
+
+def test_noalloc_resolves_colliding_hashes(B):
+    # labels of vertices without edges whose hashes share the table's fingerprint (the
+    # top 28 bits) and home slot (the low 17): the table merges them, and the
+    # confirmation has to take them apart again
+    def mix(z):
+        z ^= z >> np.uint64(30)
+        z *= np.uint64(0xbf58476d1ce4e5b9)
+        z ^= z >> np.uint64(27)
+        z *= np.uint64(0x94d049bb133111eb)
+        z ^= z >> np.uint64(31)
+        return z
+    h = mix(mix((np.arange(1 << 24, dtype=np.uint64) << np.uint64(32)) ^ np.uint64(0x13198a2e03707344)))
+    key = (h >> np.uint64(36) << np.uint64(17)) | (h & np.uint64(MAX_N * 2 - 1))
+    order = np.sort(key)
+    twice = order[1:][order[1:] == order[:-1]]
+    labels = np.flatnonzero(np.isin(key, twice))
+    assert len(twice) > 1 and len(labels) >= 2 * len(twice)
+    vl = np.tile(labels, 6).astype(np.int32)[np.random.default_rng(7).permutation(6 * len(labels))]
+    none = np.zeros(0, np.int32)
+    _check_against_oracle(B, dict(n=len(vl), src=none, dst=none, elabel=none, vlabel=vl))
+
+
 def _rejected(B, *args, match=None):
     with pytest.raises(B.BisimError) as ei:
         B.bisim_refine_round_noalloc(*args)
