@@ -150,145 +150,170 @@ __device__ __forceinline__ int dense_class(int64_t d, bool live, int small_max, 
 // class (k_layout_count), one exclusive sum of all of them, class by class
 // (counts first, then edges), and the placement (k_layout_place), which writes
 // the vertex, its position and its row offset at once. Both passes are bound by
-// the bytes they move (8 and 24 a vertex); sorting (class, vertex) pairs by radix
-// and collecting bounds, vertices, degrees and offsets in passes of their own
-// took 0.35 ms of the 10M-vertex build.
-constexpr int kLayoutTile = 1024;
+// the bytes they move (4 and 20 a vertex) as long as the instructions a vertex
+// stay few: sums and ranks taken class by class within each warp, for five or six
+// classes a warp, made them 87 and 152 us on 10M vertices; this way 28 and 59.
+constexpr int kLayoutThreads = 256;
+constexpr int kLayoutPer = 4;
+constexpr int kLayoutTile = kLayoutThreads * kLayoutPer;
+constexpr int kLayoutWarps = kLayoutThreads / 32;
 constexpr int kLayoutClasses = static_cast<int>(kDDead) + 1;
 struct LayoutBounds {
     int64_t edge[kDClasses + 1];                                     // first edge of each class; all of them
     int32_t pos[kDClasses + 1];                                      // first position of each class; the live ones' number
 };
 static_assert(sizeof(LayoutBounds) <= 256, "pinned blocks hold 256 bytes");
+static_assert(kLayoutClasses <= 32 && kLayoutTile * 32 <= 65536, "class and place in the tile in 16 bits");
 
-struct LayoutShared {
-    unsigned cnt[32][kLayoutClasses];                                // per warp, later exclusive over the warps
-    unsigned long long edges[32][kLayoutClasses];
-};
+// This thread's vertices of the tile: those of its lane in its warp's four runs of 32.
+__device__ __forceinline__ int64_t layout_vertex(int k) {
+    return static_cast<int64_t>(blockIdx.x) * kLayoutTile + (threadIdx.x >> 5) * 32 * kLayoutPer + k * 32 + lane_id();
+}
 
-// This thread's class; the warp's totals per class go to sh. RANK: also the
-// thread's rank among the warp's vertices of the class and the edges of those
-// before it. The sums are 32-bit unless the warp has a row that could overflow them.
-template <bool RANK>
-__device__ __forceinline__ int layout_tile(const int32_t* __restrict__ deg, const uint8_t* __restrict__ alive, int32_t n,
-                                           int small_max, int mid_max, LayoutShared& sh, unsigned* rank,
-                                           unsigned long long* before) {
-    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-    const int64_t v = static_cast<int64_t>(blockIdx.x) * kLayoutTile + threadIdx.x;
-    const int32_t d = v < n ? deg[v] : 0;
-    const int c = v < n ? dense_class(d, alive == nullptr || alive[v], small_max, mid_max) : kLayoutClasses;
-    if (lane < kLayoutClasses) {
-        sh.cnt[warp][lane] = 0u;
-        sh.edges[warp][lane] = 0ull;
-    }
-    __syncwarp();
-    const bool huge = __any_sync(0xffffffffu, static_cast<uint32_t>(d) >= 1u << 27);
-    for (unsigned todo = __ballot_sync(0xffffffffu, c < kLayoutClasses); todo;) {
-        const int lead = __ffs(todo) - 1;
-        const int lc = __shfl_sync(0xffffffffu, c, lead);
-        const unsigned same = __ballot_sync(0xffffffffu, c == lc);
-        unsigned long long sum;
-        if (huge) {
-            unsigned long long inc = c == lc ? static_cast<unsigned long long>(static_cast<int64_t>(d)) : 0ull;
+// Their degrees and classes (kLayoutClasses past the last vertex, and for what a
+// list that failed its check left as a degree: those vertices get no position).
+__device__ __forceinline__ void layout_load(const int32_t* __restrict__ deg, const uint8_t* __restrict__ alive, int32_t n,
+                                            int small_max, int mid_max, int32_t (&d)[kLayoutPer], int (&c)[kLayoutPer]) {
+    bool live[kLayoutPer];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= static_cast<unsigned>(o)) inc += y;
-            }
-            if (RANK && c == lc) *before = inc - static_cast<unsigned long long>(static_cast<int64_t>(d));
-            sum = __shfl_sync(0xffffffffu, inc, 31);
-        } else if (RANK) {
-            unsigned inc = c == lc ? static_cast<unsigned>(d) : 0u;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= static_cast<unsigned>(o)) inc += y;
-            }
-            if (c == lc) *before = inc - static_cast<unsigned>(d);
-            sum = __shfl_sync(0xffffffffu, inc, 31);
-        } else {
-            sum = __reduce_add_sync(0xffffffffu, c == lc ? static_cast<unsigned>(d) : 0u);
-        }
-        if (RANK && c == lc) *rank = static_cast<unsigned>(__popc(same & lanemask_lt()));
-        if (static_cast<int>(lane) == lead) {
-            sh.cnt[warp][lc] = static_cast<unsigned>(__popc(same));
-            sh.edges[warp][lc] = sum;
-        }
-        todo &= ~same;
+    for (int k = 0; k < kLayoutPer; ++k) {
+        const int64_t v = layout_vertex(k);
+        d[k] = v < n ? deg[v] : 0;
+        live[k] = v < n && (alive == nullptr || alive[v]);
     }
-    __syncthreads();
-    return c;
+#pragma unroll
+    for (int k = 0; k < kLayoutPer; ++k)
+        c[k] = layout_vertex(k) < n && d[k] >= 0 ? dense_class(d[k], live[k], small_max, mid_max) : kLayoutClasses;
 }
 
 // `skip` (nullable): nothing is done when the word is set.
-__global__ void __launch_bounds__(kLayoutTile) k_layout_count(const int32_t* __restrict__ deg,
-                                                              const uint8_t* __restrict__ alive, int32_t n, int small_max,
-                                                              int mid_max, int64_t tiles, int64_t* __restrict__ sums,
-                                                              const unsigned* skip) {
-    __shared__ LayoutShared sh;
+__global__ void __launch_bounds__(kLayoutThreads) k_layout_count(const int32_t* __restrict__ deg,
+                                                                 const uint8_t* __restrict__ alive, int32_t n, int small_max,
+                                                                 int mid_max, int64_t tiles, int64_t* __restrict__ sums,
+                                                                 const unsigned* skip) {
+    __shared__ unsigned cnt[32], low[32], high[32];                  // per class: vertices; edges as sums of half words
     if (skip != nullptr && *skip) return;
-    layout_tile<false>(deg, alive, n, small_max, mid_max, sh, nullptr, nullptr);
-    const unsigned warp = threadIdx.x >> 5;
-    if (warp < kLayoutClasses) {                                     // a warp per class
-        const unsigned cnt = __reduce_add_sync(0xffffffffu, sh.cnt[lane_id()][warp]);
-        unsigned long long e = sh.edges[lane_id()][warp];
+    if (threadIdx.x < 32) cnt[threadIdx.x] = low[threadIdx.x] = high[threadIdx.x] = 0u;
+    __syncthreads();
+    int32_t d[kLayoutPer];
+    int c[kLayoutPer];
+    layout_load(deg, alive, n, small_max, mid_max, d, c);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-        if (lane_id() == 0) {
-            sums[warp * tiles + blockIdx.x] = cnt;
-            sums[(kLayoutClasses + warp) * tiles + blockIdx.x] = static_cast<int64_t>(e);
+    for (int k = 0; k < kLayoutPer; ++k) {
+        const unsigned same = __match_any_sync(0xffffffffu, c[k]);
+        if (static_cast<int>(lane_id()) == __ffs(same) - 1) atomicAdd(&cnt[c[k]], static_cast<unsigned>(__popc(same)));
+        if (c[k] > 2 && d[k] != 0) {                                 // the rows of class 1 have one edge, those of 2 two
+            const unsigned x = static_cast<unsigned>(d[k]);
+            atomicAdd(&low[c[k]], x & 0xffffu);
+            if (x >> 16) atomicAdd(&high[c[k]], x >> 16);
         }
+    }
+    __syncthreads();
+    const unsigned q = threadIdx.x;
+    if (q < kLayoutClasses) {
+        const int64_t edges = q == 1 || q == 2 ? static_cast<int64_t>(q) * cnt[q]
+                                               : static_cast<int64_t>(low[q]) + (static_cast<int64_t>(high[q]) << 16);
+        sums[q * tiles + blockIdx.x] = cnt[q];
+        sums[(kLayoutClasses + q) * tiles + blockIdx.x] = edges;
     }
 }
 
-__global__ void __launch_bounds__(kLayoutTile) k_layout_place(const int32_t* __restrict__ deg,
-                                                              const uint8_t* __restrict__ alive, int32_t n, int small_max,
-                                                              int mid_max, int64_t tiles,
-                                                              const int64_t* __restrict__ sums,
-                                                              int32_t* __restrict__ vert, int32_t* __restrict__ vpos,
-                                                              int64_t* __restrict__ prp, LayoutBounds* __restrict__ bounds,
-                                                              const unsigned* skip) {
-    __shared__ LayoutShared sh;
-    __shared__ int64_t at[kLayoutClasses], eat[kLayoutClasses];
+// The tile's vertices go into class order in shared memory (ranks by match masks,
+// a warp's counts in its own row), where one sum over the degrees gives all row
+// offsets, and are written from there in runs.
+__global__ void __launch_bounds__(kLayoutThreads) k_layout_place(const int32_t* __restrict__ deg,
+                                                                 const uint8_t* __restrict__ alive, int32_t n, int small_max,
+                                                                 int mid_max, int64_t tiles,
+                                                                 const int64_t* __restrict__ sums,
+                                                                 int32_t* __restrict__ vert, int32_t* __restrict__ vpos,
+                                                                 int64_t* __restrict__ prp, LayoutBounds* __restrict__ bounds,
+                                                                 const unsigned* skip) {
+    __shared__ unsigned cnt[kLayoutWarps][32];                       // per warp, later those of the warps before it
+    __shared__ unsigned first[32];                                   // a class's first place in the tile
+    __shared__ int64_t at[32], eat[32];                              // its first position and edge
+    __shared__ __align__(16) int32_t sdeg[kLayoutTile];
+    __shared__ uint16_t who[kLayoutTile];                            // class, place among the tile's vertices
+    __shared__ int64_t edge[kLayoutTile];                            // edges of the tile before each place
+    __shared__ int64_t wsum[kLayoutWarps];
     if (skip != nullptr && *skip) return;
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     if (threadIdx.x < kLayoutClasses) {
         at[threadIdx.x] = sums[threadIdx.x * tiles + blockIdx.x];
         eat[threadIdx.x] = sums[(kLayoutClasses + threadIdx.x) * tiles + blockIdx.x] - n;   // the counts come first: n of them
     }
-    unsigned rank = 0u;
-    unsigned long long before = 0ull;
-    const int c = layout_tile<true>(deg, alive, n, small_max, mid_max, sh, &rank, &before);
-    const unsigned warp = threadIdx.x >> 5, lane = lane_id();
-    if (warp < kLayoutClasses) {                                     // a warp per class: exclusive over the 32 warps
-        const unsigned x = sh.cnt[lane][warp];
-        const unsigned long long e = sh.edges[lane][warp];
-        unsigned xi = x;
-        unsigned long long ei = e;
+    cnt[warp][lane] = 0u;
+    int32_t d[kLayoutPer];
+    int c[kLayoutPer];
+    layout_load(deg, alive, n, small_max, mid_max, d, c);
+    __syncwarp();
+    unsigned rank[kLayoutPer];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, xi, o);
-            const unsigned long long z = __shfl_up_sync(0xffffffffu, ei, o);
-            if (lane >= static_cast<unsigned>(o)) {
-                xi += y;
-                ei += z;
-            }
-        }
-        sh.cnt[lane][warp] = xi - x;
-        sh.edges[lane][warp] = ei - e;
+    for (int k = 0; k < kLayoutPer; ++k) {
+        const unsigned same = __match_any_sync(0xffffffffu, c[k]);
+        const unsigned before = cnt[warp][c[k]];
+        rank[k] = before + static_cast<unsigned>(__popc(same & lanemask_lt()));
+        __syncwarp();
+        if (static_cast<int>(lane) == __ffs(same) - 1) cnt[warp][c[k]] = before + static_cast<unsigned>(__popc(same));
+        __syncwarp();
     }
     __syncthreads();
-    if (c < kLayoutClasses) {
-        const int64_t v = static_cast<int64_t>(blockIdx.x) * kLayoutTile + threadIdx.x;
-        const int64_t p = at[c] + sh.cnt[warp][c] + rank;
-        vert[p] = static_cast<int32_t>(v);
-        vpos[v] = static_cast<int32_t>(p);
-        if (c != static_cast<int>(kDDead)) prp[p] = eat[c] + static_cast<int64_t>(sh.edges[warp][c] + before);
+    if (warp == 0) {                                                 // a lane per class, the padding last
+        unsigned total = 0u;
+#pragma unroll
+        for (int w = 0; w < kLayoutWarps; ++w) {
+            const unsigned x = cnt[w][lane];
+            cnt[w][lane] = total;
+            total += x;
+        }
+        unsigned inc = total;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= static_cast<unsigned>(o)) inc += y;
+        }
+        first[lane] = inc - total;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kLayoutPer; ++k) {
+        const unsigned p = first[c[k]] + cnt[warp][c[k]] + rank[k];
+        sdeg[p] = d[k];
+        who[p] = static_cast<uint16_t>(c[k] * kLayoutTile + static_cast<int>(warp * 32 * kLayoutPer + k * 32 + lane));
+    }
+    __syncthreads();
+    const int4 x = reinterpret_cast<const int4*>(sdeg)[threadIdx.x];
+    const int64_t s1 = x.x, s2 = s1 + x.y, s3 = s2 + x.z, s4 = s3 + x.w;
+    int64_t inc = s4;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= static_cast<unsigned>(o)) inc += y;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int64_t base = inc - s4;
+    for (unsigned w = 0; w < warp; ++w) base += wsum[w];
+    edge[threadIdx.x * kLayoutPer] = base;
+    edge[threadIdx.x * kLayoutPer + 1] = base + s1;
+    edge[threadIdx.x * kLayoutPer + 2] = base + s2;
+    edge[threadIdx.x * kLayoutPer + 3] = base + s3;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kLayoutPer; ++k) {
+        const unsigned p = k * kLayoutThreads + threadIdx.x;
+        const unsigned q = who[p] / kLayoutTile;
+        if (q >= kLayoutClasses) continue;
+        const int64_t v = static_cast<int64_t>(blockIdx.x) * kLayoutTile + who[p] % kLayoutTile;
+        const int64_t to = at[q] + (p - first[q]);
+        vert[to] = static_cast<int32_t>(v);
+        vpos[v] = static_cast<int32_t>(to);
+        if (q != kDDead) prp[to] = eat[q] + (edge[p] - edge[first[q]]);
     }
     if (blockIdx.x == 0 && threadIdx.x <= kDClasses) {
-        const int64_t first = sums[threadIdx.x * tiles], e = sums[(kLayoutClasses + threadIdx.x) * tiles] - n;
-        bounds->pos[threadIdx.x] = static_cast<int32_t>(first);
+        const int64_t begin = sums[threadIdx.x * tiles], e = sums[(kLayoutClasses + threadIdx.x) * tiles] - n;
+        bounds->pos[threadIdx.x] = static_cast<int32_t>(begin);
         bounds->edge[threadIdx.x] = e;
-        if (threadIdx.x == kDClasses) prp[first] = e;                // the end of the last live row
+        if (threadIdx.x == kDClasses) prp[begin] = e;                // the end of the last live row
     }
 }
 
@@ -1910,12 +1935,12 @@ bisim_status dense_layout_positions(bisim_ctx* ctx, const int32_t* deg, cudaStre
     const int sm = ctx->opt.small_max_degree, mm = ctx->opt.mid_max_degree;
     {
         Launch L(site_c, s, n, 0, 4.0 * n);
-        k_layout_count<<<static_cast<unsigned>(tiles), kLayoutTile, 0, s>>>(deg, ctx->alive, n, sm, mm, tiles, tsum, skip);
+        k_layout_count<<<static_cast<unsigned>(tiles), kLayoutThreads, 0, s>>>(deg, ctx->alive, n, sm, mm, tiles, tsum, skip);
     }
     exclusive_scan_i64(tsum, tsum, len, tsum + len, s);
     {
         Launch L(site_c, s, n, 0, 20.0 * n);
-        k_layout_place<<<static_cast<unsigned>(tiles), kLayoutTile, 0, s>>>(deg, ctx->alive, n, sm, mm, tiles, tsum, ctx->dvert,
+        k_layout_place<<<static_cast<unsigned>(tiles), kLayoutThreads, 0, s>>>(deg, ctx->alive, n, sm, mm, tiles, tsum, ctx->dvert,
                                                                            ctx->dvpos, ctx->dprp, dbounds, skip);
     }
     cudaMemcpyAsync(h, dbounds, sizeof(LayoutBounds), cudaMemcpyDeviceToHost, s);
