@@ -294,38 +294,27 @@ bisim_status finish_init(bisim_ctx* ctx, cudaStream_t s) {
     return BISIM_OK;
 }
 
-__global__ void k_globalize(const int64_t* __restrict__ voff, const int64_t* __restrict__ eoff, int32_t G,
-                            const int32_t* __restrict__ sl, const int32_t* __restrict__ dl, int64_t m,
-                            int32_t* __restrict__ src, int32_t* __restrict__ dst, unsigned* err) {
-    for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < m;
-         e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        int lo = 0, hi = G - 1;   // graph g with eoff[g] <= e < eoff[g+1]
+// The graph of every vertex, four vertices a thread; a warp's 128 are looked up once.
+__global__ void __launch_bounds__(256) k_graph_ids(const int64_t* __restrict__ voff, int32_t G, int32_t n,
+                                                   int32_t* __restrict__ gid) {
+    const auto graph_of = [&](int64_t v, int32_t lo, int32_t hi) {
         while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (eoff[mid] <= e) lo = mid; else hi = mid - 1;
+            const int32_t mid = lo + (hi - lo + 1) / 2;
+            if (voff[mid] <= v) lo = mid; else hi = mid - 1;
         }
-        const int64_t ng = voff[lo + 1] - voff[lo];
-        const int32_t a = sl[e], b = dl[e];
-        if (a < 0 || a >= ng || b < 0 || b >= ng) {
-            atomicOr(err, kErrBadInput);
-            src[e] = 0;
-            dst[e] = 0;
-        } else {
-            src[e] = static_cast<int32_t>(voff[lo] + a);
-            dst[e] = static_cast<int32_t>(voff[lo] + b);
-        }
+        return lo;
+    };
+    const int64_t v0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 4;
+    const int64_t w0 = v0 - 4 * (threadIdx.x & 31u), w1 = min(w0 + 127, static_cast<int64_t>(n) - 1);
+    if (w0 >= n) return;
+    const int32_t glo = graph_of(w0, 0, G - 1), ghi = graph_of(w1, glo, G - 1);
+    if (v0 >= n) return;
+    if (v0 + 4 <= n) {
+        reinterpret_cast<int4*>(gid)[v0 / 4] =
+            make_int4(graph_of(v0, glo, ghi), graph_of(v0 + 1, glo, ghi), graph_of(v0 + 2, glo, ghi), graph_of(v0 + 3, glo, ghi));
+    } else {
+        for (int64_t v = v0; v < n; ++v) gid[v] = graph_of(v, glo, ghi);
     }
-}
-
-__global__ void k_graph_ids(const int64_t* __restrict__ voff, int32_t G, int32_t n, int32_t* __restrict__ gid) {
-    const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    int lo = 0, hi = G - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (voff[mid] <= v) lo = mid; else hi = mid - 1;
-    }
-    gid[v] = lo;
 }
 
 }  // namespace
@@ -721,26 +710,19 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
     if (st == BISIM_OK) {
         cudaMemcpyAsync(ctx->voff, hv.data(), sizeof(int64_t) * (n_graphs + 1), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(deoff, he.data(), sizeof(int64_t) * (n_graphs + 1), cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(&ctx->dstate->error, 0, sizeof(unsigned), s);
         BISIM_SITE(site_g, "batch_graph_ids");
-        BISIM_SITE(site_e, "batch_globalize");
         if (n > 0)
             Launch(site_g, s, n, 0, 4.0 * n),
-            k_graph_ids<<<(n + 255) / 256, 256, 0, s>>>(ctx->voff, n_graphs, n, ctx->gid);
-        if (m > 0)
-            Launch(site_e, s, 0, m, 16.0 * m),
-            k_globalize<<<static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 1 << 16)), 256, 0, s>>>(
-                ctx->voff, deoff, n_graphs, static_cast<const int32_t*>(ds), static_cast<const int32_t*>(dd), m,
-                gsrc, gdst, &ctx->dstate->error);
-        cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
-        if ((e = cudaStreamSynchronize(s))) st = cuda_error(ctx, e, "globalize batched edges");
-        else if (ctx->hstate->error & kErrBadInput) st = set_error(ctx, BISIM_EINVAL, "a graph-local edge endpoint is out of range");
+            k_graph_ids<<<(n + 1023) / 1024, 256, 0, s>>>(ctx->voff, n_graphs, n, ctx->gid);
     }
+    const BatchedList batch{ctx->voff, deoff, n_graphs, gsrc, gdst};
+    const int32_t* ls = static_cast<const int32_t*>(ds);
+    const int32_t* ld = static_cast<const int32_t*>(dd);
     EdgeView view;
     const int32_t* bl = static_cast<const int32_t*>(dl);
     if (st == BISIM_OK && !edge_view_identity(ctx)) {
         // another direction or a label filter: the view keeps every graph's edges together
-        if ((st = edge_view_coo(ctx, gsrc, gdst, bl, m, deoff, n_graphs, s, &view)) == BISIM_OK) {
+        if ((st = globalize_edges(ctx, batch, ls, ld, s)) == BISIM_OK && (st = edge_view_coo(ctx, gsrc, gdst, bl, m, deoff, n_graphs, s, &view)) == BISIM_OK) {
             ctx->m = view.m;
             if ((e = cudaMemcpyAsync(he.data(), view.eoff, sizeof(int64_t) * (n_graphs + 1), cudaMemcpyDeviceToHost, s)) ||
                 (e = cudaStreamSynchronize(s)))
@@ -748,7 +730,8 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
         }
     }
     if (st == BISIM_OK)
-        st = build_from_coo(ctx, view.src ? view.src : gsrc, view.src ? view.dst : gdst, view.src ? view.lab : bl, s);
+        st = view.src ? build_from_coo(ctx, view.src, view.dst, view.lab, s)
+                      : build_from_coo(ctx, ls, ld, bl, s, nullptr, &batch);
     edge_view_free(&view, s);
     if (st == BISIM_OK) st = dense_region_table(ctx, hv.data(), n_graphs, s);
     if (st == BISIM_OK) st = segment_init(ctx, hv.data(), he.data(), n_graphs, s);

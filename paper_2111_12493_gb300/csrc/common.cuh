@@ -473,8 +473,21 @@ struct CooArrival {
     void (*arrived)(void*) = nullptr;
     void* arrived_arg = nullptr;
 };
+// A batch of graphs (device offsets of their vertices and edges in the union), whose
+// edges name graph-local ids; src and dst receive the union's.
+struct BatchedList {
+    const int64_t* voff;
+    const int64_t* eoff;
+    int32_t n_graphs;
+    int32_t* src;
+    int32_t* dst;
+};
 bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* dst,
-                            const int32_t* elab, cudaStream_t s, const CooArrival* arrival = nullptr);
+                            const int32_t* elab, cudaStream_t s, const CooArrival* arrival = nullptr,
+                            const BatchedList* batch = nullptr);
+// Only the check of graph-local ids and the union's ids.
+bisim_status globalize_edges(bisim_ctx* ctx, const BatchedList& batch, const int32_t* src, const int32_t* dst,
+                             cudaStream_t s);
 bisim_status build_from_csr(bisim_ctx* ctx, const int64_t* row_ptr, const int32_t* col,
                             const int32_t* elab, cudaStream_t s);
 

@@ -111,6 +111,108 @@ __global__ void __launch_bounds__(256) k_validate_coo(const int32_t* __restrict_
     }
 }
 
+// The graph of edge e, known to lie in [lo, hi].
+__device__ __forceinline__ int32_t graph_of(const int64_t* __restrict__ eoff, int64_t e, int32_t lo, int32_t hi) {
+    while (lo < hi) {
+        const int32_t mid = lo + (hi - lo + 1) / 2;
+        if (eoff[mid] <= e) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// The same for a batched list, whose edges name vertices of their own graph: the
+// union's ids are written to B.src and B.dst on the way (deg null: only those, and
+// the check). A warp's 128 edges are looked up once: unless a graph ends among
+// them, all have the offset of one graph. (A search over all graphs for every
+// edge, in a pass before the check: 219 and 77 us for the 37M edges of 512 graphs.)
+__global__ void __launch_bounds__(256) k_validate_local(const BatchedList B, const int32_t* __restrict__ src,
+                                                        const int32_t* __restrict__ dst, int64_t m,
+                                                        uint32_t* __restrict__ deg, int64_t* __restrict__ start, DevState* st,
+                                                        bool wide) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t quads = (m + 3) / 4;
+    const int64_t lane = threadIdx.x & 31u;
+    bool unsorted = false;
+    unsigned turn = 0;
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q - lane < quads; q += stride) {
+        const int64_t e0 = 4 * q;
+        int32_t s[6] = {-1, -1, -1, -1, -1, -1}, d[4] = {0, 0, 0, 0};    // s[0] and s[5]: the sources beside the four
+        if (wide && e0 + 4 <= m) {
+            const int4 x = __ldcs(reinterpret_cast<const int4*>(src + e0));
+            const int4 y = __ldcs(reinterpret_cast<const int4*>(dst + e0));
+            s[1] = x.x;
+            s[2] = x.y;
+            s[3] = x.z;
+            s[4] = x.w;
+            d[0] = y.x;
+            d[1] = y.y;
+            d[2] = y.z;
+            d[3] = y.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (e0 + k >= m) break;
+                s[k + 1] = src[e0 + k];
+                d[k] = dst[e0 + k];
+            }
+        }
+        if (e0 > 0 && e0 <= m) s[0] = src[e0 - 1];
+        if (e0 + 4 < m) s[5] = src[e0 + 4];
+        const int64_t w0 = 4 * (q - lane), w1 = min(w0 + 128, m - 1);    // the warp's edges and the one after
+        const int32_t glo = graph_of(B.eoff, max(w0 - 1, int64_t{0}), 0, B.n_graphs - 1);
+        const int32_t ghi = B.eoff[glo + 1] > w1 ? glo : graph_of(B.eoff, w1, glo, B.n_graphs - 1);
+        int64_t first[6], size[6];
+        if (glo == ghi) {
+            const int64_t f = B.voff[glo], z = B.voff[glo + 1] - f;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                first[k] = f;
+                size[k] = z;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int32_t g = graph_of(B.eoff, min(max(e0 + k - 1, int64_t{0}), m - 1), glo, ghi);
+                first[k] = B.voff[g];
+                size[k] = B.voff[g + 1] - first[k];
+            }
+        }
+        if (++turn <= 2u || (turn & 7u) == 0u) unsorted = cached_flag(&st->unsorted);
+        bool bad = false, back = false;
+        int32_t v[6], t[4];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = s[k] < 0 ? -1 : static_cast<int32_t>(first[k] + s[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool ok = s[k + 1] >= 0 && s[k + 1] < size[k + 1] && d[k] >= 0 && d[k] < size[k + 1];
+            t[k] = ok ? static_cast<int32_t>(first[k + 1] + d[k]) : -1;
+            if (e0 + k >= m) continue;
+            bad = bad || !ok;
+            if (!ok || unsorted || deg == nullptr) continue;
+            const int32_t x = v[k + 1];
+            back = back || v[k] > x;
+            if (v[k] != x) {
+                start[x] = e0 + k;
+                atomicAdd(&deg[x], 0u - static_cast<uint32_t>(e0 + k));
+            }
+            if (v[k + 2] != x) atomicAdd(&deg[x], static_cast<uint32_t>(e0 + k + 1));
+        }
+        if (e0 + 4 <= m) {
+            *reinterpret_cast<int4*>(B.src + e0) = make_int4(v[1], v[2], v[3], v[4]);
+            *reinterpret_cast<int4*>(B.dst + e0) = make_int4(t[0], t[1], t[2], t[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (e0 + k >= m) break;
+                B.src[e0 + k] = v[k + 1];
+                B.dst[e0 + k] = t[k];
+            }
+        }
+        if (bad) atomicOr(&st->error, kErrBadInput);
+        if (back) *reinterpret_cast<volatile unsigned*>(&st->unsorted) = 1u;
+    }
+}
+
 // The targets' check of a list whose sources k_validate_coo checked alone.
 __global__ void __launch_bounds__(256) k_validate_dst(const int32_t* __restrict__ dst, int64_t m, int32_t n,
                                                       const uint8_t* __restrict__ alive, DevState* st) {
@@ -304,7 +406,31 @@ __global__ void k_validate_csr(const int64_t* __restrict__ rp, const int32_t* __
     }
 }
 
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+void launch_validate_local(bisim_ctx* ctx, const BatchedList& B, const int32_t* src, const int32_t* dst, uint32_t* deg,
+                           int64_t* start, cudaStream_t s) {
+    const int64_t m = ctx->m;
+    if (m <= 0) return;
+    BISIM_SITE(site, "batch_globalize");
+    Launch L(site, s, 0, m, 16.0 * m);
+    k_validate_local<<<grid_for(std::min<int64_t>(cdiv(m, 4), 1 << 22), 256), 256, 0, s>>>(
+        B, src, dst, m, deg, start, ctx->dstate, aligned16(src) && aligned16(dst));
+}
+
 }  // namespace
+
+bisim_status globalize_edges(bisim_ctx* ctx, const BatchedList& batch, const int32_t* src, const int32_t* dst,
+                             cudaStream_t s) {
+    cudaMemsetAsync(&ctx->dstate->error, 0, sizeof(unsigned), s);
+    launch_validate_local(ctx, batch, src, dst, nullptr, nullptr, s);
+    cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
+    cudaError_t e;
+    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "globalize batched edges");
+    if (ctx->hstate->error & kErrBadInput)
+        return set_error(ctx, BISIM_EINVAL, "a graph-local edge endpoint is out of range");
+    return BISIM_OK;
+}
 
 // COO -> the round layout directly: out-degrees, then the positions of the
 // layout (vertices grouped by degree class) and their row offsets, then every
@@ -312,7 +438,8 @@ __global__ void k_validate_csr(const int64_t* __restrict__ rp, const int32_t* __
 // are the layout's packed rows; the vertex-ordered CSR is rebuilt from them
 // only if an update or the list-mode path asks for it.
 bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* dst,
-                            const int32_t* elab, cudaStream_t s, const CooArrival* arrival) {
+                            const int32_t* elab, cudaStream_t s, const CooArrival* arrival,
+                            const BatchedList* batch) {
     const int32_t n = ctx->n;
     const int64_t m = ctx->m;
     const int64_t cap = std::max<int64_t>(m, 1);
@@ -341,11 +468,15 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
     BISIM_SITE(site_pack, "csr_place");
     const unsigned grid = grid_for(std::min<int64_t>(m, 1 << 22), 256);
     const unsigned tile_grid = static_cast<unsigned>(std::min<int64_t>(cdiv(m, kTileEdges), 152 * 8));
-    const bool wide = (reinterpret_cast<uintptr_t>(src) & 15u) == 0 && (arrival || (reinterpret_cast<uintptr_t>(dst) & 15u) == 0);
+    const bool wide = aligned16(src) && (arrival || aligned16(dst));
     // arriving arrays: the sources are checked and counted while the targets
     // and labels are still being copied in
     if (arrival != nullptr) cudaStreamWaitEvent(s, arrival->src, 0);
-    if (m > 0)
+    if (batch != nullptr) {
+        launch_validate_local(ctx, *batch, src, dst, deg, start, s);
+        src = batch->src;
+        dst = batch->dst;
+    } else if (m > 0)
         Launch(site_val, s, 0, m, arrival ? 4.0 * m : 8.0 * m),
         k_validate_coo<<<grid_for(std::min<int64_t>(cdiv(m, 4), 1 << 22), 256), 256, 0, s>>>(
             src, arrival ? nullptr : dst, m, n, ctx->alive, deg, start, ctx->dstate, wide);
@@ -355,7 +486,8 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
     bisim_status st = dense_layout_positions(ctx, reinterpret_cast<const int32_t*>(deg), s, &ctx->dstate->unsorted);
     if (st == BISIM_OK && (ctx->hstate->error & kErrBadInput))
-        st = set_error(ctx, BISIM_EINVAL, "edge endpoint out of range [0, n) or on a dead vertex");
+        st = set_error(ctx, BISIM_EINVAL, batch ? "a graph-local edge endpoint is out of range"
+                                                : "edge endpoint out of range [0, n) or on a dead vertex");
     const bool sorted = ctx->hstate->unsorted == 0;
     if (st == BISIM_OK && !sorted && m > 0) {
         cudaMemsetAsync(deg, 0, sizeof(uint32_t) * nv, s);

@@ -589,12 +589,19 @@ __global__ void __launch_bounds__(kDeferThreads) k_verify_deferred(const int32_t
     }
 }
 
-__global__ void k_local_ids(const int32_t* __restrict__ P, const int32_t* __restrict__ gid,
-                            const int64_t* __restrict__ voff, int32_t n, int32_t* __restrict__ out) {
-    const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const int32_t p = P[v];
-    out[v] = p < 0 ? -1 : static_cast<int32_t>(p - voff[gid[v]]);
+// Graph-local ids of the blocks, four vertices a thread where `out` takes 16-byte
+// stores (`wide`).
+__global__ void __launch_bounds__(256) k_local_ids(const int32_t* __restrict__ P, const int32_t* __restrict__ gid,
+                                                   const int64_t* __restrict__ voff, int32_t n, int32_t* __restrict__ out,
+                                                   bool wide) {
+    const int64_t v0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 4;
+    const auto local = [&](int32_t p, int32_t g) { return p < 0 ? -1 : static_cast<int32_t>(p - voff[g]); };
+    if (wide && v0 + 4 <= n) {
+        const int4 p = *reinterpret_cast<const int4*>(P + v0), g = *reinterpret_cast<const int4*>(gid + v0);
+        *reinterpret_cast<int4*>(out + v0) = make_int4(local(p.x, g.x), local(p.y, g.y), local(p.z, g.z), local(p.w, g.w));
+    } else {
+        for (int64_t v = v0; v < v0 + 4 && v < n; ++v) out[v] = local(P[v], gid[v]);
+    }
 }
 
 // ----------------------------------------------------------------------------- host side
@@ -879,7 +886,8 @@ void launch_local_ids(const bisim_ctx* ctx, int32_t* out, cudaStream_t s) {
     BISIM_SITE(site, "local_ids");
     Launch L(site, s, ctx->n, 0, 8.0 * ctx->n);
     if (ctx->n > 0)
-        k_local_ids<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->P[ctx->cur], ctx->gid, ctx->voff, ctx->n, out);
+        k_local_ids<<<grid_for(cdiv(ctx->n, 4), 256), 256, 0, s>>>(ctx->P[ctx->cur], ctx->gid, ctx->voff, ctx->n, out,
+                                                                  (reinterpret_cast<uintptr_t>(out) & 15u) == 0);
 }
 
 }  // namespace bisim

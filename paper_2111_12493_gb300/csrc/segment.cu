@@ -648,9 +648,12 @@ bisim_status segment_queue(bisim_ctx* ctx, int32_t split, cudaStream_t s) {
         else big[g] = 1;
     }
     ctx->seg_n_small = static_cast<int32_t>(queue.size());
-    if (!queue.empty())
-        cudaMemcpyAsync(ctx->seg_order, queue.data(), sizeof(int32_t) * queue.size(), cudaMemcpyHostToDevice, s);
-    if (G > 0) cudaMemcpyAsync(ctx->seg_big, big.data(), G, cudaMemcpyHostToDevice, s);
+    if (queue.empty()) {                              // nothing reads the flags: the union's rounds take every graph
+        ctx->seg_split = split;
+        return BISIM_OK;
+    }
+    cudaMemcpyAsync(ctx->seg_order, queue.data(), sizeof(int32_t) * queue.size(), cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ctx->seg_big, big.data(), G, cudaMemcpyHostToDevice, s);
     cudaError_t e;
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "upload graph queue");   // the host vectors die here
     ctx->seg_split = split;
@@ -670,6 +673,25 @@ bisim_status segment_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t
     cudaError_t e;
     bisim_status pst = dense_prepare(ctx, s);        // the rows in the round layout (built by init)
     if (pst != BISIM_OK) return pst;
+    bisim_status st;
+    if ((st = segment_queue(ctx, ctx->opt.batch_split, s)) != BISIM_OK) return st;
+    const int32_t n_small = ctx->seg_n_small;
+    const bool any_big = n_small < ctx->n_graphs;
+    if (any_big && (n_small == 0 || limit <= 0)) {
+        // every graph above the split: the union's round kernels alone
+        int64_t blocks = 0;
+        int32_t rounds = 0, executed = 0;
+        if ((st = dense_rounds_all(ctx, k, cap, s, &rounds, &executed, &blocks, true)) != BISIM_OK) return st;
+        ctx->cur_k = rounds;
+        ctx->stats.rounds = rounds;
+        ctx->stats.rounds_executed = executed;
+        ctx->stats.num_blocks = blocks;
+        *out_rounds = rounds;
+        *out_executed = executed;
+        *out_blocks = blocks;
+        return BISIM_OK;
+    }
+    // state of the persistent kernel
     if (ctx->seg_hash == nullptr) {
         const size_t nv = static_cast<size_t>(std::max(n, 1));
         if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->seg_hash), sizeof(unsigned long long) * nv, s)) ||
@@ -693,24 +715,6 @@ bisim_status segment_rounds(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t
         k_seg_rows<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(ctx->dvpos, ctx->dprp, n, ctx->seg_e0,
                                                                          ctx->seg_deg);
         ctx->seg_rows_version = ctx->layout_version;
-    }
-    bisim_status st;
-    if ((st = segment_queue(ctx, ctx->opt.batch_split, s)) != BISIM_OK) return st;
-    const int32_t n_small = ctx->seg_n_small;
-    const bool any_big = n_small < ctx->n_graphs;
-    if (any_big && (n_small == 0 || limit <= 0)) {
-        // every graph above the split: the union's round kernels alone
-        int64_t blocks = 0;
-        int32_t rounds = 0, executed = 0;
-        if ((st = dense_rounds_all(ctx, k, cap, s, &rounds, &executed, &blocks, true)) != BISIM_OK) return st;
-        ctx->cur_k = rounds;
-        ctx->stats.rounds = rounds;
-        ctx->stats.rounds_executed = executed;
-        ctx->stats.num_blocks = blocks;
-        *out_rounds = rounds;
-        *out_executed = executed;
-        *out_blocks = blocks;
-        return BISIM_OK;
     }
     // graphs above the split (if any) go through the union's round kernels on
     // the caller's stream while the persistent kernel takes the others on a

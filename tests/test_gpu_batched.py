@@ -255,3 +255,34 @@ def test_autotune_picks_a_listed_split_and_keeps_results(B):
         assert (rounds, blocks) == (wr, wb)
     finally:
         B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("off", [0, 1, 3])
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_local_edges_around_graph_ends(B, off, shuffled):
+    # graphs of no, few and more edges than a thread's four or a warp's 128, vertices
+    # without a graph's edges, arrays at other alignments, edges in any order
+    rng = np.random.default_rng(31 + off)
+    graphs = []
+    for n, m in [(1, 0), (3, 1), (2, 3), (5, 0), (7, 4), (200, 127), (1, 130), (300, 129), (2, 1), (40, 900), (1, 0), (9, 3)]:
+        src = rng.integers(0, n, m)
+        graphs.append((n, src if shuffled else np.sort(src), rng.integers(0, n, m), rng.integers(0, 3, m), rng.integers(0, 2, n)))
+    b = _concat(graphs)
+    shift = lambda a, k: _dev(np.concatenate([np.full(k, 1, np.int32), a]))[k:]
+    def init(b):
+        return B.summarize_init_batched(_dev(b["vertex_offsets"]), _dev(b["edge_offsets"]), shift(b["src_local"], off),
+                                        shift(b["dst_local"], (off * 2) % 4), _dev(b["elabel"]), _dev(b["vlabel"]))
+    want, _, _ = oracle_batched(b, 2)
+    ctx = init(b)
+    B.bisim_iterate(ctx, 2)
+    _same(B.get_partition(ctx).cpu().numpy(), want, "local edges")
+    B.summarize_destroy(ctx)
+    # an id of the next graph, at either end of a graph's edges
+    for g in (2, 5, 9):
+        for e in (b["edge_offsets"][g], b["edge_offsets"][g + 1] - 1):
+            for name in ("src_local", "dst_local"):
+                bad = dict(b)
+                bad[name] = b[name].copy()
+                bad[name][e] = graphs[g][0]
+                with pytest.raises(B.BisimError, match="graph-local"):
+                    init(bad)
