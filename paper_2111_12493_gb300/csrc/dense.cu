@@ -398,55 +398,78 @@ __global__ void k_unpack_big(const int32_t* __restrict__ vert, int64_t first, co
     }
 }
 
-// Rows of out-degree <= 256: one warp per 32 consecutive positions. The warp's
-// output range is contiguous, so it is written word by word across the lanes;
-// each word finds its source row by a binary search over the warp's 33 row
-// offsets in shared memory.
-__global__ void __launch_bounds__(256) k_dense_pack_rows(const int32_t* __restrict__ vert, int64_t count,
+// Rows of out-degree <= 256. Positions before `split` (the thread classes): a warp
+// per 32 consecutive ones, whose rows are about equally long (they lie in class
+// order) and of at most 32 edges: eight lanes a row, sixteen rows' loads in flight
+// in the warp. From `split` on a warp per kPackLong rows, one after the other.
+// (Writing the warp's contiguous range word by word, each word's row found by
+// a binary search over the 33 offsets, took 77 us for 4M edges in 400k rows; this
+// takes 13, and 37 with 32 of the longer rows a warp.)
+constexpr int kPackLong = 2;
+__global__ void __launch_bounds__(256) k_dense_pack_rows(const int32_t* __restrict__ vert, int64_t split, int64_t count,
                                                          const int64_t* __restrict__ prp,
                                                          const int64_t* __restrict__ rp,
                                                          const int32_t* __restrict__ col,
                                                          const int32_t* __restrict__ elab,
                                                          unsigned long long* __restrict__ pe) {
-    __shared__ int64_t off_all[8][33];
-    __shared__ int64_t src_all[8][32];
-    const int warp = threadIdx.x >> 5;
-    const unsigned lane = lane_id();
-    const int64_t p0 = (static_cast<int64_t>(blockIdx.x) * 8 + warp) * 32;
-    if (p0 >= count) return;                             // whole warp leaves together
-    int64_t* off = off_all[warp];
-    int64_t* src = src_all[warp];
-    const int64_t pend = min(count, p0 + 32);
-    const int64_t p = p0 + lane;
-    const bool act = p < count;
-    off[lane] = prp[act ? p : pend];                     // rows past the end start at the end
-    if (lane == 0) off[32] = prp[pend];
-    src[lane] = act ? rp[vert[p]] : 0;
-    __syncwarp();
-    const int64_t o1 = off[32];
-    constexpr int kAtOnce = 4;                           // words a lane looks up before it loads any of them
-    for (int64_t o = off[0] + lane; o < o1; o += 32 * kAtOnce) {
-        int64_t e[kAtOnce];
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kAtOnce = 4;
+    const int lane = static_cast<int>(lane_id());
+    const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / 32, shorts = (split + 31) / 32;
+    const bool long_rows = w >= shorts;                  // the same for the whole warp
+    const int rows = long_rows ? kPackLong : 32;
+    const int64_t first = long_rows ? split + (w - shorts) * kPackLong : w * 32;
+    const int64_t end = long_rows ? count : split, p = first + lane;
+    if (first >= end) return;
+    int64_t to = 0, from = 0;
+    int d = 0;
+    if (lane < rows && p < end) {
+        to = prp[p];
+        d = static_cast<int>(prp[p + 1] - to);
+        from = rp[vert[p]];
+    }
+    if (!long_rows) {
+        const int widest = __reduce_max_sync(kAll, d);
+        const int sub = lane & 7;
+        for (int r0 = 0; r0 < 8; r0 += kAtOnce) {
+            int64_t f[kAtOnce], t[kAtOnce];
+            int n[kAtOnce];
 #pragma unroll
-        for (int k = 0; k < kAtOnce; ++k) {
-            const int64_t w = o + 32 * k;
-            int lo = 0, hi = 31;                         // the last row starting at or before w
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (off[mid] <= w) lo = mid; else hi = mid - 1;
+            for (int k = 0; k < kAtOnce; ++k) {
+                const int row = (r0 + k) * 4 + (lane >> 3);
+                f[k] = __shfl_sync(kAll, from, row);
+                t[k] = __shfl_sync(kAll, to, row);
+                n[k] = __shfl_sync(kAll, d, row);
             }
-            e[k] = src[lo] + (w - off[lo]);
-        }
-        int32_t l[kAtOnce], t[kAtOnce];
+            for (int j = sub; j < widest; j += 8) {
+                int32_t c[kAtOnce], l[kAtOnce];
 #pragma unroll
-        for (int k = 0; k < kAtOnce; ++k) {
-            if (o + 32 * k >= o1) break;
-            l[k] = __ldcs(elab + e[k]);
-            t[k] = __ldcs(col + e[k]);
-        }
+                for (int k = 0; k < kAtOnce; ++k) {
+                    c[k] = j < n[k] ? __ldcs(col + f[k] + j) : 0;
+                    l[k] = j < n[k] ? __ldcs(elab + f[k] + j) : 0;
+                }
 #pragma unroll
-        for (int k = 0; k < kAtOnce; ++k)
-            if (o + 32 * k < o1) pe[o + 32 * k] = pack_edge(l[k], t[k]);
+                for (int k = 0; k < kAtOnce; ++k)
+                    if (j < n[k]) pe[t[k] + j] = pack_edge(l[k], c[k]);
+            }
+        }
+    } else {
+        for (int row = 0; row < kPackLong; ++row) {
+            const int64_t f = __shfl_sync(kAll, from, row), t = __shfl_sync(kAll, to, row);
+            const int n = __shfl_sync(kAll, d, row);
+            for (int j0 = lane; j0 < n; j0 += 32 * kAtOnce) {
+                int32_t c[kAtOnce], l[kAtOnce];
+#pragma unroll
+                for (int k = 0; k < kAtOnce; ++k) {
+                    const int j = j0 + 32 * k;
+                    c[k] = j < n ? __ldcs(col + f + j) : 0;
+                    l[k] = j < n ? __ldcs(elab + f + j) : 0;
+                }
+#pragma unroll
+                for (int k = 0; k < kAtOnce; ++k)
+                    if (j0 + 32 * k < n) pe[t + j0 + 32 * k] = pack_edge(l[k], c[k]);
+            }
+        }
     }
 }
 
@@ -1898,13 +1921,13 @@ void free_hub_layout(bisim_ctx* ctx, cudaStream_t s) {
 void pack_rows_from_csr(bisim_ctx* ctx, cudaStream_t s) {
     BISIM_SITE(site_p, "dense_pack");
     const int64_t* begin = ctx->dbegin;
-    const int64_t small = begin[kDMid0];                 // rows of at most 256 edges: a warp per 32 rows
+    const int64_t small = begin[kDMid0];                 // rows of at most 256 edges
     const int64_t mid = begin[kDHub] - small;
     const int64_t edges = ctx->dedge_begin[kDHub];
     Launch L(site_p, s, begin[kDHub], edges, 16.0 * edges + 20.0 * begin[kDHub]);
     if (small > 0)
-        k_dense_pack_rows<<<grid_for(small, 256), 256, 0, s>>>(ctx->dvert, small, ctx->dprp, ctx->row_ptr, ctx->col,
-                                                              ctx->elab, ctx->dpe);
+        k_dense_pack_rows<<<grid_for((cdiv(begin[kDWarp0], 32) + cdiv(small - begin[kDWarp0], kPackLong)) * 32, 256), 256, 0, s>>>(
+            ctx->dvert, begin[kDWarp0], small, ctx->dprp, ctx->row_ptr, ctx->col, ctx->elab, ctx->dpe);
     if (mid > 0)
         k_dense_pack_big<<<static_cast<unsigned>(mid), 256, 0, s>>>(ctx->dvert, small, ctx->dprp, ctx->row_ptr,
                                                                    ctx->col, ctx->elab, ctx->dpe);

@@ -99,6 +99,23 @@ def test_edge_arrays_at_any_alignment(B, off, m):
         a[m // 2] = keep
 
 
+@pytest.mark.parametrize("shorts,longs", [(0, 1), (1, 0), (31, 2), (32, 3), (33, 40), (200, 1)])
+@pytest.mark.parametrize("thresholds", [{}, dict(small_max_degree=0)])
+def test_rows_packed_from_a_csr(B, shorts, longs, thresholds):
+    # rows up to 32 edges a group of lanes each, up to 256 a warp each, at the ends of their warps
+    rng = np.random.default_rng(shorts + longs)
+    deg = rng.permutation(np.concatenate([rng.integers(0, 33, shorts), rng.choice([33, 34, 127, 128, 129, 255, 256], longs)]))
+    n, m = len(deg), int(deg.sum())
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    col, lab = rng.integers(0, n, m).astype(np.int32), rng.integers(0, 5, m).astype(np.int32)
+    vl = rng.integers(0, 3, n).astype(np.int32)
+    with B.summarize_init(n, _dev(rp), _dev(col), _dev(lab), _dev(vl), options=B.default_options(**thresholds)) as ctx:
+        for k in (1, 2):
+            want, _, _ = oracle.refine(n, np.repeat(np.arange(n), deg).astype(np.int32), col, lab, vl, k)
+            B.bisim_iterate(ctx, k)
+            assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 3001])
 @pytest.mark.parametrize("thresholds", [{}, dict(small_max_degree=4, mid_max_degree=300), dict(small_max_degree=0, mid_max_degree=0)])
 def test_layout_tiles_and_classes(B, n, thresholds):
