@@ -282,15 +282,13 @@ bisim_status finish_init(bisim_ctx* ctx, cudaStream_t s) {
     if ((st = alloc_refine_state(ctx, s)) != BISIM_OK) return st;
     if (ctx->opt.mem_budget_bytes > 0 && ctx->device_bytes > ctx->opt.mem_budget_bytes)
         return set_error(ctx, BISIM_ENOMEM, "context exceeds the memory budget");
-    if ((st = compute_p0(ctx, s)) != BISIM_OK) return st;
-    cudaMemcpyAsync(ctx->P[0], ctx->P0, sizeof(int32_t) * std::max(ctx->n, 1), cudaMemcpyDeviceToDevice, s);
+    // also the current partition; its read-back is the call's last synchronisation
+    if ((st = compute_p0(ctx, s, ctx->P[0])) != BISIM_OK) return st;
     ctx->cur = 0;
     ctx->stats.n_vertices = ctx->n;
     ctx->stats.n_edges = ctx->m;
     ctx->stats.n_graphs = ctx->n_graphs;
     ctx->stats.device_bytes = ctx->device_bytes;
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e) return cuda_error(ctx, e, "initialise partition");
     return BISIM_OK;
 }
 
@@ -581,11 +579,21 @@ bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges
             *out = ctx;
             return BISIM_OK;
         }
-    } else if (edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK &&
-               (st = build_from_csr(ctx, row_ptr, col, edge_label, s)) == BISIM_OK &&
-               (st = finish_init(ctx, s)) == BISIM_OK) {
-        *out = ctx;
-        return BISIM_OK;
+    } else if (edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK) {
+        // P_0 does not look at the edges: one synchronisation for it and their check
+        unsigned* found = static_cast<unsigned*>(pinned_take());
+        if (found == nullptr) st = set_error(ctx, BISIM_ENOMEM, "pinned check word");
+        if (st == BISIM_OK && (st = build_from_csr(ctx, row_ptr, col, edge_label, s, found)) == BISIM_OK) {
+            st = finish_init(ctx, s);
+            const cudaError_t e = st == BISIM_OK ? cudaSuccess : cudaStreamSynchronize(s);
+            if (e) st = cuda_error(ctx, e, "validate CSR");
+            else if (csr_checked(ctx, *found) != BISIM_OK) st = BISIM_EINVAL;
+        }
+        if (found != nullptr) pinned_give(found);
+        if (st == BISIM_OK) {
+            *out = ctx;
+            return BISIM_OK;
+        }
     }
     std::string msg = ctx->err;
     destroy_ctx(ctx);

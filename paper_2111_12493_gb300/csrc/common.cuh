@@ -488,8 +488,11 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
 // Only the check of graph-local ids and the union's ids.
 bisim_status globalize_edges(bisim_ctx* ctx, const BatchedList& batch, const int32_t* src, const int32_t* dst,
                              cudaStream_t s);
+// `later` (pinned, nullable): what the check found is only copied there, and the
+// caller looks (csr_checked) after its next synchronisation of `s`.
 bisim_status build_from_csr(bisim_ctx* ctx, const int64_t* row_ptr, const int32_t* col,
-                            const int32_t* elab, cudaStream_t s);
+                            const int32_t* elab, cudaStream_t s, unsigned* later = nullptr);
+bisim_status csr_checked(bisim_ctx* ctx, unsigned error);
 
 
 // ----------------------------------------------------------------------------- dynamic adjacency (store.cu)
@@ -503,7 +506,8 @@ bisim_status csr_from_store(bisim_ctx* ctx, cudaStream_t s);
 
 // ----------------------------------------------------------------------------- refinement (refine.cu)
 
-bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s);
+// P_0 into ctx->P0 (and `also`); synchronises.
+bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s, int32_t* also = nullptr);
 // Advances the signature table's epoch (clearing the table when it wraps).
 TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s);
 // One signature round over the vertices of `B` (all of them, or the `vcount`

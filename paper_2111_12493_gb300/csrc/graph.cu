@@ -543,7 +543,7 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
 }
 
 bisim_status build_from_csr(bisim_ctx* ctx, const int64_t* row_ptr, const int32_t* col,
-                            const int32_t* elab, cudaStream_t s) {
+                            const int32_t* elab, cudaStream_t s, unsigned* later) {
     const int32_t n = ctx->n;
     const int64_t m = ctx->m;
     cudaError_t e;
@@ -560,9 +560,17 @@ bisim_status build_from_csr(bisim_ctx* ctx, const int64_t* row_ptr, const int32_
     Launch(site_vcsr, s, n + 1, m, 8.0 * (n + 1) + 4.0 * m),
     k_validate_csr<<<grid_for(std::min<int64_t>(std::max<int64_t>(m, n + 1), 1 << 22), 256), 256, 0, s>>>(
         ctx->row_ptr, ctx->col, n, m, ctx->alive, &ctx->dstate->error);
+    if (later != nullptr) {
+        cudaMemcpyAsync(later, &ctx->dstate->error, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+        return BISIM_OK;
+    }
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "validate CSR");
-    if (ctx->hstate->error & kErrBadInput)
+    return csr_checked(ctx, ctx->hstate->error);
+}
+
+bisim_status csr_checked(bisim_ctx* ctx, unsigned error) {
+    if (error & kErrBadInput)
         return set_error(ctx, BISIM_EINVAL, "malformed CSR: row_ptr not a prefix sum of [0, m], a target out of range, or an edge on a dead vertex");
     return BISIM_OK;
 }

@@ -486,36 +486,40 @@ __global__ void __launch_bounds__(256) k_p0_insert(int32_t n, const uint8_t* __r
 }
 
 // Confirm each vertex against its slot's smallest vertex. Equal: that vertex is
-// its block id. Different: queue it for the next level.
+// its block id (which goes to `also` as well, when given). Different: queue it for
+// the next level.
 template <class Mode>
 __global__ void k_resolve_verify(const int32_t* __restrict__ list, int64_t count,
                                  const uint8_t* __restrict__ alive, Mode M,
                                  const uint32_t* __restrict__ slot, const Slot* __restrict__ slots,
                                  int32_t* __restrict__ Pout, int32_t* __restrict__ next,
-                                 int32_t* __restrict__ deferred, DevState* st, int32_t n_total) {
+                                 int32_t* __restrict__ deferred, DevState* st, int32_t n_total,
+                                 int32_t* __restrict__ also) {
     const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x;
     const int64_t i = i0 + threadIdx.x;
     bool is_block = false, push = false, defer = false;
     int32_t v = -1;
     if (i < count) {
         v = list ? list[i] : static_cast<int32_t>(i);
-        if (!list && alive && !alive[v]) {
-            Pout[v] = -1;
-        } else {
+        int32_t block = -1;
+        if (list || !alive || alive[v]) {
             const uint32_t sv = slot[v];
             const int32_t r = sv == ~0u ? -1 : table_rep(slots, sv);
             if (r < 0 || r >= n_total) {          // failed insert: reported through st->error
                 atomicOr(&st->error, kErrTableFull);
-                Pout[v] = -1;
             } else if (r == v) {
-                Pout[v] = v;
+                block = v;
                 is_block = true;
             } else {
                 const int eq = M.compare(v, r);
-                if (eq == 1) Pout[v] = r;
+                if (eq == 1) block = r;
                 else if (eq == 0) push = true;
                 else defer = true;
             }
+        }
+        if (!push && !defer) {
+            Pout[v] = block;
+            if (also) also[v] = block;
         }
     }
     const unsigned bb = __ballot_sync(0xffffffffu, is_block);
@@ -642,7 +646,7 @@ void launch_deferred(bisim_ctx* ctx, const Mode& M, int32_t* Pout, int32_t* next
 
 template <class Mode>
 bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist, int64_t vcount, cudaStream_t s,
-                     int64_t* blocks) {
+                     int64_t* blocks, int32_t* also = nullptr) {
     const int32_t n = ctx->n;
     const int64_t nv = vlist ? vcount : n;
     cudaError_t e;
@@ -652,7 +656,7 @@ bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist
         Launch L(site, s, nv, 0, Mode::kVerifyBytesPerVertex * nv);
         k_resolve_verify<Mode><<<grid_for(nv, 256), 256, 0, s>>>(vlist, nv, ctx->alive, M, ctx->slot,
                                                                  ctx->table, Pout, ctx->ulist[0], ctx->dlist,
-                                                                 ctx->dstate, n);
+                                                                 ctx->dstate, n, also);
     }
     if (nv > 0) launch_deferred(ctx, M, Pout, ctx->ulist[0], s);
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
@@ -677,7 +681,7 @@ bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist
             Launch L(site_v, s, cu, 0, 0.0);
             k_resolve_verify<Mode><<<grid_for(cu, 256), 256, 0, s>>>(ctx->ulist[which], cu, ctx->alive, M, ctx->slot,
                                                                       ctx->table, Pout, ctx->ulist[which ^ 1],
-                                                                      ctx->dlist, ctx->dstate, n);
+                                                                      ctx->dlist, ctx->dstate, n, also);
         }
         launch_deferred(ctx, M, Pout, ctx->ulist[which ^ 1], s);
         cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
@@ -798,7 +802,7 @@ bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s) {
     return BISIM_OK;
 }
 
-bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s) {
+bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s, int32_t* also) {
     TableRef t = next_epoch(ctx, s);
     LabelMode M{ctx->vlabel, ctx->gid};
     if (ctx->n > 0) {
@@ -808,7 +812,8 @@ bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s) {
             ctx->n, ctx->alive, M, ctx->slot, t, &ctx->dstate->error);
     }
     int64_t blocks = 0;
-    bisim_status st = resolve(ctx, M, ctx->P0, nullptr, 0, s, &blocks);
+    static_assert(!LabelMode::kDefers, "a deferred comparison would have to write `also` too");
+    bisim_status st = resolve(ctx, M, ctx->P0, nullptr, 0, s, &blocks, also);
     if (st != BISIM_OK) return st;
     ctx->last_blocks = blocks;
     ctx->stats.num_blocks = blocks;
