@@ -47,6 +47,59 @@ void pinned_give(void* p) {
     g_pinned_free.push_back(p);
 }
 
+// Branches are kept for the next caller, of any context: at most kBranchesKept per
+// device, more are destroyed when they are joined. What a branch has in flight then
+// is ordered before its join, so whoever takes it next is only queued behind it.
+namespace {
+constexpr size_t kBranchesKept = 8;
+std::mutex g_branch_mu;
+std::vector<Branch> g_branches[64];
+
+void branch_destroy(const Branch& b) {
+    if (b.s) cudaStreamDestroy(b.s);                    // its work in flight completes first
+    if (b.fork) cudaEventDestroy(b.fork);
+    if (b.join) cudaEventDestroy(b.join);
+}
+}  // namespace
+
+Branch branch_fork(int device, cudaStream_t s) {
+    Branch b;
+    if (device < 0 || device >= 64) return b;
+    {
+        std::lock_guard<std::mutex> lk(g_branch_mu);
+        if (!g_branches[device].empty()) {
+            b = g_branches[device].back();
+            g_branches[device].pop_back();
+        }
+    }
+    if (b.s == nullptr && (cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking) != cudaSuccess ||
+                           cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) != cudaSuccess ||
+                           cudaEventCreateWithFlags(&b.join, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaGetLastError();
+        branch_destroy(b);
+        return Branch{};
+    }
+    cudaEventRecord(b.fork, s);
+    cudaStreamWaitEvent(b.s, b.fork, 0);
+    return b;
+}
+
+void branch_join(int device, Branch* b, cudaStream_t s) {
+    if (b->s == nullptr) return;
+    cudaEventRecord(b->join, b->s);
+    cudaStreamWaitEvent(s, b->join, 0);
+    const Branch done = *b;
+    *b = Branch{};
+    {
+        std::lock_guard<std::mutex> lk(g_branch_mu);
+        if (g_branches[device].size() < kBranchesKept) {
+            g_branches[device].push_back(done);
+            return;
+        }
+    }
+    branch_destroy(done);
+}
+
 // Whether the kernels of the current device may read `p` in place: managed
 // memory, or device memory of the current device. Memory of another GPU is
 // not (no peer mapping is assumed): it is staged through a copy like host memory.
@@ -113,6 +166,7 @@ void destroy_ctx(bisim_ctx* ctx) {
     // it: the pool then hands the memory straight to the next context, which a
     // free still pending on the device would make it map afresh
     cudaStream_t s = static_cast<cudaStream_t>(ctx->last_stream);
+    branch_join(ctx->device, &ctx->p0_branch, s);        // an init that failed beside its P_0
     for (void* p : ctx->allocs) cudaFreeAsync(p, s);
     if (ctx->dstate) cudaFreeAsync(ctx->dstate, s);
     cudaStreamSynchronize(s);
@@ -151,7 +205,7 @@ bisim_status new_ctx(bisim_ctx** out, int32_t n, int64_t m, const bisim_options*
     cudaError_t e = cudaGetDevice(&ctx->device);
     if (e) { delete ctx; return cuda_error(nullptr, e, "cudaGetDevice"); }
     setup_pool(ctx->device);
-    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->dstate), sizeof(DevState), s))) {
+    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->dstate), 2 * sizeof(DevState), s))) {
         destroy_ctx(ctx);
         return cuda_error(nullptr, e, "allocate context state");
     }
@@ -160,8 +214,9 @@ bisim_status new_ctx(bisim_ctx** out, int32_t n, int64_t m, const bisim_options*
         destroy_ctx(ctx);
         return set_error(nullptr, BISIM_ENOMEM, "pinned host memory for the context state");
     }
-    cudaMemsetAsync(ctx->dstate, 0, sizeof(DevState), s);
-    std::memset(ctx->hstate, 0, sizeof(DevState));
+    static_assert(2 * sizeof(DevState) <= kPinnedBlock, "the mirror's block");
+    cudaMemsetAsync(ctx->dstate, 0, 2 * sizeof(DevState), s);
+    std::memset(ctx->hstate, 0, 2 * sizeof(DevState));
     bisim_status st = edge_view_setup(ctx, opt, s);
     if (st != BISIM_OK) {
         const std::string msg = ctx->err;
@@ -279,11 +334,11 @@ bisim_status coo_arrive(bisim_ctx* ctx, const int32_t* src, const int32_t* dst, 
 
 bisim_status finish_init(bisim_ctx* ctx, cudaStream_t s) {
     bisim_status st;
-    if ((st = alloc_refine_state(ctx, s)) != BISIM_OK) return st;
+    if (!ctx->p0_pending && (st = p0_begin(ctx, s, false)) != BISIM_OK) return st;
     if (ctx->opt.mem_budget_bytes > 0 && ctx->device_bytes > ctx->opt.mem_budget_bytes)
         return set_error(ctx, BISIM_ENOMEM, "context exceeds the memory budget");
     // also the current partition; its read-back is the call's last synchronisation
-    if ((st = compute_p0(ctx, s, ctx->P[0])) != BISIM_OK) return st;
+    if ((st = p0_end(ctx, s)) != BISIM_OK) return st;
     ctx->cur = 0;
     ctx->stats.n_vertices = ctx->n;
     ctx->stats.n_edges = ctx->m;
@@ -558,7 +613,8 @@ bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges
         destroy_ctx(ctx);
         return set_error(nullptr, BISIM_EINVAL, "a required array is NULL");
     }
-    if (!edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK) {
+    if (!edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK &&
+        (st = p0_begin(ctx, s, true)) == BISIM_OK) {
         // another direction or a label filter: the CSR's edges as a list, then the view's COO path
         std::vector<void*> temps;
         const void *drp = nullptr, *dc = nullptr, *dl = nullptr;
@@ -579,7 +635,8 @@ bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges
             *out = ctx;
             return BISIM_OK;
         }
-    } else if (edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK) {
+    } else if (edge_view_identity(ctx) && (st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK &&
+               (st = p0_begin(ctx, s, true)) == BISIM_OK) {
         // P_0 does not look at the edges: one synchronisation for it and their check
         unsigned* found = static_cast<unsigned*>(pinned_take());
         if (found == nullptr) st = set_error(ctx, BISIM_ENOMEM, "pinned check word");
@@ -652,7 +709,7 @@ bisim_status summarize_init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_e
         destroy_ctx(ctx);
         return set_error(nullptr, st, msg);
     }
-    if ((st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK) {
+    if ((st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK && (st = p0_begin(ctx, s, true)) == BISIM_OK) {
         if ((e = stage(src, eb, s, &ds, temps)) || (e = stage(dst, eb, s, &dd, temps)) ||
             (e = stage(edge_label, eb, s, &dl, temps)))
             st = cuda_error(ctx, e, "stage edge arrays");
@@ -722,6 +779,7 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
         if (n > 0)
             Launch(site_g, s, n, 0, 4.0 * n),
             k_graph_ids<<<(n + 1023) / 1024, 256, 0, s>>>(ctx->voff, n_graphs, n, ctx->gid);
+        st = p0_begin(ctx, s, true);
     }
     const BatchedList batch{ctx->voff, deoff, n_graphs, gsrc, gdst};
     const int32_t* ls = static_cast<const int32_t*>(ds);

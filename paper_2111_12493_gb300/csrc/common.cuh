@@ -258,6 +258,13 @@ struct Buf {
     size_t bytes = 0;
 };
 
+// A stream of its own for part of a call's kernels, with the events that put it
+// between two points of the caller's stream.
+struct Branch {
+    cudaStream_t s = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+
 }  // namespace bisim
 
 // ----------------------------------------------------------------------------- context
@@ -357,8 +364,10 @@ struct bisim_ctx {
     // collision resolution
     int32_t* ulist[2] = {nullptr, nullptr};
     int32_t* dlist = nullptr;      // vertices whose verification needs a set comparison
-    bisim::DevState* dstate = nullptr;
+    bisim::DevState* dstate = nullptr;   // [2]: the second is P_0's while it runs beside the build
     bisim::DevState* hstate = nullptr;   // pinned mirror
+    bool p0_pending = false;             // p0_begin ran and p0_end did not
+    bisim::Branch p0_branch;
 
     // updates
     int32_t* esrc = nullptr;       // source vertex of every CSR edge (kept once updates start)
@@ -445,6 +454,10 @@ CtxPiece ctx_piece(T** p, size_t count) {
 // Whether the kernels of the current device may use `p` in place (api.cu).
 bool device_accessible(const void* p);
 // 256-byte pinned host blocks from process-lifetime slabs (nullptr if none can be had).
+// Forks from `s`. A branch without a stream (none could be had) stands for `s` itself.
+// After the join (which has to come, on the same stream) the branch is gone.
+Branch branch_fork(int device, cudaStream_t s);
+void branch_join(int device, Branch* b, cudaStream_t s);
 void* pinned_take();
 void pinned_give(void* p);
 
@@ -506,8 +519,13 @@ bisim_status csr_from_store(bisim_ctx* ctx, cudaStream_t s);
 
 // ----------------------------------------------------------------------------- refinement (refine.cu)
 
-// P_0 into ctx->P0 (and `also`); synchronises.
-bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s, int32_t* also = nullptr);
+// P_0 into ctx->P0; synchronises.
+bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s);
+// The refinement state, and P_0 into ctx->P0 and ctx->P[0]. An `early` call, as soon
+// as the vertex arrays (and graphs) are there, starts it beside the build where that
+// pays, else does nothing; p0_end synchronises `s` and has the result.
+bisim_status p0_begin(bisim_ctx* ctx, cudaStream_t s, bool early);
+bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s);
 // Advances the signature table's epoch (clearing the table when it wraps).
 TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s);
 // One signature round over the vertices of `B` (all of them, or the `vcount`
@@ -517,7 +535,6 @@ TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s);
 bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
                              const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s,
                              int64_t* out_blocks);
-bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s);
 void pin_partition_in_l2(bisim_ctx* ctx, const int32_t* P, cudaStream_t s);
 void unpin_partition(bisim_ctx* ctx, cudaStream_t s);
 void launch_local_ids(const bisim_ctx* ctx, int32_t* out, cudaStream_t s);

@@ -1731,62 +1731,6 @@ DenseView dense_view(bisim_ctx* ctx) {
 }
 
 
-// A stream of its own for part of a round's signature kernels, with the events that
-// put it between two points of the caller's stream. Kept for the next round of any
-// context: at most kBranchesKept per device, more are destroyed when they are given
-// back. What a branch still has in flight then is ordered before its join, so
-// whoever takes it next is only queued behind it.
-struct Branch {
-    cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-};
-constexpr size_t kBranchesKept = 8;
-std::mutex g_branch_mu;
-std::vector<Branch> g_branches[64];
-
-void branch_destroy(const Branch& b) {
-    if (b.s) cudaStreamDestroy(b.s);
-    if (b.fork) cudaEventDestroy(b.fork);
-    if (b.join) cudaEventDestroy(b.join);
-}
-
-// Forks from `s`; a branch without a stream (none could be had) runs on `s` itself.
-Branch branch_fork(int device, cudaStream_t s) {
-    Branch b;
-    if (device < 0 || device >= 64) return b;
-    {
-        std::lock_guard<std::mutex> lk(g_branch_mu);
-        if (!g_branches[device].empty()) {
-            b = g_branches[device].back();
-            g_branches[device].pop_back();
-        }
-    }
-    if (b.s == nullptr && (cudaStreamCreateWithFlags(&b.s, cudaStreamNonBlocking) != cudaSuccess ||
-                           cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) != cudaSuccess ||
-                           cudaEventCreateWithFlags(&b.join, cudaEventDisableTiming) != cudaSuccess)) {
-        cudaGetLastError();
-        branch_destroy(b);
-        return Branch{};
-    }
-    cudaEventRecord(b.fork, s);
-    cudaStreamWaitEvent(b.s, b.fork, 0);
-    return b;
-}
-
-void branch_join(int device, const Branch& b, cudaStream_t s) {
-    if (b.s == nullptr) return;
-    cudaEventRecord(b.join, b.s);
-    cudaStreamWaitEvent(s, b.join, 0);
-    {
-        std::lock_guard<std::mutex> lk(g_branch_mu);
-        if (g_branches[device].size() < kBranchesKept) {
-            g_branches[device].push_back(b);
-            return;
-        }
-    }
-    branch_destroy(b);                                  // its work in flight completes first
-}
-
 // Everything of one round P[0] -> P[1] that needs no host decision:
 // signatures of the listed vertices of every class, then level 0 of the
 // renumbering. P[1] already holds P_i (the end of the previous round copied
@@ -1822,7 +1766,7 @@ void launch_round(bisim_ctx* ctx, cudaStream_t s, const TableRef& t, const int32
     // neither: the three run beside each other, the longer rows first. Not while
     // launches are timed, nor in a captured round.
     const bool beside = !prof_enabled() && round_no == nullptr && db[kDMid0] > db[0];
-    const Branch hubs = beside && ctx->n_dhub > 0 && ctx->n_dchunks > 0 ? branch_fork(ctx->device, s) : Branch{};
+    Branch hubs = beside && ctx->n_dhub > 0 && ctx->n_dchunks > 0 ? branch_fork(ctx->device, s) : Branch{};
     if (ctx->n_dhub > 0) {
         const cudaStream_t hs = hubs.s ? hubs.s : s;
         if (ctx->n_dchunks > 0) {
@@ -1838,7 +1782,7 @@ void launch_round(bisim_ctx* ctx, cudaStream_t s, const TableRef& t, const int32
         Launch L(site_hf, hs, 0, 0, 0.0);
         k_dense_hub_finalize<<<grid_for(ctx->n_dhub, 128), 128, 0, hs>>>(D, H);
     }
-    const Branch mids = beside && db[kDHub] > db[kDMid0] ? branch_fork(ctx->device, s) : Branch{};
+    Branch mids = beside && db[kDHub] > db[kDMid0] ? branch_fork(ctx->device, s) : Branch{};
     {
         const cudaStream_t ms = mids.s ? mids.s : s;
         launch_mid<8192, 512>(ctx, kDMid0 + 4, D, ms, site_mid[4]);
@@ -1863,8 +1807,8 @@ void launch_round(bisim_ctx* ctx, cudaStream_t s, const TableRef& t, const int32
         Launch L(site_w, s, 0, 0, 0.0);
         k_dense_warp_sig<<<persistent_grid(k_dense_warp_sig, kThreads, 0, cdiv(verts, kThreads / 32)), kThreads, 0, s>>>(D);
     }
-    branch_join(ctx->device, mids, s);
-    branch_join(ctx->device, hubs, s);
+    branch_join(ctx->device, &mids, s);
+    branch_join(ctx->device, &hubs, s);
     launch_level(ctx, s, D, t, 0, nullptr, ctx->dbegin[kDClasses], ctx->ulist[0]);
 }
 

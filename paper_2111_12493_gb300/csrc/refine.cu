@@ -629,7 +629,7 @@ TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s) {
 namespace {
 
 template <class Mode>
-void launch_deferred(bisim_ctx* ctx, const Mode& M, int32_t* Pout, int32_t* next, cudaStream_t s) {
+void launch_deferred(bisim_ctx* ctx, const Mode& M, int32_t* Pout, int32_t* next, DevState* ds, cudaStream_t s) {
     if constexpr (Mode::kDefers) {
         static bool attr_set = false;
         if (!attr_set) {
@@ -640,60 +640,76 @@ void launch_deferred(bisim_ctx* ctx, const Mode& M, int32_t* Pout, int32_t* next
         BISIM_SITE(site, "verify_deferred");
         Launch L(site, s, 0, 0, 0.0);
         k_verify_deferred<<<kDeferGrid, kDeferThreads, kDeferSmem, s>>>(ctx->dlist, M, ctx->slot, ctx->table, Pout,
-                                                                         next, ctx->dstate);
+                                                                         next, ds);
     }
 }
 
+// The confirmation of level 0 and its read-back, with the state words `ds` / `hs`;
+// resolve_settle, once they have arrived, runs the collision levels that are needed.
 template <class Mode>
-bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist, int64_t vcount, cudaStream_t s,
-                     int64_t* blocks, int32_t* also = nullptr) {
+void resolve_launch(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist, int64_t vcount, cudaStream_t s,
+                    int32_t* also, DevState* ds, DevState* hs) {
     const int32_t n = ctx->n;
     const int64_t nv = vlist ? vcount : n;
-    cudaError_t e;
-    cudaMemsetAsync(ctx->dstate, 0, sizeof(DevState), s);
+    cudaMemsetAsync(ds, 0, sizeof(DevState), s);
     if (nv > 0) {
         BISIM_SITE(site, Mode::kVerifySite);
         Launch L(site, s, nv, 0, Mode::kVerifyBytesPerVertex * nv);
         k_resolve_verify<Mode><<<grid_for(nv, 256), 256, 0, s>>>(vlist, nv, ctx->alive, M, ctx->slot,
                                                                  ctx->table, Pout, ctx->ulist[0], ctx->dlist,
-                                                                 ctx->dstate, n, also);
+                                                                 ds, n, also);
     }
-    if (nv > 0) launch_deferred(ctx, M, Pout, ctx->ulist[0], s);
-    cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
-    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify signatures");
+    if (nv > 0) launch_deferred(ctx, M, Pout, ctx->ulist[0], ds, s);
+    cudaMemcpyAsync(hs, ds, sizeof(DevState), cudaMemcpyDeviceToHost, s);
+}
+
+template <class Mode>
+bisim_status resolve_settle(bisim_ctx* ctx, Mode M, int32_t* Pout, cudaStream_t s, int64_t* blocks, int32_t* also,
+                            DevState* ds, DevState* hs) {
+    const int32_t n = ctx->n;
+    cudaError_t e;
     int which = 0;
     uint32_t level = 0;
-    while (ctx->hstate->error == 0 && ctx->hstate->unresolved > 0) {
+    while (hs->error == 0 && hs->unresolved > 0) {
         if (++level > static_cast<uint32_t>(kMaxLevels))
             return set_error(ctx, BISIM_ETIMEOUT, "hash collision resolution did not converge");
-        const int64_t cu = ctx->hstate->unresolved;
+        const int64_t cu = hs->unresolved;
         TableRef t = next_epoch(ctx, s);
-        cudaMemsetAsync(&ctx->dstate->unresolved, 0, sizeof(unsigned), s);
-        cudaMemsetAsync(&ctx->dstate->deferred, 0, sizeof(unsigned), s);
+        cudaMemsetAsync(&ds->unresolved, 0, sizeof(unsigned), s);
+        cudaMemsetAsync(&ds->deferred, 0, sizeof(unsigned), s);
         BISIM_SITE(site_i, "collision_insert");
         BISIM_SITE(site_v, "collision_verify");
         {
             Launch L(site_i, s, cu, 0, 0.0);
             k_resolve_insert<Mode><<<grid_for(cu, 256), 256, 0, s>>>(ctx->ulist[which], cu, ctx->alive, M, level,
-                                                                      ctx->slot, t, &ctx->dstate->error);
+                                                                      ctx->slot, t, &ds->error);
         }
         {
             Launch L(site_v, s, cu, 0, 0.0);
             k_resolve_verify<Mode><<<grid_for(cu, 256), 256, 0, s>>>(ctx->ulist[which], cu, ctx->alive, M, ctx->slot,
                                                                       ctx->table, Pout, ctx->ulist[which ^ 1],
-                                                                      ctx->dlist, ctx->dstate, n, also);
+                                                                      ctx->dlist, ds, n, also);
         }
-        launch_deferred(ctx, M, Pout, ctx->ulist[which ^ 1], s);
-        cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
+        launch_deferred(ctx, M, Pout, ctx->ulist[which ^ 1], ds, s);
+        cudaMemcpyAsync(hs, ds, sizeof(DevState), cudaMemcpyDeviceToHost, s);
         if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "resolve hash collisions");
         which ^= 1;
         ctx->stats.collision_levels += 1;
     }
-    if (ctx->hstate->error & kErrTableFull) return set_error(ctx, BISIM_ETIMEOUT, "signature table probe limit reached");
-    if (ctx->hstate->error & kErrHubFull) return set_error(ctx, BISIM_ETIMEOUT, "hub dedup table probe limit reached");
-    if (ctx->hstate->error) return set_error(ctx, BISIM_EINVAL, "device reported invalid input");
-    *blocks = static_cast<int64_t>(ctx->hstate->blocks);
+    if (hs->error & kErrTableFull) return set_error(ctx, BISIM_ETIMEOUT, "signature table probe limit reached");
+    if (hs->error & kErrHubFull) return set_error(ctx, BISIM_ETIMEOUT, "hub dedup table probe limit reached");
+    if (hs->error) return set_error(ctx, BISIM_EINVAL, "device reported invalid input");
+    *blocks = static_cast<int64_t>(hs->blocks);
     return BISIM_OK;
+}
+
+template <class Mode>
+bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist, int64_t vcount, cudaStream_t s,
+                     int64_t* blocks) {
+    resolve_launch(ctx, M, Pout, vlist, vcount, s, nullptr, ctx->dstate, ctx->hstate);
+    cudaError_t e;
+    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify signatures");
+    return resolve_settle(ctx, M, Pout, s, blocks, nullptr, ctx->dstate, ctx->hstate);
 }
 
 // Algorithmic bytes of the signature kernels: per edge col 4 + label 4 + the
@@ -780,6 +796,9 @@ void unpin_partition(bisim_ctx* ctx, cudaStream_t s) {
     cudaGetLastError();
 }
 
+namespace {
+
+// The table is left to be cleared.
 bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s) {
     const int32_t n = ctx->n;
     const int64_t m = ctx->m;
@@ -797,27 +816,71 @@ bisim_status alloc_refine_state(bisim_ctx* ctx, cudaStream_t s) {
                                  ctx_piece(&ctx->ulist[1], nv), ctx_piece(&ctx->dlist, nv), ctx_piece(&ctx->table, ns)},
                                 s)))
         return cuda_error(ctx, e, "alloc refinement state");
-    cudaMemsetAsync(ctx->table, 0, sizeof(Slot) * ns, s);
-    if ((e = cudaGetLastError())) return cuda_error(ctx, e, "init refine state");
     return BISIM_OK;
 }
 
-bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s, int32_t* also) {
+LabelMode label_mode(const bisim_ctx* ctx) { return LabelMode{ctx->vlabel, ctx->gid}; }
+
+void p0_launch(bisim_ctx* ctx, cudaStream_t s, int32_t* also, DevState* ds, DevState* hs, int ctas_per_sm = 8) {
+    static_assert(!LabelMode::kDefers, "a deferred comparison would have to write `also` too");
     TableRef t = next_epoch(ctx, s);
-    LabelMode M{ctx->vlabel, ctx->gid};
+    const LabelMode M = label_mode(ctx);
     if (ctx->n > 0) {
         BISIM_SITE(site, "label_insert");
         Launch L(site, s, ctx->n, 0, 20.0 * ctx->n);   // label 4 B + one 16-byte table slot
-        k_p0_insert<<<static_cast<unsigned>(std::min<int64_t>(cdiv(ctx->n, kP0Tile), 152 * 8)), 256, 0, s>>>(
-            ctx->n, ctx->alive, M, ctx->slot, t, &ctx->dstate->error);
+        k_p0_insert<<<static_cast<unsigned>(std::min<int64_t>(cdiv(ctx->n, kP0Tile), 152 * ctas_per_sm)), 256, 0, s>>>(
+            ctx->n, ctx->alive, M, ctx->slot, t, &ds->error);
     }
+    resolve_launch(ctx, M, ctx->P0, nullptr, 0, s, also, ds, hs);
+}
+
+bisim_status p0_settle(bisim_ctx* ctx, cudaStream_t s, int32_t* also, DevState* ds, DevState* hs) {
     int64_t blocks = 0;
-    static_assert(!LabelMode::kDefers, "a deferred comparison would have to write `also` too");
-    bisim_status st = resolve(ctx, M, ctx->P0, nullptr, 0, s, &blocks, also);
+    const bisim_status st = resolve_settle(ctx, label_mode(ctx), ctx->P0, s, &blocks, also, ds, hs);
     if (st != BISIM_OK) return st;
     ctx->last_blocks = blocks;
     ctx->stats.num_blocks = blocks;
     return BISIM_OK;
+}
+
+// From this many vertices on P_0 runs on a branch beside the build: its kernels wait
+// for a map in shared memory and hardly use memory, the build's passes for memory.
+// (10M vertices: 88 + 50 us of kernels, the one-off 3.55 to 3.47 ms; batch of 512
+// graphs, 7.4M vertices, 2.17 to 2.05.) Below, the build's first kernels would only
+// start later: 180 against 183 us at 1k vertices.
+constexpr int32_t kP0BesideMin = 1 << 16;
+
+}  // namespace
+
+bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s) {
+    p0_launch(ctx, s, nullptr, ctx->dstate, ctx->hstate);
+    cudaError_t e;
+    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify labels");
+    return p0_settle(ctx, s, nullptr, ctx->dstate, ctx->hstate);
+}
+
+bisim_status p0_begin(bisim_ctx* ctx, cudaStream_t s, bool early) {
+    const bool beside = early && ctx->n >= kP0BesideMin && !prof_enabled();
+    if (early && !beside) return BISIM_OK;
+    bisim_status st = alloc_refine_state(ctx, s);
+    if (st != BISIM_OK) return st;
+    if (beside) ctx->p0_branch = branch_fork(ctx->device, s);
+    const cudaStream_t ps = ctx->p0_branch.s ? ctx->p0_branch.s : s;
+    cudaMemsetAsync(ctx->table, 0, sizeof(Slot) * ctx->nslots, ps);
+    // on a branch its CTAs leave half of every SM to the build
+    p0_launch(ctx, ps, ctx->P[0], ctx->dstate + 1, ctx->hstate + 1, ctx->p0_branch.s ? 4 : 8);
+    ctx->p0_pending = true;
+    cudaError_t e;
+    if ((e = cudaGetLastError())) return cuda_error(ctx, e, "init refine state");
+    return BISIM_OK;
+}
+
+bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s) {
+    branch_join(ctx->device, &ctx->p0_branch, s);
+    ctx->p0_pending = false;
+    cudaError_t e;
+    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify labels");
+    return p0_settle(ctx, s, ctx->P[0], ctx->dstate + 1, ctx->hstate + 1);
 }
 
 bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
