@@ -381,11 +381,23 @@ __global__ void __launch_bounds__(kTileThreads) k_place_coo(const int32_t* __res
     }
 }
 
-__global__ void k_validate_csr(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                               int32_t n, int64_t m, const uint8_t* __restrict__ alive,
-                               unsigned* err) {
+// The check of a CSR, which also makes the context's copy of it (the `to` arrays;
+// null: the given ones are the copy). Four edges a thread in 16-byte accesses where
+// `wide` says that the given arrays take them: three copies and then a check of one
+// edge a thread took 28 and 20 us for 4M edges; this takes 17.
+struct CsrCopy {
+    int64_t* rp;
+    int32_t* col;
+    int32_t* elab;
+};
+
+__global__ void __launch_bounds__(256) k_validate_csr(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
+                                                      const int32_t* __restrict__ elab, int32_t n, int64_t m,
+                                                      const uint8_t* __restrict__ alive, const CsrCopy to, bool wide,
+                                                      unsigned* err) {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    bool bad = false;
     for (int64_t v = t0; v <= n; v += stride) {
         int64_t a = rp[v];
         bool ok = a >= 0 && a <= m;
@@ -396,14 +408,28 @@ __global__ void k_validate_csr(const int64_t* __restrict__ rp, const int32_t* __
             ok = ok && b >= a;
             if (alive != nullptr && !alive[v]) ok = ok && b == a;
         }
-        if (!ok) atomicOr(err, kErrBadInput);
+        if (to.rp != nullptr) to.rp[v] = a;
+        bad = bad || !ok;
     }
-    for (int64_t e = t0; e < m; e += stride) {
-        int32_t d = col[e];
-        bool ok = d >= 0 && d < n;
-        if (ok && alive != nullptr) ok = alive[d];
-        if (!ok) atomicOr(err, kErrBadInput);
+    const auto check = [&](int32_t d) { return d >= 0 && d < n && (alive == nullptr || alive[d]); };
+    const int64_t quads = wide ? m / 4 : 0;
+    for (int64_t q = t0; q < quads; q += stride) {
+        const int4 d = reinterpret_cast<const int4*>(col)[q];
+        if (to.col != nullptr) {
+            reinterpret_cast<int4*>(to.col)[q] = d;
+            reinterpret_cast<int4*>(to.elab)[q] = __ldcs(reinterpret_cast<const int4*>(elab) + q);
+        }
+        bad = bad || !check(d.x) || !check(d.y) || !check(d.z) || !check(d.w);
     }
+    for (int64_t e = 4 * quads + t0; e < m; e += stride) {
+        const int32_t d = col[e];
+        if (to.col != nullptr) {
+            to.col[e] = d;
+            to.elab[e] = elab[e];
+        }
+        bad = bad || !check(d);
+    }
+    if (bad) atomicOr(err, kErrBadInput);
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -550,16 +576,24 @@ bisim_status build_from_csr(bisim_ctx* ctx, const int64_t* row_ptr, const int32_
     if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->row_ptr), sizeof(int64_t) * (n + 1), s))) return cuda_error(ctx, e, "alloc row_ptr");
     if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->col), sizeof(int32_t) * std::max<int64_t>(m, 1), s))) return cuda_error(ctx, e, "alloc col");
     if ((e = ctx_alloc(ctx, reinterpret_cast<void**>(&ctx->elab), sizeof(int32_t) * std::max<int64_t>(m, 1), s))) return cuda_error(ctx, e, "alloc elab");
-    cudaMemcpyAsync(ctx->row_ptr, row_ptr, sizeof(int64_t) * (n + 1), cudaMemcpyDefault, s);
-    if (m > 0) {
-        cudaMemcpyAsync(ctx->col, col, sizeof(int32_t) * m, cudaMemcpyDefault, s);
-        cudaMemcpyAsync(ctx->elab, elab, sizeof(int32_t) * m, cudaMemcpyDefault, s);
+    CsrCopy to{ctx->row_ptr, ctx->col, ctx->elab};
+    if (!device_accessible(row_ptr) || (m > 0 && (!device_accessible(col) || !device_accessible(elab)))) {
+        cudaMemcpyAsync(ctx->row_ptr, row_ptr, sizeof(int64_t) * (n + 1), cudaMemcpyDefault, s);
+        if (m > 0) {
+            cudaMemcpyAsync(ctx->col, col, sizeof(int32_t) * m, cudaMemcpyDefault, s);
+            cudaMemcpyAsync(ctx->elab, elab, sizeof(int32_t) * m, cudaMemcpyDefault, s);
+        }
+        row_ptr = ctx->row_ptr;
+        col = ctx->col;
+        elab = ctx->elab;
+        to = CsrCopy{nullptr, nullptr, nullptr};
     }
     cudaMemsetAsync(&ctx->dstate->error, 0, sizeof(unsigned), s);
     BISIM_SITE(site_vcsr, "validate_csr");
-    Launch(site_vcsr, s, n + 1, m, 8.0 * (n + 1) + 4.0 * m),
-    k_validate_csr<<<grid_for(std::min<int64_t>(std::max<int64_t>(m, n + 1), 1 << 22), 256), 256, 0, s>>>(
-        ctx->row_ptr, ctx->col, n, m, ctx->alive, &ctx->dstate->error);
+    const unsigned grid = static_cast<unsigned>(std::min<int64_t>(cdiv(std::max<int64_t>(cdiv(m, 4), n + 1), 256), 152 * 8));
+    Launch(site_vcsr, s, n + 1, m, (to.rp ? 16.0 : 8.0) * (n + 1) + (to.rp ? 16.0 : 4.0) * m),
+    k_validate_csr<<<grid, 256, 0, s>>>(row_ptr, col, elab, n, m, ctx->alive, to, aligned16(col) && aligned16(elab),
+                                        &ctx->dstate->error);
     if (later != nullptr) {
         cudaMemcpyAsync(later, &ctx->dstate->error, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
         return BISIM_OK;

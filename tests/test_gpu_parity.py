@@ -424,3 +424,60 @@ def test_autotune_keeps_results_and_picks_listed_settings(B):
         want, wr, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], k, 10)
         assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want) and rounds == wr
     B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [(1 << 16) - 1, 1 << 16, 70_001])
+@pytest.mark.parametrize("form", ["coo", "csr"])
+def test_p0_beside_the_build(B, n, form):
+    # from 2^16 vertices on P_0 runs beside the build: its result, and an init that
+    # refuses its edges while P_0 is under way
+    rng = np.random.default_rng(n)
+    m = 2 * n
+    src = np.sort(rng.integers(0, n, m)).astype(np.int32)
+    dst, lab = rng.integers(0, n, m).astype(np.int32), rng.integers(0, 3, m).astype(np.int32)
+    vl = rng.integers(0, 1000, n).astype(np.int32)
+    rp = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))]).astype(np.int64)
+
+    def init(dst):
+        if form == "csr":
+            return B.summarize_init(n, _dev(rp), _dev(dst), _dev(lab), _dev(vl))
+        return B.summarize_init_coo(n, _dev(src), _dev(dst), _dev(lab), _dev(vl))
+
+    bad = dst.copy()
+    bad[m // 2] = n
+    for _ in range(2):
+        with pytest.raises(B.BisimError):
+            init(bad)
+        with init(dst) as ctx:
+            want, _, _ = oracle.refine(n, src, dst, lab, vl, 0)
+            assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+            B.bisim_iterate(ctx, 1)
+            want, _, _ = oracle.refine(n, src, dst, lab, vl, 1)
+            assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("off", [0, 1, 2])
+@pytest.mark.parametrize("m", [1, 3, 4, 5, 4099])
+@pytest.mark.parametrize("where", ["device", "host"])
+def test_csr_arrays_at_any_alignment(B, off, m, where):
+    # the check of a CSR makes the context's copy of it, four edges at a time where
+    # the arrays allow it; the copy shows in the summary's edges
+    import torch
+    rng = np.random.default_rng(m)
+    n = 40
+    src = np.sort(rng.integers(0, n, m)).astype(np.int32)
+    dst, lab = rng.integers(0, n, m).astype(np.int32), rng.integers(0, 2, m).astype(np.int32)
+    vl = rng.integers(0, 2, n).astype(np.int32)
+    rp = np.concatenate([[0], np.cumsum(np.bincount(src, minlength=n))]).astype(np.int64)
+    put = (lambda a: _dev(a)) if where == "device" else (lambda a: torch.from_numpy(np.ascontiguousarray(a)))
+    shift = lambda a, k: put(np.concatenate([np.full(k, 7, np.int32), a]))[k:]
+    want, _, _ = oracle.refine(n, src, dst, lab, vl, 2)
+    with B.summarize_init(n, put(rp), shift(dst, off), shift(lab, (2 * off) % 4), put(vl)) as ctx:
+        B.bisim_iterate(ctx, 2)
+        assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+        s, l, t = (x.cpu().numpy() for x in B.get_summary_edges(ctx)[:3])
+        assert sorted(zip(s, l, t)) == sorted(set(zip(want[src], lab, want[dst])))
+    bad = dst.copy()
+    bad[m - 1] = n
+    with pytest.raises(B.BisimError, match="malformed CSR"):
+        B.summarize_init(n, put(rp), shift(bad, off), shift(lab, off), put(vl))
