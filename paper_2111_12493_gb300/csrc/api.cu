@@ -205,7 +205,7 @@ bisim_status new_ctx(bisim_ctx** out, int32_t n, int64_t m, const bisim_options*
     cudaError_t e = cudaGetDevice(&ctx->device);
     if (e) { delete ctx; return cuda_error(nullptr, e, "cudaGetDevice"); }
     setup_pool(ctx->device);
-    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->dstate), 2 * sizeof(DevState), s))) {
+    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&ctx->dstate), kStateStride * sizeof(DevState) + sizeof(DevState), s))) {
         destroy_ctx(ctx);
         return cuda_error(nullptr, e, "allocate context state");
     }
@@ -215,7 +215,7 @@ bisim_status new_ctx(bisim_ctx** out, int32_t n, int64_t m, const bisim_options*
         return set_error(nullptr, BISIM_ENOMEM, "pinned host memory for the context state");
     }
     static_assert(2 * sizeof(DevState) <= kPinnedBlock, "the mirror's block");
-    cudaMemsetAsync(ctx->dstate, 0, 2 * sizeof(DevState), s);
+    cudaMemsetAsync(ctx->dstate, 0, sizeof(DevState), s);
     std::memset(ctx->hstate, 0, 2 * sizeof(DevState));
     bisim_status st = edge_view_setup(ctx, opt, s);
     if (st != BISIM_OK) {
@@ -232,6 +232,7 @@ bisim_status new_ctx(bisim_ctx** out, int32_t n, int64_t m, const bisim_options*
 bisim_status build_from_coo_view(bisim_ctx* ctx, const int32_t* src, const int32_t* dst, const int32_t* lab,
                                  cudaStream_t s) {
     if (edge_view_identity(ctx)) return build_from_coo(ctx, src, dst, lab, s);
+    if (edge_view_reversal(ctx)) return build_from_coo(ctx, dst, src, lab, s);
     EdgeView v;
     bisim_status st = edge_view_coo(ctx, src, dst, lab, ctx->m, nullptr, 0, s, &v);
     if (st == BISIM_OK) {
@@ -786,7 +787,8 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
     const int32_t* ld = static_cast<const int32_t*>(dd);
     EdgeView view;
     const int32_t* bl = static_cast<const int32_t*>(dl);
-    if (st == BISIM_OK && !edge_view_identity(ctx)) {
+    if (edge_view_reversal(ctx)) std::swap(ls, ld);
+    else if (st == BISIM_OK && !edge_view_identity(ctx)) {
         // another direction or a label filter: the view keeps every graph's edges together
         if ((st = globalize_edges(ctx, batch, ls, ld, s)) == BISIM_OK && (st = edge_view_coo(ctx, gsrc, gdst, bl, m, deoff, n_graphs, s, &view)) == BISIM_OK) {
             ctx->m = view.m;

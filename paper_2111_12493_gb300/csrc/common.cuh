@@ -125,7 +125,11 @@ struct DevState {
     unsigned int pairs;             // dense rounds: small pairs left to a warp comparison
     unsigned int listed;            // dense rounds: positions that need the table this round
     unsigned int unsorted;          // COO build: some edge's source is smaller than the one before it
+    unsigned int bad_label;         // edge view: a label the forward-backward direction cannot take
 };
+
+// Kernels that run beside each other do not share a cache line of state.
+constexpr int kStateStride = 8;
 
 __device__ __forceinline__ unsigned long long table_read(const TableRef& t, uint64_t pos) {
     return *reinterpret_cast<volatile unsigned long long*>(&t.slots[pos].w);
@@ -364,7 +368,7 @@ struct bisim_ctx {
     // collision resolution
     int32_t* ulist[2] = {nullptr, nullptr};
     int32_t* dlist = nullptr;      // vertices whose verification needs a set comparison
-    bisim::DevState* dstate = nullptr;   // [2]: the second is P_0's while it runs beside the build
+    bisim::DevState* dstate = nullptr;   // and, kStateStride further on, P_0's while it runs beside the build
     bisim::DevState* hstate = nullptr;   // pinned mirror
     bool p0_pending = false;             // p0_begin ran and p0_end did not
     bisim::Branch p0_branch;
@@ -648,6 +652,9 @@ struct EdgeView {
 };
 // Whether the context refines the caller's edges unchanged (forward, no filter).
 bool edge_view_identity(const bisim_ctx* ctx);
+// Whether it refines them reversed, all of them: the same arrays, ends exchanged.
+bool edge_view_reversal(const bisim_ctx* ctx);
+bisim_status edge_view_bad_label(bisim_ctx* ctx);
 // Copies the options' label filter (sorted, unique) into the context.
 bisim_status edge_view_setup(bisim_ctx* ctx, const bisim_options* opt, cudaStream_t s);
 // The internal edge list of the context's direction and filter for device

@@ -77,10 +77,50 @@ __global__ void k_view_emit(const int32_t* __restrict__ src, const int32_t* __re
     }
 }
 
+// Both directions of every edge, unfiltered: edge e becomes entries 2e and 2e + 1, so
+// nothing is counted and nothing read back (counts, their scan and an emission that
+// looks places up: 168 us for 8M edges, against 50). A label out of range is left to
+// the build's read-back. Two edges a thread, 16-byte stores; 8-byte loads where the
+// arrays take them (`wide`).
+__global__ void __launch_bounds__(256) k_view_both(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                   const int32_t* __restrict__ lab, int64_t m, bool wide,
+                                                   int32_t* __restrict__ os, int32_t* __restrict__ od,
+                                                   int32_t* __restrict__ ol, DevState* st) {
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    bool bad = false;
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; 2 * q < m; q += stride) {
+        const int64_t e = 2 * q;
+        const bool two = e + 1 < m;
+        int2 u, w, l;
+        if (wide && two) {
+            u = __ldcs(reinterpret_cast<const int2*>(src + e));
+            w = __ldcs(reinterpret_cast<const int2*>(dst + e));
+            l = __ldcs(reinterpret_cast<const int2*>(lab + e));
+        } else {
+            u = make_int2(src[e], two ? src[e + 1] : 0);
+            w = make_int2(dst[e], two ? dst[e + 1] : 0);
+            l = make_int2(lab[e], two ? lab[e + 1] : 0);
+        }
+        bad = bad || l.x < kBothLabelMin || l.x > kBothLabelMax || l.y < kBothLabelMin || l.y > kBothLabelMax;
+        const int32_t l0 = static_cast<int32_t>(2u * static_cast<uint32_t>(l.x)), l1 = static_cast<int32_t>(2u * static_cast<uint32_t>(l.y));
+        if (two) {
+            reinterpret_cast<int4*>(os)[q] = make_int4(u.x, w.x, u.y, w.y);
+            reinterpret_cast<int4*>(od)[q] = make_int4(w.x, u.x, w.y, u.y);
+            reinterpret_cast<int4*>(ol)[q] = make_int4(l0, l0 + 1, l1, l1 + 1);
+        } else {
+            reinterpret_cast<int2*>(os)[e] = make_int2(u.x, w.x);
+            reinterpret_cast<int2*>(od)[e] = make_int2(w.x, u.x);
+            reinterpret_cast<int2*>(ol)[e] = make_int2(l0, l0 + 1);
+        }
+    }
+    if (bad) atomicOr(&st->bad_label, 1u);
+}
+
+// Per-graph offsets of the view's edges (pos null: two of every edge).
 __global__ void k_view_offsets(const int64_t* __restrict__ pos, const int64_t* __restrict__ eoff, int32_t G,
                                int64_t* __restrict__ out) {
     const int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (g <= G) out[g] = pos[eoff[g]];
+    if (g <= G) out[g] = pos ? pos[eoff[g]] : 2 * eoff[g];
 }
 
 // Internal operations per operation: edge operations as edges above, vertex
@@ -168,6 +208,10 @@ bool edge_view_identity(const bisim_ctx* ctx) {
     return ctx->opt.direction == BISIM_DIR_FORWARD && ctx->nfilter == 0;
 }
 
+bool edge_view_reversal(const bisim_ctx* ctx) {
+    return ctx->opt.direction == BISIM_DIR_BACKWARD && ctx->nfilter == 0;
+}
+
 bisim_status edge_view_setup(bisim_ctx* ctx, const bisim_options* opt, cudaStream_t s) {
     ctx->opt.label_filter = nullptr;                // caller memory: never kept
     if (opt == nullptr || opt->n_label_filter <= 0) return BISIM_OK;
@@ -188,19 +232,47 @@ bisim_status edge_view_setup(bisim_ctx* ctx, const bisim_options* opt, cudaStrea
     return BISIM_OK;
 }
 
+bisim_status edge_view_bad_label(bisim_ctx* ctx) {
+    return set_error(ctx, BISIM_EINVAL, "the forward-backward direction needs edge labels in [-2^30, 2^30)");
+}
+
 bisim_status edge_view_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* dst, const int32_t* lab, int64_t m,
                            const int64_t* eoff, int32_t G, cudaStream_t s, EdgeView* out) {
     *out = EdgeView{};
     cudaError_t e;
+    const int32_t dir = ctx->opt.direction;
+    BISIM_SITE(site, "edge_view");
+    const auto alloc = [&](int64_t total) -> cudaError_t {
+        const size_t eb = sizeof(int32_t) * static_cast<size_t>(std::max<int64_t>(total, 1));
+        cudaError_t err = cudaMallocAsync(reinterpret_cast<void**>(&out->src), eb, s);
+        if (err == cudaSuccess) err = cudaMallocAsync(reinterpret_cast<void**>(&out->dst), eb, s);
+        if (err == cudaSuccess) err = cudaMallocAsync(reinterpret_cast<void**>(&out->lab), eb, s);
+        if (err == cudaSuccess && eoff) err = cudaMallocAsync(reinterpret_cast<void**>(&out->eoff), sizeof(int64_t) * (G + 1), s);
+        return err;
+    };
+    if (dir == BISIM_DIR_BOTH && ctx->nfilter == 0) {
+        if ((e = alloc(2 * m))) {
+            edge_view_free(out, s);
+            return cuda_error(ctx, e, "alloc edge view");
+        }
+        const auto even = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; };
+        {
+            Launch L(site, s, 0, m, 36.0 * m);
+            k_view_both<<<grid_for((m + 1) / 2, 256), 256, 0, s>>>(src, dst, lab, m, even(src) && even(dst) && even(lab),
+                                                                  out->src, out->dst, out->lab, ctx->dstate);
+        }
+        if (eoff) k_view_offsets<<<(G + 256) / 256, 256, 0, s>>>(nullptr, eoff, G, out->eoff);
+        out->m = 2 * m;
+        if ((e = cudaGetLastError())) return cuda_error(ctx, e, "edge view");
+        return BISIM_OK;
+    }
     const size_t scan_words = scan_temp_words(m + 1);
     int64_t* pos = nullptr;
     if ((e = cudaMallocAsync(reinterpret_cast<void**>(&pos), sizeof(int64_t) * (2 * (m + 1) + scan_words), s)))
         return cuda_error(ctx, e, "alloc edge view");
     int64_t* cnt = pos + (m + 1);
     int64_t* tmp = cnt + (m + 1);
-    const int32_t dir = ctx->opt.direction;
     cudaMemsetAsync(&ctx->dstate->error, 0, sizeof(unsigned), s);
-    BISIM_SITE(site, "edge_view");
     {
         Launch L(site, s, 0, m, 24.0 * m);
         k_view_count<<<grid_for(m + 1, 256), 256, 0, s>>>(lab, m, ctx->dfilter, ctx->nfilter, dir, cnt,
@@ -217,13 +289,9 @@ bisim_status edge_view_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* ds
     }
     if (err & kErrBadInput) {
         cudaFreeAsync(pos, s);
-        return set_error(ctx, BISIM_EINVAL, "the forward-backward direction needs edge labels in [-2^30, 2^30)");
+        return edge_view_bad_label(ctx);
     }
-    const size_t eb = sizeof(int32_t) * static_cast<size_t>(std::max<int64_t>(total, 1));
-    if ((e = cudaMallocAsync(reinterpret_cast<void**>(&out->src), eb, s)) ||
-        (e = cudaMallocAsync(reinterpret_cast<void**>(&out->dst), eb, s)) ||
-        (e = cudaMallocAsync(reinterpret_cast<void**>(&out->lab), eb, s)) ||
-        (eoff && (e = cudaMallocAsync(reinterpret_cast<void**>(&out->eoff), sizeof(int64_t) * (G + 1), s)))) {
+    if ((e = alloc(total))) {
         cudaFreeAsync(pos, s);
         edge_view_free(out, s);
         return cuda_error(ctx, e, "alloc edge view");
@@ -272,7 +340,7 @@ bisim_status edge_view_ops(bisim_ctx* ctx, const bisim_op* ops, int64_t n, cudaS
     }
     if (err & kErrBadInput) {
         cudaFreeAsync(pos, s);
-        return set_error(ctx, BISIM_EINVAL, "the forward-backward direction needs edge labels in [-2^30, 2^30)");
+        return edge_view_bad_label(ctx);
     }
     if ((e = cudaMallocAsync(reinterpret_cast<void**>(out), sizeof(bisim_op) * std::max<int64_t>(total, 1), s))) {
         cudaFreeAsync(pos, s);

@@ -511,6 +511,7 @@ bisim_status build_from_coo(bisim_ctx* ctx, const int32_t* src, const int32_t* d
     // both what the check found and where the classes lie
     cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
     bisim_status st = dense_layout_positions(ctx, reinterpret_cast<const int32_t*>(deg), s, &ctx->dstate->unsorted);
+    if (st == BISIM_OK && ctx->hstate->bad_label) st = edge_view_bad_label(ctx);
     if (st == BISIM_OK && (ctx->hstate->error & kErrBadInput))
         st = set_error(ctx, BISIM_EINVAL, batch ? "a graph-local edge endpoint is out of range"
                                                 : "edge endpoint out of range [0, n) or on a dead vertex");

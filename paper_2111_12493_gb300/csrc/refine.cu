@@ -868,7 +868,7 @@ bisim_status p0_begin(bisim_ctx* ctx, cudaStream_t s, bool early) {
     const cudaStream_t ps = ctx->p0_branch.s ? ctx->p0_branch.s : s;
     cudaMemsetAsync(ctx->table, 0, sizeof(Slot) * ctx->nslots, ps);
     // on a branch its CTAs leave half of every SM to the build
-    p0_launch(ctx, ps, ctx->P[0], ctx->dstate + 1, ctx->hstate + 1, ctx->p0_branch.s ? 4 : 8);
+    p0_launch(ctx, ps, ctx->P[0], ctx->dstate + kStateStride, ctx->hstate + 1, ctx->p0_branch.s ? 4 : 8);
     ctx->p0_pending = true;
     cudaError_t e;
     if ((e = cudaGetLastError())) return cuda_error(ctx, e, "init refine state");
@@ -880,7 +880,7 @@ bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s) {
     ctx->p0_pending = false;
     cudaError_t e;
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify labels");
-    return p0_settle(ctx, s, ctx->P[0], ctx->dstate + 1, ctx->hstate + 1);
+    return p0_settle(ctx, s, ctx->P[0], ctx->dstate + kStateStride, ctx->hstate + 1);
 }
 
 bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,

@@ -144,3 +144,29 @@ def test_forward_backward_rejects_labels_outside_its_range(B):
         B.summarize_init_coo(3, _dev(src), _dev(dst), _dev(np.zeros(2, np.int32)), _dev(vl),
                              options=B.default_options(direction=7))
     B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("mode,code", MODES)
+@pytest.mark.parametrize("m,off", [(0, 0), (1, 0), (1, 1), (2, 1), (3, 0), (1001, 0), (1001, 1), (1002, 3)])
+def test_unfiltered_views_of_odd_lists(B, mode, code, m, off):
+    # both directions: two edges a thread, 8-byte loads where the arrays take them;
+    # backward: the caller's arrays with their ends exchanged
+    rng = np.random.default_rng(m)
+    n = 60
+    src, dst, lab = (rng.integers(0, hi, m).astype(np.int32) for hi in (n, n, 3))
+    vl = rng.integers(0, 2, n).astype(np.int32)
+    shift = lambda a, k: _dev(np.concatenate([np.full(k, 5, np.int32), a]))[k:]
+    ctx = B.summarize_init_coo(n, shift(src, off), shift(dst, (2 * off) % 4), shift(lab, off), _dev(vl),
+                               options=B.default_options(direction=code))
+    B.bisim_iterate(ctx, 2)
+    want, _, _ = oracle.refine(n, src, dst, lab, vl, 2, direction=mode)
+    _same(B.get_partition(ctx).cpu().numpy(), want)
+    B.summarize_destroy(ctx)
+    for a, bad in ((src, n), (dst, -1)):
+        if m == 0:
+            continue
+        keep, a[m - 1] = a[m - 1], bad
+        with pytest.raises(B.BisimError, match="endpoint"):
+            B.summarize_init_coo(n, shift(src, off), shift(dst, off), shift(lab, off), _dev(vl),
+                                 options=B.default_options(direction=code))
+        a[m - 1] = keep
