@@ -890,12 +890,44 @@ bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pi
                             ? GraphView{ctx->xro, ctx->xlen, nullptr, nullptr, ctx->xpe, Pin, hout}
                             : GraphView{ctx->row_ptr, nullptr, ctx->col, ctx->elab, nullptr, Pin, hout};
     TableRef t = next_epoch(ctx, s);
-    if (B.n_hub > 0) {
-        cudaMemsetAsync(B.tab, 0, sizeof(unsigned long long) * B.tab_words, s);
-        cudaMemsetAsync(B.acc, 0, sizeof(HubAcc) * B.n_hub, s);
-    }
     const int64_t* cb = B.begin;
     unsigned* err = &ctx->dstate->error;
+    // the hubs' chain, the CTA classes and the others run beside each other (the
+    // first two leave most of an SM's warps unused), the longer rows first
+    Branch hubs = B.n_chunks > 0 && !prof_enabled() ? branch_fork(ctx->device, s) : Branch{};
+    if (B.n_hub > 0) {
+        const cudaStream_t hs = hubs.s ? hubs.s : s;
+        cudaMemsetAsync(B.tab, 0, sizeof(unsigned long long) * B.tab_words, hs);
+        cudaMemsetAsync(B.acc, 0, sizeof(HubAcc) * B.n_hub, hs);
+        if (B.n_chunks > 0) {
+            BISIM_SITE(site_hi, "hub_insert");
+            BISIM_SITE(site_hf, "hub_finalize");
+            const int64_t hub_edges = B.edges[kClassHub];
+            {
+                Launch L1(site_hi, hs, 0, hub_edges, kSigBytesPerEdge * hub_edges);
+                k_hub_insert<<<static_cast<unsigned>(B.n_chunks), 256, 0, hs>>>(B.chunks, G, B.toff, B.tmask, B.tab, B.acc,
+                                                                               ctx->skey, err);
+            }
+            Launch L2(site_hf, hs, B.n_hub, 0, kSigBytesPerVertex * B.n_hub);
+            k_hub_finalize<<<grid_for(B.n_hub, 128), 128, 0, hs>>>(B.hub_list, B.n_hub, G, B.acc, ctx->cnt, ctx->slot, t,
+                                                                  err);
+        }
+    }
+    const int64_t ctas = cb[kClassHub] - cb[kSmallClasses + 3];
+    Branch mids = ctas > 0 && cb[kSmallClasses + 3] > cb[0] && !prof_enabled() ? branch_fork(ctx->device, s) : Branch{};
+    const cudaStream_t ms = mids.s ? mids.s : s;
+    auto mid = [&](int c) {
+        const int k = kSmallClasses + c;
+        return std::make_tuple(B.class_list + cb[k], cb[k + 1] - cb[k], B.edges[k]);
+    };
+    { auto [l, c, e] = mid(7); if (c > 0) launch_mid<8192>(ctx, l, c, e, G, t, ms); }
+    { auto [l, c, e] = mid(6); if (c > 0) launch_mid<4096>(ctx, l, c, e, G, t, ms); }
+    { auto [l, c, e] = mid(5); if (c > 0) launch_mid<2048>(ctx, l, c, e, G, t, ms); }
+    { auto [l, c, e] = mid(4); if (c > 0) launch_mid<1024>(ctx, l, c, e, G, t, ms); }
+    { auto [l, c, e] = mid(3); if (c > 0) launch_mid<512>(ctx, l, c, e, G, t, ms); }
+    { auto [l, c, e] = mid(2); if (c > 0) launch_mid<256>(ctx, l, c, e, G, t, s); }
+    { auto [l, c, e] = mid(1); if (c > 0) launch_mid<128>(ctx, l, c, e, G, t, s); }
+    { auto [l, c, e] = mid(0); if (c > 0) launch_mid<64>(ctx, l, c, e, G, t, s); }
     static const int small_site[kSmallClasses] = {prof_site("sig_small_4"), prof_site("sig_small_8"),
                                                    prof_site("sig_small_16"), prof_site("sig_small_32")};
     auto small = [&](int c, auto kern) {
@@ -907,35 +939,12 @@ bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pi
                                                    ctx->slot, t, err);
         }
     };
-    small(0, k_sig_small<4>);
-    small(1, k_sig_small<8>);
-    small(2, k_sig_small<16>);
     small(3, k_sig_small<32>);
-    auto mid = [&](int c) {
-        const int k = kSmallClasses + c;
-        return std::make_tuple(B.class_list + cb[k], cb[k + 1] - cb[k], B.edges[k]);
-    };
-    { auto [l, c, e] = mid(0); if (c > 0) launch_mid<64>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(1); if (c > 0) launch_mid<128>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(2); if (c > 0) launch_mid<256>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(3); if (c > 0) launch_mid<512>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(4); if (c > 0) launch_mid<1024>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(5); if (c > 0) launch_mid<2048>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(6); if (c > 0) launch_mid<4096>(ctx, l, c, e, G, t, s); }
-    { auto [l, c, e] = mid(7); if (c > 0) launch_mid<8192>(ctx, l, c, e, G, t, s); }
-    if (B.n_chunks > 0) {
-        BISIM_SITE(site_hi, "hub_insert");
-        BISIM_SITE(site_hf, "hub_finalize");
-        const int64_t hub_edges = B.edges[kClassHub];
-        {
-            Launch L1(site_hi, s, 0, hub_edges, kSigBytesPerEdge * hub_edges);
-            k_hub_insert<<<static_cast<unsigned>(B.n_chunks), 256, 0, s>>>(B.chunks, G, B.toff, B.tmask, B.tab, B.acc,
-                                                                          ctx->skey, err);
-        }
-        Launch L2(site_hf, s, B.n_hub, 0, kSigBytesPerVertex * B.n_hub);
-        k_hub_finalize<<<grid_for(B.n_hub, 128), 128, 0, s>>>(B.hub_list, B.n_hub, G, B.acc, ctx->cnt, ctx->slot, t,
-                                                             err);
-    }
+    small(2, k_sig_small<16>);
+    small(1, k_sig_small<8>);
+    small(0, k_sig_small<4>);
+    branch_join(ctx->device, &mids, s);
+    branch_join(ctx->device, &hubs, s);
     cudaError_t e;
     if ((e = cudaGetLastError())) return cuda_error(ctx, e, "launch signature kernels");
     SigMode M;
