@@ -535,10 +535,14 @@ TableRef next_epoch(bisim_ctx* ctx, cudaStream_t s);
 // One signature round over the vertices of `B` (all of them, or the `vcount`
 // listed in `vlist` for verification): Pout[v] = smallest listed vertex with
 // v's exact signature over the labelling Pin; hout[v] (nullable) receives the
-// signature hash that was inserted.
-bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
-                             const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s,
-                             int64_t* out_blocks);
+// signature hash that was inserted. signature_launch leaves its state's copy to
+// ctx->hstate under way; once `s` is synchronised, signature_settle reports errors
+// and runs the collision levels, if any (*changed). Until then a vertex whose hash
+// collided stands for itself in Pout.
+bisim_status signature_launch(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
+                              const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s);
+bisim_status signature_settle(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
+                              unsigned long long* hout, cudaStream_t s, bool* changed);
 void pin_partition_in_l2(bisim_ctx* ctx, const int32_t* P, cudaStream_t s);
 void unpin_partition(bisim_ctx* ctx, cudaStream_t s);
 void launch_local_ids(const bisim_ctx* ctx, int32_t* out, cudaStream_t s);

@@ -1193,9 +1193,9 @@ void launch_frontier(bisim_ctx* ctx, Scratch& S, int j, const uint8_t* a, const 
 }
 
 // One level over the frontier launch_frontier made. Host round trips: one
-// read-back of the frontier's sizes and buckets, the signature round's own,
-// and one per probe round that still has candidates. The level's block-id and
-// index checks are read back once for all levels by inc_finish.
+// read-back of the frontier's sizes and buckets, one of the signature round and the
+// first probe round, and one per further probe round that still has candidates. The
+// level's block-id and index checks are read back once for all levels by inc_finish.
 bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cudaStream_t s) {
     Work& W = S.W;
     Level L = level_view(ctx, j);
@@ -1247,26 +1247,30 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
                                                           ctx->opt.hash_bits >= 64 ? ~0ull : ((1ull << ctx->opt.hash_bits) - 1));
         } else {
             if ((st = finish_buckets(ctx, S, LB, s)) != BISIM_OK) return st;
-            int64_t blocks = 0;
-            st = signature_round(ctx, LB.B, ctx->lid[j - 1], W.grp, W.FL, fl, W.h, s, &blocks);
+            st = signature_launch(ctx, LB.B, ctx->lid[j - 1], W.grp, W.FL, fl, W.h, s);
             if (st != BISIM_OK) {
                 if (LB.hubmem) cudaFreeAsync(LB.hubmem, s);
                 return st;
             }
         }
-        Launch Lk(site_group, s, fl, 0, 24.0 * fl);
-        k_group_init<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, W);
-        k_group_stats<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, W);
     }
     // 3. match live blocks: probe, compare the candidates (their number is read
     // on the device), probe again; the host only looks when a probe round
-    // still leaves candidates (different signatures under one hash)
+    // still leaves candidates (different signatures under one hash), and with the
+    // first of them at the signatures: groups whose hashes collided were taken apart
+    // too far until then, so they are made and matched again
     const uint64_t hmask = ctx->opt.hash_bits >= 64 ? ~0ull : ((1ull << ctx->opt.hash_bits) - 1);
-    if (fl > 0) {
+    const auto group_and_probe = [&] {
+        {
+            Launch Lk(site_group, s, fl, 0, 24.0 * fl);
+            k_group_init<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, W);
+            k_group_stats<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, W);
+        }
         Launch Lk(site_probe, s, fl, 0, 32.0 * fl);
         cudaMemsetAsync(&W.counters[2], 0, 8, s);
         k_probe<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, L, W, j, ctx->vlabel, hmask);
-    }
+    };
+    if (fl > 0) group_and_probe();
     for (int iter = 0; fl > 0 && j > 0; ++iter) {
         if (iter > 1 << 16) {
             if (LB.hubmem) cudaFreeAsync(LB.hubmem, s);
@@ -1300,6 +1304,18 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
         }
         cudaMemcpyAsync(&S.h->ncand, &W.counters[2], 8, cudaMemcpyDeviceToHost, s);
         if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "probe blocks");
+        if (iter == 0) {
+            bool changed = false;
+            st = signature_settle(ctx, LB.B, ctx->lid[j - 1], W.grp, W.h, s, &changed);
+            if (st != BISIM_OK) {
+                if (LB.hubmem) cudaFreeAsync(LB.hubmem, s);
+                return st;
+            }
+            if (changed) {
+                group_and_probe();
+                continue;
+            }
+        }
         if (S.h->ncand == 0) break;
     }
     if (LB.hubmem) cudaFreeAsync(LB.hubmem, s);

@@ -517,7 +517,9 @@ __global__ void k_resolve_verify(const int32_t* __restrict__ list, int64_t count
                 else defer = true;
             }
         }
-        if (!push && !defer) {
+        if (push || defer) {
+            Pout[v] = v;               // alone until it is decided, for who looks before the levels have run
+        } else {
             Pout[v] = block;
             if (also) also[v] = block;
         }
@@ -703,15 +705,6 @@ bisim_status resolve_settle(bisim_ctx* ctx, Mode M, int32_t* Pout, cudaStream_t 
     return BISIM_OK;
 }
 
-template <class Mode>
-bisim_status resolve(bisim_ctx* ctx, Mode M, int32_t* Pout, const int32_t* vlist, int64_t vcount, cudaStream_t s,
-                     int64_t* blocks) {
-    resolve_launch(ctx, M, Pout, vlist, vcount, s, nullptr, ctx->dstate, ctx->hstate);
-    cudaError_t e;
-    if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "verify signatures");
-    return resolve_settle(ctx, M, Pout, s, blocks, nullptr, ctx->dstate, ctx->hstate);
-}
-
 // Algorithmic bytes of the signature kernels: per edge col 4 + label 4 + the
 // gathered P_i[w] 4; per vertex row_ptr 4 + P_i[v] 4 + one 16-byte table slot.
 constexpr double kSigBytesPerEdge = 12.0;
@@ -883,12 +876,39 @@ bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s) {
     return p0_settle(ctx, s, ctx->P[0], ctx->dstate + kStateStride, ctx->hstate + 1);
 }
 
-bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
-                             const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s,
-                             int64_t* out_blocks) {
-    const GraphView G = ctx->store_ready
-                            ? GraphView{ctx->xro, ctx->xlen, nullptr, nullptr, ctx->xpe, Pin, hout}
+namespace {
+
+GraphView graph_view(const bisim_ctx* ctx, const int32_t* Pin, unsigned long long* hout) {
+    return ctx->store_ready ? GraphView{ctx->xro, ctx->xlen, nullptr, nullptr, ctx->xpe, Pin, hout}
                             : GraphView{ctx->row_ptr, nullptr, ctx->col, ctx->elab, nullptr, Pin, hout};
+}
+
+SigMode sig_mode(const bisim_ctx* ctx, const Buckets& B, const GraphView& G) {
+    SigMode M;
+    M.G = G;
+    M.cnt = ctx->cnt;
+    M.skey = ctx->skey;
+    M.H = HubView{B.hub_list, B.n_hub, B.toff, B.tmask, B.tab, B.acc};
+    // lists of up to small_max entries are sorted (thread-per-vertex classes); the
+    // incremental path sets its own limit per batch
+    M.small_max = ctx->store_ready ? ctx->inc_small_max : ctx->opt.small_max_degree;
+    M.mid_max = ctx->opt.mid_max_degree;
+    return M;
+}
+
+}  // namespace
+
+bisim_status signature_settle(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
+                              unsigned long long* hout, cudaStream_t s, bool* changed) {
+    int64_t blocks = 0;
+    *changed = ctx->hstate->error == 0 && ctx->hstate->unresolved > 0;
+    return resolve_settle(ctx, sig_mode(ctx, B, graph_view(ctx, Pin, hout)), Pout, s, &blocks, nullptr, ctx->dstate,
+                          ctx->hstate);
+}
+
+bisim_status signature_launch(bisim_ctx* ctx, const Buckets& B, const int32_t* Pin, int32_t* Pout,
+                              const int32_t* vlist, int64_t vcount, unsigned long long* hout, cudaStream_t s) {
+    const GraphView G = graph_view(ctx, Pin, hout);
     TableRef t = next_epoch(ctx, s);
     const int64_t* cb = B.begin;
     unsigned* err = &ctx->dstate->error;
@@ -947,16 +967,8 @@ bisim_status signature_round(bisim_ctx* ctx, const Buckets& B, const int32_t* Pi
     branch_join(ctx->device, &hubs, s);
     cudaError_t e;
     if ((e = cudaGetLastError())) return cuda_error(ctx, e, "launch signature kernels");
-    SigMode M;
-    M.G = G;
-    M.cnt = ctx->cnt;
-    M.skey = ctx->skey;
-    M.H = HubView{B.hub_list, B.n_hub, B.toff, B.tmask, B.tab, B.acc};
-    // lists of up to small_max entries are sorted (thread-per-vertex classes); the
-    // incremental path sets its own limit per batch
-    M.small_max = ctx->store_ready ? ctx->inc_small_max : ctx->opt.small_max_degree;
-    M.mid_max = ctx->opt.mid_max_degree;
-    return resolve(ctx, M, Pout, vlist, vcount, s, out_blocks);
+    resolve_launch(ctx, sig_mode(ctx, B, G), Pout, vlist, vcount, s, nullptr, ctx->dstate, ctx->hstate);
+    return BISIM_OK;
 }
 
 void launch_local_ids(const bisim_ctx* ctx, int32_t* out, cudaStream_t s) {
