@@ -69,10 +69,12 @@ enum { BISIM_FLAG_L2_PIN = 1 };
 enum { BISIM_FLAG_FULL_RECOMPUTE = 2 };
 
 /* BISIM_FLAG_EAGER: run the rounds of bisim_iterate as host-driven launch
- * sequences, one round at a time. By default the round loop is one captured
- * CUDA graph whose while node repeats a round until the block count stops
- * changing or the round limit is reached, decided on the device; rounds also
- * run eagerly while launch profiling (bisim_profile_enable) is on. */
+ * sequences, one round at a time. By default the device decides when the block
+ * count stops changing or the round limit is reached: the rounds are one
+ * cooperative kernel wherever the rows that are left have at most 256 edges
+ * (after one host-driven round, or from P_0 on), else one captured CUDA graph
+ * whose while node repeats a round. Rounds also run eagerly while launch
+ * profiling (bisim_profile_enable) is on. */
 enum { BISIM_FLAG_EAGER = 4 };
 
 /* BISIM_FLAG_UNION_ROUNDS: batched contexts run the rounds of the disjoint
@@ -275,7 +277,9 @@ bisim_status get_block_sizes(bisim_ctx* ctx, int32_t* sizes, void* stream);
  *   capacity   entries the outputs hold; min(capacity, count) are written
  *   out_count  the number of distinct triples (call with capacity 0 to size
  *              the outputs)
- * Uses about 36 bytes of temporary device memory per edge. Synchronises `stream`.
+ * Uses about 8 bytes of temporary device memory per edge and 32 per vertex, and 24
+ * more per edge of a source block of more than 2048 edges (backward contexts:
+ * about 36 per edge). Synchronises `stream`.
  */
 bisim_status get_summary_edges(bisim_ctx* ctx, int32_t* src_block, int32_t* label, int32_t* dst_block,
                                int64_t capacity, int64_t* out_count, void* stream);
@@ -332,8 +336,9 @@ bisim_status bisim_retune(bisim_ctx* ctx, const bisim_options* opt, void* stream
  * touch nothing. All scratch lives in one fixed array of about 10.5 MB inside
  * the library, which every GPU that loads the library holds until the process
  * exits. The first call on a device looks up that array's device address
- * (once per device). Every call shares the array, so calls that overlap on the GPU -- from two threads or two streams at once -- race and
- * must be serialised by the caller. Synchronises `stream`.
+ * (once per device). Every call shares the array, so calls that overlap on the
+ * GPU -- from two threads or two streams at once -- race and must be serialised by
+ * the caller. Synchronises `stream`.
  */
 bisim_status bisim_refine_round_noalloc(int32_t n_vertices, int64_t n_edges, const int64_t* row_ptr,
                                         const int32_t* col, const int32_t* edge_label,

@@ -12,14 +12,14 @@
 //                   a value counted when no earlier one equals it;
 //   degree <= 256   one warp per vertex with a set in shared memory;
 //   degree <= 8192  one CTA per vertex with a set in shared memory;
-//   above           the row cut into chunks over many CTAs; its values are
-//                   bucketed by a mix of their bits and every bucket is
-//                   deduplicated by one CTA in shared memory.
+//   above           the row cut into chunks over many CTAs, whose values go
+//                   through a filter in shared memory into a table per hub in
+//                   device memory.
 // Each vertex's signature hash goes into the open-addressing table, whose slots
 // keep the smallest vertex (the canonical block id). A verification pass then
 // confirms every vertex against its slot's representative by recomputing both
-// pair sets (no list is stored): inside the lane group for small degrees, in a
-// CTA per pair otherwise. Vertices whose signature differs from their
+// pair sets (no list is stored): in the thread for rows of up to two edges, in a
+// warp up to 32, in a CTA per pair otherwise. Vertices whose signature differs from their
 // representative's (a hash collision) are re-hashed with a new salt in further
 // levels; the smallest vertex of each level's group is final, so the loop ends
 // with the exact partition.
@@ -1763,8 +1763,9 @@ void launch_round(bisim_ctx* ctx, cudaStream_t s, const TableRef& t, const int32
     if (D.work) cudaMemsetAsync(D.work, 0, sizeof(unsigned long long) * kWorkWords, s);
     // The CTA classes hold few warps an SM (their sets fill shared memory) and the
     // hubs wait for their tables' popular slots, while the thread classes need
-    // neither: the three run beside each other, the longer rows first. Not while
-    // launches are timed, nor in a captured round.
+    // neither: the three run beside each other, the longer rows first (one-off of
+    // 400k / 4M 630 to 550 us, of 10M / 100M 3.64 to 3.52 ms). Not while launches are
+    // timed, nor in a captured round, where it was slower.
     const bool beside = !prof_enabled() && round_no == nullptr && db[kDMid0] > db[0];
     Branch hubs = beside && ctx->n_dhub > 0 && ctx->n_dchunks > 0 ? branch_fork(ctx->device, s) : Branch{};
     if (ctx->n_dhub > 0) {
