@@ -379,7 +379,7 @@ def rounds_roofline(bisim, torch, W, d_in, stream, peak, executed):
     """Per round i: survey bytes of the rows and vertices it processed / its event time.
 
     Round i's time is T(i) - T(i-1), T(k) the best event time of bisim_iterate(k)
-    on a resident context (captured device-side loop); its work is counted on the
+    on a resident context (loop decided on the device); its work is counted on the
     device in an eager profiled run of the same k. Workloads with many rounds
     report rounds 1-3 and the mean of the rest."""
     ctx = W.init_only(bisim, d_in)
@@ -594,7 +594,7 @@ def run_ours(args, world, rank, local):
                                 **({"batch_split": int(W.options.batch_split) if W.options else None}
                                    if W.batched else {})}),
             "iterate_only": {"value": iterate_only, "unit": UNIT, "rounds_executed": int(it_exec),
-                             "note": "bisim_iterate alone on a resident context (round graph already captured)"},
+                             "note": "bisim_iterate alone on a resident context"},
             "profiled_steps": {"ms_per_step": profiled_ms / args.steps,
                                "note": "the timed steps again with per-launch CUDA events (rounds run eagerly); "
                                        "kernels and roofline come from these"},
