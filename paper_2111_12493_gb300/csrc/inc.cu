@@ -23,6 +23,7 @@
 // The output partition names each level-k block by its smallest member.
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -923,19 +924,29 @@ constexpr int kHubPrefetch = 2048;     // hub records read back with the level's
 constexpr size_t kHubStageBytes = size_t{1} << 20;   // pinned stage of a frontier's hub layout
 constexpr int64_t kThreadClassOps = 20000;   // batches above this use thread-per-vertex classes
 
+// A level's words: cleared together when the level begins, and read back together,
+// with the first hub records, which follow them on the device.
+struct alignas(256) LevelWords {
+    unsigned long long counters[16];         // Work::counters
+    unsigned long long count[kNumClasses];   // live frontier per class: vertices, row entries
+    unsigned long long edges[kNumClasses];
+    unsigned n_hubs;
+    unsigned tiers[4];                       // in-row tasks per tier
+    unsigned pad;
+    int64_t begin[kNumClasses + 1];          // first vertex of each class, by k_class_scan
+    unsigned long long cursor[kNumClasses];
+};
+
 // Host copies of everything a level pass reads back, in pinned memory so that
 // the copies queue behind the level's kernels and one synchronisation covers them.
 struct HostStage {
-    unsigned long long counters[16];
-    int64_t begin[kNumClasses + 1];
-    unsigned long long edges[kNumClasses];
-    unsigned n_hubs;
+    LevelWords w;
+    HubInfo hubs[kHubPrefetch];
     unsigned err;
     unsigned long long ncand;
     int64_t bnext[kMaxIncLevels + 1];
     unsigned long long acc[kMaxIncLevels + 1][4];
     long long fc[kMaxIncLevels + 1][3];
-    HubInfo hubs[kHubPrefetch];
 };
 
 // Work buffers of the incremental path, kept between batches.
@@ -947,12 +958,8 @@ struct Scratch {
     unsigned long long* dacc = nullptr;   // [kMaxIncLevels + 1][4] per-level accumulators (k_settle)
     long long* dfree = nullptr;        // [kMaxIncLevels + 1][3] free-list counters (Level::fc)
     int32_t* blist = nullptr;          // [n] live frontier grouped by class
-    int64_t* dbegin = nullptr;         // [kNumClasses + 1]
-    unsigned long long* ccount = nullptr;   // [kNumClasses] vertices per class
-    unsigned long long* cedges = nullptr;   // [kNumClasses] row entries per class
-    unsigned long long* ccursor = nullptr;  // [kNumClasses]
+    LevelWords* words = nullptr;       // the level's (W.counters is its first member), followed by hubs
     HubInfo* hubs = nullptr;           // [n]
-    unsigned* n_hubs = nullptr;
     int32_t* clist = nullptr;          // [n] vertices whose block changed one level down
     unsigned long long* chcount = nullptr;
     TierLists tiers{};                 // in-row tasks, [n] per tier
@@ -971,14 +978,13 @@ cudaError_t alloc_scratch(bisim_ctx* ctx, Scratch& S, cudaStream_t s) {
     auto need = [&](size_t b) { bytes += (b + 255) & ~size_t(255); };
     need(4 * n); need(4 * n); need(8 * n); need(4 * n); need(4 * n); need(4 * n); need(4 * n); need(8 * n);
     need(4 * bc); need(4 * bc); need(4 * dw); need(4 * bc); need(4 * bc);
-    need(4 * n); need(4 * n); need(8 * 16); need(4 * n); need(4 * n); need(n); need(n); need(n); need(n); need(4 * n);
+    need(4 * n); need(4 * n); need(4 * n); need(4 * n); need(n); need(n); need(n); need(n); need(4 * n);
     size_t lslots = 64;
     while (lslots < 2 * n) lslots <<= 1;
     need(8 * lslots);
     need(8 * L); need(32 * L); need(24 * L); need(32);
-    need(4 * n); need(8 * (kNumClasses + 1)); need(8 * kNumClasses); need(8 * kNumClasses); need(8 * kNumClasses);
-    need(sizeof(HubInfo) * std::max<size_t>(n, kHubPrefetch)); need(16);
-    need(4 * n); need(16); need(3 * sizeof(RowTask) * n); need(16);
+    need(4 * n); need(sizeof(LevelWords)); need(sizeof(HubInfo) * std::max<size_t>(n, kHubPrefetch));
+    need(4 * n); need(16); need(3 * sizeof(RowTask) * n);
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&S.base), bytes, s);
     if (e) return e;
     S.bytes = bytes;
@@ -1013,13 +1019,13 @@ cudaError_t alloc_scratch(bisim_ctx* ctx, Scratch& S, cudaStream_t s) {
     W.dlist = reinterpret_cast<int32_t*>(carve(4 * bc));
     W.cand = reinterpret_cast<int32_t*>(carve(4 * n));
     W.candb = reinterpret_cast<int32_t*>(carve(4 * n));
-    W.counters = reinterpret_cast<unsigned long long*>(carve(8 * 16));
     W.F = reinterpret_cast<int32_t*>(carve(4 * n));
     W.FL = reinterpret_cast<int32_t*>(carve(4 * n));
     W.inF = reinterpret_cast<uint8_t*>(carve(n));
+    W.recomp = reinterpret_cast<uint8_t*>(carve(n));       // in this order: clear_level_flags
     W.changed = reinterpret_cast<uint8_t*>(carve(n));
+    S.chcount = reinterpret_cast<unsigned long long*>(carve(16));
     W.next = reinterpret_cast<uint8_t*>(carve(n));
-    W.recomp = reinterpret_cast<uint8_t*>(carve(n));
     S.FX = reinterpret_cast<int32_t*>(carve(4 * n));
     S.ltab = reinterpret_cast<unsigned long long*>(carve(8 * lslots));
     S.dbnext = reinterpret_cast<int64_t*>(carve(8 * L));
@@ -1030,16 +1036,12 @@ cudaError_t alloc_scratch(bisim_ctx* ctx, Scratch& S, cudaStream_t s) {
     W.n = ctx->n;
     W.bcap = ctx->bcap;
     S.blist = reinterpret_cast<int32_t*>(carve(4 * n));
-    S.dbegin = reinterpret_cast<int64_t*>(carve(8 * (kNumClasses + 1)));
-    S.ccount = reinterpret_cast<unsigned long long*>(carve(8 * kNumClasses));
-    S.cedges = reinterpret_cast<unsigned long long*>(carve(8 * kNumClasses));
-    S.ccursor = reinterpret_cast<unsigned long long*>(carve(8 * kNumClasses));
+    S.words = reinterpret_cast<LevelWords*>(carve(sizeof(LevelWords)));
     S.hubs = reinterpret_cast<HubInfo*>(carve(sizeof(HubInfo) * std::max<size_t>(n, kHubPrefetch)));
-    S.n_hubs = reinterpret_cast<unsigned*>(carve(16));
+    W.counters = S.words->counters;
     S.clist = reinterpret_cast<int32_t*>(carve(4 * n));
-    S.chcount = reinterpret_cast<unsigned long long*>(carve(16));
     RowTask* tasks = reinterpret_cast<RowTask*>(carve(3 * sizeof(RowTask) * n));
-    S.tiers = TierLists{{tasks, tasks + n, tasks + 2 * n}, reinterpret_cast<unsigned*>(carve(16))};
+    S.tiers = TierLists{{tasks, tasks + n, tasks + 2 * n}, S.words->tiers};
     cudaMemsetAsync(W.err, 0, 32, s);
     cudaMemsetAsync(S.dbnext, 0, 8 * L, s);
     cudaMemsetAsync(S.dacc, 0, 32 * L, s);
@@ -1062,23 +1064,28 @@ void free_scratch(Scratch* S, cudaStream_t s) {
     delete S;
 }
 
+// The level's words start at zero (before anything of the level is launched).
+void clear_level_words(Scratch& S, cudaStream_t s) { cudaMemsetAsync(S.words, 0, offsetof(LevelWords, begin), s); }
+
+// After the frontier has been made from them: the changed flags and their count, the
+// next level's in-neighbour flags and, above level 0, the recompute flags (this
+// level's assign sets the next level's).
+void clear_level_flags(Scratch& S, int j, cudaStream_t s) {
+    uint8_t* from = j > 0 ? S.W.recomp : S.W.changed;
+    cudaMemsetAsync(from, 0, static_cast<size_t>(S.W.next - from) + S.W.n, s);
+}
+
 // Degree buckets of the live frontier, launched before the level's read-back.
 void launch_buckets(bisim_ctx* ctx, Scratch& S, cudaStream_t s) {
     const unsigned long long* dfl = &S.W.counters[7];
-    cudaMemsetAsync(S.ccount, 0, 8 * kNumClasses, s);
-    cudaMemsetAsync(S.cedges, 0, 8 * kNumClasses, s);
-    cudaMemsetAsync(S.n_hubs, 0, 4, s);
+    LevelWords& D = *S.words;
     BISIM_SITE(site, "inc_buckets");
     Launch L(site, s, 0, 0, 0.0);
     const int sm = ctx->inc_small_max, mm = ctx->opt.mid_max_degree;
-    k_class_count<<<kDevGrid, 256, 0, s>>>(S.W.FL, dfl, ctx->xlen, sm, mm, S.ccount, S.cedges);
-    k_class_scan<<<1, 32, 0, s>>>(S.ccount, S.dbegin, S.ccursor);
-    k_class_scatter<<<kDevGrid, 256, 0, s>>>(S.W.FL, dfl, ctx->xro, ctx->xlen, sm, mm, S.ccursor, S.blist, S.hubs,
-                                            S.n_hubs);
-    cudaMemcpyAsync(S.h->begin, S.dbegin, sizeof(S.h->begin), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(S.h->edges, S.cedges, sizeof(S.h->edges), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(&S.h->n_hubs, S.n_hubs, 4, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(S.h->hubs, S.hubs, sizeof(S.h->hubs), cudaMemcpyDeviceToHost, s);
+    k_class_count<<<kDevGrid, 256, 0, s>>>(S.W.FL, dfl, ctx->xlen, sm, mm, D.count, D.edges);
+    k_class_scan<<<1, 32, 0, s>>>(D.count, D.begin, D.cursor);
+    k_class_scatter<<<kDevGrid, 256, 0, s>>>(S.W.FL, dfl, ctx->xro, ctx->xlen, sm, mm, D.cursor, S.blist, S.hubs,
+                                            &D.n_hubs);
 }
 
 // After the read-back: the Buckets view, and the hub chunks laid out on the
@@ -1092,9 +1099,9 @@ bisim_status finish_buckets(bisim_ctx* ctx, Scratch& S, ListBuckets& out, cudaSt
     Buckets& B = out.B;
     cudaError_t e;
     B.class_list = S.blist;
-    for (int c = 0; c <= kNumClasses; ++c) B.begin[c] = S.h->begin[c];
-    for (int c = 0; c < kNumClasses; ++c) B.edges[c] = static_cast<int64_t>(S.h->edges[c]);
-    B.n_hub = S.h->n_hubs;
+    for (int c = 0; c <= kNumClasses; ++c) B.begin[c] = S.h->w.begin[c];
+    for (int c = 0; c < kNumClasses; ++c) B.edges[c] = static_cast<int64_t>(S.h->w.edges[c]);
+    B.n_hub = S.h->w.n_hubs;
     if (B.n_hub == 0) return BISIM_OK;
     std::vector<HubInfo> hubs(S.h->hubs, S.h->hubs + std::min<int64_t>(B.n_hub, kHubPrefetch));
     if (B.n_hub > kHubPrefetch) {
@@ -1185,7 +1192,6 @@ void launch_frontier(bisim_ctx* ctx, Scratch& S, int j, const uint8_t* a, const 
                      const uint8_t* d, cudaStream_t s) {
     Work& W = S.W;
     const int32_t n = ctx->n;
-    cudaMemsetAsync(&W.counters[6], 0, 24, s);
     if (n > 0)
         k_frontier<<<grid_for(cdiv(n, 16), 256), 256, 0, s>>>(a, b, c, d, ctx->alive, n, j > 0 ? ctx->lid[j - 1] : nullptr,
                                                     j > 0 ? ctx->bcnt[j - 1] : nullptr, ctx->lstale[j], W.F, W.FL,
@@ -1212,7 +1218,6 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
     BISIM_SITE(site_assign, "inc_assign");
     BISIM_SITE(site_retire, "inc_retire");
     // 1. frontier vertices leave their old blocks (sizes read on the device)
-    cudaMemsetAsync(W.counters, 0, 8 * 6, s);
     {
         Launch Lk(site_remove, s, 0, 0, 0.0);
         k_remove<<<kDevGrid, 256, 0, s>>>(W.F, L, W);
@@ -1220,12 +1225,14 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
         k_rescan<<<kDevGrid, 256, 0, s>>>(n, ctx->alive, L, W);
     }
     if (j > 0) launch_buckets(ctx, S, s);
-    cudaMemcpyAsync(S.h->counters, W.counters, sizeof(S.h->counters), cudaMemcpyDeviceToHost, s);
+    const size_t back = sizeof(LevelWords) + (j > 0 ? sizeof(S.h->hubs) : 0);
+    static_assert(offsetof(HostStage, hubs) == sizeof(LevelWords), "one copy brings both");
+    cudaMemcpyAsync(&S.h->w, S.words, back, cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "frontier sizes");
-    const int64_t ntouched = static_cast<int64_t>(S.h->counters[0]);
-    const int64_t f = static_cast<int64_t>(S.h->counters[6]);
-    const int64_t fl = static_cast<int64_t>(S.h->counters[7]);
-    const int64_t fx = static_cast<int64_t>(S.h->counters[8]);
+    const int64_t ntouched = static_cast<int64_t>(S.h->w.counters[0]);
+    const int64_t f = static_cast<int64_t>(S.h->w.counters[6]);
+    const int64_t fl = static_cast<int64_t>(S.h->w.counters[7]);
+    const int64_t fx = static_cast<int64_t>(S.h->w.counters[8]);
     *frontier = fl + fx;
     unsigned long long* acc = S.dacc + 4 * j;
     if (fx > 0) {
@@ -1267,10 +1274,9 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
             k_group_stats<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, W);
         }
         Launch Lk(site_probe, s, fl, 0, 32.0 * fl);
-        cudaMemsetAsync(&W.counters[2], 0, 8, s);
         k_probe<<<grid_for(fl, 256), 256, 0, s>>>(W.FL, fl, L, W, j, ctx->vlabel, hmask);
     };
-    if (fl > 0) group_and_probe();
+    if (fl > 0) group_and_probe();                   // the candidates' count is still zero
     for (int iter = 0; fl > 0 && j > 0; ++iter) {
         if (iter > 1 << 16) {
             if (LB.hubmem) cudaFreeAsync(LB.hubmem, s);
@@ -1312,6 +1318,7 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
                 return st;
             }
             if (changed) {
+                cudaMemsetAsync(&W.counters[2], 0, 8, s);
                 group_and_probe();
                 continue;
             }
@@ -1533,6 +1540,7 @@ bisim_status inc_build(bisim_ctx* ctx, cudaStream_t s) {
     int64_t fl = 0;
     st = BISIM_OK;
     for (int j = 0; st == BISIM_OK && j <= K; ++j) {
+        clear_level_words(S, s);
         launch_frontier(ctx, S, j, nullptr, nullptr, nullptr, nullptr, s);
         cudaMemsetAsync(S.chcount, 0, 8, s);          // k_assign lists changed vertices (at most n)
         st = level_pass(ctx, j, S, &fl, s);
@@ -1570,11 +1578,10 @@ bisim_status inc_update(bisim_ctx* ctx, const uint8_t* vchanged, const uint8_t* 
     Work& W = S.W;
     int64_t total = 0;
     for (int j = 0; st == BISIM_OK && j <= K; ++j) {
+        clear_level_words(S, s);
         if (j > 0) {
             // F_j: block changed one level down, out-edges changed, or an out-edge into a
             // changed vertex (its source is in the changed vertex's in-row)
-            cudaMemsetAsync(W.next, 0, n, s);
-            cudaMemsetAsync(S.tiers.cnt, 0, 16, s);
             if (n > 0) {
                 BISIM_SITE(site, "inc_in_neighbours");
                 Launch L(site, s, n, 0, 1.0 * n);
@@ -1582,12 +1589,10 @@ bisim_status inc_update(bisim_ctx* ctx, const uint8_t* vchanged, const uint8_t* 
                 run_tiers(S.tiers, MarkSources{ctx->ype, W.next}, s);
             }
             launch_frontier(ctx, S, j, W.next, W.changed, rowchg, W.recomp, s);
-            cudaMemsetAsync(W.recomp, 0, n, s);       // this level's assign flags the next level's
         } else {
             launch_frontier(ctx, S, j, vchanged, nullptr, nullptr, nullptr, s);
         }
-        cudaMemsetAsync(W.changed, 0, n, s);
-        cudaMemsetAsync(S.chcount, 0, 8, s);          // the level lists its changed vertices
+        clear_level_flags(S, j, s);                   // the level lists its changed vertices
         int64_t fl = 0;
         st = level_pass(ctx, j, S, &fl, s);
         total += fl;

@@ -879,9 +879,9 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
         B.skh = kh1;
         B.skp = kp1;
     }
-    cudaMemsetAsync(killed, 0, n + 1, s);
-    cudaMemsetAsync(B.counters, 0, 8 * 4, s);
-    for (int q = 3; q < 8; ++q) cudaMemsetAsync(tab_arrays[q], 0, 4 * static_cast<size_t>(tsize), s);
+    // the table's last five arrays and the counters behind them (`killed`, like the
+    // caller's other flags, is zero already)
+    cudaMemsetAsync(tab_arrays[3], 0, static_cast<size_t>(reinterpret_cast<char*>(B.counters + 4) - reinterpret_cast<char*>(tab_arrays[3])), s);
     if (alive0 && n > 0) cudaMemcpyAsync(alive0, ctx->alive, n, cudaMemcpyDeviceToDevice, s);
     if (nv > 0) {
         Launch L(site_ops, s, 0, 0, 16.0 * nv);
@@ -1074,8 +1074,7 @@ bisim_status apply_ops_to_store(bisim_ctx* ctx, const bisim_op* d_ops, int64_t n
     // source row a key names is scanned once per pass
     if (ne > 0) {
         Launch L(site, s, 0, 0, 0.0);
-        cudaMemsetAsync(cnts, 0, 32, s);
-        cudaMemsetAsync(n_touched, 0, 8, s);
+        cudaMemsetAsync(cnts, 0, 40, s);                   // both lists and n_touched behind them
         k_mark_kinds<<<grid_for(ne, 256), 256, 0, s>>>(d_ops, B.skp, ne, T);
         k_key_rows<<<grid_for(ne, 256), 256, 0, s>>>(B.keyslot, ne, T, ctx->xmark, ctx->dmark, touched_o, touched_i,
                                                      n_touched);
