@@ -1,9 +1,10 @@
-// One refinement round of forward k-bisimulation (Algorithm 4, Section 3.3.1),
-// made exact.
+// P_0, and the signature round of the incremental levels: one refinement round of
+// forward k-bisimulation (Algorithm 4, Section 3.3.1) over listed vertices, made
+// exact.
 //
 // Per round i -> i+1 every live vertex v
 //   1. gathers the pairs (l, P_i[w]) of its out-edges (SignalMessages: a pull over
-//      the out-CSR instead of messages pushed along reversed edges),
+//      its row instead of messages pushed along reversed edges),
 //   2. removes duplicates (MergeMessages) -- by sorting for small and mid
 //      degrees, by a per-hub hash set for hubs,
 //   3. hashes (P_i[v], set) order-independently (Hash, with the own block in the
@@ -41,34 +42,25 @@ __device__ __forceinline__ unsigned lanemask_lt() { return (1u << lane_id()) - 1
 
 // ----------------------------------------------------------------------------- views
 
-// Rows come from the CSR (row v = [rp[v], rp[v + 1]) of col / elab) or from the
-// incremental path's row store (row v = rl[v] packed entries from rp[v], some
-// deleted, some pointing at dead vertices: those do not count).
+// Rows of the incremental path's store: row v is rl[v] packed entries from rp[v],
+// some deleted, some pointing at dead vertices: those do not count.
 struct GraphView {
     const int64_t* rp;
-    const int32_t* rl;                 // store row lengths (null: CSR)
-    const int32_t* col;
-    const int32_t* elab;
-    const unsigned long long* pe;      // store entries (null: CSR)
+    const int32_t* rl;
+    const unsigned long long* pe;
     const int32_t* P;                  // P_i (-1 for a dead vertex)
     unsigned long long* hout;          // nullable: receives each vertex's signature hash
 };
 
-__device__ __forceinline__ int row_len(const GraphView& G, int32_t v) {
-    return G.rl ? G.rl[v] : static_cast<int>(G.rp[v + 1] - G.rp[v]);
-}
+__device__ __forceinline__ int row_len(const GraphView& G, int32_t v) { return G.rl[v]; }
 
 // Pair value of row entry e; false when the entry does not count.
 __device__ __forceinline__ bool entry_value(const GraphView& G, int64_t e, unsigned long long* mv) {
-    if (G.pe) {
-        const unsigned long long x = __ldcs(G.pe + e);
-        if (x == kRowTomb) return false;
-        const int32_t p = __ldg(G.P + static_cast<int32_t>(static_cast<uint32_t>(x)));
-        if (p < 0) return false;
-        *mv = pair_value(static_cast<int32_t>(x >> 32), p);
-        return true;
-    }
-    *mv = pair_value(__ldcs(G.elab + e), __ldg(G.P + __ldcs(G.col + e)));
+    const unsigned long long x = __ldcs(G.pe + e);
+    if (x == kRowTomb) return false;
+    const int32_t p = __ldg(G.P + static_cast<int32_t>(static_cast<uint32_t>(x)));
+    if (p < 0) return false;
+    *mv = pair_value(static_cast<int32_t>(x >> 32), p);
     return true;
 }
 
@@ -705,8 +697,8 @@ bisim_status resolve_settle(bisim_ctx* ctx, Mode M, int32_t* Pout, cudaStream_t 
     return BISIM_OK;
 }
 
-// Algorithmic bytes of the signature kernels: per edge col 4 + label 4 + the
-// gathered P_i[w] 4; per vertex row_ptr 4 + P_i[v] 4 + one 16-byte table slot.
+// Algorithmic bytes of the signature kernels: per entry the word 8 + the gathered
+// P_i[w] 4; per vertex row offset 4 + P_i[v] 4 + one 16-byte table slot.
 constexpr double kSigBytesPerEdge = 12.0;
 constexpr double kSigBytesPerVertex = 24.0;
 
@@ -879,8 +871,7 @@ bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s) {
 namespace {
 
 GraphView graph_view(const bisim_ctx* ctx, const int32_t* Pin, unsigned long long* hout) {
-    return ctx->store_ready ? GraphView{ctx->xro, ctx->xlen, nullptr, nullptr, ctx->xpe, Pin, hout}
-                            : GraphView{ctx->row_ptr, nullptr, ctx->col, ctx->elab, nullptr, Pin, hout};
+    return GraphView{ctx->xro, ctx->xlen, ctx->xpe, Pin, hout};
 }
 
 SigMode sig_mode(const bisim_ctx* ctx, const Buckets& B, const GraphView& G) {
@@ -889,9 +880,8 @@ SigMode sig_mode(const bisim_ctx* ctx, const Buckets& B, const GraphView& G) {
     M.cnt = ctx->cnt;
     M.skey = ctx->skey;
     M.H = HubView{B.hub_list, B.n_hub, B.toff, B.tmask, B.tab, B.acc};
-    // lists of up to small_max entries are sorted (thread-per-vertex classes); the
-    // incremental path sets its own limit per batch
-    M.small_max = ctx->store_ready ? ctx->inc_small_max : ctx->opt.small_max_degree;
+    // lists of up to small_max entries are sorted (thread-per-vertex classes)
+    M.small_max = ctx->inc_small_max;
     M.mid_max = ctx->opt.mid_max_degree;
     return M;
 }
