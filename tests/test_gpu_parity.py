@@ -481,3 +481,22 @@ def test_csr_arrays_at_any_alignment(B, off, m, where):
     bad[m - 1] = n
     with pytest.raises(B.BisimError, match="malformed CSR"):
         B.summarize_init(n, put(rp), shift(bad, off), shift(lab, off), put(vl))
+
+
+@pytest.mark.parametrize("m", [(1 << 20) - 1, 1 << 20, (1 << 20) + 33])
+@pytest.mark.parametrize("order", ["sorted", "shuffled", "last two exchanged"])
+def test_long_lists_are_looked_at_first(B, m, order):
+    # from 2^20 edges on some places of the list are looked at before its check: what
+    # they show, and what only the check can find
+    rng = np.random.default_rng(m)
+    n = 4000
+    src = np.sort(rng.integers(0, n, m)).astype(np.int32)
+    src[-1] = n - 1
+    src[-2] = n - 2
+    if order == "shuffled":
+        src = src[rng.permutation(m)]
+    elif order != "sorted":
+        src[-2:] = src[:-3:-1].copy()
+    g = dict(n=n, src=src, dst=rng.integers(0, n, m).astype(np.int32), elabel=rng.integers(0, 9, m).astype(np.int32),
+             vlabel=rng.integers(0, 3, n).astype(np.int32))
+    check(B, g, [1])
