@@ -4,6 +4,7 @@
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 
@@ -113,6 +114,21 @@ bool device_accessible(const void* p) {
     if (a.type != cudaMemoryTypeDevice) return false;
     int cur = -1;
     return cudaGetDevice(&cur) == cudaSuccess && a.device == cur;
+}
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> allowed;
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& have = allowed[{device, kernel}];
+    if (have >= bytes) return cudaSuccess;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)))) return e;
+    have = bytes;
+    return cudaSuccess;
 }
 
 namespace {

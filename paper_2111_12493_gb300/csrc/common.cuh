@@ -457,6 +457,9 @@ CtxPiece ctx_piece(T** p, size_t count) {
 }
 // Whether the kernels of the current device may use `p` in place (api.cu).
 bool device_accessible(const void* p);
+// Lets `kernel` be launched with `bytes` of dynamic shared memory on the current
+// device (more than 48 KB have to be allowed, on every device by itself).
+cudaError_t allow_smem(const void* kernel, size_t bytes);
 // 256-byte pinned host blocks from process-lifetime slabs (nullptr if none can be had).
 // Forks from `s`. A branch without a stream (none could be had) stands for `s` itself.
 // After the join (which has to come, on the same stream) the branch is gone.
@@ -472,11 +475,12 @@ size_t scan_temp_words(int64_t n);
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 
 // Stable LSD radix sort of (u32 key, u64 value) pairs on the low `bits` key bits.
-// Buffers are ping-ponged; returns 0 if the result ended in (k0, v0), 1 if in (k1, v1).
+// Buffers are ping-ponged; *which is 0 if the result ended in (k0, v0), 1 if in (k1, v1).
+// On an error (a launch that was refused) neither holds it.
 size_t radix_temp_words(int64_t m);
 // `site_name` names the launch-timing sites of the passes ("<name>_hist", "<name>_scatter").
-int radix_sort_pairs(uint32_t* k0, uint64_t* v0, uint32_t* k1, uint64_t* v1, int64_t m, int bits,
-                     int64_t* tmp, cudaStream_t s, const char* site_name = "radix");
+cudaError_t radix_sort_pairs(uint32_t* k0, uint64_t* v0, uint32_t* k1, uint64_t* v1, int64_t m, int bits,
+                             int64_t* tmp, cudaStream_t s, const char* site_name, int* which);
 
 // ----------------------------------------------------------------------------- graph build (graph.cu)
 

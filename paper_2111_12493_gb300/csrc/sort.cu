@@ -5,7 +5,6 @@
 // stable scatter in which every warp ranks its own items with match masks and
 // the tile is put in digit order in shared memory before it is written.
 #include <algorithm>
-#include <mutex>
 #include <string>
 
 #include "common.cuh"
@@ -188,13 +187,10 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(
 }
 
 template <int ITEMS>
-void radix_pass(const uint32_t* ki, const uint64_t* vi, uint32_t* ko, uint64_t* vo, int64_t m, int shift, int64_t ntiles,
+cudaError_t radix_pass(const uint32_t* ki, const uint64_t* vi, uint32_t* ko, uint64_t* vo, int64_t m, int shift, int64_t ntiles,
                 int64_t* counts, int64_t* offs, int64_t* stmp, int site_h, int site_s, cudaStream_t s) {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_radix_scatter<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(sizeof(RadixShared<ITEMS>)));
-    });
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_radix_scatter<ITEMS>), sizeof(RadixShared<ITEMS>));
+    if (e) return e;
     {
         Launch L(site_h, s, 0, m, 4.0 * m);
         k_radix_hist<ITEMS><<<static_cast<unsigned>(ntiles), kRadixThreads, 0, s>>>(ki, m, shift, counts, ntiles);
@@ -203,6 +199,7 @@ void radix_pass(const uint32_t* ki, const uint64_t* vi, uint32_t* ko, uint64_t* 
     Launch L(site_s, s, 0, m, 24.0 * m);
     k_radix_scatter<ITEMS><<<static_cast<unsigned>(ntiles), kRadixThreads, sizeof(RadixShared<ITEMS>), s>>>(
         ki, vi, ko, vo, m, shift, offs, ntiles);
+    return cudaGetLastError();
 }
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -340,38 +337,41 @@ size_t radix_temp_words(int64_t m) {
     return static_cast<size_t>(2 * nc) + scan_temp_words(nc);
 }
 
-int radix_sort_pairs(uint32_t* k0, uint64_t* v0, uint32_t* k1, uint64_t* v1, int64_t m, int bits,
-                     int64_t* tmp, cudaStream_t s, const char* site_name) {
-    if (m <= 0 || bits <= 0) return 0;
+cudaError_t radix_sort_pairs(uint32_t* k0, uint64_t* v0, uint32_t* k1, uint64_t* v1, int64_t m, int bits,
+                             int64_t* tmp, cudaStream_t s, const char* site_name, int* which) {
+    *which = 0;
+    if (m <= 0 || bits <= 0) return cudaSuccess;
     if (m <= kSmallSortMax) {
         BISIM_SITE(site_small, "small_sort");
         Launch L(site_small, s, 0, m, 24.0 * m);
         const int mi = static_cast<int>(m);
         if (m <= 2 * kSmallSortThreads) k_small_sort<2><<<1, kSmallSortThreads, 0, s>>>(k0, v0, k1, v1, mi, bits);
         else k_small_sort<8><<<1, kSmallSortThreads, 0, s>>>(k0, v0, k1, v1, mi, bits);
-        return 1;
+        *which = 1;
+        return cudaGetLastError();
     }
     const int64_t ntiles = radix_tiles(m);
     const int64_t nc = ntiles * kRadixBins;
     int64_t* counts = tmp;
     int64_t* offs = tmp + nc;
     int64_t* stmp = tmp + 2 * nc;
-    int which = 0;
     for (int shift = 0; shift < bits; shift += 8) {
-        const uint32_t* ki = which ? k1 : k0;
-        const uint64_t* vi = which ? v1 : v0;
-        uint32_t* ko = which ? k0 : k1;
-        uint64_t* vo = which ? v0 : v1;
+        const uint32_t* ki = *which ? k1 : k0;
+        const uint64_t* vi = *which ? v1 : v0;
+        uint32_t* ko = *which ? k0 : k1;
+        uint64_t* vo = *which ? v0 : v1;
         // the site's passes are timed apart from other callers' (the CSR build's
         // full-size passes are the ones the benchmark's roofline names)
-        const std::string name = site_name ? site_name : "radix";
+        const std::string name = site_name;
         const int site_h = prof_site((name + "_hist").c_str());
         const int site_s = prof_site((name + "_scatter").c_str());
-        if (m <= kRadixShort) radix_pass<kRadixShortItems>(ki, vi, ko, vo, m, shift, ntiles, counts, offs, stmp, site_h, site_s, s);
-        else radix_pass<kRadixItems>(ki, vi, ko, vo, m, shift, ntiles, counts, offs, stmp, site_h, site_s, s);
-        which ^= 1;
+        const cudaError_t e =
+            m <= kRadixShort ? radix_pass<kRadixShortItems>(ki, vi, ko, vo, m, shift, ntiles, counts, offs, stmp, site_h, site_s, s)
+                             : radix_pass<kRadixItems>(ki, vi, ko, vo, m, shift, ntiles, counts, offs, stmp, site_h, site_s, s);
+        if (e) return e;
+        *which ^= 1;
     }
-    return which;
+    return cudaSuccess;
 }
 
 }  // namespace bisim

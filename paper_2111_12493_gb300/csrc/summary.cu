@@ -618,22 +618,28 @@ bisim_status summary_by_radix(bisim_ctx* ctx, cudaStream_t s, char** out_base, c
         k_summary_keys<<<grid_for(cdiv(m, kKeyTile) * 256, 256), 256, 0, s>>>(ctx->row_ptr, n, ctx->col, ctx->elab, m,
                                                                                 P, ctx->opt.direction, k0, v0);
     }
+    const auto fail = [&](cudaError_t err, const char* what) {
+        cudaFreeAsync(base, s);
+        return cuda_error(ctx, err, what);
+    };
     // pass A: by target block (stable), the result in (k0, v0) or (k1, v1)
-    int w = radix_sort_pairs(k0, v0, k1, v1, m, bits_for(n), tmp, s, "summary_radix");
+    int w = 0;
+    if ((e = radix_sort_pairs(k0, v0, k1, v1, m, bits_for(n), tmp, s, "summary_radix", &w))) return fail(e, "summary sort");
     uint32_t* ka = w ? k1 : k0;
     uint64_t* va = w ? v1 : v0;
     uint32_t* kb = w ? k0 : k1;
     uint64_t* vb = w ? v0 : v1;
     k_summary_to_label<<<grid_for(m, 256), 256, 0, s>>>(ka, va, m, kb, vb);
     // pass B: by label
-    w = radix_sort_pairs(kb, vb, ka, va, m, 32, tmp, s, "summary_radix");
+    if ((e = radix_sort_pairs(kb, vb, ka, va, m, 32, tmp, s, "summary_radix", &w))) return fail(e, "summary sort");
     uint32_t* kc = w ? ka : kb;
     uint64_t* vc = w ? va : vb;
     uint32_t* kd = w ? kb : ka;
     uint64_t* vd = w ? vb : va;
     k_summary_to_source<<<grid_for(m, 256), 256, 0, s>>>(kc, vc, m, kd, vd);
     // pass C: by source block (dead-endpoint edges carry n and sort last)
-    w = radix_sort_pairs(kd, vd, kc, vc, m, bits_for(static_cast<int64_t>(n) + 1), tmp, s, "summary_radix");
+    if ((e = radix_sort_pairs(kd, vd, kc, vc, m, bits_for(static_cast<int64_t>(n) + 1), tmp, s, "summary_radix", &w)))
+        return fail(e, "summary sort");
     const uint32_t* kf = w ? kc : kd;
     const uint64_t* vf = w ? vc : vd;
     {
@@ -643,10 +649,7 @@ bisim_status summary_by_radix(bisim_ctx* ctx, cudaStream_t s, char** out_base, c
         k_summary_emit<<<grid_for(m, 256), 256, 0, s>>>(kf, vf, m, n, at, os, ol, ot);
     }
     cudaMemcpyAsync(&count, at + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    if ((e = cudaStreamSynchronize(s))) {
-        cudaFreeAsync(base, s);
-        return cuda_error(ctx, e, "summary edges");
-    }
+    if ((e = cudaStreamSynchronize(s))) return fail(e, "summary edges");
     if (cur - base != static_cast<ptrdiff_t>(bytes) || count < 0 || count > m) {
         cudaFreeAsync(base, s);
         return set_error(ctx, BISIM_ECUDA, "summary edges: inconsistent scratch layout or count");
@@ -757,32 +760,38 @@ bisim_status summary_by_segment(bisim_ctx* ctx, cudaStream_t s, char** out_base,
         exclusive_scan_i64(len, first, big + 1, btmp, s);
         k_big_gather<<<grid_for(cdiv(bm, kKeyTile) * 256, 256), 256, 0, s>>>(off, L, static_cast<int32_t>(big), first, bm, seg,
                                                                            one ? tbits : 0, lbits, lo, hi, ka, va);
-        // the result of each sort in (ka, va), the other pair free
-        auto sort = [&](int bits) {
-            if (radix_sort_pairs(ka, va, kb, vb, bm, bits, btmp, s, "summary_radix")) {
-                std::swap(ka, kb);
-                std::swap(va, vb);
-            }
-        };
+        // the result of each sort in (ka, va), the other pair free; after a sort that
+        // failed nothing is looked up by its keys any more
         auto turn = [&] {
             std::swap(ka, kb);
             std::swap(va, vb);
         };
+        auto sort = [&](int bits) {
+            int w = 0;
+            e = radix_sort_pairs(ka, va, kb, vb, bm, bits, btmp, s, "summary_radix", &w);
+            if (w) turn();
+            return e == cudaSuccess;
+        };
         if (one) {
-            sort(std::min(32, tbits + lbits + sbits));
-            if (tbits + lbits + sbits > 32) {
-                k_big_high<<<grid_for(bm, 256), 256, 0, s>>>(va, bm, ka);
-                sort(tbits + lbits + sbits - 32);
+            if (sort(std::min(32, tbits + lbits + sbits))) {
+                if (tbits + lbits + sbits > 32) {
+                    k_big_high<<<grid_for(bm, 256), 256, 0, s>>>(va, bm, ka);
+                    sort(tbits + lbits + sbits - 32);
+                }
+                k_big_split<<<grid_for(bm, 256), 256, 0, s>>>(ka, va, bm, tbits, lbits, lo);
             }
-            k_big_split<<<grid_for(bm, 256), 256, 0, s>>>(ka, va, bm, tbits, lbits, lo);
-        } else {
-            sort(tbits);
+        } else if (sort(tbits)) {
             k_big_to_label<<<grid_for(bm, 256), 256, 0, s>>>(ka, va, bm, lo, hi, kb, vb);
             turn();
-            sort(lbits);
-            k_big_to_segment<<<grid_for(bm, 256), 256, 0, s>>>(ka, va, bm, lo, kb, vb);
-            turn();
-            sort(sbits);
+            if (sort(lbits)) {
+                k_big_to_segment<<<grid_for(bm, 256), 256, 0, s>>>(ka, va, bm, lo, kb, vb);
+                turn();
+                sort(sbits);
+            }
+        }
+        if (e) {
+            cudaFreeAsync(more, s);
+            return fail(e, "summary sort");
         }
         int64_t* rank = reinterpret_cast<int64_t*>(vb);
         k_big_heads<<<grid_for(bm + 1, 256), 256, 0, s>>>(ka, va, bm, rank);

@@ -846,7 +846,12 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     }
     int vbits = 1;                                          // keys 0 .. n
     while (vbits < 32 && (int64_t{1} << vbits) <= n) ++vbits;
-    const int which = radix_sort_pairs(vk0, vv0, vk1, vv1, nops, vbits, B.tmp, s, "update_radix");
+    int which = 0;
+    if ((e = radix_sort_pairs(vk0, vv0, vk1, vv1, nops, vbits, B.tmp, s, "update_radix", &which))) {
+        cudaFreeAsync(B.base, s);
+        B.base = nullptr;
+        return cuda_error(ctx, e, "sort vertex operations");
+    }
     const uint32_t* vkey = which ? vk1 : vk0;
     const uint64_t* vpos = which ? vv1 : vv0;
     // 2. EDGE_ADD liveness and edge-key hashes (before the host looks: one read-back
@@ -870,15 +875,16 @@ bisim_status batch_begin(bisim_ctx* ctx, const bisim_op* d_ops, int64_t nops, si
     B.V = VertexOps{vkey, vpos, B.nv, d_ops, ctx->alive};
     const int64_t nv = B.nv, ne = B.ne;
 
-    // ---- from here on the batch is valid and the graph changes ----
     // stable sort of the edge operations by key hash: operations of one key stay
     // in batch order
-    B.skh = kh0;
-    B.skp = kp0;
-    if (ne > 0 && radix_sort_pairs(kh0, kp0, kh1, kp1, ne, hbits, B.tmp, s, "update_radix")) {
-        B.skh = kh1;
-        B.skp = kp1;
+    if ((e = radix_sort_pairs(kh0, kp0, kh1, kp1, ne, hbits, B.tmp, s, "update_radix", &which))) {
+        cudaFreeAsync(B.base, s);
+        B.base = nullptr;
+        return cuda_error(ctx, e, "sort edge operations");
     }
+    B.skh = which ? kh1 : kh0;
+    B.skp = which ? kp1 : kp0;
+    // ---- from here on the batch is valid and the graph changes ----
     // the table's last five arrays and the counters behind them (`killed`, like the
     // caller's other flags, is zero already)
     cudaMemsetAsync(tab_arrays[3], 0, static_cast<size_t>(reinterpret_cast<char*>(B.counters + 4) - reinterpret_cast<char*>(tab_arrays[3])), s);
