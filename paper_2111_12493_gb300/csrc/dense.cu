@@ -1542,11 +1542,6 @@ HubSets hub_sets(const bisim_ctx* ctx) {
     return HubSets{ctx->dbegin[kDHub], ctx->n_dhub, ctx->htab, ctx->dedge_begin[kDHub], ctx->dacc};
 }
 
-template <class K>
-void allow_smem(K kernel, size_t bytes) {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-}
-
 // Algorithmic bytes: the signature kernels move per edge the packed (label,
 // target) word 8 + the gathered P_i[w] 4, per vertex the list entry 4, the row
 // offset 8, the vertex id 4, P_i[v] 4 and the 16-byte signature record written
@@ -1600,16 +1595,18 @@ void launch_mid(bisim_ctx* ctx, int cls, const DenseView& D, cudaStream_t s, int
     k_dense_mid_sig<N, T><<<grid, T, smem, s>>>(cls, D, 4 + (cls - kDMid0));
 }
 
-// Kernel attributes (shared memory above 48 KB), set once before any launch or capture.
+// Kernel attributes (shared memory above 48 KB, on the current device) and the
+// persistent grids, looked up before any launch or capture.
 void set_attributes() {
+    const auto allow = [](auto kernel, size_t bytes) { allow_smem(reinterpret_cast<const void*>(kernel), bytes); };
+    allow(k_dense_mid_sig<512, 256>, sizeof(unsigned long long) * 2 * 512);
+    allow(k_dense_mid_sig<1024, 256>, sizeof(unsigned long long) * 2 * 1024);
+    allow(k_dense_mid_sig<2048, 512>, sizeof(unsigned long long) * 2 * 2048);
+    allow(k_dense_mid_sig<4096, 512>, sizeof(unsigned long long) * 2 * 4096);
+    allow(k_dense_mid_sig<8192, 512>, sizeof(unsigned long long) * 2 * 8192);
+    allow(k_dense_compare_cta, kCompareSmem);
     static std::once_flag once;
     std::call_once(once, []() {
-        allow_smem(k_dense_mid_sig<512, 256>, sizeof(unsigned long long) * 2 * 512);
-        allow_smem(k_dense_mid_sig<1024, 256>, sizeof(unsigned long long) * 2 * 1024);
-        allow_smem(k_dense_mid_sig<2048, 512>, sizeof(unsigned long long) * 2 * 2048);
-        allow_smem(k_dense_mid_sig<4096, 512>, sizeof(unsigned long long) * 2 * 4096);
-        allow_smem(k_dense_mid_sig<8192, 512>, sizeof(unsigned long long) * 2 * 8192);
-        allow_smem(k_dense_compare_cta, kCompareSmem);
         persistent_grid(k_hub_clear, kThreads, 0, 1);
         persistent_grid(k_hub_insert, kThreads, kHubInsertSmem, 1);
         persistent_grid(k_dense_thread_sig<8>, kThreads, 0, 1);

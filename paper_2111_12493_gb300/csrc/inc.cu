@@ -1284,12 +1284,7 @@ bisim_status level_pass(bisim_ctx* ctx, int j, Scratch& S, int64_t* frontier, cu
         }
         Level Lp = level_view(ctx, j - 1);
         const Buckets& B = LB.B;
-        static bool attr = false;
-        if (!attr) {
-            cudaFuncSetAttribute(k_compare<kCmpLargeSlots>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(sizeof(unsigned long long) * kCmpLargeSlots));
-            attr = true;
-        }
+        allow_smem(reinterpret_cast<const void*>(k_compare<kCmpLargeSlots>), sizeof(unsigned long long) * kCmpLargeSlots);
         {
             Launch Lk(site_compare, s, 0, 0, 0.0);
             k_compare<kCmpSmallSlots><<<kCmpGrid, kCmpThreads, sizeof(unsigned long long) * kCmpSmallSlots, s>>>(

@@ -625,12 +625,7 @@ namespace {
 template <class Mode>
 void launch_deferred(bisim_ctx* ctx, const Mode& M, int32_t* Pout, int32_t* next, DevState* ds, cudaStream_t s) {
     if constexpr (Mode::kDefers) {
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaFuncSetAttribute(k_verify_deferred, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kDeferSmem));
-            attr_set = true;
-        }
+        allow_smem(reinterpret_cast<const void*>(k_verify_deferred), kDeferSmem);
         BISIM_SITE(site, "verify_deferred");
         Launch L(site, s, 0, 0, 0.0);
         k_verify_deferred<<<kDeferGrid, kDeferThreads, kDeferSmem, s>>>(ctx->dlist, M, ctx->slot, ctx->table, Pout,
@@ -725,11 +720,7 @@ void launch_cta_mid(bisim_ctx* ctx, const int32_t* list, int64_t count, int64_t 
                     cudaStream_t s) {
     constexpr int T = N <= 1024 ? 256 : 512;
     const size_t smem = sizeof(unsigned long long) * 2 * N;
-    static bool attr_set = false;   // per process; the attribute belongs to the function
-    if (!attr_set && smem > 48 * 1024) {
-        cudaFuncSetAttribute(k_sig_mid<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        attr_set = true;
-    }
+    allow_smem(reinterpret_cast<const void*>(k_sig_mid<N, T>), smem);
     static const int site = prof_site(N == 64 ? "sig_mid_64" : N == 128 ? "sig_mid_128" : N == 256 ? "sig_mid_256"
                                       : N == 512 ? "sig_mid_512" : N == 1024 ? "sig_mid_1024" : N == 2048 ? "sig_mid_2048"
                                       : N == 4096 ? "sig_mid_4096" : "sig_mid_8192");

@@ -596,12 +596,12 @@ __global__ void k_seg_rows(const int32_t* __restrict__ vpos, const int64_t* __re
 }
 
 int seg_grid(int32_t G, bool beside_union) {
+    allow_smem(reinterpret_cast<const void*>(k_segments), kSegSmem);
     static int per_sm = -1, sms = 0;
     if (per_sm < 0) {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_segments, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSegSmem));
         int b = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_segments, kSegThreads, kSegSmem) != cudaSuccess) b = 1;
         per_sm = std::max(b, 1);

@@ -43,11 +43,39 @@ void sort_on_two_devices() {
     expect(sort() == cudaErrorInvalidValue, "shared memory that could not be had went unnoticed");
 }
 
+// So do the kernels of the wide rows, in the rounds and in the incremental levels.
+void wide_rows_on_two_devices() {
+    bisim_ctx c;
+    c.n = 1000;
+    c.m = 100000;
+    c.opt.hash_bits = 64;
+    c.opt.mid_max_degree = kMidMaxN;
+    c.dense_ready = true;
+    c.nslots = 2048;
+    for (int q = 0; q <= kDClasses; ++q) c.dbegin[q] = 10 * q;
+    Buckets B{};
+    for (int q = 0; q <= kNumClasses; ++q) B.begin[q] = 10 * q;
+    void* state = nullptr;
+    cudaMallocAsync(&state, 4096, nullptr);
+    c.dstate = static_cast<DevState*>(state);
+    c.hstate = static_cast<DevState*>(pinned_take());
+    cudaMallocAsync(&state, sizeof(Slot) * c.nslots, nullptr);
+    c.table = static_cast<Slot*>(state);
+    for (int device : {0, 1}) {
+        fake::runtime().device = c.device = device;
+        int64_t blocks = 0;
+        expect(dense_round(&c, nullptr, &blocks) == BISIM_OK, "a round failed");
+        expect(signature_launch(&c, B, nullptr, nullptr, nullptr, 10, nullptr, nullptr) == BISIM_OK, "signatures failed");
+        expect(fake::runtime().refused == 0, "a kernel asked for shared memory that was not allowed on its device");
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const std::map<std::string, std::function<void()>> scenarios = {
         {"sort_on_two_devices", sort_on_two_devices},
+        {"wide_rows_on_two_devices", wide_rows_on_two_devices},
     };
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) {
