@@ -1036,11 +1036,11 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
 
 // Cooperative launches of this process follow one another on a device, whatever
 // their streams: each waits for the event recorded after the one before, so that
-// two of them never share the SMs half resident.
+// two of them never share the SMs half resident. That includes launches on equal
+// handles: the per-thread default stream is another stream in every thread.
 struct CoopLane {
     std::mutex mu;
     cudaEvent_t done[64] = {};
-    cudaStream_t last[64] = {};
 };
 
 CoopLane& coop_lane() {
@@ -1056,11 +1056,10 @@ cudaError_t launch_in_lane(int device, const void* kernel, unsigned grid, unsign
     cudaError_t e;
     if (lane.done[device] == nullptr) {
         if ((e = cudaEventCreateWithFlags(&lane.done[device], cudaEventDisableTiming))) return e;
-    } else if (lane.last[device] != s) {
-        if ((e = cudaStreamWaitEvent(s, lane.done[device], 0))) return e;
+    } else if ((e = cudaStreamWaitEvent(s, lane.done[device], 0))) {
+        return e;
     }
     if ((e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(threads), args, smem, s))) return e;
-    lane.last[device] = s;
     return cudaEventRecord(lane.done[device], s);
 }
 

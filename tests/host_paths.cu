@@ -70,12 +70,48 @@ void wide_rows_on_two_devices() {
     }
 }
 
+// A context of `n` vertices with short rows, laid out as far as the round loop's host code looks.
+bisim_ctx& looping_context(int32_t n) {
+    bisim_ctx& c = *new bisim_ctx();
+    c.n = n;
+    c.m = n;
+    c.opt.hash_bits = 64;
+    c.dense_ready = true;
+    c.nslots = 2048;
+    for (int q = 1; q <= kDClasses; ++q) c.dbegin[q] = n;
+    return c;
+}
+
+// Two loops on the per-thread default stream may come from two threads, for which
+// the one handle names two streams: the second waits for the first all the same.
+void loops_on_one_handle() {
+    bisim_ctx* c[2] = {&looping_context(1 << 20), &looping_context(1 << 20)};
+    const auto& calls = fake::runtime().calls;
+    cudaEvent_t last = nullptr;
+    for (int i = 0; i < 2; ++i) {
+        fake::runtime().on_launch = [&](const void*, bool) {
+            static_cast<LoopState*>(c[i]->hloop)->stop = kStopDone;
+            return cudaSuccess;
+        };
+        LoopState init{}, out{};
+        expect(round_loop(c[i], cudaStreamPerThread, true, init, nullptr, &out) == BISIM_OK, "a loop failed");
+        size_t at = calls.size();
+        while (at > 0 && calls[at - 1].what != "cooperative") --at;
+        expect(at > 0, "the loop was not a cooperative launch");
+        if (at == 0) return;
+        if (i == 1) expect(at > 1 && calls[at - 2].what == "wait" && calls[at - 2].event == last, "the second loop did not wait for the first");
+        expect(at < calls.size() && calls[at].what == "record", "no event follows the loop");
+        if (at < calls.size()) last = calls[at].event;
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
     const std::map<std::string, std::function<void()>> scenarios = {
         {"sort_on_two_devices", sort_on_two_devices},
         {"wide_rows_on_two_devices", wide_rows_on_two_devices},
+        {"loops_on_one_handle", loops_on_one_handle},
     };
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) {

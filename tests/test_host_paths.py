@@ -32,7 +32,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["sort_on_two_devices", "wide_rows_on_two_devices"])
+@pytest.mark.parametrize("scenario", ["sort_on_two_devices", "wide_rows_on_two_devices", "loops_on_one_handle"])
 def test_host_path(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
