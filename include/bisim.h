@@ -73,7 +73,8 @@ enum { BISIM_FLAG_FULL_RECOMPUTE = 2 };
  * count stops changing or the round limit is reached: the rounds are one
  * cooperative kernel wherever the rows that are left have at most 256 edges
  * (after one host-driven round, or from P_0 on), else one captured CUDA graph
- * whose while node repeats a round. Rounds also run eagerly while launch
+ * whose while node repeats a round (also where the cooperative kernel is refused
+ * its SMs, or waits for them for seconds). Rounds also run eagerly while launch
  * profiling (bisim_profile_enable) is on. */
 enum { BISIM_FLAG_EAGER = 4 };
 

@@ -477,7 +477,8 @@ bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
     bool done = limit <= 0;
     // on the device as far as it goes: one round of the kernels of every class and
     // the cooperative loop, then (while rows above 256 edges stay listed) the
-    // captured graph; a hash collision ends either one's last round here
+    // captured graph; a hash collision ends either one's last round here. Where the
+    // loop cannot run or gives up, the rounds start from P_0 again without it.
     const bool device_loop = round_loop_usable(ctx);
     bool collided = false;
     for (int part = 0; part < 2 && !done && !collided && device_loop; ++part) {
@@ -486,6 +487,11 @@ bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
         bisim_status st = part == 0 ? dense_round_then_loop(ctx, s, limit, fixpoint, prev, from_p0, &g)
                                     : dense_graph_rounds(ctx, s, limit - executed, fixpoint, prev, &g);
         if (st != BISIM_OK) return st;
+        if (g.stop == kStopLost) {
+            int64_t dropped = 0;
+            if ((st = dense_rounds_begin(ctx, s, nullptr, &prev, &dropped)) != BISIM_OK) return st;
+            continue;
+        }
         const int32_t before = executed;
         executed += g.executed;
         if (g.stop == kStopDone) {

@@ -343,6 +343,7 @@ struct bisim_ctx {
     void* dloop = nullptr;                           // loop state on the device
     void* hloop = nullptr;                           // its pinned host mirror
     int32_t loop_copy = 0;                           // cooperative loop: which copy of its counters the next launch uses
+    uint32_t loop_polls = 0;                         // cooperative loop: polls of a barrier before it gives up, 0: as usual
     int64_t round_graph_launches = 0;                // kernels in one captured round
 
     // batched contexts: the persistent per-graph kernel (segment.cu)

@@ -46,7 +46,8 @@ constexpr int kLoopGroups = 4;            // degree <= 8, <= 16, <= 32, <= 256: 
 constexpr int kHotSlots = 64;
 constexpr int kSeenSlots = 1024;
 constexpr int kLoopWarpSet = 512;         // slots of a warp's set: twice the longest row
-constexpr unsigned kSpinLimit = 1u << 22; // polls of a barrier before the kernel gives up (seconds)
+constexpr unsigned kSpinLimit = 1u << 22; // polls of a barrier before the kernel gives up (seconds): the rounds
+                                          // then run again without it
 constexpr int kUnits = 4;                 // work units a warp takes between two flushes of the CTA
 constexpr int kStage = kUnits * 32;
 constexpr uint8_t kCold = 255;
@@ -112,6 +113,7 @@ struct LoopView {
     int32_t n;
     int32_t copy;                         // which LoopCopy this launch uses
     int32_t cluster;                      // the grid is one cluster
+    unsigned polls;                       // kSpinLimit, or what a test sets
     int32_t start;                        // 1: from P_0 with every live position listed; 0: from act[0] / aoff and *L
     LoopState init;                       // start: the loop state to begin with
 };
@@ -192,7 +194,7 @@ __device__ bool arrive_and_wait(const LoopView& V, unsigned k, Shared& sh) {
         const unsigned target = gridDim.x * k;
         unsigned spin = 0;
         while (load_acquire(&c->arrived) < target) {
-            if (++spin > kSpinLimit || ((spin & 255u) == 0u && load_acquire(&V.ctl->abort) != 0u)) {
+            if (++spin > V.polls || ((spin & 255u) == 0u && load_acquire(&V.ctl->abort) != 0u)) {
                 atomicExch(&V.ctl->abort, 1u);
                 sh.ok = 0;
                 break;
@@ -1173,6 +1175,7 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     V.copy = ctx->loop_copy;
     ctx->loop_copy ^= 1;
     V.start = start ? 1 : 0;
+    V.polls = ctx->loop_polls ? ctx->loop_polls : kSpinLimit;
     V.init = init;
     std::memset(h, 0, sizeof(*h));
     h->stop = kStopLost;                                   // overwritten by the kernel
@@ -1203,21 +1206,22 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     } else {
         e = launch_in_lane(ctx->device, kernel, grid, threads, args, smem, s);
     }
-    if (e) {
-        ctx->loop_copy ^= 1;                               // the launch that would have cleared the other copy is missing
-        return cuda_error(ctx, e, "launch round loop");
-    }
-    prof_add_launches(1);
+    // refused (too few SMs for a grid that has to be resident as a whole): no result either
+    if (e) cudaGetLastError();
+    else prof_add_launches(1);
     if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "round loop");
     *out = *h;
     if (out->stop == kStopLost) {
-        cudaMemsetAsync(V.ctl, 0, sizeof(LoopCtl), s);
-        cudaStreamSynchronize(s);
-        ctx->epoch32 = kEpochCycle;
-        return set_error(ctx, BISIM_ETIMEOUT, "round loop: a grid barrier ran out of polls");
+        cudaMemsetAsync(V.ctl, 0, sizeof(LoopCtl), s);     // both copies of the counters
+        ctx->epoch32 = kEpochCycle;                        // the next epoch starts with a blank table
+        return BISIM_OK;
     }
     if (!regions) ctx->epoch32 = static_cast<uint32_t>(out->epoch) + kEpochCycle;
     return BISIM_OK;
 }
 
 }  // namespace bisim
+
+extern "C" void bisim_loop_polls(bisim_ctx* ctx, uint32_t polls) {
+    if (ctx != nullptr) ctx->loop_polls = polls;
+}

@@ -13,7 +13,7 @@ enum : int32_t {
     kStopCollision = 2,     // the last round's hash collisions are left to the host
     kStopError = 3,         // error bits in the status word
     kStopWideRows = 4,      // cooperative kernel: rows above 256 edges are listed; nothing was done
-    kStopLost = 5,          // cooperative kernel: no result came back
+    kStopLost = 5,          // cooperative kernel: it could not run, or gave up at a barrier
 };
 
 // State of a run of rounds (device memory, and its pinned mirror).
@@ -58,8 +58,15 @@ bisim_status round_loop_state(bisim_ctx* ctx, cudaStream_t s);
 // state to begin with), or from the current list and the loop state in device
 // memory. The result is in P[0] unless out->stop is kStopCollision or
 // kStopError: then the last round stands as the host-driven levels expect it.
+// kStopLost: the partition and the list are left anyhow, and the rounds have to
+// start from P_0 again without the loop.
 // `ccount`: the list's per-class survivor counters. Synchronises s.
 bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopState& init, unsigned long long* ccount,
                         LoopState* out);
 
 }  // namespace bisim
+
+// Sets the polls after which the context's loop gives up at a barrier (0: the
+// usual number, a few seconds), so that tests see what follows. Not part of the
+// public interface.
+extern "C" void bisim_loop_polls(bisim_ctx* ctx, uint32_t polls);

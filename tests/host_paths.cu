@@ -5,6 +5,7 @@
 #include <functional>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "bisim.h"
@@ -105,6 +106,46 @@ void loops_on_one_handle() {
     }
 }
 
+// A loop that is refused its SMs, or gives up at a barrier, leaves the rounds to
+// the captured graph, from P_0 again.
+void rounds_without_the_loop() {
+    bisim_ctx& c = looping_context(1 << 20);
+    const auto device_array = [](auto** p, size_t count) {
+        void* q = nullptr;
+        cudaMallocAsync(&q, count * sizeof(**p), nullptr);
+        *p = static_cast<std::remove_reference_t<decltype(*p)>>(q);
+    };
+    device_array(&c.P0, c.n);
+    device_array(&c.P[0], c.n);
+    device_array(&c.P[1], c.n);
+    device_array(&c.djoined, c.n);
+    device_array(&c.dstate, 1);
+    device_array(&c.table, c.nslots);
+    c.hstate = static_cast<DevState*>(pinned_take());
+    for (int i = 0; i < c.n; ++i) c.P0[i] = 7;
+    c.last_blocks = 5;
+    for (const bool refuse : {true, false}) {
+        int graphs = 0;
+        c.P[0][1] = 0;                          // as if the loop had got some way
+        fake::runtime().on_launch = [&](const void* kernel, bool cooperative) {
+            if (cooperative) return refuse ? cudaErrorCooperativeLaunchTooLarge : cudaSuccess;
+            if (kernel == nullptr) {            // the graph
+                ++graphs;
+                LoopState* L = static_cast<LoopState*>(c.dloop);
+                expect(L->prev_blocks == 5 && L->limit == 3 && c.P[0][1] == 7, "the graph did not start from P_0");
+                L->stop = kStopDone;
+                L->executed = L->rounds = 3;
+                L->blocks = 11;
+            }
+            return cudaSuccess;
+        };
+        int32_t rounds = 0, executed = 0;
+        int64_t blocks = 0;
+        expect(dense_rounds_all(&c, 3, 0, nullptr, &rounds, &executed, &blocks, true) == BISIM_OK, "the rounds failed");
+        expect(graphs == 1 && rounds == 3 && executed == 3 && blocks == 11, "the graph's result is not the call's");
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -112,6 +153,7 @@ int main(int argc, char** argv) {
         {"sort_on_two_devices", sort_on_two_devices},
         {"wide_rows_on_two_devices", wide_rows_on_two_devices},
         {"loops_on_one_handle", loops_on_one_handle},
+        {"rounds_without_the_loop", rounds_without_the_loop},
     };
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) {

@@ -122,3 +122,29 @@ def test_one_cta_with_a_warp_row_as_the_first_call():
             "c = B.summarize_init_coo(3, i([0] * 40 + [1]), i([k % 3 for k in range(40)] + [2]), i(list(range(40)) + [0]), i([0, 0, 0]));"
             "assert B.bisim_iterate(c, 1)[1] == 3; assert B.get_partition(c).tolist() == [0, 1, 2]")
     subprocess.run([sys.executable, "-c", code], check=True, timeout=300)
+
+
+@pytest.mark.parametrize("hub", [0, 300])
+@pytest.mark.parametrize("degree", [3, 20])
+def test_rounds_go_on_without_a_loop_that_gave_up(B, degree, hub):
+    """With one poll a barrier the CTAs give up while others are on their way; the rounds then run again from P_0 by
+    the captured graph. The next call has the loop back."""
+    import torch
+    g = rows_graph(60_000, degree, seed=degree)
+    if hub:
+        # a wide row that is alone in its block from round 1 on, so that the loop takes over after it
+        rng = np.random.default_rng(hub)
+        for k, more in (("src", np.full(hub, 17)), ("dst", rng.integers(0, g["n"], hub)), ("elabel", 2 + np.arange(hub))):
+            g[k] = np.concatenate([g[k], more]).astype(np.int32)
+    want, rounds, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], oracle.FIXPOINT, 20)
+    t = {k: torch.from_numpy(g[k]).cuda() for k in ("src", "dst", "elabel", "vlabel")}
+    with B.summarize_init_coo(g["n"], t["src"], t["dst"], t["elabel"], t["vlabel"]) as ctx:
+        launches = []
+        for polls in (0, 1, 0):
+            B._lib.bisim_loop_polls(ctx.ptr, polls)
+            before = B.bisim_launch_count()
+            got = B.bisim_iterate(ctx, oracle.FIXPOINT, 20)
+            launches.append(B.bisim_launch_count() - before)
+            assert got == (rounds, len(np.unique(want)))
+            assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+        assert launches[1] > launches[0] == launches[2]

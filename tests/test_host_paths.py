@@ -32,7 +32,8 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["sort_on_two_devices", "wide_rows_on_two_devices", "loops_on_one_handle"])
+@pytest.mark.parametrize("scenario", ["sort_on_two_devices", "wide_rows_on_two_devices", "loops_on_one_handle",
+                                      "rounds_without_the_loop"])
 def test_host_path(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
