@@ -364,6 +364,25 @@ bisim_status finish_init(bisim_ctx* ctx, cudaStream_t s) {
     return BISIM_OK;
 }
 
+// The end of an init that failed. *again: a device allocation failed while P_0's
+// state was there beside the build's scratch.
+bisim_status init_failed(bisim_ctx* ctx, bisim_status st, bool* again) {
+    const std::string msg = ctx->err;
+    *again = ctx->out_of_memory && ctx->p0_early;
+    destroy_ctx(ctx);
+    return set_error(nullptr, st, msg);
+}
+
+// Beside the build, P_0 holds 32 bytes a vertex and the table before the build's
+// scratch, the staged arrays and the edge view are gone (0.45 GB at 10M vertices).
+// Where that is too much, the init starts over with P_0 after the build.
+template <class F>
+bisim_status init_in_memory(const F& init) {
+    bool again = false;
+    const bisim_status st = init(false, &again);
+    return again ? init(true, &again) : st;
+}
+
 // The graph of every vertex, four vertices a thread; a warp's 128 are looked up once.
 __global__ void __launch_bounds__(256) k_graph_ids(const int64_t* __restrict__ voff, int32_t G, int32_t n,
                                                    int32_t* __restrict__ gid) {
@@ -398,6 +417,7 @@ bisim_status set_error(bisim_ctx* ctx, bisim_status st, const std::string& msg) 
 bisim_status cuda_error(bisim_ctx* ctx, cudaError_t e, const char* what) {
     std::string msg = std::string(what) + ": " + cudaGetErrorString(e);
     cudaGetLastError();
+    if (ctx != nullptr && e == cudaErrorMemoryAllocation) ctx->out_of_memory = true;
     return set_error(ctx, BISIM_ECUDA, msg);
 }
 
@@ -624,13 +644,15 @@ void bisim_default_options(bisim_options* opt) {
     opt->batch_split = 0;
 }
 
-bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int64_t* row_ptr,
-                            const int32_t* col, const int32_t* edge_label, const int32_t* vertex_label,
-                            const uint8_t* alive, const bisim_options* opt, void* stream) {
+static bisim_status init_csr(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int64_t* row_ptr,
+                             const int32_t* col, const int32_t* edge_label, const int32_t* vertex_label,
+                             const uint8_t* alive, const bisim_options* opt, void* stream, bool p0_after,
+                             bool* again) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bisim_ctx* ctx = nullptr;
     bisim_status st = new_ctx(out, n_vertices, n_edges, opt, s, &ctx);
     if (st != BISIM_OK) return st;
+    ctx->p0_after = p0_after;
     if (row_ptr == nullptr || (n_vertices > 0 && vertex_label == nullptr) ||
         (n_edges > 0 && (col == nullptr || edge_label == nullptr))) {
         destroy_ctx(ctx);
@@ -675,18 +697,27 @@ bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges
             return BISIM_OK;
         }
     }
-    std::string msg = ctx->err;
-    destroy_ctx(ctx);
-    return set_error(nullptr, st, msg);
+    return init_failed(ctx, st, again);
 }
 
-bisim_status summarize_init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int32_t* src,
-                                const int32_t* dst, const int32_t* edge_label, const int32_t* vertex_label,
-                                const uint8_t* alive, const bisim_options* opt, void* stream) {
+bisim_status summarize_init(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int64_t* row_ptr,
+                            const int32_t* col, const int32_t* edge_label, const int32_t* vertex_label,
+                            const uint8_t* alive, const bisim_options* opt, void* stream) {
+    return init_in_memory([&](bool p0_after, bool* again) {
+        return init_csr(out, n_vertices, n_edges, row_ptr, col, edge_label, vertex_label, alive, opt, stream, p0_after,
+                        again);
+    });
+}
+
+static bisim_status init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int32_t* src,
+                             const int32_t* dst, const int32_t* edge_label, const int32_t* vertex_label,
+                             const uint8_t* alive, const bisim_options* opt, void* stream, bool p0_after,
+                             bool* again) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bisim_ctx* ctx = nullptr;
     bisim_status st = new_ctx(out, n_vertices, n_edges, opt, s, &ctx);
     if (st != BISIM_OK) return st;
+    ctx->p0_after = p0_after;
     if ((n_vertices > 0 && vertex_label == nullptr) ||
         (n_edges > 0 && (src == nullptr || dst == nullptr || edge_label == nullptr))) {
         destroy_ctx(ctx);
@@ -728,9 +759,7 @@ bisim_status summarize_init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_e
             *out = ctx;
             return BISIM_OK;
         }
-        std::string msg = ctx->err;
-        destroy_ctx(ctx);
-        return set_error(nullptr, st, msg);
+        return init_failed(ctx, st, again);
     }
     if ((st = copy_vertex_arrays(ctx, vertex_label, alive, s)) == BISIM_OK && (st = p0_begin(ctx, s, true)) == BISIM_OK) {
         if ((e = stage(src, eb, s, &ds, temps)) || (e = stage(dst, eb, s, &dd, temps)) ||
@@ -745,15 +774,22 @@ bisim_status summarize_init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_e
         *out = ctx;
         return BISIM_OK;
     }
-    std::string msg = ctx->err;
-    destroy_ctx(ctx);
-    return set_error(nullptr, st, msg);
+    return init_failed(ctx, st, again);
 }
 
-bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int64_t* vertex_offsets,
-                                    const int64_t* edge_offsets, const int32_t* src_local,
-                                    const int32_t* dst_local, const int32_t* edge_label,
-                                    const int32_t* vertex_label, const bisim_options* opt, void* stream) {
+bisim_status summarize_init_coo(bisim_ctx** out, int32_t n_vertices, int64_t n_edges, const int32_t* src,
+                                const int32_t* dst, const int32_t* edge_label, const int32_t* vertex_label,
+                                const uint8_t* alive, const bisim_options* opt, void* stream) {
+    return init_in_memory([&](bool p0_after, bool* again) {
+        return init_coo(out, n_vertices, n_edges, src, dst, edge_label, vertex_label, alive, opt, stream, p0_after,
+                        again);
+    });
+}
+
+static bisim_status init_batched(bisim_ctx** out, int32_t n_graphs, const int64_t* vertex_offsets,
+                                 const int64_t* edge_offsets, const int32_t* src_local, const int32_t* dst_local,
+                                 const int32_t* edge_label, const int32_t* vertex_label, const bisim_options* opt,
+                                 void* stream, bool p0_after, bool* again) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (out == nullptr) return set_error(nullptr, BISIM_EINVAL, "out pointer is NULL");
     *out = nullptr;
@@ -774,6 +810,7 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
     bisim_ctx* ctx = nullptr;
     bisim_status st = new_ctx(out, n, m, opt, s, &ctx);
     if (st != BISIM_OK) return st;
+    ctx->p0_after = p0_after;
     ctx->n_graphs = n_graphs;
     if ((n > 0 && vertex_label == nullptr) || (m > 0 && (src_local == nullptr || dst_local == nullptr || edge_label == nullptr))) {
         destroy_ctx(ctx);
@@ -833,9 +870,17 @@ bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int
         *out = ctx;
         return BISIM_OK;
     }
-    std::string msg = ctx->err;
-    destroy_ctx(ctx);
-    return set_error(nullptr, st, msg);
+    return init_failed(ctx, st, again);
+}
+
+bisim_status summarize_init_batched(bisim_ctx** out, int32_t n_graphs, const int64_t* vertex_offsets,
+                                    const int64_t* edge_offsets, const int32_t* src_local,
+                                    const int32_t* dst_local, const int32_t* edge_label,
+                                    const int32_t* vertex_label, const bisim_options* opt, void* stream) {
+    return init_in_memory([&](bool p0_after, bool* again) {
+        return init_batched(out, n_graphs, vertex_offsets, edge_offsets, src_local, dst_local, edge_label, vertex_label,
+                            opt, stream, p0_after, again);
+    });
 }
 
 bisim_status bisim_iterate(bisim_ctx* ctx, int32_t k, int32_t cap, int32_t* out_rounds, int64_t* out_num_blocks,

@@ -372,6 +372,9 @@ struct bisim_ctx {
     bisim::DevState* dstate = nullptr;   // and, kStateStride further on, P_0's while it runs beside the build
     bisim::DevState* hstate = nullptr;   // pinned mirror
     bool p0_pending = false;             // p0_begin ran and p0_end did not
+    bool p0_after = false;               // P_0 follows the build (less memory at its peak)
+    bool p0_early = false;               // P_0 was begun before the build
+    bool out_of_memory = false;          // a device allocation failed
     bisim::Branch p0_branch;
 
     // updates
@@ -532,7 +535,8 @@ bisim_status csr_from_store(bisim_ctx* ctx, cudaStream_t s);
 bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s);
 // The refinement state, and P_0 into ctx->P0 and ctx->P[0]. An `early` call, as soon
 // as the vertex arrays (and graphs) are there, starts it beside the build where that
-// pays, else does nothing; p0_end synchronises `s` and has the result.
+// pays (unless p0_after is set), else does nothing; p0_end synchronises `s` and has
+// the result.
 bisim_status p0_begin(bisim_ctx* ctx, cudaStream_t s, bool early);
 bisim_status p0_end(bisim_ctx* ctx, cudaStream_t s);
 // Advances the signature table's epoch (clearing the table when it wraps).

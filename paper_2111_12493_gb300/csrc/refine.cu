@@ -836,8 +836,9 @@ bisim_status compute_p0(bisim_ctx* ctx, cudaStream_t s) {
 }
 
 bisim_status p0_begin(bisim_ctx* ctx, cudaStream_t s, bool early) {
-    const bool beside = early && ctx->n >= kP0BesideMin && !prof_enabled();
+    const bool beside = early && !ctx->p0_after && ctx->n >= kP0BesideMin && !prof_enabled();
     if (early && !beside) return BISIM_OK;
+    ctx->p0_early = beside;
     bisim_status st = alloc_refine_state(ctx, s);
     if (st != BISIM_OK) return st;
     if (beside) ctx->p0_branch = branch_fork(ctx->device, s);

@@ -146,6 +146,47 @@ void rounds_without_the_loop() {
     }
 }
 
+// An init that does not fit with P_0 beside the build fits with P_0 after it.
+void init_at_the_memory_limit() {
+    const int32_t n = 200000, graphs = 2;
+    const int64_t m = 1000000;
+    int32_t* a[4];                              // sources, targets, labels; vertex labels
+    for (int32_t*& p : a) {
+        void* q = nullptr;
+        cudaMallocAsync(&q, sizeof(int32_t) * m, nullptr);
+        p = static_cast<int32_t*>(q);
+    }
+    const std::vector<int64_t> vo = {0, n / 2, n}, eo = {0, m / 2, m};
+    void* rp = nullptr;
+    cudaMallocAsync(&rp, sizeof(int64_t) * (n + 1), nullptr);
+    bisim_options o;
+    bisim_default_options(&o);
+    const std::map<std::string, std::function<bisim_status(bisim_ctx**)>> inits = {
+        {"edge list", [&](bisim_ctx** c) { return summarize_init_coo(c, n, m, a[0], a[1], a[2], a[3], nullptr, &o, nullptr); }},
+        {"CSR", [&](bisim_ctx** c) { return summarize_init(c, n, m, static_cast<int64_t*>(rp), a[1], a[2], a[3], nullptr, &o, nullptr); }},
+        {"batch", [&](bisim_ctx** c) { return summarize_init_batched(c, graphs, vo.data(), eo.data(), a[0], a[1], a[2], a[3], &o, nullptr); }},
+    };
+    fake::Runtime& R = fake::runtime();
+    const size_t before = R.live;
+    for (const int direction : {BISIM_DIR_FORWARD, BISIM_DIR_BOTH}) {
+        o.direction = direction;
+        for (const auto& [what, init] : inits) {
+            if (what == "CSR" && direction == BISIM_DIR_FORWARD) continue;      // nothing is staged: no peak to avoid
+            bisim_ctx* c = nullptr;
+            R.limit = ~size_t{0};
+            R.peak = before;
+            expect(init(&c) == BISIM_OK, what.c_str());
+            summarize_destroy(c);
+            R.limit = R.peak - 1;
+            expect(init(&c) == BISIM_OK, (what + ", a byte below the peak").c_str());
+            summarize_destroy(c);
+            R.limit = before + 1000;
+            expect(init(&c) != BISIM_OK && c == nullptr, (what + ", next to no memory").c_str());
+            expect(R.live == before, (what + ": memory is left behind").c_str());
+        }
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -154,6 +195,7 @@ int main(int argc, char** argv) {
         {"wide_rows_on_two_devices", wide_rows_on_two_devices},
         {"loops_on_one_handle", loops_on_one_handle},
         {"rounds_without_the_loop", rounds_without_the_loop},
+        {"init_at_the_memory_limit", init_at_the_memory_limit},
     };
     const auto s = scenarios.find(argc > 1 ? argv[1] : "");
     if (s == scenarios.end()) {

@@ -33,7 +33,7 @@ def program(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["sort_on_two_devices", "wide_rows_on_two_devices", "loops_on_one_handle",
-                                      "rounds_without_the_loop"])
+                                      "rounds_without_the_loop", "init_at_the_memory_limit"])
 def test_host_path(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
