@@ -245,3 +245,32 @@ def test_noalloc_rejects_memory_of_another_device(B):
         vl = torch.from_numpy(g["vlabel"]).to("cuda:0")
         out = torch.empty(g["n"], dtype=torch.int32, device="cuda:0")
         _rejected(B, g["n"], d_rp, d_col, d_lab, vl, out, match="current device")
+
+
+@pytest.mark.parametrize("n,wide,degree", [(153, 4, 300), (10_000, 20, 8000), (19_457, 300, 600), (60_000, 800, 1000)])
+def test_noalloc_wide_rows_side_by_side(B, n, wide, degree):
+    """Rows that take a whole CTA, at the first ids and spread over all: the same partitions as the oracle's, and
+    side by side they are not one CTA's work (up to eight times the time of the spread ones, when they were)."""
+    import time
+
+    import torch
+    rng = np.random.default_rng(n)
+    took = []
+    for ids in (np.arange(wide), np.sort(rng.choice(n, wide, replace=False))):
+        d = np.full(n, 2)
+        d[ids] = degree
+        m = int(d.sum())
+        g = dict(n=n, src=np.repeat(np.arange(n), d).astype(np.int32), dst=rng.integers(0, n, m).astype(np.int32),
+                 elabel=rng.integers(0, 3, m).astype(np.int32), vlabel=rng.integers(0, 2, n).astype(np.int32))
+        g["dst"][degree * 2:degree * 3] = g["dst"][degree:degree * 2]      # two of the first rows alike
+        g["elabel"][degree * 2:degree * 3] = g["elabel"][degree:degree * 2]
+        _check_against_oracle(B, g)
+        rp, col, lab, vl = _dev(*_csr(g), g["vlabel"])
+        out = torch.empty(n, dtype=torch.int32, device="cuda")
+        best = 1.0
+        for _ in range(30):
+            t = time.perf_counter()
+            B.bisim_refine_round_noalloc(n, rp, col, lab, vl, out)
+            best = min(best, time.perf_counter() - t)
+        took.append(best)
+    assert took[0] < 2.5 * took[1], took
