@@ -1350,23 +1350,28 @@ __global__ void k_active_init(int32_t* __restrict__ act, int64_t n_live, int64_t
 }
 
 constexpr int kCompareGrid = 304;                      // persistent grids: two CTAs per SM
-constexpr int kCompareWarpGrid = 1216;                 // eight per SM: 32 pairs a warp, all warps in flight
+constexpr int kCompareWarpGrid = 1216;                 // eight per SM
+constexpr unsigned kCompareWarps = 6080;               // warps of it that are resident (48 registers)
 
-// Pairs whose rows have at most 32 edges, 32 pairs to a warp. A pair with at
-// most eight edges on both sides is compared by its lane: r's values in
-// registers, v's four at a time, S_v inside S_r iff each is among them (the
-// sizes are equal). The others take the whole warp one after the other: lane j
-// holds the j-th pair value of each row. (One warp per pair throughout was bound
-// by the latency of four dependent loads a pair: 0.33 of the 0.73 ms of a 1M chain
-// graph's rounds.) The pair count is read on the device.
+// Pairs whose rows have at most 32 edges, up to 32 pairs to a warp (fewer of a short
+// list, but no fewer than eight). A pair with at most eight edges on both sides is
+// compared by its lane: r's values in registers, v's four at a time, S_v inside S_r
+// iff each is among them (the sizes are equal). The others go four at a time, eight
+// lanes a pair, four values of each row a lane. (One warp per pair throughout was
+// bound by the latency of four dependent loads a pair: 0.33 of the 0.73 ms of a 1M
+// chain graph's rounds. The wide pairs one after the other by the whole warp, 32 of
+// them: one round on 20k vertices of 16 edges, 20k pairs, took 143 us, with
+// a warp a pair 120, takes 123; on 2M vertices 1,110 and now 960.) The pair count is
+// read on the device.
 __global__ void __launch_bounds__(kThreads) k_dense_compare_warp(const int2* __restrict__ pairs, const DenseView D,
                                                                  int32_t* __restrict__ Pout,
                                                                  int32_t* __restrict__ next, DevState* st) {
     const unsigned count = *reinterpret_cast<volatile unsigned*>(&st->pairs);
     const unsigned lane = lane_id();
-    const unsigned threads = gridDim.x * kThreads;
-    for (unsigned b = blockIdx.x * kThreads + (threadIdx.x & ~31u); b < count; b += threads) {
-        const bool in = b + lane < count;
+    const unsigned warps = gridDim.x * (kThreads / 32);
+    const unsigned per = max(8u, min(32u, (count + kCompareWarps - 1) / kCompareWarps));
+    for (unsigned b = (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * per; b < count; b += warps * per) {
+        const bool in = lane < per && b + lane < count;
         int2 pr = make_int2(0, 0);
         int64_t ev = 0, er = 0;
         int dv = 0, dr = 0;
@@ -1404,20 +1409,45 @@ __global__ void __launch_bounds__(kThreads) k_dense_compare_warp(const int2* __r
                 }
             }
         }
-        for (unsigned todo = __ballot_sync(0xffffffffu, in && !small); todo; todo &= todo - 1u) {
-            const int q = __ffs(todo) - 1;
+        // the others four at a time, eight lanes a pair
+        unsigned todo = __ballot_sync(0xffffffffu, in && !small);
+        while (todo) {
+            unsigned mine = todo;                                    // from the (lane / 8)-th pair that is left on
+            for (unsigned k = 0; k < lane / 8; ++k) mine &= mine - 1u;
+            const int q = mine ? __ffs(mine) - 1 : 0;
             const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
-            const int qdv = __shfl_sync(0xffffffffu, dv, q), qdr = __shfl_sync(0xffffffffu, dr, q);
-            const bool ha = static_cast<int>(lane) < qdv, hb = static_cast<int>(lane) < qdr;
-            const uint64_t va = ha ? packed_pair_value(D.pe[qev + lane], D.P) : 0ull;
-            const uint64_t vb = hb ? packed_pair_value(D.pe[qer + lane], D.P) : 0ull;
-            bool found = false;
-            for (int k = 0; k < qdr; ++k) {
-                const uint64_t bk = __shfl_sync(0xffffffffu, vb, k);   // every lane takes part in every shuffle
-                found = found || bk == va;
+            const int gdv = __shfl_sync(0xffffffffu, dv, q), gdr = __shfl_sync(0xffffffffu, dr, q);
+            const int qdv = mine ? gdv : 0, qdr = mine ? gdr : 0;
+            const int sub = static_cast<int>(lane & 7u);
+            uint64_t va[4], vb[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                va[j] = sub + 8 * j < qdv ? D.pe[qev + sub + 8 * j] : 0ull;
+                vb[j] = sub + 8 * j < qdr ? D.pe[qer + sub + 8 * j] : 0ull;
             }
-            const bool miss = __any_sync(0xffffffffu, ha && !found);
-            if (static_cast<int>(lane) == q) same = !miss;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (sub + 8 * j < qdv) va[j] = packed_pair_value(va[j], D.P);
+                if (sub + 8 * j < qdr) vb[j] = packed_pair_value(vb[j], D.P);
+            }
+            unsigned found = 0u;                                     // which of the lane's four are among r's
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (__all_sync(0xffffffffu, qdr <= 8 * i)) break;
+                for (int k = 0; k < 8; ++k) {
+                    const uint64_t bk = __shfl_sync(0xffffffffu, vb[i], k, 8);   // every lane takes part
+                    const bool is = 8 * i + k < qdr;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (is && va[j] == bk) found |= 1u << j;
+                }
+            }
+            bool miss = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) miss = miss || (sub + 8 * j < qdv && !((found >> j) & 1u));
+            const unsigned missed = __ballot_sync(0xffffffffu, miss);
+            for (int g = 0; g < 4 && todo; ++g, todo &= todo - 1u)   // the same for the whole warp
+                if (static_cast<int>(lane) == __ffs(todo) - 1) same = ((missed >> (8 * g)) & 0xffu) == 0u;
         }
         const unsigned words = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(dv + dr));
         if (lane == 0) atomicAdd(&st->aux, static_cast<unsigned long long>(words));

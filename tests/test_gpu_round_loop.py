@@ -148,3 +148,12 @@ def test_rounds_go_on_without_a_loop_that_gave_up(B, degree, hub):
             assert got == (rounds, len(np.unique(want)))
             assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
         assert launches[1] > launches[0] == launches[2]
+
+
+@pytest.mark.parametrize("bits", [2, 64])
+@pytest.mark.parametrize("n,degree", [(25, 9), (26, 32), (800, 17), (20_000, 24), (20_000, 8)])
+def test_pairs_of_the_single_class_kernels(B, n, degree, bits):
+    """Equal and (with two bits of hash) unequal rows of 8 to 33 edges, compared eight lanes a pair in the kernels of
+    host-driven rounds: lists shorter than a warp's pairs, and longer than all warps'."""
+    check(B, rows_graph(n, degree, seed=n + degree), [1, 2],
+          options=B.default_options(flags=B.FLAG_EAGER, hash_bits=bits))
