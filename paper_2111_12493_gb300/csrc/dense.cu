@@ -1173,8 +1173,9 @@ __global__ void __launch_bounds__(kThreads) k_dense_verify(const int32_t* __rest
 // not alone in their block, in order. Tiles of kActTile entries, four
 // consecutive entries per thread (eight left most CTAs idle once the list is
 // short: 2.725 against 2.679 ms for the five rounds of the 10M-vertex graph);
-// `stop` (the captured loop's decision, null for host-driven rounds) skips all
-// of it when the host must first resolve the round's hash collisions.
+// `stop` (the device's decision, null for host-driven rounds) skips all of it
+// when the host must first resolve the round's hash collisions, and the list when
+// no round follows.
 constexpr int kActPer = 4;
 constexpr int kActTile = kThreads * kActPer;
 
@@ -1250,7 +1251,7 @@ __global__ void __launch_bounds__(kThreads) k_active_count(const DenseView D, co
 // Pass 2 (one CTA): exclusive scan of the tile counts; the new length goes to tcount[slot_total].
 __global__ void __launch_bounds__(1024) k_active_scan(const int64_t* __restrict__ aoff, int64_t* __restrict__ tcount,
                                                       int64_t slot_total, const int32_t* stop) {
-    if (stop != nullptr && *stop >= 2) return;
+    if (stop != nullptr && *stop != kStopNo) return;
     const int64_t tiles = (aoff[kDClasses] + kActTile - 1) / kActTile;
     const int64_t total = cta_exclusive_scan(tcount, tcount, tiles);
     if (threadIdx.x == 0) tcount[slot_total] = total;
@@ -1260,7 +1261,7 @@ __global__ void __launch_bounds__(1024) k_active_scan(const int64_t* __restrict_
 __global__ void __launch_bounds__(kThreads) k_active_scatter(const DenseView D, const int64_t* __restrict__ toff,
                                                              int32_t* __restrict__ next, const int32_t* stop) {
     __shared__ unsigned wpre[kThreads / 32];
-    if (stop != nullptr && *stop >= 2) return;
+    if (stop != nullptr && *stop != kStopNo) return;
     const int64_t count = D.aoff[kDClasses];
     const int64_t tiles = (count + kActTile - 1) / kActTile;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -1296,7 +1297,7 @@ __global__ void __launch_bounds__(kThreads) k_active_scatter(const DenseView D, 
 __global__ void __launch_bounds__(kThreads) k_active_finish(const int32_t* __restrict__ next, int32_t* __restrict__ act,
                                                             int64_t* __restrict__ aoff, const int64_t* __restrict__ total,
                                                             unsigned long long* __restrict__ ccount, const int32_t* stop) {
-    if (stop != nullptr && *stop >= 2) return;
+    if (stop != nullptr && *stop != kStopNo) return;
     const int64_t len = *total;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         int64_t run = 0;
@@ -1730,7 +1731,7 @@ ClassBounds class_bounds(const bisim_ctx* ctx) {
 
 // End of a round: P_{i+1} of the listed vertices into the input buffer and the
 // list compacted to the vertices still not alone (see k_active_count). `stop`
-// is the captured loop's decision, or null for host-driven rounds.
+// is the device's decision, or null for host-driven rounds.
 void launch_round_end(bisim_ctx* ctx, cudaStream_t s, const DenseView& D, const int32_t* stop,
                       const int32_t* Pfrom = nullptr) {
     BISIM_SITE(site, "active_compact");
@@ -2373,10 +2374,30 @@ bisim_status dense_round_then_loop(bisim_ctx* ctx, cudaStream_t s, int32_t limit
     init.fixpoint = fixpoint ? 1 : 0;
     init.rounds = limit;
     bisim_status st;
+    cudaError_t e;
+    const auto fill = [&](const LoopState& r) {
+        out->executed = r.executed;
+        out->rounds = r.rounds;
+        out->blocks = static_cast<int64_t>(r.blocks);
+        out->prev = static_cast<int64_t>(r.prev_blocks);
+        out->stop = r.stop;
+        return BISIM_OK;
+    };
     set_attributes();                          // a collision's levels on the host need them too
     if (!from_p0) {
         if ((st = round_loop_state(ctx, s)) != BISIM_OK) return st;
         launch_round(ctx, s, level_table(ctx, s));
+        if (limit == 1) {
+            // no list for a next round and no loop: six launches fewer, of which a
+            // small graph's one round took 20 us longer than as a captured graph
+            cudaMemcpyAsync(ctx->hstate, ctx->dstate, sizeof(DevState), cudaMemcpyDeviceToHost, s);
+            if ((e = cudaStreamSynchronize(s))) return cuda_error(ctx, e, "dense round");
+            loop_advance(init, ctx->hstate->blocks, ctx->hstate->unresolved, ctx->hstate->error);
+            if (init.stop == kStopDone &&
+                (e = cudaMemcpyAsync(ctx->P[0], ctx->P[1], sizeof(int32_t) * ctx->n, cudaMemcpyDeviceToDevice, s)))
+                return cuda_error(ctx, e, "dense round");
+            return fill(init);
+        }
         LoopState* L = static_cast<LoopState*>(ctx->dloop);
         BISIM_SITE(site_ck, "round_check");
         {
@@ -2387,12 +2408,7 @@ bisim_status dense_round_then_loop(bisim_ctx* ctx, cudaStream_t s, int32_t limit
     }
     LoopState r;
     if ((st = round_loop(ctx, s, from_p0, init, class_counts(ctx), &r)) != BISIM_OK) return st;
-    out->executed = r.executed;
-    out->rounds = r.rounds;
-    out->blocks = static_cast<int64_t>(r.blocks);
-    out->prev = static_cast<int64_t>(r.prev_blocks);
-    out->stop = r.stop;
-    return BISIM_OK;
+    return fill(r);
 }
 
 bisim_status dense_graph_rounds(bisim_ctx* ctx, cudaStream_t s, int32_t limit, bool fixpoint, int64_t prev_blocks,

@@ -29,6 +29,13 @@ def rows_graph(n, degree, seed, copies=3, n_labels=2):
     return dict(n=n, src=cat(src), dst=cat(dst), elabel=cat(lab), vlabel=rng.integers(0, 2, n).astype(np.int32))
 
 
+def with_hub(g, edges):
+    """The graph with a row of `edges` more edges, whose vertex is alone in its block from round 1 on."""
+    rng = np.random.default_rng(edges)
+    more = dict(src=np.full(edges, 17), dst=rng.integers(0, g["n"], edges), elabel=2 + np.arange(edges))
+    return dict(g, **{k: np.concatenate([g[k], more[k]]).astype(np.int32) for k in more})
+
+
 def path_graph(lengths, marked=()):
     n = int(sum(lengths))
     ends = np.cumsum(lengths) - 1
@@ -132,10 +139,7 @@ def test_rounds_go_on_without_a_loop_that_gave_up(B, degree, hub):
     import torch
     g = rows_graph(60_000, degree, seed=degree)
     if hub:
-        # a wide row that is alone in its block from round 1 on, so that the loop takes over after it
-        rng = np.random.default_rng(hub)
-        for k, more in (("src", np.full(hub, 17)), ("dst", rng.integers(0, g["n"], hub)), ("elabel", 2 + np.arange(hub))):
-            g[k] = np.concatenate([g[k], more]).astype(np.int32)
+        g = with_hub(g, hub)
     want, rounds, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], oracle.FIXPOINT, 20)
     t = {k: torch.from_numpy(g[k]).cuda() for k in ("src", "dst", "elabel", "vlabel")}
     with B.summarize_init_coo(g["n"], t["src"], t["dst"], t["elabel"], t["vlabel"]) as ctx:
@@ -157,3 +161,29 @@ def test_pairs_of_the_single_class_kernels(B, n, degree, bits):
     host-driven rounds: lists shorter than a warp's pairs, and longer than all warps'."""
     check(B, rows_graph(n, degree, seed=n + degree), [1, 2],
           options=B.default_options(flags=B.FLAG_EAGER, hash_bits=bits))
+
+
+@pytest.mark.parametrize("bits", [3, 64])
+@pytest.mark.parametrize("hub", [300, 9000])
+def test_one_round_of_every_class(B, hub, bits):
+    """A single round beside wide rows ends without a list or a loop, also where the fixpoint's cap is 1, where the
+    round changes nothing and where it meets collisions; what follows works on its partition."""
+    import torch
+    options = B.default_options(hash_bits=bits)
+    g = with_hub(rows_graph(2000, 5, seed=hub), hub)
+    check(B, g, [1], options=options)
+    check(B, g, [oracle.FIXPOINT], cap=1, options=options)
+    ring = dict(n=1000, src=np.arange(1000, dtype=np.int32), dst=np.roll(np.arange(1000, dtype=np.int32), 1),
+                elabel=np.zeros(1000, np.int32), vlabel=np.zeros(1000, np.int32))
+    ring["src"], ring["dst"] = np.append(ring["src"], np.full(hub, 17, np.int32)), np.append(ring["dst"], np.arange(hub, dtype=np.int32) % 1000)
+    ring["elabel"] = np.zeros(len(ring["src"]), np.int32)
+    check(B, ring, [1, oracle.FIXPOINT], cap=1, options=options)
+    check(B, ring, [oracle.FIXPOINT], options=options)
+    t = {k: torch.from_numpy(g[k]).cuda() for k in ("src", "dst", "elabel", "vlabel")}
+    with B.summarize_init_coo(g["n"], t["src"], t["dst"], t["elabel"], t["vlabel"], options=options) as ctx:
+        B.bisim_iterate(ctx, 1)
+        want, _, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], 1, 0)
+        assert np.array_equal(B.get_block_sizes(ctx).cpu().numpy(), np.bincount(want, minlength=g["n"]))
+        B.bisim_iterate(ctx, 3)
+        want, _, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], 3, 0)
+        assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
