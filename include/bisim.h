@@ -279,8 +279,9 @@ bisim_status get_block_sizes(bisim_ctx* ctx, int32_t* sizes, void* stream);
  *   out_count  the number of distinct triples (call with capacity 0 to size
  *              the outputs)
  * Uses about 8 bytes of temporary device memory per edge and 32 per vertex, and 24
- * more per edge of a source block of more than 2048 edges (backward contexts:
- * about 36 per edge). Synchronises `stream`.
+ * more per edge of a source block of more than 2048 edges (backward contexts, and
+ * graphs of millions of vertices and fewer edges than vertices: about 36 per
+ * edge). Synchronises `stream`.
  */
 bisim_status get_summary_edges(bisim_ctx* ctx, int32_t* src_block, int32_t* label, int32_t* dst_block,
                                int64_t capacity, int64_t* out_count, void* stream);

@@ -18,8 +18,9 @@
 // are sorted in a warp's registers (several at once), up to 256 in a warp's
 // shared memory, up to 2048 in a CTA's; the keys of longer ones are brought
 // together and radix-sorted by target block, label and segment. A backward
-// context's rows hold the edges by target: there the triples of all edges are
-// radix-sorted by target block, label and source block.
+// context's rows hold the edges by target: there, and where few edges lie between
+// many vertices, the triples of all edges are radix-sorted by target block, label and
+// source block.
 //
 // On a 1M / 10M power-law graph at k = 2 (9.7M summary edges) ten radix passes over
 // all edges took 2.0 of 2.26 ms.
@@ -579,8 +580,15 @@ __global__ void __launch_bounds__(256) k_seg_emit(const int64_t* __restrict__ at
     }
 }
 
-// A backward context: the triples of all edges sorted by target block, label
-// and source block. *out_base (freed by the caller) holds the compacted triples
+// The segments take a dozen passes over all blocks, the radix sorts ten over all
+// edges: many vertices with few edges between them are better sorted. us by segments
+// and by radix, vertices and edges in millions: 1 and 0.5 280 / 457; 3 and 0.3 457 /
+// 430; 3 and 1.5 564 / 617; 10 and 0.5 794 / 490; 10 and 5 1,328 / 1,059; 10 and 10
+// 1,515 / 1,803; 30 and 3 1,749 / 880; 30 and 15 3,500 / 2,680.
+bool fewer_edges_than_passes_over_blocks(int64_t n, int64_t m) { return 10 * m < 7 * (n - 1250000); }
+
+// A backward context, or few edges for its vertices: the triples of all edges sorted
+// by target block, label and source block. *out_base (freed by the caller) holds the compacted triples
 // os, ol, ot.
 bisim_status summary_by_radix(bisim_ctx* ctx, cudaStream_t s, char** out_base, const int32_t** out_os,
                               const int32_t** out_ol, const int32_t** out_ot, int64_t* out_count) {
@@ -862,18 +870,18 @@ bisim_status get_summary_edges(bisim_ctx* ctx, int32_t* src_block, int32_t* labe
     const int32_t n = ctx->n;
     const int64_t m = ctx->m;
     if (n == 0 || m == 0) return BISIM_OK;
-    const bool backward = ctx->opt.direction == BISIM_DIR_BACKWARD;
+    const bool by_radix = ctx->opt.direction == BISIM_DIR_BACKWARD || fewer_edges_than_passes_over_blocks(n, m);
     char* base = nullptr;
     const int32_t *os = nullptr, *ol = nullptr, *ot = nullptr;
     const unsigned long long* seg = nullptr;
     const int64_t *off = nullptr, *at = nullptr;
     int64_t count = 0;
-    st = backward ? summary_by_radix(ctx, s, &base, &os, &ol, &ot, &count)
+    st = by_radix ? summary_by_radix(ctx, s, &base, &os, &ol, &ot, &count)
                   : summary_by_segment(ctx, s, &base, &seg, &off, &at, &count);
     if (st != BISIM_OK) return st;
     const int64_t take = std::min(capacity, count);
     char* stage = nullptr;
-    if (!backward && take > 0) {
+    if (!by_radix && take > 0) {
         // straight into the caller's arrays where a kernel may write them
         int32_t* o[3] = {src_block, label, dst_block};
         const bool direct = device_accessible(src_block) && device_accessible(label) && device_accessible(dst_block);

@@ -180,3 +180,29 @@ def test_big_segments_whose_triples_exceed_a_word(B):
     want = np.unique(np.stack([src, lab, dst], 1).astype(np.int64), axis=0).T
     assert np.array_equal(got, want)
     B.summarize_destroy(ctx)
+
+
+@pytest.mark.parametrize("direction", [0, 2])
+@pytest.mark.parametrize("m", [68_000, 72_000])
+def test_few_edges_between_many_vertices(B, m, direction):
+    """On both sides of the line below which the triples are sorted, not the blocks' segments (0.7 edges for every
+    vertex above 1.25 million); forward-backward contexts hold every edge twice."""
+    rng = np.random.default_rng(m)
+    n = 1_350_000
+    m //= 2 if direction == 2 else 1
+    src, dst = (rng.integers(0, n, m).astype(np.int32) for _ in range(2))
+    src[: m // 4] = 5                                       # one long row, and repeated triples
+    lab, vl = rng.integers(-3, 3, m).astype(np.int32), rng.integers(0, 3, n).astype(np.int32)
+    alive = np.ones(n, np.uint8)
+    alive[rng.integers(0, n, 1000)] = 0
+    alive[5] = 1
+    keep = alive[src].astype(bool) & alive[dst].astype(bool)
+    src, dst, lab = src[keep], dst[keep], lab[keep]
+    with B.summarize_init_coo(n, _dev(src), _dev(dst), _dev(lab), _dev(vl), alive=_dev(alive),
+                              options=B.default_options(direction=direction)) as ctx:
+        B.bisim_iterate(ctx, 1)
+        P = B.get_partition(ctx).cpu().numpy()
+        if direction == 0:
+            want, _, _ = oracle.refine(n, src, dst, lab, vl, 1, 0, alive=alive)
+            assert np.array_equal(P, want)
+        assert _gpu_summary(B, ctx) == oracle.summary_edges(src, dst, lab, P)
