@@ -4,16 +4,19 @@
 // What it replaces is a loop of about a dozen kernels a round. Each of those is
 // near empty once the list is short (a late round of a power-law graph) or the
 // graph is small, and a round then costs its launches: 77 us on 300k vertices in
-// paths, 60 us on 10k vertices. Here a round is two or three phases with a grid
-// barrier after each, one CTA per SM (on small graphs one cluster, or one CTA):
+// paths, 60 us on 10k vertices. Here a round is two phases with a grid barrier after
+// each, one CTA per SM (on small graphs one cluster, or one CTA):
 //   A  the entries of the list that are not alone in their block compute their
-//      signatures
-//   B  every entry is confirmed by an exact comparison, inside the thread for
-//      rows of at most eight edges, in the warp for longer ones: in a round that
-//      splits most blocks against the smallest vertex of its slot of the
-//      signature table (which phase A filled), else against the smallest vertex
-//      of its present block; those that differ from it enter the table
-//   C  (only then, and only them) and are confirmed against their slots
+//      signatures and enter them into the table
+//   B  every entry is confirmed against the smallest vertex of its slot by an exact
+//      comparison, inside the thread for rows of at most eight edges, in the warp
+//      for longer ones
+// (Rounds that split few blocks compared every entry with its present block's smallest
+// vertex first, and only those that differed entered the table, in a third phase: it
+// was slower. us to the fixpoint with and without: 600 rounds on 300k vertices in paths
+// 14,900 / 13,700, 100 rounds on 1M 6,230 / 5,030 and on 100k 1,940 / 1,990; paths with
+// one extra edge per 100 vertices, 300k and 1M, 530 / 257 and 827 / 473; two edges a
+// vertex with two labels, 200k, 445 / 174.)
 //
 // The list is cut among the CTAs at the start and each keeps its part to the end
 // (dealt in units of up to 32 entries, rotated from row to row so that no period
@@ -52,11 +55,9 @@ constexpr int kUnits = 4;                 // work units a warp takes between two
 constexpr int kStage = kUnits * 32;
 constexpr uint8_t kCold = 255;
 
-// Values of an entry's `own` flag. 1 with joined = 0: alone in its block.
+// Values of an entry's `own` flag.
 constexpr uint8_t kMember = 0;            // not its block's smallest vertex
 constexpr uint8_t kOwner = 1;             // the smallest vertex; joined says whether others are in the block
-constexpr uint8_t kOwnerLeft = 3;         // ... and some left since: joined may be out of date
-constexpr uint8_t kOwnerAsks = 5;         // ... and this round those that stay set it anew
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -103,7 +104,6 @@ struct LoopView {
     uint64_t nslots;
     uint32_t epoch;                       // the table's last epoch (kEpochCycle: blank it first)
     int32_t* unresolved;
-    int32_t* split;                       // entries that left their block's smallest vertex this round
     DevState* st;
     LoopCtl* ctl;
     LoopState* L;
@@ -129,7 +129,6 @@ struct Shared {
     unsigned zero[kLoopWarps];
     int32_t seen[kSeenSlots];                 // positions whose joined flag this CTA has set this round
     unsigned next_cnt[kLoopGroups];           // entries of the next list so far
-    unsigned split;                           // entries of the split list so far
     unsigned owned;                           // entries that are their block's id
     unsigned error;                           // kErr* bits
     unsigned flags;                           // barrier result: kAny* of all CTAs
@@ -161,7 +160,7 @@ __device__ __forceinline__ void distinct_of_warp(uint64_t val, bool has, uint64_
 
 // ----------------------------------------------------------------------------- barrier
 
-constexpr unsigned kAnySplit = 1u, kAnyUnresolved = 2u, kAnyError = 4u;
+constexpr unsigned kAnyUnresolved = 1u, kAnyError = 2u;
 
 __device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
     unsigned v;
@@ -269,8 +268,10 @@ __device__ __forceinline__ int32_t list_at(const List& l, int g, unsigned j) {
     return l.buf ? l.buf[at] : static_cast<int32_t>(at);
 }
 
-// Entry i of the CTA's groups in turn: its place among all entries.
-__device__ __forceinline__ int64_t place_of(const List& l, unsigned i, int* group, unsigned* j) {
+__device__ __forceinline__ unsigned list_size(const List& l) { return l.cnt[0] + l.cnt[1] + l.cnt[2] + l.cnt[3]; }
+
+// Entry i of the CTA's groups in turn.
+__device__ __forceinline__ int32_t entry_of(const List& l, unsigned i) {
     int g = 0;
 #pragma unroll
     for (int q = 0; q < kLoopGroups - 1; ++q) {
@@ -279,19 +280,7 @@ __device__ __forceinline__ int64_t place_of(const List& l, unsigned i, int* grou
             g = q + 1;
         }
     }
-    *group = g;
-    *j = i;
-    return dealt(l, g, i);
-}
-
-__device__ __forceinline__ unsigned list_size(const List& l) { return l.cnt[0] + l.cnt[1] + l.cnt[2] + l.cnt[3]; }
-
-__device__ __forceinline__ int32_t entry_of(const List& l, unsigned i) {
-    int g;
-    unsigned j;
-    const int64_t place = place_of(l, i, &g, &j);
-    const int64_t at = l.base[g] + place;
-    return l.buf ? l.buf[at] : static_cast<int32_t>(at);
+    return list_at(l, g, i);
 }
 
 // ----------------------------------------------------------------------------- table
@@ -354,10 +343,10 @@ __device__ __forceinline__ void put_sig(const LoopView& V, int64_t pos, uint64_t
 
 // ----------------------------------------------------------------------------- phase A
 
-// What a round is: its first of the launch (every entry stays, the list is
-// kept as it is), and whether every entry enters the table.
+// What a round is: `first` of the launch, when every entry stays and the list is
+// kept as it is.
 struct Round {
-    bool first, insert;
+    bool first;
     const int32_t* Pin;
     int32_t* Pout;
     int32_t* next;                        // buffer of the next list
@@ -365,19 +354,8 @@ struct Round {
 };
 
 // Does the entry stay on the list? Not when its vertex is alone in its block.
-// An owner whose block lost members asks those that stay, once.
 __device__ __forceinline__ bool stays_listed(const LoopView& V, const Round& R, int32_t pos) {
-    if (R.first) return true;
-    const uint8_t o = V.own[pos];
-    if (o == kMember) return true;
-    if (o == kOwnerLeft) {
-        V.own[pos] = kOwnerAsks;
-        V.joined[pos] = 0;
-        return true;
-    }
-    if (!V.joined[pos]) return false;
-    if (o == kOwnerAsks) V.own[pos] = kOwner;
-    return true;
+    return R.first || V.own[pos] == kMember || V.joined[pos];
 }
 
 // A unit of up to 32 short rows (group 0): a thread per vertex. The entries that
@@ -430,29 +408,27 @@ __device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, 
         h = hash & R.t.hmask;
     }
     unsigned hot = kCold;
-    if (R.insert) {                                                // the same for the whole grid
-        if (stay) {
-            V.joined[pos] = 0;
-            table_span(V, v, &base, &mask);
-        }
-        unsigned members;
-        const int rep = combine(stay, h, base, v, &members);
-        const bool doer = stay && rep == static_cast<int>(lane_id());
-        if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
-            // popular in the warp: combine over the CTA too, at the flush
-            const unsigned at = static_cast<unsigned>(h ^ (h >> 29)) & (kHotSlots - 1);
-            const unsigned long long prev = atomicCAS(&sh.hot_key[at], 0ull, static_cast<unsigned long long>(h));
-            if (prev == 0ull || prev == h) {
-                atomicMin(&sh.hot_min[at], static_cast<unsigned>(v));
-                hot = at;
-            }
-        }
-        uint32_t sl = ~0u;
-        if (doer && hot == kCold) sl = table_insert_in(R.t, h, v, static_cast<uint64_t>(base), mask, &sh.error);
-        sl = __shfl_sync(0xffffffffu, sl, rep);
-        hot = __shfl_sync(0xffffffffu, hot, rep);
-        if (stay && hot == kCold) V.slot[pos] = sl;
+    if (stay) {
+        V.joined[pos] = 0;
+        table_span(V, v, &base, &mask);
     }
+    unsigned members;
+    const int rep = combine(stay, h, base, v, &members);
+    const bool doer = stay && rep == static_cast<int>(lane_id());
+    if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
+        // popular in the warp: combine over the CTA too, at the flush
+        const unsigned at = static_cast<unsigned>(h ^ (h >> 29)) & (kHotSlots - 1);
+        const unsigned long long prev = atomicCAS(&sh.hot_key[at], 0ull, static_cast<unsigned long long>(h));
+        if (prev == 0ull || prev == h) {
+            atomicMin(&sh.hot_min[at], static_cast<unsigned>(v));
+            hot = at;
+        }
+    }
+    uint32_t sl = ~0u;
+    if (doer && hot == kCold) sl = table_insert_in(R.t, h, v, static_cast<uint64_t>(base), mask, &sh.error);
+    sl = __shfl_sync(0xffffffffu, sl, rep);
+    hot = __shfl_sync(0xffffffffu, hot, rep);
+    if (stay && hot == kCold) V.slot[pos] = sl;
     const unsigned stays = __ballot_sync(0xffffffffu, stay);
     if (stay) {
         const int at = *staged + __popc(stays & ((1u << lane_id()) - 1u));
@@ -562,14 +538,12 @@ __device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, co
         put_sig(V, pos, hash, cnt, own);
         h = hash & R.t.hmask;
     }
-    if (R.insert) {
-        if (stay) {
-            V.joined[pos] = 0;
-            table_span(V, v, &base, &mask);
-        }
-        const uint32_t sl = insert_warp(R.t, stay, h, base, mask, v, &sh.error);
-        if (stay) V.slot[pos] = sl;
+    if (stay) {
+        V.joined[pos] = 0;
+        table_span(V, v, &base, &mask);
     }
+    const uint32_t sl = insert_warp(R.t, stay, h, base, mask, v, &sh.error);
+    if (stay) V.slot[pos] = sl;
     if (!R.first && stays) {
         unsigned at = 0;
         if (lane == 0) at = atomicAdd(&sh.next_cnt[g], static_cast<unsigned>(__popc(stays)));
@@ -636,7 +610,7 @@ __device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared
     }
 }
 
-// ----------------------------------------------------------------------------- phases B and C
+// ----------------------------------------------------------------------------- phase B
 
 // Is every pair value of row [ea, ea + da) among those of row [eb, eb + db)?
 // All lanes of the warp take part; at most 256 entries each.
@@ -755,11 +729,10 @@ __device__ __forceinline__ void add_owned(unsigned owned, Shared& sh) {
     if (lane_id() == 0 && owned) atomicAdd(&sh.owned, owned);
 }
 
-// Confirms the CTA's entries pos_of(i), i < total, against their table slots'
-// smallest vertices. (Two entries a thread at once: no faster.)
-template <class F>
-__device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, unsigned total, const F& pos_of,
-                                             Shared& sh) {
+// Confirms the CTA's entries against their table slots' smallest vertices. (Two
+// entries a thread at once: no faster.)
+__device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, const List& l, Shared& sh) {
+    const unsigned total = list_size(l);
     const unsigned lane = lane_id();
     unsigned owned = 0;
     for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
@@ -767,7 +740,7 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
         bool test = false, push = false;
         int4 a{}, c{};
         if (b + lane < total) {
-            p.pos = pos_of(b + lane);
+            p.pos = entry_of(l, b + lane);
             const uint32_t sv = V.slot[p.pos];
             p.v = __ldg(V.vert + p.pos);
             p.r = sv == ~0u ? -1 : table_rep(V.t.slots, sv);
@@ -792,75 +765,6 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
     add_owned(owned, sh);
 }
 
-// Phase B of a round whose blocks mostly hold: every entry against the smallest
-// vertex b of its present block. b stays in the part of its block that keeps the
-// block's id, whatever happens to the others, so a vertex with b's signature
-// needs neither the table nor a flag; those that leave b enter the table, and b
-// asks next round whether it is alone now (see stays_listed).
-__device__ __forceinline__ void keep_or_split(const LoopView& V, const Round& R, const List& l, Shared& sh) {
-    const unsigned total = list_size(l);
-    const unsigned lane = lane_id();
-    unsigned owned = 0;
-    for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
-        const unsigned i = b + lane;
-        Pair p{-1, -1, -1, -1};
-        bool test = false, leave = false, asks = false;
-        int4 a{}, c{};
-        if (i < total) {
-            p.pos = entry_of(l, i);
-            p.v = __ldg(V.vert + p.pos);
-            a = record(V, p.pos);
-            p.r = a.w;
-            if (p.r == p.v) {
-                R.Pout[p.v] = p.v;
-                ++owned;
-            } else {
-                p.rpos = __ldg(V.vpos + p.r);
-                c = record(V, p.rpos);
-                asks = V.own[p.rpos] == kOwnerAsks;
-                test = a.x == c.x && a.y == c.y && a.z == c.z;
-                leave = !test;
-            }
-        }
-        const bool join = confirm(V, p, test, false, a, c, R);
-        if (join && asks) mark_joined(V, p.rpos, sh);
-        const unsigned leaves = __ballot_sync(0xffffffffu, leave);
-        if (leaves) {
-            unsigned at = 0;
-            if (lane == 0) at = atomicAdd(&sh.split, static_cast<unsigned>(__popc(leaves)));
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(leaves & ((1u << lane) - 1u));
-            if (leave) {
-                int g;
-                unsigned j;
-                const int64_t to = place_of(l, at, &g, &j);
-                V.split[V.gb[g] + to] = p.pos;                     // one place per entry, as on the list
-                if (__ldcg(V.own + p.rpos) != kOwnerLeft) V.own[p.rpos] = kOwnerLeft;
-            }
-        }
-    }
-    add_owned(owned, sh);
-    __syncthreads();
-    // those that leave enter the table, equal signatures of a warp as one
-    const unsigned split = sh.split;
-    for (unsigned b = threadIdx.x - lane; b < split; b += blockDim.x) {
-        const bool on = b + lane < split;
-        int32_t pos = 0, v = 0;
-        uint64_t h = 0, mask = 0;
-        int64_t base = 0;
-        if (on) {
-            int g;
-            unsigned j;
-            const int64_t from = place_of(l, b + lane, &g, &j);
-            pos = V.split[V.gb[g] + from];
-            v = __ldg(V.vert + pos);
-            h = V.sig[pos].hash & R.t.hmask;
-            table_span(V, v, &base, &mask);
-        }
-        const uint32_t sl = insert_warp(R.t, on, h, base, mask, v, &sh.error);
-        if (on) V.slot[pos] = sl;
-    }
-}
-
 // ----------------------------------------------------------------------------- the loop
 
 // The list and the state of a round that ended in a hash collision (or an
@@ -880,10 +784,6 @@ __device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int 
             const int32_t x = V.P[0][v];
             V.P[0][v] = V.P[1][v];
             V.P[1][v] = x;
-        }
-        if (V.own[pos] > kOwner) {                                 // whether it is alone is not known: listed on
-            V.own[pos] = kOwner;
-            V.joined[pos] = 1;
         }
     }
     if (!grid_barrier(V, ++*bar, sh)) return false;
@@ -953,7 +853,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
     int nbuf = V.start ? 0 : 1;                            // the list buffer the next list goes to
     int out = 1;
     bool fine = true;
-    int64_t grown = 0, listed_before = 0;
     Round R;
     R.Pin = V.start ? V.P0 : V.P[0];
     R.t = V.t;
@@ -970,14 +869,9 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
         R.t.epoch = static_cast<uint64_t>(ep) << 32;
         R.Pout = V.P[out];
         R.next = V.act[nbuf];
-        // most listed vertices keep their block's smallest vertex when the last
-        // round made few new blocks: then the table is for those that do not (a
-        // chain graph's second round splits most of its million vertices after a
-        // first that made one new block for every five)
-        R.insert = R.first || grown * 32 >= listed_before;
         for (int i = threadIdx.x; i < kSeenSlots; i += blockDim.x) sh.seen[i] = -1;
         if (threadIdx.x < kLoopGroups) sh.next_cnt[threadIdx.x] = 0u;
-        if (threadIdx.x == 0) sh.split = sh.owned = 0u;
+        if (threadIdx.x == 0) sh.owned = 0u;
         __syncthreads();
         phase_a(V, R, l, sh, sets);
         if (!(fine = grid_barrier(V, ++bar, sh))) break;
@@ -990,30 +884,13 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
             }
             nbuf ^= 1;
         }
-        bool confirmed = R.insert;
-        if (R.insert) verify_slots(V, R, list_size(l), [&](unsigned i) { return entry_of(l, i); }, sh);
-        else keep_or_split(V, R, l, sh);
+        verify_slots(V, R, l, sh);
         __syncthreads();
         // unresolved entries are rare: every CTA looks at the counter
-        for (;;) {
-            const unsigned flags = (sh.split ? kAnySplit : 0u) | (sh.error ? kAnyError : 0u) |
-                                   (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
-            if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
-            if (confirmed || !(sh.flags & kAnySplit)) break;
-            verify_slots(V, R, sh.split, [&](unsigned i) {
-                int g;
-                unsigned j;
-                const int64_t from = place_of(l, i, &g, &j);
-                return V.split[V.gb[g] + from];
-            }, sh);
-            confirmed = true;
-            __syncthreads();
-        }
-        if (!fine) break;
+        const unsigned flags = (sh.error ? kAnyError : 0u) | (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
+        if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
         const unsigned listed = sh.total[0];
         const unsigned long long blocks = static_cast<unsigned long long>(V.n_live - listed) + sh.total[1];
-        grown = static_cast<int64_t>(blocks - S.prev_blocks);
-        listed_before = listed;
         loop_advance(S, blocks, sh.flags & kAnyUnresolved, sh.flags & kAnyError);
         if (S.stop == kStopDone) {
             if (out != 0)                                  // the result belongs in P[0]
@@ -1162,7 +1039,6 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     V.t.hmask = hb >= 64 ? ~0ull : ((1ull << hb) - 1ull);
     V.epoch = regions || ctx->epoch32 == 0 ? kEpochCycle : (ctx->epoch32 - 1) % kEpochCycle + 1;
     V.unresolved = ctx->ulist[0];
-    V.split = ctx->ulist[1];
     V.st = ctx->dstate;
     V.L = static_cast<LoopState*>(ctx->dloop);
     V.ctl = reinterpret_cast<LoopCtl*>(static_cast<char*>(ctx->dloop) + ls);
