@@ -1410,46 +1410,9 @@ __global__ void __launch_bounds__(kThreads) k_dense_compare_warp(const int2* __r
                 }
             }
         }
-        // the others four at a time, eight lanes a pair
-        unsigned todo = __ballot_sync(0xffffffffu, in && !small);
-        while (todo) {
-            unsigned mine = todo;                                    // from the (lane / 8)-th pair that is left on
-            for (unsigned k = 0; k < lane / 8; ++k) mine &= mine - 1u;
-            const int q = mine ? __ffs(mine) - 1 : 0;
-            const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
-            const int gdv = __shfl_sync(0xffffffffu, dv, q), gdr = __shfl_sync(0xffffffffu, dr, q);
-            const int qdv = mine ? gdv : 0, qdr = mine ? gdr : 0;
-            const int sub = static_cast<int>(lane & 7u);
-            uint64_t va[4], vb[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                va[j] = sub + 8 * j < qdv ? D.pe[qev + sub + 8 * j] : 0ull;
-                vb[j] = sub + 8 * j < qdr ? D.pe[qer + sub + 8 * j] : 0ull;
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (sub + 8 * j < qdv) va[j] = packed_pair_value(va[j], D.P);
-                if (sub + 8 * j < qdr) vb[j] = packed_pair_value(vb[j], D.P);
-            }
-            unsigned found = 0u;                                     // which of the lane's four are among r's
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (__all_sync(0xffffffffu, qdr <= 8 * i)) break;
-                for (int k = 0; k < 8; ++k) {
-                    const uint64_t bk = __shfl_sync(0xffffffffu, vb[i], k, 8);   // every lane takes part
-                    const bool is = 8 * i + k < qdr;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (is && va[j] == bk) found |= 1u << j;
-                }
-            }
-            bool miss = false;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) miss = miss || (sub + 8 * j < qdv && !((found >> j) & 1u));
-            const unsigned missed = __ballot_sync(0xffffffffu, miss);
-            for (int g = 0; g < 4 && todo; ++g, todo &= todo - 1u)   // the same for the whole warp
-                if (static_cast<int>(lane) == __ffs(todo) - 1) same = ((missed >> (8 * g)) & 0xffu) == 0u;
-        }
+        const bool inside = rows_inside(in && !small, ev, dv, er, dr, D.pe,
+                                        [&](unsigned long long w) { return packed_pair_value(w, D.P); });
+        if (!small) same = inside;
         const unsigned words = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(dv + dr));
         if (lane == 0) atomicAdd(&st->aux, static_cast<unsigned long long>(words));
         if (in && same) {

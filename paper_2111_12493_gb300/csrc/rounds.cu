@@ -9,8 +9,8 @@
 //   A  the entries of the list that are not alone in their block compute their
 //      signatures and enter them into the table
 //   B  every entry is confirmed against the smallest vertex of its slot by an exact
-//      comparison, inside the thread for rows of at most eight edges, in the warp
-//      for longer ones
+//      comparison, inside the thread for rows of at most eight edges; the pairs
+//      with longer rows are shared out to the CTA's warps afterwards
 // (Rounds that split few blocks compared every entry with its present block's smallest
 // vertex first, and only those that differed entered the table, in a third phase: it
 // was slower. us to the fixpoint with and without: 600 rounds on 300k vertices in paths
@@ -104,6 +104,7 @@ struct LoopView {
     uint64_t nslots;
     uint32_t epoch;                       // the table's last epoch (kEpochCycle: blank it first)
     int32_t* unresolved;
+    int32_t* wide;                        // entries that confirm_wide compares, at their CTA's places
     DevState* st;
     LoopCtl* ctl;
     LoopState* L;
@@ -130,6 +131,7 @@ struct Shared {
     int32_t seen[kSeenSlots];                 // positions whose joined flag this CTA has set this round
     unsigned next_cnt[kLoopGroups];           // entries of the next list so far
     unsigned owned;                           // entries that are their block's id
+    unsigned wide;                            // entries on the wide list
     unsigned error;                           // kErr* bits
     unsigned flags;                           // barrier result: kAny* of all CTAs
     unsigned total[2];                        // barrier result: listed, owned
@@ -270,17 +272,28 @@ __device__ __forceinline__ int32_t list_at(const List& l, int g, unsigned j) {
 
 __device__ __forceinline__ unsigned list_size(const List& l) { return l.cnt[0] + l.cnt[1] + l.cnt[2] + l.cnt[3]; }
 
-// Entry i of the CTA's groups in turn.
-__device__ __forceinline__ int32_t entry_of(const List& l, unsigned i) {
+// Entry i of the CTA's groups in turn: its group, and i becomes its number in it.
+__device__ __forceinline__ int group_of(const List& l, unsigned* i) {
     int g = 0;
 #pragma unroll
     for (int q = 0; q < kLoopGroups - 1; ++q) {
-        if (g == q && i >= l.cnt[q]) {
-            i -= l.cnt[q];
+        if (g == q && *i >= l.cnt[q]) {
+            *i -= l.cnt[q];
             g = q + 1;
         }
     }
+    return g;
+}
+
+__device__ __forceinline__ int32_t entry_of(const List& l, unsigned i) {
+    const int g = group_of(l, &i);
     return list_at(l, g, i);
+}
+
+// A place among all positions that is this CTA's alone, one for each of its entries.
+__device__ __forceinline__ int64_t place_of(const LoopView& V, const List& l, unsigned i) {
+    const int g = group_of(l, &i);
+    return V.gb[g] + dealt(l, g, i);
 }
 
 // ----------------------------------------------------------------------------- table
@@ -612,28 +625,6 @@ __device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared
 
 // ----------------------------------------------------------------------------- phase B
 
-// Is every pair value of row [ea, ea + da) among those of row [eb, eb + db)?
-// All lanes of the warp take part; at most 256 entries each.
-__device__ bool row_inside(const LoopView& V, const int32_t* P, int64_t ea, int da, int64_t eb, int db) {
-    const int lane = static_cast<int>(lane_id());
-    bool miss = false;
-    for (int a0 = 0; a0 < da && !miss; a0 += 32) {
-        const bool ha = a0 + lane < da;
-        const uint64_t a = ha ? word_value(__ldg(V.pe + ea + a0 + lane), P) : 0ull;
-        bool found = !ha;
-        for (int b0 = 0; b0 < db; b0 += 32) {
-            const uint64_t b = b0 + lane < db ? word_value(__ldg(V.pe + eb + b0 + lane), P) : 0ull;
-            const int lim = min(32, db - b0);
-            for (int k = 0; k < lim; ++k) {
-                const uint64_t bk = __shfl_sync(0xffffffffu, b, k);    // every lane takes part in every shuffle
-                found = found || bk == a;
-            }
-        }
-        miss = __any_sync(0xffffffffu, !found);
-    }
-    return !miss;
-}
-
 // One entry and the representative it is to be confirmed against.
 struct Pair {
     int32_t pos, v, r, rpos;              // rpos < 0: nothing to confirm
@@ -655,12 +646,27 @@ __device__ __forceinline__ void mark_joined(const LoopView& V, int32_t rpos, Sha
     V.joined[rpos] = 1;
 }
 
+// The entry joins the representative's block, or (with `push`) goes on the
+// unresolved list. For the whole warp.
+__device__ __forceinline__ void settle(const LoopView& V, const Round& R, const Pair& p, bool join, bool push, Shared& sh) {
+    if (join) {
+        R.Pout[p.v] = p.r;
+        mark_joined(V, p.rpos, sh);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, push);
+    if (m) {
+        unsigned at = 0;
+        if (lane_id() == 0) at = atomicAdd(&V.ctl->copy[V.copy].unresolved, static_cast<unsigned>(__popc(m)));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (push) V.unresolved[at + __popc(m & ((1u << lane_id()) - 1u))] = p.pos;
+    }
+}
+
 // Confirms the lanes' pairs exactly: with `test`, the records a and c have
-// equal own blocks and sizes. Returns whether the entry joins the
-// representative's block; the others (and those with `push`) go on the unresolved list.
+// equal own blocks and sizes. Returns whether a row is too long for that
+// (confirm_wide decides then).
 __device__ __forceinline__ bool confirm(const LoopView& V, const Pair& p, bool test, bool push, const int4& a,
-                                        const int4& c, const Round& R) {
-    const unsigned lane = lane_id();
+                                        const int4& c, const Round& R, Shared& sh) {
     bool join = false, wide = false;
     int64_t ev = 0, er = 0;
     int dv = 0, dr = 0;
@@ -702,25 +708,8 @@ __device__ __forceinline__ bool confirm(const LoopView& V, const Pair& p, bool t
             wide = true;
         }
     }
-    for (unsigned todo = __ballot_sync(0xffffffffu, wide); todo; todo &= todo - 1u) {
-        const int q = __ffs(todo) - 1;
-        const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
-        const int qdv = __shfl_sync(0xffffffffu, dv, q), qdr = __shfl_sync(0xffffffffu, dr, q);
-        const bool same = row_inside(V, R.Pin, qev, qdv, qer, qdr);
-        if (static_cast<int>(lane) == q) {
-            join = same;
-            push = !same;
-        }
-    }
-    if (join) R.Pout[p.v] = p.r;
-    const unsigned m = __ballot_sync(0xffffffffu, push);
-    if (m) {
-        unsigned at = 0;
-        if (lane == 0) at = atomicAdd(&V.ctl->copy[V.copy].unresolved, static_cast<unsigned>(__popc(m)));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (push) V.unresolved[at + __popc(m & ((1u << lane) - 1u))] = p.pos;
-    }
-    return join;
+    settle(V, R, p, join, push, sh);
+    return wide;
 }
 
 // Adds the threads' counts to the CTA's.
@@ -760,9 +749,81 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
                 push = !test;
             }
         }
-        if (confirm(V, p, test, push, a, c, R)) mark_joined(V, p.rpos, sh);
+        const bool wide = confirm(V, p, test, push, a, c, R, sh);
+        const unsigned m = __ballot_sync(0xffffffffu, wide);
+        if (m) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&sh.wide, static_cast<unsigned>(__popc(m)));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (wide) V.wide[place_of(V, l, at)] = p.pos;
+        }
     }
     add_owned(owned, sh);
+}
+
+// Pairs with a row of more than eight edges, cut evenly among the CTA's warps: rows
+// of up to 32 edges eight lanes a pair, longer ones through a set in shared memory.
+// (Each compared by the warp that met it, against 32 shuffles of the other row at a
+// time, a CTA's few wide pairs were one warp's: 1,000 vertices of 250 edges with equal
+// sets took 678 us a round, 98 in the kernels of the single classes.)
+__device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, Shared& sh, unsigned long long* sets) {
+    const unsigned count = sh.wide, lane = lane_id(), warp = threadIdx.x >> 5, warps = blockDim.x / 32;
+    const unsigned per = max(4u, min(32u, (count + warps - 1) / warps));
+    const auto value = [&](unsigned long long w) { return word_value(w, R.Pin); };
+    for (unsigned b = warp * per; b < count; b += warps * per) {
+        const bool in = lane < per && b + lane < count;
+        Pair p{-1, -1, -1, -1};
+        int64_t ev = 0, er = 0;
+        int dv = 0, dr = 0;
+        if (in) {
+            p.pos = V.wide[place_of(V, l, b + lane)];
+            p.v = __ldg(V.vert + p.pos);
+            p.r = table_rep(V.t.slots, V.slot[p.pos]);
+            p.rpos = __ldg(V.vpos + p.r);
+            ev = __ldg(V.prp + p.pos);
+            dv = static_cast<int>(__ldg(V.prp + p.pos + 1) - ev);
+            er = __ldg(V.prp + p.rpos);
+            dr = static_cast<int>(__ldg(V.prp + p.rpos + 1) - er);
+        }
+        const bool by_eights = in && dv <= 32 && dr <= 32;
+        bool same = rows_inside(by_eights, ev, dv, er, dr, V.pe, value);
+        unsigned long long* tab = sets + warp * kLoopWarpSet;
+        for (unsigned todo = __ballot_sync(0xffffffffu, in && !by_eights); todo; todo &= todo - 1u) {
+            const int q = __ffs(todo) - 1;
+            const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
+            const int qdv = __shfl_sync(0xffffffffu, dv, q), qdr = __shfl_sync(0xffffffffu, dr, q);
+            uint32_t size = 64;
+            while (size < 2u * static_cast<uint32_t>(qdr)) size <<= 1;
+            for (uint32_t j = lane; j < size; j += 32) tab[j] = 0ull;
+            if (lane == 0) sh.zero[warp] = 0u;
+            __syncwarp();
+            bool miss = false;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {                 // r's row into the set, then v's against it
+                const int64_t e = pass ? qev : qer;
+                const int d = pass ? qdv : qdr;
+                uint64_t x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int j = k * 32 + static_cast<int>(lane);
+                    x[k] = j < d ? __ldg(V.pe + e + j) : 0ull;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (k * 32 + static_cast<int>(lane) < d) x[k] = value(x[k]);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (k * 32 + static_cast<int>(lane) >= d) break;
+                    if (pass == 0) smem_set_insert(tab, size - 1, &sh.zero[warp], x[k]);
+                    else miss = miss || !smem_set_contains(tab, size - 1, sh.zero[warp], x[k]);
+                }
+                __syncwarp();
+            }
+            miss = __any_sync(0xffffffffu, miss);
+            if (static_cast<int>(lane) == q) same = !miss;
+        }
+        settle(V, R, p, in && same, in && !same, sh);
+    }
 }
 
 // ----------------------------------------------------------------------------- the loop
@@ -871,7 +932,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
         R.next = V.act[nbuf];
         for (int i = threadIdx.x; i < kSeenSlots; i += blockDim.x) sh.seen[i] = -1;
         if (threadIdx.x < kLoopGroups) sh.next_cnt[threadIdx.x] = 0u;
-        if (threadIdx.x == 0) sh.owned = 0u;
+        if (threadIdx.x == 0) sh.owned = sh.wide = 0u;
         __syncthreads();
         phase_a(V, R, l, sh, sets);
         if (!(fine = grid_barrier(V, ++bar, sh))) break;
@@ -886,6 +947,10 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
         }
         verify_slots(V, R, l, sh);
         __syncthreads();
+        if (sh.wide) {
+            confirm_wide(V, R, l, sh, sets);
+            __syncthreads();
+        }
         // unresolved entries are rare: every CTA looks at the counter
         const unsigned flags = (sh.error ? kAnyError : 0u) | (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
         if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
@@ -1039,6 +1104,7 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     V.t.hmask = hb >= 64 ? ~0ull : ((1ull << hb) - 1ull);
     V.epoch = regions || ctx->epoch32 == 0 ? kEpochCycle : (ctx->epoch32 - 1) % kEpochCycle + 1;
     V.unresolved = ctx->ulist[0];
+    V.wide = ctx->ulist[1];
     V.st = ctx->dstate;
     V.L = static_cast<LoopState*>(ctx->dloop);
     V.ctl = reinterpret_cast<LoopCtl*>(static_cast<char*>(ctx->dloop) + ls);

@@ -48,6 +48,57 @@ __host__ __device__ inline void loop_advance(LoopState& L, unsigned long long bl
     L.blocks = blocks;
 }
 
+// For the lanes with `on`: is every pair value of the row [ev, ev + dv) of the packed
+// rows among those of [er, er + dr)? Rows of at most 32 edges; the whole warp takes
+// part. Four pairs at a time, eight lanes a pair, four values of each row a lane.
+// `value`: the pair value of a packed word.
+template <class Value>
+__device__ __forceinline__ bool rows_inside(bool on, int64_t ev, int dv, int64_t er, int dr,
+                                            const unsigned long long* __restrict__ pe, const Value& value) {
+    const unsigned lane = threadIdx.x & 31u;
+    const int sub = static_cast<int>(lane & 7u);
+    bool inside = false;
+    unsigned todo = __ballot_sync(0xffffffffu, on);
+    while (todo) {
+        unsigned mine = todo;                                        // from the (lane / 8)-th pair that is left on
+        for (unsigned k = 0; k < lane / 8; ++k) mine &= mine - 1u;
+        const int q = mine ? __ffs(mine) - 1 : 0;
+        const int64_t qev = __shfl_sync(0xffffffffu, ev, q), qer = __shfl_sync(0xffffffffu, er, q);
+        const int gdv = __shfl_sync(0xffffffffu, dv, q), gdr = __shfl_sync(0xffffffffu, dr, q);
+        const int qdv = mine ? gdv : 0, qdr = mine ? gdr : 0;
+        uint64_t va[4], vb[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            va[j] = sub + 8 * j < qdv ? pe[qev + sub + 8 * j] : 0ull;
+            vb[j] = sub + 8 * j < qdr ? pe[qer + sub + 8 * j] : 0ull;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (sub + 8 * j < qdv) va[j] = value(va[j]);
+            if (sub + 8 * j < qdr) vb[j] = value(vb[j]);
+        }
+        unsigned found = 0u;                                         // which of the lane's four are among r's
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (__all_sync(0xffffffffu, qdr <= 8 * i)) break;
+            for (int k = 0; k < 8; ++k) {
+                const uint64_t b = __shfl_sync(0xffffffffu, vb[i], k, 8);   // every lane takes part
+                const bool is = 8 * i + k < qdr;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (is && va[j] == b) found |= 1u << j;
+            }
+        }
+        bool miss = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) miss = miss || (sub + 8 * j < qdv && !((found >> j) & 1u));
+        const unsigned missed = __ballot_sync(0xffffffffu, miss);
+        for (int g = 0; g < 4 && todo; ++g, todo &= todo - 1u)       // the same for the whole warp
+            if (static_cast<int>(lane) == __ffs(todo) - 1) inside = ((missed >> (8 * g)) & 0xffu) == 0u;
+    }
+    return inside;
+}
+
 // Whether runs of rounds may go through the cooperative kernel at all.
 bool round_loop_usable(const bisim_ctx* ctx);
 // Whether it covers the whole graph (no live vertex above 256 edges).

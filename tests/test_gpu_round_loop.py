@@ -187,3 +187,38 @@ def test_one_round_of_every_class(B, hub, bits):
         B.bisim_iterate(ctx, 3)
         want, _, _ = oracle.refine(g["n"], g["src"], g["dst"], g["elabel"], g["vlabel"], 3, 0)
         assert np.array_equal(B.get_partition(ctx).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("bits", [2, 64])
+@pytest.mark.parametrize("n,degree", [(40, 12), (1000, 33), (1000, 250), (30_000, 30), (9000, 90)])
+def test_wide_pairs_are_shared_out(B, n, degree, bits):
+    """Long rows of few values (two labels, two blocks): every entry is a pair with a wide row. Few of them to a CTA
+    and several to a warp, equal and (with two bits of hash) unequal."""
+    rng = np.random.default_rng(degree)
+    g = dict(n=n, src=np.repeat(np.arange(n), degree).astype(np.int32),
+             dst=rng.integers(0, n, n * degree).astype(np.int32),
+             elabel=rng.integers(0, 2, n * degree).astype(np.int32), vlabel=rng.integers(0, 2, n).astype(np.int32))
+    rare = rng.integers(0, n, n // 10)                      # rows that miss a pair
+    g["elabel"][(rare[:, None] * degree + np.arange(degree)).ravel()] = 0
+    check(B, g, [1, 2, oracle.FIXPOINT], options=B.default_options(hash_bits=bits))
+
+
+def test_wide_pairs_do_not_wait_for_one_warp(B):
+    """1,000 rows of 250 edges, all pairs (two labels) against none (many labels): 14 times the time when the warp
+    that met a CTA's pairs compared them all."""
+    import time
+
+    import torch
+    rng = np.random.default_rng(1)
+    n, d = 1000, 250
+    took = []
+    for labels, blocks in ((2, 2), (1000, 200)):
+        a = [np.repeat(np.arange(n), d), rng.integers(0, n, n * d), rng.integers(0, labels, n * d), rng.integers(0, blocks, n)]
+        with B.summarize_init_coo(n, *(torch.from_numpy(x.astype(np.int32)).cuda() for x in a)) as ctx:
+            best = 1.0
+            for _ in range(30):
+                t = time.perf_counter()
+                B.bisim_iterate(ctx, 1)
+                best = min(best, time.perf_counter() - t)
+        took.append(best)
+    assert took[0] < 4 * took[1], took
