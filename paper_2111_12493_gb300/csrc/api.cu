@@ -555,15 +555,23 @@ bisim_status dense_rounds_run(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
     return BISIM_OK;
 }
 
-// The cooperative loop takes the first round too when it covers every row and
-// the graph has at most this many vertices. Above it the first round's list is
-// long enough for the kernels of the single classes, which keep twice the warps
-// resident. us to the fixpoint with the loop from P_0 against the kernels of one
-// round first: power-law rows of at most 256 edges, 1M vertices 329 / 384, 2M
-// 524 / 544, 4M 995 / 953, 8M 1962 / 1713; uniform graphs of five edges a vertex
-// 295 / 369, 517 / 566, 974 / 1003, 2073 / 1969; chains with two extra edges
-// 324 / 416, 536 / 671, 977 / 1165, 2019 / 2326.
-constexpr int64_t kLoopStartMax = int64_t{1} << 22;
+// The cooperative loop takes the first round too when it covers every row, the graph
+// has at most kLoopStartMax vertices, and of rows above eight edges at most
+// kLoopStartRows, with at most kLoopStartEdges. Above that the first round is long
+// enough for the kernels of the single classes, which keep twice the warps resident
+// and take a row of 9 to 32 edges by a thread, the loop by a warp. us to the fixpoint
+// with the loop from P_0 / with the kernels of one round first:
+//   rows of two edges     1M 169 / 205, 2M 306 / 312, 4M 626 / 528, 8M 1,351 / 1,046
+//   uniform, mean five    1M 275 / 338, 2M 494 / 530, 4M 961 / 965, 8M 2,056 / 1,942
+//   chains, two extra     1M 293 / 391, 2M 517 / 639, 4M 958 / 1,186, 8M 1,895 / 2,208
+//   rows of ten edges     200k 116 / 137, 500k 197 / 177, 1M 318 / 238, 4M 1,110 / 598
+//   rows of 30 edges      100k 120 / 150, 200k 167 / 184, 500k 334 / 295
+//   rows of 100 edges     50k 146 / 158, 100k 226 / 213, 200k 354 / 311
+//   uniform, mean ten     500k 210 / 236, 1M 322 / 310, 2M 576 / 459, 4M 1,105 / 773
+//   power law to 256      500k 182 / 224, 1M 297 / 291, 2M 491 / 447, 4M 872 / 718
+constexpr int64_t kLoopStartMax = int64_t{3} << 20;
+constexpr int64_t kLoopStartRows = 400000;
+constexpr int64_t kLoopStartEdges = 6000000;
 
 bisim_status dense_rounds_all(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream_t s, int32_t* out_rounds,
                               int32_t* out_executed, int64_t* out_blocks, bool allow_graph) {
@@ -572,7 +580,9 @@ bisim_status dense_rounds_all(bisim_ctx* ctx, int32_t k, int32_t cap, cudaStream
     const int32_t limit = k == BISIM_FIXPOINT ? cap : k;
     if ((st = dense_prepare(ctx, s)) != BISIM_OK) return st;
     const bool from_p0 = limit > 0 && round_loop_usable(ctx) && round_loop_covers(ctx) &&
-                         ctx->dbegin[kDClasses] <= kLoopStartMax;
+                         ctx->dbegin[kDClasses] <= kLoopStartMax &&
+                         ctx->dbegin[kDClasses] - ctx->dbegin[kDRows8] <= kLoopStartRows &&
+                         ctx->dedge_begin[kDClasses] - ctx->dedge_begin[kDRows8] <= kLoopStartEdges;
     if (from_p0) {
         if (ctx->opt.mem_budget_bytes > 0 && ctx->device_bytes > ctx->opt.mem_budget_bytes)
             return set_error(ctx, BISIM_ENOMEM, "context exceeds the memory budget");

@@ -28,6 +28,7 @@ constexpr uint8_t kClassDead = 255;
 //   7..9   one warp per vertex, shared-memory set of 2N slots, N = 64, 128, 256
 //   10..14 one CTA per vertex, N = 512 .. 8192
 //   15     hubs: rows cut into chunks over many CTAs, values deduplicated by bucket
+constexpr int kDRows8 = 5;                // first class of more than eight edges
 constexpr int kDWarp0 = 7;
 constexpr int kDMid0 = 10;
 constexpr int kDHub = 15;

@@ -222,3 +222,14 @@ def test_wide_pairs_do_not_wait_for_one_warp(B):
                 best = min(best, time.perf_counter() - t)
         took.append(best)
     assert took[0] < 4 * took[1], took
+
+
+@pytest.mark.parametrize("n", [400_000, 400_001])
+def test_first_round_on_both_sides_of_its_line(B, n):
+    """Up to 400,000 rows above eight edges are the loop's from P_0 on; more have their first round in the kernels of
+    the single classes."""
+    rng = np.random.default_rng(n)
+    d = 9
+    g = dict(n=n, src=np.repeat(np.arange(n), d).astype(np.int32), dst=rng.integers(0, n, n * d).astype(np.int32),
+             elabel=rng.integers(0, 2, n * d).astype(np.int32), vlabel=rng.integers(0, 2, n).astype(np.int32))
+    check(B, g, [1, 2])
