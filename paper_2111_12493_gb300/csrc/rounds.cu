@@ -4,19 +4,17 @@
 // What it replaces is a loop of about a dozen kernels a round. Each of those is
 // near empty once the list is short (a late round of a power-law graph) or the
 // graph is small, and a round then costs its launches: 77 us on 300k vertices in
-// paths, 60 us on 10k vertices. Here a round is two phases with a grid barrier after
-// each, one CTA per SM (on small graphs one cluster, or one CTA):
+// paths, 60 us on 10k vertices. Here a round is two or three phases with a grid
+// barrier after each, one CTA per SM (on small graphs one cluster, or one CTA):
 //   A  the entries of the list that are not alone in their block compute their
-//      signatures and enter them into the table
-//   B  every entry is confirmed against the smallest vertex of its slot by an exact
-//      comparison, inside the thread for rows of at most eight edges; the pairs
-//      with longer rows are shared out to the CTA's warps afterwards
-// (Rounds that split few blocks compared every entry with its present block's smallest
-// vertex first, and only those that differed entered the table, in a third phase: it
-// was slower. us to the fixpoint with and without: 600 rounds on 300k vertices in paths
-// 14,900 / 13,700, 100 rounds on 1M 6,230 / 5,030 and on 100k 1,940 / 1,990; paths with
-// one extra edge per 100 vertices, 300k and 1M, 530 / 257 and 827 / 473; two edges a
-// vertex with two labels, 200k, 445 / 174.)
+//      signatures
+//   B  every entry is confirmed by an exact comparison, inside the thread for rows of
+//      at most eight edges (the pairs with longer rows are shared out to the CTA's
+//      warps afterwards), against the smallest vertex of its slot of the signature
+//      table, which phase A filled; in a round that is likely to keep many small
+//      blocks (see keeps_blocks) against the smallest vertex of its present block,
+//      and those that differ from it enter the table instead
+//   C  (only then, and only them) and are confirmed against their slots
 //
 // The list is cut among the CTAs at the start and each keeps its part to the end
 // (dealt in units of up to 32 entries, rotated from row to row so that no period
@@ -58,6 +56,8 @@ constexpr uint8_t kCold = 255;
 // Values of an entry's `own` flag.
 constexpr uint8_t kMember = 0;            // not its block's smallest vertex
 constexpr uint8_t kOwner = 1;             // the smallest vertex; joined says whether others are in the block
+constexpr uint8_t kOwnerLeft = 3;         // ... and some left since: joined may be out of date
+constexpr uint8_t kOwnerAsks = 5;         // ... and this round those that stay set it anew
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -105,6 +105,7 @@ struct LoopView {
     uint32_t epoch;                       // the table's last epoch (kEpochCycle: blank it first)
     int32_t* unresolved;
     int32_t* wide;                        // entries that confirm_wide compares, at their CTA's places
+    int32_t* split;                       // entries that left their block's smallest vertex this round, the same
     DevState* st;
     LoopCtl* ctl;
     LoopState* L;
@@ -132,6 +133,7 @@ struct Shared {
     unsigned next_cnt[kLoopGroups];           // entries of the next list so far
     unsigned owned;                           // entries that are their block's id
     unsigned wide;                            // entries on the wide list
+    unsigned split;                           // and on the split list
     unsigned error;                           // kErr* bits
     unsigned flags;                           // barrier result: kAny* of all CTAs
     unsigned total[2];                        // barrier result: listed, owned
@@ -162,7 +164,7 @@ __device__ __forceinline__ void distinct_of_warp(uint64_t val, bool has, uint64_
 
 // ----------------------------------------------------------------------------- barrier
 
-constexpr unsigned kAnyUnresolved = 1u, kAnyError = 2u;
+constexpr unsigned kAnySplit = 1u, kAnyUnresolved = 2u, kAnyError = 4u;
 
 __device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
     unsigned v;
@@ -357,9 +359,9 @@ __device__ __forceinline__ void put_sig(const LoopView& V, int64_t pos, uint64_t
 // ----------------------------------------------------------------------------- phase A
 
 // What a round is: `first` of the launch, when every entry stays and the list is
-// kept as it is.
+// kept as it is, and whether every entry enters the table.
 struct Round {
-    bool first;
+    bool first, insert;
     const int32_t* Pin;
     int32_t* Pout;
     int32_t* next;                        // buffer of the next list
@@ -367,13 +369,26 @@ struct Round {
 };
 
 // Does the entry stay on the list? Not when its vertex is alone in its block.
+// An owner whose block lost members asks those that stay, once.
+template <bool KEEPS>
 __device__ __forceinline__ bool stays_listed(const LoopView& V, const Round& R, int32_t pos) {
-    return R.first || V.own[pos] == kMember || V.joined[pos];
+    if (R.first) return true;
+    const uint8_t o = V.own[pos];
+    if (o == kMember) return true;
+    if (KEEPS && o == kOwnerLeft) {
+        V.own[pos] = kOwnerAsks;
+        V.joined[pos] = 0;
+        return true;
+    }
+    if (!V.joined[pos]) return false;
+    if (KEEPS && o == kOwnerAsks) V.own[pos] = kOwner;
+    return true;
 }
 
 // A unit of up to 32 short rows (group 0): a thread per vertex. The entries that
 // stay listed are staged in shared memory; the CTA's flush appends them to its
 // next list.
+template <bool KEEPS>
 __device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, const List& l, unsigned j0, Shared& sh,
                                              int warp, int* staged) {
     const unsigned j = j0 + lane_id();
@@ -387,7 +402,7 @@ __device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, 
         v = __ldg(V.vert + pos);
         e0 = __ldg(V.prp + pos);
         d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
-        stay = stays_listed(V, R, pos);
+        stay = stays_listed<KEEPS>(V, R, pos);
         own = R.Pin[v];
     }
     // the list is grouped by degree, so the warp's longest row is mostly short:
@@ -421,27 +436,29 @@ __device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, 
         h = hash & R.t.hmask;
     }
     unsigned hot = kCold;
-    if (stay) {
-        V.joined[pos] = 0;
-        table_span(V, v, &base, &mask);
-    }
-    unsigned members;
-    const int rep = combine(stay, h, base, v, &members);
-    const bool doer = stay && rep == static_cast<int>(lane_id());
-    if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
-        // popular in the warp: combine over the CTA too, at the flush
-        const unsigned at = static_cast<unsigned>(h ^ (h >> 29)) & (kHotSlots - 1);
-        const unsigned long long prev = atomicCAS(&sh.hot_key[at], 0ull, static_cast<unsigned long long>(h));
-        if (prev == 0ull || prev == h) {
-            atomicMin(&sh.hot_min[at], static_cast<unsigned>(v));
-            hot = at;
+    if (!KEEPS || R.insert) {                                      // the same for the whole grid
+        if (stay) {
+            V.joined[pos] = 0;
+            table_span(V, v, &base, &mask);
         }
+        unsigned members;
+        const int rep = combine(stay, h, base, v, &members);
+        const bool doer = stay && rep == static_cast<int>(lane_id());
+        if (doer && members >= 4u && V.gid == nullptr && h != 0ull) {
+            // popular in the warp: combine over the CTA too, at the flush
+            const unsigned at = static_cast<unsigned>(h ^ (h >> 29)) & (kHotSlots - 1);
+            const unsigned long long prev = atomicCAS(&sh.hot_key[at], 0ull, static_cast<unsigned long long>(h));
+            if (prev == 0ull || prev == h) {
+                atomicMin(&sh.hot_min[at], static_cast<unsigned>(v));
+                hot = at;
+            }
+        }
+        uint32_t sl = ~0u;
+        if (doer && hot == kCold) sl = table_insert_in(R.t, h, v, static_cast<uint64_t>(base), mask, &sh.error);
+        sl = __shfl_sync(0xffffffffu, sl, rep);
+        hot = __shfl_sync(0xffffffffu, hot, rep);
+        if (stay && hot == kCold) V.slot[pos] = sl;
     }
-    uint32_t sl = ~0u;
-    if (doer && hot == kCold) sl = table_insert_in(R.t, h, v, static_cast<uint64_t>(base), mask, &sh.error);
-    sl = __shfl_sync(0xffffffffu, sl, rep);
-    hot = __shfl_sync(0xffffffffu, hot, rep);
-    if (stay && hot == kCold) V.slot[pos] = sl;
     const unsigned stays = __ballot_sync(0xffffffffu, stay);
     if (stay) {
         const int at = *staged + __popc(stays & ((1u << lane_id()) - 1u));
@@ -454,6 +471,7 @@ __device__ __forceinline__ void unit_threads(const LoopView& V, const Round& R, 
 // A unit of up to `per` rows of group g (9 to 256 edges): a warp per row, several
 // rows of at most 32 edges at a time to keep their loads in flight together.
 // Lane q keeps the result of row q, and the lanes finish all of them together.
+template <bool KEEPS>
 __device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, const List& l, int g, unsigned j0,
                                            unsigned per, Shared& sh, int warp, unsigned long long* sets) {
     const unsigned lane = lane_id();
@@ -467,7 +485,7 @@ __device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, co
         v = __ldg(V.vert + pos);
         e0 = __ldg(V.prp + pos);
         d = static_cast<int>(__ldg(V.prp + pos + 1) - e0);
-        stay = stays_listed(V, R, pos);
+        stay = stays_listed<KEEPS>(V, R, pos);
         own = R.Pin[v];
         if (!stay) R.Pout[v] = own;
     }
@@ -551,12 +569,14 @@ __device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, co
         put_sig(V, pos, hash, cnt, own);
         h = hash & R.t.hmask;
     }
-    if (stay) {
-        V.joined[pos] = 0;
-        table_span(V, v, &base, &mask);
+    if (!KEEPS || R.insert) {
+        if (stay) {
+            V.joined[pos] = 0;
+            table_span(V, v, &base, &mask);
+        }
+        const uint32_t sl = insert_warp(R.t, stay, h, base, mask, v, &sh.error);
+        if (stay) V.slot[pos] = sl;
     }
-    const uint32_t sl = insert_warp(R.t, stay, h, base, mask, v, &sh.error);
-    if (stay) V.slot[pos] = sl;
     if (!R.first && stays) {
         unsigned at = 0;
         if (lane == 0) at = atomicAdd(&sh.next_cnt[g], static_cast<unsigned>(__popc(stays)));
@@ -572,6 +592,7 @@ __device__ __forceinline__ void unit_warps(const LoopView& V, const Round& R, co
 // work: 32 short rows, or up to 32 longer ones (fewer when there are not enough
 // to go round). After every kUnits units the CTA enters its hot signatures, one
 // insert each, and appends its staged rows to its next list.
+template <bool KEEPS>
 __device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared& sh, unsigned long long* sets) {
     const int warp = static_cast<int>(threadIdx.x >> 5);
     const unsigned lane = lane_id();
@@ -585,10 +606,10 @@ __device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared
         for (int k = 0; k < kUnits; ++k) {
             const unsigned u = u0 + k * warps + warp;
             if (u >= units) break;                                 // the same for the whole warp
-            if (u >= end1) unit_threads(V, R, l, (u - end1) * 32, sh, warp, &staged);
-            else if (u < end3) unit_warps(V, R, l, 3, u * per3, per3, sh, warp, sets);
-            else if (u < end2) unit_warps(V, R, l, 2, (u - end3) * per2, per2, sh, warp, sets);
-            else unit_warps(V, R, l, 1, (u - end2) * per1, per1, sh, warp, sets);
+            if (u >= end1) unit_threads<KEEPS>(V, R, l, (u - end1) * 32, sh, warp, &staged);
+            else if (u < end3) unit_warps<KEEPS>(V, R, l, 3, u * per3, per3, sh, warp, sets);
+            else if (u < end2) unit_warps<KEEPS>(V, R, l, 2, (u - end3) * per2, per2, sh, warp, sets);
+            else unit_warps<KEEPS>(V, R, l, 1, (u - end2) * per1, per1, sh, warp, sets);
         }
         if (lane == 0) sh.wcnt[warp] = static_cast<unsigned>(staged);
         __syncthreads();
@@ -623,7 +644,7 @@ __device__ void phase_a(const LoopView& V, const Round& R, const List& l, Shared
     }
 }
 
-// ----------------------------------------------------------------------------- phase B
+// ----------------------------------------------------------------------------- phases B and C
 
 // One entry and the representative it is to be confirmed against.
 struct Pair {
@@ -646,12 +667,13 @@ __device__ __forceinline__ void mark_joined(const LoopView& V, int32_t rpos, Sha
     V.joined[rpos] = 1;
 }
 
-// The entry joins the representative's block, or (with `push`) goes on the
-// unresolved list. For the whole warp.
-__device__ __forceinline__ void settle(const LoopView& V, const Round& R, const Pair& p, bool join, bool push, Shared& sh) {
+// The entry joins the representative's block (with `mark` the representative is
+// told), or (with `push`) goes on the unresolved list. For the whole warp.
+__device__ __forceinline__ void settle(const LoopView& V, const Round& R, const Pair& p, bool join, bool mark, bool push,
+                                       Shared& sh) {
     if (join) {
         R.Pout[p.v] = p.r;
-        mark_joined(V, p.rpos, sh);
+        if (mark) mark_joined(V, p.rpos, sh);
     }
     const unsigned m = __ballot_sync(0xffffffffu, push);
     if (m) {
@@ -662,11 +684,11 @@ __device__ __forceinline__ void settle(const LoopView& V, const Round& R, const 
     }
 }
 
-// Confirms the lanes' pairs exactly: with `test`, the records a and c have
-// equal own blocks and sizes. Returns whether a row is too long for that
-// (confirm_wide decides then).
-__device__ __forceinline__ bool confirm(const LoopView& V, const Pair& p, bool test, bool push, const int4& a,
-                                        const int4& c, const Round& R, Shared& sh) {
+// Confirms the lanes' pairs exactly: with `test`, the records a and c have equal own
+// blocks and sizes. Pairs with a row too long for that go on the wide list
+// (confirm_wide).
+__device__ __forceinline__ void confirm(const LoopView& V, const Round& R, const List& l, const Pair& p, bool test,
+                                        bool mark, bool push, const int4& a, const int4& c, Shared& sh) {
     bool join = false, wide = false;
     int64_t ev = 0, er = 0;
     int dv = 0, dr = 0;
@@ -708,8 +730,14 @@ __device__ __forceinline__ bool confirm(const LoopView& V, const Pair& p, bool t
             wide = true;
         }
     }
-    settle(V, R, p, join, push, sh);
-    return wide;
+    settle(V, R, p, join, mark, push, sh);
+    const unsigned m = __ballot_sync(0xffffffffu, wide);
+    if (m) {
+        unsigned at = 0;
+        if (lane_id() == 0) at = atomicAdd(&sh.wide, static_cast<unsigned>(__popc(m)));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane_id()) - 1u));
+        if (wide) V.wide[place_of(V, l, at)] = p.pos;
+    }
 }
 
 // Adds the threads' counts to the CTA's.
@@ -718,10 +746,11 @@ __device__ __forceinline__ void add_owned(unsigned owned, Shared& sh) {
     if (lane_id() == 0 && owned) atomicAdd(&sh.owned, owned);
 }
 
-// Confirms the CTA's entries against their table slots' smallest vertices. (Two
-// entries a thread at once: no faster.)
-__device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, const List& l, Shared& sh) {
-    const unsigned total = list_size(l);
+// Confirms the CTA's entries pos_of(i), i < total, against their table slots'
+// smallest vertices. (Two entries a thread at once: no faster.)
+template <class F>
+__device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, const List& l, unsigned total,
+                                             const F& pos_of, Shared& sh) {
     const unsigned lane = lane_id();
     unsigned owned = 0;
     for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
@@ -729,7 +758,7 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
         bool test = false, push = false;
         int4 a{}, c{};
         if (b + lane < total) {
-            p.pos = entry_of(l, b + lane);
+            p.pos = pos_of(b + lane);
             const uint32_t sv = V.slot[p.pos];
             p.v = __ldg(V.vert + p.pos);
             p.r = sv == ~0u ? -1 : table_rep(V.t.slots, sv);
@@ -749,24 +778,82 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
                 push = !test;
             }
         }
-        const bool wide = confirm(V, p, test, push, a, c, R, sh);
-        const unsigned m = __ballot_sync(0xffffffffu, wide);
-        if (m) {
+        confirm(V, R, l, p, test, true, push, a, c, sh);
+    }
+    add_owned(owned, sh);
+}
+
+// Phase B of a round that is likely to keep its blocks: every entry against the
+// smallest vertex b of its present block. b stays in the part of its block that keeps
+// the block's id, whatever happens to the others, so a vertex with b's signature needs
+// neither the table nor a flag; those that leave b go on the split list, and b asks next
+// round whether it is alone now (see stays_listed).
+__device__ __forceinline__ void keep_or_split(const LoopView& V, const Round& R, const List& l, Shared& sh) {
+    const unsigned total = list_size(l);
+    const unsigned lane = lane_id();
+    unsigned owned = 0;
+    for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
+        Pair p{-1, -1, -1, -1};
+        bool test = false, leave = false, asks = false;
+        int4 a{}, c{};
+        if (b + lane < total) {
+            p.pos = entry_of(l, b + lane);
+            p.v = __ldg(V.vert + p.pos);
+            a = record(V, p.pos);
+            p.r = a.w;
+            if (p.r == p.v) {
+                R.Pout[p.v] = p.v;
+                ++owned;
+            } else {
+                p.rpos = __ldg(V.vpos + p.r);
+                c = record(V, p.rpos);
+                asks = V.own[p.rpos] == kOwnerAsks;
+                test = a.x == c.x && a.y == c.y && a.z == c.z;
+                leave = !test;
+            }
+        }
+        confirm(V, R, l, p, test, asks, false, a, c, sh);
+        const unsigned leaves = __ballot_sync(0xffffffffu, leave);
+        if (leaves) {
             unsigned at = 0;
-            if (lane == 0) at = atomicAdd(&sh.wide, static_cast<unsigned>(__popc(m)));
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-            if (wide) V.wide[place_of(V, l, at)] = p.pos;
+            if (lane == 0) at = atomicAdd(&sh.split, static_cast<unsigned>(__popc(leaves)));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(leaves & ((1u << lane) - 1u));
+            if (leave) {
+                V.split[place_of(V, l, at)] = p.pos;
+                if (__ldcg(V.own + p.rpos) != kOwnerLeft) V.own[p.rpos] = kOwnerLeft;
+            }
         }
     }
     add_owned(owned, sh);
+}
+
+// The entries of the split list enter the table, equal signatures of a warp as one.
+__device__ __forceinline__ void insert_split(const LoopView& V, const Round& R, const List& l, Shared& sh) {
+    const unsigned split = sh.split, lane = lane_id();
+    for (unsigned b = threadIdx.x - lane; b < split; b += blockDim.x) {
+        const bool on = b + lane < split;
+        int32_t pos = 0, v = 0;
+        uint64_t h = 0, mask = 0;
+        int64_t base = 0;
+        if (on) {
+            pos = V.split[place_of(V, l, b + lane)];
+            v = __ldg(V.vert + pos);
+            h = V.sig[pos].hash & R.t.hmask;
+            table_span(V, v, &base, &mask);
+        }
+        const uint32_t sl = insert_warp(R.t, on, h, base, mask, v, &sh.error);
+        if (on) V.slot[pos] = sl;
+    }
 }
 
 // Pairs with a row of more than eight edges, cut evenly among the CTA's warps: rows
 // of up to 32 edges eight lanes a pair, longer ones through a set in shared memory.
 // (Each compared by the warp that met it, against 32 shuffles of the other row at a
 // time, a CTA's few wide pairs were one warp's: 1,000 vertices of 250 edges with equal
-// sets took 678 us a round, 98 in the kernels of the single classes.)
-__device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, Shared& sh, unsigned long long* sets) {
+// sets took 678 us a round, 98 in the kernels of the single classes.) `keep`: against
+// the present block's smallest vertex, as keep_or_split, else the table slot's.
+__device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, bool keep, Shared& sh,
+                             unsigned long long* sets) {
     const unsigned count = sh.wide, lane = lane_id(), warp = threadIdx.x >> 5, warps = blockDim.x / 32;
     const unsigned per = max(4u, min(32u, (count + warps - 1) / warps));
     const auto value = [&](unsigned long long w) { return word_value(w, R.Pin); };
@@ -778,7 +865,7 @@ __device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, S
         if (in) {
             p.pos = V.wide[place_of(V, l, b + lane)];
             p.v = __ldg(V.vert + p.pos);
-            p.r = table_rep(V.t.slots, V.slot[p.pos]);
+            p.r = keep ? record(V, p.pos).w : table_rep(V.t.slots, V.slot[p.pos]);
             p.rpos = __ldg(V.vpos + p.r);
             ev = __ldg(V.prp + p.pos);
             dv = static_cast<int>(__ldg(V.prp + p.pos + 1) - ev);
@@ -822,7 +909,8 @@ __device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, S
             miss = __any_sync(0xffffffffu, miss);
             if (static_cast<int>(lane) == q) same = !miss;
         }
-        settle(V, R, p, in && same, in && !same, sh);
+        const bool mark = !keep || (in && V.own[p.rpos] == kOwnerAsks);
+        settle(V, R, p, in && same, mark, in && !same, sh);
     }
 }
 
@@ -831,6 +919,7 @@ __device__ void confirm_wide(const LoopView& V, const Round& R, const List& l, S
 // The list and the state of a round that ended in a hash collision (or an
 // error) as the host-driven levels expect them: P_i in P[0], P_{i+1} as far as
 // it is known in P[1], the list in act[0] / aoff, the counts in the status word.
+template <bool KEEPS>
 __device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int out, unsigned long long blocks,
                           unsigned listed, unsigned* bar, Shared& sh) {
     LoopCopy* c = &V.ctl->copy[V.copy];
@@ -845,6 +934,10 @@ __device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int 
             const int32_t x = V.P[0][v];
             V.P[0][v] = V.P[1][v];
             V.P[1][v] = x;
+        }
+        if (KEEPS && V.own[pos] > kOwner) {                        // whether it is alone is not known: listed on
+            V.own[pos] = kOwner;
+            V.joined[pos] = 1;
         }
     }
     if (!grid_barrier(V, ++*bar, sh)) return false;
@@ -881,6 +974,25 @@ __device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int 
     return true;
 }
 
+// Whether the next round is likely to keep most blocks, and those small: the last one
+// made few new ones of its listed entries, and its blocks had at most kKeepSize of them
+// on average. Then comparing with them saves an insert at a random slot per entry, and
+// entries cannot leave without new blocks in proportion. Large blocks are entered once
+// per CTA and warp, which costs less than the comparison, and can lose half their entries
+// for one new block. us to the fixpoint with no such round, with the first condition
+// alone, with both: power law 1.4M / 4M 613 / 563 / 565, 1M / 5M 512 / 460 / 467, 4M /
+// 16M 1,220 / 1,145 / 1,147; beside a wide row, paths of 300k vertices with 3,000 more
+// edges 332 / 503 / 334, two edges a vertex with two labels, 200k, 248 / 426 / 250, 600
+// rounds of paths on 300k 13,260 / 15,600 / 13,560.
+constexpr int64_t kKeepSize = 32;
+__device__ __forceinline__ bool keeps_blocks(int64_t grown, int64_t owned, int64_t listed) {
+    return grown * 32 < listed && listed <= owned * kKeepSize;
+}
+
+// KEEPS: with rounds that keep_or_split begins. For loops after a round of the single
+// classes; those from P_0 on gain nothing by them (uniform graphs and chains 0 to 3%),
+// and the rest of the kernel is 2% to 3% slower with them in it.
+template <bool KEEPS>
 __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V) {
     extern __shared__ unsigned long long sets[];           // a set per warp, when warp-class rows exist
     __shared__ Shared sh;
@@ -913,7 +1025,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
     unsigned bar = 0;
     int nbuf = V.start ? 0 : 1;                            // the list buffer the next list goes to
     int out = 1;
-    bool fine = true;
+    bool fine = true, keep = false;
     Round R;
     R.Pin = V.start ? V.P0 : V.P[0];
     R.t = V.t;
@@ -930,11 +1042,12 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
         R.t.epoch = static_cast<uint64_t>(ep) << 32;
         R.Pout = V.P[out];
         R.next = V.act[nbuf];
+        R.insert = !KEEPS || !keep;
         for (int i = threadIdx.x; i < kSeenSlots; i += blockDim.x) sh.seen[i] = -1;
         if (threadIdx.x < kLoopGroups) sh.next_cnt[threadIdx.x] = 0u;
-        if (threadIdx.x == 0) sh.owned = sh.wide = 0u;
+        if (threadIdx.x == 0) sh.owned = sh.wide = sh.split = 0u;
         __syncthreads();
-        phase_a(V, R, l, sh, sets);
+        phase_a<KEEPS>(V, R, l, sh, sets);
         if (!(fine = grid_barrier(V, ++bar, sh))) break;
         if (!R.first) {
             l.buf = R.next;
@@ -945,17 +1058,27 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
             }
             nbuf ^= 1;
         }
-        verify_slots(V, R, l, sh);
+        if (KEEPS && keep) keep_or_split(V, R, l, sh);
+        else verify_slots(V, R, l, list_size(l), [&](unsigned i) { return entry_of(l, i); }, sh);
         __syncthreads();
-        if (sh.wide) {
-            confirm_wide(V, R, l, sh, sets);
+        for (bool against_block = KEEPS && keep;; against_block = false) {
+            if (sh.wide) confirm_wide(V, R, l, KEEPS && against_block, sh, sets);
+            if (KEEPS && against_block && sh.split) insert_split(V, R, l, sh);
+            __syncthreads();
+            // unresolved entries are rare: every CTA looks at the counter
+            const unsigned flags = (sh.split ? kAnySplit : 0u) | (sh.error ? kAnyError : 0u) |
+                                   (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
+            if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
+            if (!KEEPS || !against_block || !(sh.flags & kAnySplit)) break;
+            if (threadIdx.x == 0) sh.wide = 0u;
+            __syncthreads();
+            verify_slots(V, R, l, sh.split, [&](unsigned i) { return V.split[place_of(V, l, i)]; }, sh);
             __syncthreads();
         }
-        // unresolved entries are rare: every CTA looks at the counter
-        const unsigned flags = (sh.error ? kAnyError : 0u) | (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
-        if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
+        if (!fine) break;
         const unsigned listed = sh.total[0];
         const unsigned long long blocks = static_cast<unsigned long long>(V.n_live - listed) + sh.total[1];
+        keep = keeps_blocks(static_cast<int64_t>(blocks - S.prev_blocks), sh.total[1], listed);
         loop_advance(S, blocks, sh.flags & kAnyUnresolved, sh.flags & kAnyError);
         if (S.stop == kStopDone) {
             if (out != 0)                                  // the result belongs in P[0]
@@ -964,7 +1087,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
                     V.P[0][v] = V.P[1][v];
                 }
         } else if (S.stop != kStopNo) {
-            if (!(fine = hand_back(V, l, R, out, blocks, listed, &bar, sh))) break;
+            if (!(fine = hand_back<KEEPS>(V, l, R, out, blocks, listed, &bar, sh))) break;
         }
         R.Pin = R.Pout;
         out ^= 1;
@@ -1025,6 +1148,7 @@ cudaLaunchAttribute cluster_attribute(unsigned size) {
 }
 
 // The largest cluster of full SMs the device takes (16 where a GPC has them, else 8).
+template <bool KEEPS>
 int largest_cluster(int device, size_t smem) {
     static std::mutex mu;
     static int known[64][2] = {};
@@ -1032,16 +1156,16 @@ int largest_cluster(int device, size_t smem) {
     std::lock_guard<std::mutex> lk(mu);
     int& k = known[device][smem ? 1 : 0];
     if (k == 0) {
-        cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_round_loop<KEEPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(sizeof(unsigned long long) * kLoopWarps * kLoopWarpSet));
-        cudaFuncSetAttribute(k_round_loop, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(k_round_loop<KEEPS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         for (k = 16; k > 1; k >>= 1) {
             cudaLaunchConfig_t cfg = cluster_config(static_cast<unsigned>(k), kLoopThreads, smem);
             cudaLaunchAttribute attr = cluster_attribute(static_cast<unsigned>(k));
             cfg.attrs = &attr;
             cfg.numAttrs = 1;
             int fit = 0;
-            if (cudaOccupancyMaxActiveClusters(&fit, k_round_loop, &cfg) == cudaSuccess && fit > 0) break;
+            if (cudaOccupancyMaxActiveClusters(&fit, k_round_loop<KEEPS>, &cfg) == cudaSuccess && fit > 0) break;
             cudaGetLastError();
         }
     }
@@ -1105,6 +1229,7 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     V.epoch = regions || ctx->epoch32 == 0 ? kEpochCycle : (ctx->epoch32 - 1) % kEpochCycle + 1;
     V.unresolved = ctx->ulist[0];
     V.wide = ctx->ulist[1];
+    V.split = ctx->dlist;
     V.st = ctx->dstate;
     V.L = static_cast<LoopState*>(ctx->dloop);
     V.ctl = reinterpret_cast<LoopCtl*>(static_cast<char*>(ctx->dloop) + ls);
@@ -1132,12 +1257,12 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     const int64_t units = cdiv(gb[1], 32) + gb[4] - gb[1];
     const unsigned threads = units <= static_cast<int64_t>(sms) * 16 ? 512 : kLoopThreads;
     const int64_t want = std::max<int64_t>(1, std::min<int64_t>(sms, cdiv(units, threads / 32)));
-    const int cl = largest_cluster(ctx->device, smem);     // also sets the kernel's attributes, so always asked
+    const int cl = start ? largest_cluster<false>(ctx->device, smem) : largest_cluster<true>(ctx->device, smem);   // also sets the kernel's attributes, so always asked
     const bool cluster = want > 1 && want <= cl;
     const unsigned grid = static_cast<unsigned>(want);
     V.cluster = cluster ? 1 : 0;
     void* args[] = {&V};
-    const void* kernel = reinterpret_cast<const void*>(k_round_loop);
+    const void* kernel = start ? reinterpret_cast<const void*>(k_round_loop<false>) : reinterpret_cast<const void*>(k_round_loop<true>);
     if (grid == 1 || cluster) {
         cudaLaunchConfig_t cfg = cluster_config(grid, threads, smem);
         cudaLaunchAttribute attr = cluster_attribute(grid);

@@ -233,3 +233,20 @@ def test_first_round_on_both_sides_of_its_line(B, n):
     g = dict(n=n, src=np.repeat(np.arange(n), d).astype(np.int32), dst=rng.integers(0, n, n * d).astype(np.int32),
              elabel=rng.integers(0, 2, n * d).astype(np.int32), vlabel=rng.integers(0, 2, n).astype(np.int32))
     check(B, g, [1, 2])
+
+
+@pytest.mark.parametrize("bits", [6, 64])
+@pytest.mark.parametrize("degree", [3, 14, 60])
+@pytest.mark.parametrize("tails", [1, 40])
+def test_rounds_that_keep_small_blocks(B, tails, degree, bits):
+    """Triplets with equal rows stay blocks of three from the first rounds on, while paths beside them split one
+    vertex each off a block for 30 rounds more; a wide row makes the loop start after a round of the single classes,
+    where such rounds compare with the blocks first."""
+    g = rows_graph(3000, degree, seed=degree + tails)
+    n, length = g["n"], 30
+    v = np.arange(tails * length)
+    v = v[v % length != length - 1] + n
+    path = dict(src=v, dst=v + 1, elabel=np.zeros(len(v)))
+    g = dict(n=n + tails * length, vlabel=np.append(g["vlabel"], np.zeros(tails * length, np.int32)),
+             **{k: np.concatenate([g[k], path[k]]).astype(np.int32) for k in path})
+    check(B, with_hub(g, 300), [2, 5, 29, oracle.FIXPOINT], options=B.default_options(hash_bits=bits))
