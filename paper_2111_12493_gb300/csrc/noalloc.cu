@@ -191,28 +191,37 @@ struct RoundShared {
     unsigned blocks;
 };
 
-// The items are dealt to the CTAs one at a time, the CTAs turned from round to round
-// so that no period of the ids lands on one of them: a CTA's t-th item. Its warps
-// take turns at them (item t is lane t / warps of warp t % warps). With consecutive
-// items a CTA's and a warp's, wide rows that lie side by side (ids by degree) were
-// one CTA's or one warp's, one after the other: 20 rows of 8000 edges first among 10k
-// vertices took 626 us and take 95, 500 of 300 edges 232 and 71.
-__device__ __forceinline__ int64_t dealt_item(int64_t t) {
-    return t * gridDim.x + (blockIdx.x + t * 61) % gridDim.x;
+// The items are dealt to the CTAs in units of 1 << shift consecutive ones, the CTAs
+// turned from round to round so that no period of the ids lands on one of them: a
+// CTA's t-th item. Its warps take turns at the units too (my_item). With consecutive
+// items a CTA's and a warp's, wide rows that lie side by side (ids by degree) were one
+// CTA's or one warp's, one after the other: 20 rows of 8000 edges first among 10k
+// vertices took 626 us and take 95, 500 of 300 edges 232 and 71. From 96 items a CTA
+// on a unit has four, which keep the short rows' loads together: 65k vertices of four
+// edges and two labels 49 us one at a time, 43 in fours (and the 20 rows 177).
+__device__ __forceinline__ int64_t dealt_item(int64_t t, int shift) {
+    const int64_t u = t >> shift;
+    return ((u * gridDim.x + (blockIdx.x + u * 61) % gridDim.x) << shift) + (t & ((1 << shift) - 1));
 }
+
+__device__ __forceinline__ int my_item(int warp, int warps, int lane, int shift) {
+    return ((((lane >> shift) * warps) + warp) << shift) + (lane & ((1 << shift) - 1));
+}
+
+int item_shift(int per_cta) { return per_cta >= 96 ? 2 : 0; }
 
 // Pass 1. A CTA takes `per_cta` vertices at a time, one a lane.
 template <int LANE, int THREADS>
-__global__ void __launch_bounds__(THREADS) k_noalloc_sign(const RoundView V, int per_cta) {
+__global__ void __launch_bounds__(THREADS) k_noalloc_sign(const RoundView V, int per_cta, int shift) {
     extern __shared__ unsigned long long sets[];
     __shared__ RoundShared sh;
     const int warp = static_cast<int>(threadIdx.x >> 5), warps = static_cast<int>(blockDim.x >> 5);
     const int lane = static_cast<int>(lane_id());
-    const int mine = lane * warps + warp;                   // of the CTA's items
+    const int mine = my_item(warp, warps, lane, shift);     // of the CTA's items
     if (threadIdx.x == 0) sh.listed = 0u;
     __syncthreads();
     for (int64_t t0 = 0; t0 * gridDim.x < V.n; t0 += per_cta) {
-        const int64_t i = dealt_item(t0 + mine);
+        const int64_t i = dealt_item(t0 + mine, shift);
         const int32_t v = static_cast<int32_t>(i);
         int32_t own = 0;
         int64_t b = 0;
@@ -303,18 +312,19 @@ __device__ __forceinline__ bool group_same(const unsigned long long* a, const un
 // list of the next collision level. Does nothing when pass 1 refused the input.
 template <int LANE, int THREADS>
 __global__ void __launch_bounds__(THREADS) k_noalloc_verify(const RoundView V, const int32_t* __restrict__ list,
-                                                            int32_t count, int per_cta, int32_t* __restrict__ next) {
+                                                            int32_t count, int per_cta, int shift,
+                                                            int32_t* __restrict__ next) {
     extern __shared__ unsigned long long sets[];
     __shared__ RoundShared sh;
     if (*reinterpret_cast<volatile unsigned*>(&V.st->error) != 0u) return;   // the same for the whole grid: only pass 1 sets it
     const int warp = static_cast<int>(threadIdx.x >> 5);
     const int lane = static_cast<int>(lane_id());
     const int warps = static_cast<int>(blockDim.x >> 5);
-    const int mine = lane * warps + warp;                   // of the CTA's items
+    const int mine = my_item(warp, warps, lane, shift);     // of the CTA's items
     if (threadIdx.x == 0) sh.listed = sh.blocks = 0u;
     __syncthreads();
     for (int64_t t0 = 0; t0 * gridDim.x < count; t0 += per_cta) {
-        const int64_t i = dealt_item(t0 + mine);
+        const int64_t i = dealt_item(t0 + mine, shift);
         int32_t v = -1, r = -1;
         int c = -1;                                     // size of the sets to compare
         bool own = false, push = false;
@@ -526,18 +536,21 @@ extern "C" bisim_status bisim_refine_round_noalloc(int32_t n_vertices, int64_t n
     // small CTAs while they are enough, so that a short list still meets every SM
     const unsigned threads = long_rows ? 1024 : n <= sms * 128 ? 128 : 512;
     // the vertices dealt evenly to the SMs, as far as a CTA has lanes for them
-    const auto per_cta = [&](int32_t count) { return std::min<int32_t>((count + sms - 1) / sms, static_cast<int32_t>(threads)); };
+    const auto per_cta = [&](int32_t count) {
+        const int32_t even = (count + sms - 1) / sms, unit = 1 << item_shift(even);
+        return std::min<int32_t>((even + unit - 1) / unit * unit, static_cast<int32_t>(threads));
+    };
     const auto grid = [&](int32_t count) { return std::min<unsigned>((count + per_cta(count) - 1) / per_cta(count), sms); };
     const auto verify = [&](const int32_t* from, int32_t count, int32_t* next) {
-        if (long_rows) k_noalloc_verify<8, 1024><<<grid(count), threads, kRoundSmem, s>>>(V, from, count, per_cta(count), next);
-        else k_noalloc_verify<32, 512><<<grid(count), threads, kRoundSmem, s>>>(V, from, count, per_cta(count), next);
+        if (long_rows) k_noalloc_verify<8, 1024><<<grid(count), threads, kRoundSmem, s>>>(V, from, count, per_cta(count), item_shift(per_cta(count)), next);
+        else k_noalloc_verify<32, 512><<<grid(count), threads, kRoundSmem, s>>>(V, from, count, per_cta(count), item_shift(per_cta(count)), next);
     };
     BISIM_SITE(site_sign, "noalloc_sign");
     BISIM_SITE(site_verify, "noalloc_verify");
     {
         Launch L(site_sign, s, n, m, 28.0 * n + 20.0 * m);
-        if (long_rows) k_noalloc_sign<8, 1024><<<grid(n), threads, kRoundSmem, s>>>(V, per_cta(n));
-        else k_noalloc_sign<32, 512><<<grid(n), threads, kRoundSmem, s>>>(V, per_cta(n));
+        if (long_rows) k_noalloc_sign<8, 1024><<<grid(n), threads, kRoundSmem, s>>>(V, per_cta(n), item_shift(per_cta(n)));
+        else k_noalloc_sign<32, 512><<<grid(n), threads, kRoundSmem, s>>>(V, per_cta(n), item_shift(per_cta(n)));
     }
     {
         Launch L(site_verify, s, n, m, 48.0 * n + 16.0 * m);

@@ -247,7 +247,7 @@ def test_noalloc_rejects_memory_of_another_device(B):
         _rejected(B, g["n"], d_rp, d_col, d_lab, vl, out, match="current device")
 
 
-@pytest.mark.parametrize("n,wide,degree", [(153, 4, 300), (10_000, 20, 8000), (19_457, 300, 600), (60_000, 800, 1000)])
+@pytest.mark.parametrize("n,wide,degree", [(153, 4, 300), (10_000, 20, 8000), (19_457, 300, 600), (14_441, 300, 600), (60_000, 800, 1000)])
 def test_noalloc_wide_rows_side_by_side(B, n, wide, degree):
     """Rows that take a whole CTA, at the first ids and spread over all: the same partitions as the oracle's, and
     side by side they are not one CTA's work (up to eight times the time of the spread ones, when they were)."""
