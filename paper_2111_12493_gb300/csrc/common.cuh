@@ -465,11 +465,11 @@ bool device_accessible(const void* p);
 // Lets `kernel` be launched with `bytes` of dynamic shared memory on the current
 // device (more than 48 KB have to be allowed, on every device by itself).
 cudaError_t allow_smem(const void* kernel, size_t bytes);
-// 256-byte pinned host blocks from process-lifetime slabs (nullptr if none can be had).
 // Forks from `s`. A branch without a stream (none could be had) stands for `s` itself.
 // After the join (which has to come, on the same stream) the branch is gone.
 Branch branch_fork(int device, cudaStream_t s);
 void branch_join(int device, Branch* b, cudaStream_t s);
+// 256-byte pinned host blocks from process-lifetime slabs (nullptr if none can be had).
 void* pinned_take();
 void pinned_give(void* p);
 

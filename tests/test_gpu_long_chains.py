@@ -9,10 +9,10 @@ so the fixpoint needs as many rounds as the path is long. The closed form
     every vertex closer to the sink is alone, so there are min(i+1, m+1)
     blocks, and the fixpoint is reached at r = m.
 
-These tests run that form at m = 1000 through the captured device-side round
-loop (table epochs wrap every 15 rounds, the active list shrinks by one
-vertex per round) and through host-driven rounds, and many identical paths
-(every vertex active in every round) against the oracle.
+These tests run that form at m = 1000 through the cooperative round loop, the
+captured graph (table epochs wrap every 15 rounds, the active list shrinks by
+one vertex per round) and host-driven rounds, and many identical paths (every
+vertex active in every round) against the oracle.
 """
 
 import numpy as np
@@ -53,25 +53,43 @@ def _closed_form(m, k):
     return np.where(dist >= k, 0, i).astype(np.int32)
 
 
-@pytest.mark.parametrize("eager", [False, True], ids=["captured-loop", "eager"])
-def test_path_of_1001_vertices_needs_exactly_1000_rounds(B, eager):
+def _with_wide_twins(g):
+    """Two more vertices of another label with 300 parallel edges each to the path's sink: one block of two in every
+    round, whose wide rows keep the rounds in the captured graph."""
+    n = g["n"]
+    twins = np.repeat([n, n + 1], 300).astype(np.int32)
+    return dict(n=n + 2, src=np.append(g["src"], twins), dst=np.append(g["dst"], np.full(600, n - 1, np.int32)),
+                elabel=np.append(g["elabel"], np.zeros(600, np.int32)), vlabel=np.append(g["vlabel"], [1, 1]).astype(np.int32))
+
+
+@pytest.mark.parametrize("route", ["cooperative-loop", "captured-graph", "eager"])
+def test_path_of_1001_vertices_needs_exactly_1000_rounds(B, route):
     m = 1000
     g = _paths(1, m + 1)
-    flags = B.FLAG_EAGER if eager else 0
+    flags = B.FLAG_EAGER if route == "eager" else 0
+    twins = 0
+    if route == "captured-graph":
+        g = _with_wide_twins(g)
+        twins = 1
+
+    def path_part(P):
+        assert not twins or (P[m + 1:] == m + 1).all()
+        return P[:m + 1]
+
     ctx = B.summarize_init_coo(g["n"], _dev(g["src"]), _dev(g["dst"]), _dev(g["elabel"]), _dev(g["vlabel"]),
                                options=B.default_options(flags=flags))
     rounds, blocks = B.bisim_iterate(ctx, B.FIXPOINT, 5000)
-    assert rounds == m and blocks == m + 1
+    assert rounds == m and blocks == m + 1 + twins
     assert B.bisim_get_stats(ctx)["rounds_executed"] == m + 1
-    assert np.array_equal(B.get_partition(ctx).cpu().numpy(), _closed_form(m, m))
+    assert np.array_equal(path_part(B.get_partition(ctx).cpu().numpy()), _closed_form(m, m))
     # sampled rounds, across epoch wraps (every 15) and past the fixpoint
     for k in (1, 2, 14, 15, 16, 17, 30, 31, 499, 998, 999, 1000, 1001, 1500):
         rounds, blocks = B.bisim_iterate(ctx, k, 0)
-        assert rounds == k and blocks == min(k + 1, m + 1), (k, blocks)
-        assert np.array_equal(B.get_partition(ctx).cpu().numpy(), _closed_form(m, k)), k
+        assert rounds == k and blocks == min(k + 1, m + 1) + twins, (k, blocks)
+        assert np.array_equal(path_part(B.get_partition(ctx).cpu().numpy()), _closed_form(m, k)), k
     # the fixpoint with a cap below it stops at the cap
     rounds, blocks = B.bisim_iterate(ctx, B.FIXPOINT, 300)
-    assert rounds == 300 and blocks == 301
+    assert rounds == 300 and blocks == 301 + twins
     B.summarize_destroy(ctx)
 
 
