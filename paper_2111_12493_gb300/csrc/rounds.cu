@@ -11,9 +11,9 @@
 //   B  every entry is confirmed by an exact comparison, inside the thread for rows of
 //      at most eight edges (the pairs with longer rows are shared out to the CTA's
 //      warps afterwards), against the smallest vertex of its slot of the signature
-//      table, which phase A filled; in a round that is likely to keep many small
-//      blocks (see keeps_blocks) against the smallest vertex of its present block,
-//      and those that differ from it enter the table instead
+//      table, which phase A filled; in a round that is likely to keep most blocks
+//      (see keeps_blocks) against the smallest vertex of its present block, and those
+//      that differ from it enter the table instead
 //   C  (only then, and only them) and are confirmed against their slots
 //
 // The list is cut among the CTAs at the start and each keeps its part to the end
@@ -62,7 +62,8 @@ constexpr uint8_t kOwnerAsks = 5;         // ... and this round those that stay 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // What one barrier carries: the CTAs' listed (high half) and owned entries
-// added up, and the union of their kAny* flags.
+// added up, the number of CTAs that raise each of three flags (8 bits each), and
+// above those the CTAs' moved entries.
 struct __align__(16) BarrierSum {
     unsigned long long counts;
     unsigned long long flags;
@@ -134,9 +135,10 @@ struct Shared {
     unsigned owned;                           // entries that are their block's id
     unsigned wide;                            // entries on the wide list
     unsigned split;                           // and on the split list
+    unsigned moved;                           // members that are in another block now
     unsigned error;                           // kErr* bits
     unsigned flags;                           // barrier result: kAny* of all CTAs
-    unsigned total[2];                        // barrier result: listed, owned
+    unsigned total[3];                        // barrier result: listed, owned, moved
     int ok;
 };
 
@@ -214,24 +216,28 @@ __device__ bool grid_barrier(const LoopView& V, unsigned k, Shared& sh) {
     return arrive_and_wait(V, k, sh);
 }
 
-// The same with the sum of all CTAs' counts and the union of their flags, in
+// The same with the sums of all CTAs' counts and the union of their flags, in
 // sh.total and sh.flags. Three sums rotate: that of barrier k + 1 is cleared
 // before anyone leaves barrier k, and was last read before anyone reached k - 1.
 __device__ bool grid_barrier(const LoopView& V, unsigned k, unsigned flags, unsigned listed, unsigned owned,
-                             Shared& sh) {
+                             unsigned moved, Shared& sh) {
     LoopCopy* c = &V.ctl->copy[V.copy];
     __syncthreads();
     if (threadIdx.x == 0) {
         if (blockIdx.x == 0) c->sum[(k + 1) % 3] = BarrierSum{0ull, 0ull};
         atomicAdd(&c->sum[k % 3].counts, (static_cast<unsigned long long>(listed) << 32) | owned);
-        if (flags) atomicOr(&c->sum[k % 3].flags, static_cast<unsigned long long>(flags));
+        const unsigned long long raised = (flags & kAnySplit ? 1ull : 0ull) | (flags & kAnyUnresolved ? 1ull << 8 : 0ull) |
+                                          (flags & kAnyError ? 1ull << 16 : 0ull) | static_cast<unsigned long long>(moved) << 24;
+        if (raised) atomicAdd(&c->sum[k % 3].flags, raised);
     }
     const bool fine = arrive_and_wait(V, k, sh);
     if (threadIdx.x == 0) {
         const ulonglong2 t = __ldcg(reinterpret_cast<const ulonglong2*>(&c->sum[k % 3]));
         sh.total[0] = static_cast<unsigned>(t.x >> 32);
         sh.total[1] = static_cast<unsigned>(t.x);
-        sh.flags = static_cast<unsigned>(t.y);
+        sh.total[2] = static_cast<unsigned>(t.y >> 24);
+        sh.flags = (t.y & 0xffull ? kAnySplit : 0u) | (t.y & 0xff00ull ? kAnyUnresolved : 0u) |
+                   (t.y & 0xff0000ull ? kAnyError : 0u);
     }
     __syncthreads();
     return fine;
@@ -748,11 +754,11 @@ __device__ __forceinline__ void add_owned(unsigned owned, Shared& sh) {
 
 // Confirms the CTA's entries pos_of(i), i < total, against their table slots'
 // smallest vertices. (Two entries a thread at once: no faster.)
-template <class F>
+template <bool KEEPS, class F>
 __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, const List& l, unsigned total,
                                              const F& pos_of, Shared& sh) {
     const unsigned lane = lane_id();
-    unsigned owned = 0;
+    unsigned owned = 0, moved = 0;
     for (unsigned b = threadIdx.x - lane; b < total; b += blockDim.x) {
         Pair p{-1, -1, -1, -1};
         bool test = false, push = false;
@@ -776,11 +782,16 @@ __device__ __forceinline__ void verify_slots(const LoopView& V, const Round& R, 
                 V.own[p.pos] = kMember;
                 test = a.z == c.z && a.w == c.w;
                 push = !test;
+                if (KEEPS && a.w != p.r) ++moved;
             }
         }
         confirm(V, R, l, p, test, true, push, a, c, sh);
     }
     add_owned(owned, sh);
+    if (KEEPS) {
+        moved = __reduce_add_sync(0xffffffffu, moved);
+        if (lane == 0 && moved) atomicAdd(&sh.moved, moved);
+    }
 }
 
 // Phase B of a round that is likely to keep its blocks: every entry against the
@@ -974,24 +985,31 @@ __device__ bool hand_back(const LoopView& V, const List& l, const Round& R, int 
     return true;
 }
 
-// Whether the next round is likely to keep most blocks, and those small: the last one
-// made few new ones of its listed entries, and its blocks had at most kKeepSize of them
-// on average. Then comparing with them saves an insert at a random slot per entry, and
-// entries cannot leave without new blocks in proportion. Large blocks are entered once
-// per CTA and warp, which costs less than the comparison, and can lose half their entries
-// for one new block. us to the fixpoint with no such round, with the first condition
-// alone, with both: power law 1.4M / 4M 613 / 563 / 565, 1M / 5M 512 / 460 / 467, 4M /
-// 16M 1,220 / 1,145 / 1,147; beside a wide row, paths of 300k vertices with 3,000 more
-// edges 332 / 503 / 334, two edges a vertex with two labels, 200k, 248 / 426 / 250, 600
-// rounds of paths on 300k 13,260 / 15,600 / 13,560.
+// Whether the next round is likely to keep most blocks. Then comparing with them saves
+// an insert at a random or a popular slot per entry; what has to pay for it is the third
+// phase, and the entries that leave, one by one. Two signs of it, from the last round:
+// few new blocks, and blocks of at most kKeepSize listed entries on average (entries
+// cannot leave small blocks without new ones in proportion); or few entries in another
+// block than before on a long list (13 us for the phase and 5 ns for an entry that
+// leaves, against 50 ps an insert). us to the fixpoint with no such round, with any
+// round that made few new blocks, with these two: power law 1.4M / 4M 613 / 561 / 562,
+// 4M / 16M 1,220 / 1,147 / 1,158, with a label filter 500k / 1.5M 494 / 413 / 423 and 3M /
+// 9M 1,267 / 1,130 / 1,137; beside a wide row, paths of 300k vertices with 3,000 more edges
+// 330 / 503 / 332, two edges a vertex with two labels, 200k, 246 / 400 / 248, 600 rounds
+// of paths on 300k 13,270 / 15,920 / 13,740.
 constexpr int64_t kKeepSize = 32;
-__device__ __forceinline__ bool keeps_blocks(int64_t grown, int64_t owned, int64_t listed) {
-    return grown * 32 < listed && listed <= owned * kKeepSize;
+constexpr int64_t kKeepListed = 210000;
+constexpr int64_t kKeepMoved = 200;
+__device__ __forceinline__ bool keeps_blocks(int64_t grown, int64_t moved, int64_t owned, int64_t listed) {
+    return (grown * 32 < listed && listed <= owned * kKeepSize) || kKeepListed + kKeepMoved * (moved + grown) < listed;
 }
 
-// KEEPS: with rounds that keep_or_split begins. For loops after a round of the single
-// classes; those from P_0 on gain nothing by them (uniform graphs and chains 0 to 3%),
-// and the rest of the kernel is 2% to 3% slower with them in it.
+// KEEPS: with rounds that keep_or_split begins. The rest of the kernel is 2% to 3%
+// slower with them in it, so loops from P_0 on have them only where many vertices have
+// no edges and stay in large blocks: a fourth of them, on a list long enough (chains
+// with two extra edges a vertex behind a label filter, 56% without edges, 500k 431 to
+// 380 us, 3M 1,579 to 1,482; unfiltered ones 186 to 190 and 697 to 717, uniform graphs of
+// mean five 178 to 182 and 713 to 730).
 template <bool KEEPS>
 __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V) {
     extern __shared__ unsigned long long sets[];           // a set per warp, when warp-class rows exist
@@ -1045,7 +1063,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
         R.insert = !KEEPS || !keep;
         for (int i = threadIdx.x; i < kSeenSlots; i += blockDim.x) sh.seen[i] = -1;
         if (threadIdx.x < kLoopGroups) sh.next_cnt[threadIdx.x] = 0u;
-        if (threadIdx.x == 0) sh.owned = sh.wide = sh.split = 0u;
+        if (threadIdx.x == 0) sh.owned = sh.wide = sh.split = sh.moved = 0u;
         __syncthreads();
         phase_a<KEEPS>(V, R, l, sh, sets);
         if (!(fine = grid_barrier(V, ++bar, sh))) break;
@@ -1059,7 +1077,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
             nbuf ^= 1;
         }
         if (KEEPS && keep) keep_or_split(V, R, l, sh);
-        else verify_slots(V, R, l, list_size(l), [&](unsigned i) { return entry_of(l, i); }, sh);
+        else verify_slots<KEEPS>(V, R, l, list_size(l), [&](unsigned i) { return entry_of(l, i); }, sh);
         __syncthreads();
         for (bool against_block = KEEPS && keep;; against_block = false) {
             if (sh.wide) confirm_wide(V, R, l, KEEPS && against_block, sh, sets);
@@ -1068,17 +1086,17 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_round_loop(const LoopView V
             // unresolved entries are rare: every CTA looks at the counter
             const unsigned flags = (sh.split ? kAnySplit : 0u) | (sh.error ? kAnyError : 0u) |
                                    (__ldcg(&V.ctl->copy[V.copy].unresolved) ? kAnyUnresolved : 0u);
-            if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh))) break;
+            if (!(fine = grid_barrier(V, ++bar, flags, list_size(l), sh.owned, sh.moved + sh.split, sh))) break;
             if (!KEEPS || !against_block || !(sh.flags & kAnySplit)) break;
             if (threadIdx.x == 0) sh.wide = 0u;
             __syncthreads();
-            verify_slots(V, R, l, sh.split, [&](unsigned i) { return V.split[place_of(V, l, i)]; }, sh);
+            verify_slots<false>(V, R, l, sh.split, [&](unsigned i) { return V.split[place_of(V, l, i)]; }, sh);
             __syncthreads();
         }
         if (!fine) break;
         const unsigned listed = sh.total[0];
         const unsigned long long blocks = static_cast<unsigned long long>(V.n_live - listed) + sh.total[1];
-        keep = keeps_blocks(static_cast<int64_t>(blocks - S.prev_blocks), sh.total[1], listed);
+        if (KEEPS) keep = keeps_blocks(static_cast<int64_t>(blocks - S.prev_blocks), sh.total[2], sh.total[1], listed);
         loop_advance(S, blocks, sh.flags & kAnyUnresolved, sh.flags & kAnyError);
         if (S.stop == kStopDone) {
             if (out != 0)                                  // the result belongs in P[0]
@@ -1257,12 +1275,13 @@ bisim_status round_loop(bisim_ctx* ctx, cudaStream_t s, bool start, const LoopSt
     const int64_t units = cdiv(gb[1], 32) + gb[4] - gb[1];
     const unsigned threads = units <= static_cast<int64_t>(sms) * 16 ? 512 : kLoopThreads;
     const int64_t want = std::max<int64_t>(1, std::min<int64_t>(sms, cdiv(units, threads / 32)));
-    const int cl = start ? largest_cluster<false>(ctx->device, smem) : largest_cluster<true>(ctx->device, smem);   // also sets the kernel's attributes, so always asked
+    const bool keeps = !start || (V.n_live > kKeepListed && 4 * (db[1] - db[0]) >= V.n_live);
+    const int cl = keeps ? largest_cluster<true>(ctx->device, smem) : largest_cluster<false>(ctx->device, smem);   // also sets the kernel's attributes, so always asked
     const bool cluster = want > 1 && want <= cl;
     const unsigned grid = static_cast<unsigned>(want);
     V.cluster = cluster ? 1 : 0;
     void* args[] = {&V};
-    const void* kernel = start ? reinterpret_cast<const void*>(k_round_loop<false>) : reinterpret_cast<const void*>(k_round_loop<true>);
+    const void* kernel = keeps ? reinterpret_cast<const void*>(k_round_loop<true>) : reinterpret_cast<const void*>(k_round_loop<false>);
     if (grid == 1 || cluster) {
         cudaLaunchConfig_t cfg = cluster_config(grid, threads, smem);
         cudaLaunchAttribute attr = cluster_attribute(grid);

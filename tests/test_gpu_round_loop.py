@@ -250,3 +250,14 @@ def test_rounds_that_keep_small_blocks(B, tails, degree, bits):
     g = dict(n=n + tails * length, vlabel=np.append(g["vlabel"], np.zeros(tails * length, np.int32)),
              **{k: np.concatenate([g[k], path[k]]).astype(np.int32) for k in path})
     check(B, with_hub(g, 300), [2, 5, 29, oracle.FIXPOINT], options=B.default_options(hash_bits=bits))
+
+
+@pytest.mark.parametrize("bits", [10, 64])
+def test_rounds_that_keep_large_blocks(B, bits):
+    """20 paths of 11,000 vertices: 20 entries of a long list leave the large block in every round; a wide row makes
+    the loop start after a round of the single classes, where such rounds compare with the blocks first."""
+    g = with_hub(path_graph([11_000] * 20, marked=(7, 30_000)), 300)
+    check(B, g, [3, 24], options=B.default_options(hash_bits=bits))
+    # from P_0 on beside as many vertices without edges
+    g = path_graph([11_000] * 20 + [1] * 80_000, marked=(7, 30_000, 250_000))
+    check(B, g, [3, 24], options=B.default_options(hash_bits=bits))
